@@ -139,23 +139,28 @@ __device__ __forceinline__ void slide(uint32_t (&plane)[NP][WPL], int np, const 
     }
 }
 
-// One step of the look-ahead rule: `want` of the candidates at most may move in; the best take the free capacity, the
-// next ones replace residents of lower key, worst first. H is updated; I units came in, `swaps` of them for a resident.
-// The number of swaps is the largest m for which the (insf + m)-th best candidate's key exceeds the m-th lowest
-// resident key, i.e. for which some threshold t has at least insf + m candidates with key >= t and m residents with
-// key < t: the maximum over t of min(C(t) - insf, R(t)), C falling and R rising in t, found where they cross.
+// One step of the look-ahead rule: at most `want` of the candidates move in, the best first; they take the free
+// capacity, then the next ones replace residents of lower key, lowest first. H is updated; I units came in, `swaps` of
+// them for a resident. kb = want less the free capacity bounds the swaps from one side, the keys from the other: m swaps
+// are possible iff some threshold t has insf + m candidates with key >= t and m residents with key < t, so their number
+// is the maximum over t of min(C(t) - insf, R(t)), C falling and R rising in t, reached where the two cross.
+//   quota: the want-th best candidate and the kb-th lowest resident, both descents side by side; right when the first
+//          key is above the second.
+//   cross: the crossing, one descent over both sets; right when it gives at most kb swaps, and then its threshold cuts
+//          both sets: candidates above it and residents below it move, of those at it as many as are still to move.
+// Either is one count per plane. `limited` remembers which was right at the step before and goes first.
 template <int WPL, int NP, bool MULTI>
 __device__ __forceinline__ void exchange_units(const uint32_t (&plane)[NP][WPL], int np, const uint32_t (&cand)[WPL],
                                                uint32_t want, uint32_t free_slots, uint32_t (&H)[WPL],
-                                               CtaSum<MULTI>& sum, uint32_t& I, uint32_t& swaps)
+                                               CtaSum<MULTI>& sum, bool& limited, uint32_t& I, uint32_t& swaps)
 {
     const uint32_t insf = min(want, free_slots), kb = want - insf;
-    swaps = 0;
-    uint32_t mc[WPL], mr[WPL];
-    if (kb) {                                            // warp- and CTA-uniform
+    uint32_t mc[WPL], mr[WPL], in[WPL], out[WPL], needC, needR;   // ties at the thresholds, units beyond them
+    for (bool quota = limited || kb == 0;; quota = !quota) {      // two passes at most
 #pragma unroll
-        for (int j = 0; j < WPL; ++j) { mc[j] = cand[j]; mr[j] = H[j]; }
-        uint32_t above = 0, below = 0;                   // candidates above, residents below the keys still open
+        for (int j = 0; j < WPL; ++j) { mc[j] = cand[j]; mr[j] = H[j]; in[j] = 0u; out[j] = 0u; }
+        uint32_t above = 0, below = 0, keyC = 0, keyR = 0;
+        needC = want; needR = kb;
 #pragma unroll
         for (int b = NP - 1; b >= 0; --b) {
             if (b >= np) continue;
@@ -163,41 +168,40 @@ __device__ __forceinline__ void exchange_units(const uint32_t (&plane)[NP][WPL],
 #pragma unroll
             for (int j = 0; j < WPL; ++j) c += (__popc(mc[j] & plane[b][j]) << 16) + __popc(mr[j] & ~plane[b][j]);
             c = sum(c);
-            const uint32_t hi = above + (c >> 16), lo = below + (c & 0xFFFFu);   // C and R at the threshold with bit b set
-            const bool up = hi >= insf + lo;
-            if (up) below = lo; else above = hi;
-            const uint32_t flip = up ? 0u : 0xFFFFFFFFu;
+            const uint32_t cc = c >> 16, cr = c & 0xFFFFu;
+            uint32_t tc, tr;                              // all ones: go on among the set bits (C), among the clear ones (R)
+            if (quota) {
+                tc = needC <= cc ? 0xFFFFFFFFu : 0u;
+                tr = needR <= cr ? 0xFFFFFFFFu : 0u;
+                needC -= cc & ~tc; needR -= cr & ~tr;
+                keyC |= tc & (1u << b); keyR |= ~tr & (1u << b);
+            } else {
+                tc = above + cc >= insf + below + cr ? 0xFFFFFFFFu : 0u;
+                tr = ~tc;
+                above += cc & ~tc; below += cr & tc;
+            }
 #pragma unroll
-            for (int j = 0; j < WPL; ++j) { mc[j] &= plane[b][j] ^ flip; mr[j] &= plane[b][j] ^ flip; }
+            for (int j = 0; j < WPL; ++j) {
+                const uint32_t p = plane[b][j];
+                in[j] |= mc[j] & p & ~tc;
+                mc[j] &= ~(p ^ tc);
+                out[j] |= mr[j] & ~p & ~tr;
+                mr[j] &= p ^ tr;
+            }
         }
-        swaps = min(kb, max(below, above > insf ? above - insf : 0u));
+        if (quota) {
+            swaps = kb;
+            if (kb == 0 || keyC > keyR) break;
+            limited = false;
+        } else {
+            swaps = max(below, above > insf ? above - insf : 0u);
+            needC = insf + swaps - above; needR = swaps - below;
+            if (swaps <= kb) break;
+            limited = true;
+        }
     }
     I = insf + swaps;
     if (!I) return;
-    // the I best candidates and the `swaps` worst residents: sets beyond the thresholds, ties at them
-    uint32_t in[WPL], out[WPL], needC = I, needR = swaps;
-#pragma unroll
-    for (int j = 0; j < WPL; ++j) { mc[j] = cand[j]; mr[j] = H[j]; in[j] = 0u; out[j] = 0u; }
-#pragma unroll
-    for (int b = NP - 1; b >= 0; --b) {
-        if (b >= np) continue;
-        uint32_t c = 0;
-#pragma unroll
-        for (int j = 0; j < WPL; ++j) c += (__popc(mc[j] & plane[b][j]) << 16) + __popc(mr[j] & ~plane[b][j]);
-        c = sum(c);
-        const uint32_t cc = c >> 16, cr = c & 0xFFFFu;
-        const uint32_t tc = needC <= cc ? 0xFFFFFFFFu : 0u, tr = needR <= cr ? 0xFFFFFFFFu : 0u;
-        if (!tc) needC -= cc;
-        if (!tr) needR -= cr;
-#pragma unroll
-        for (int j = 0; j < WPL; ++j) {
-            const uint32_t p = plane[b][j];
-            in[j] |= mc[j] & p & ~tc;
-            mc[j] &= ~(p ^ tc);
-            out[j] |= mr[j] & ~p & ~tr;
-            mr[j] &= p ^ tr;
-        }
-    }
     const uint32_t bf = sum.before((popcn(mc) << 16) + popcn(mr));
     first_bits(mc, bf >> 16, needC);
     first_bits(mr, bf & 0xFFFFu, needR);
@@ -259,6 +263,7 @@ lookahead_kernel(const uint32_t* __restrict__ A, const uint32_t* __restrict__ ro
             load_row(A + (size_t)t * W32, W32, w0, a);
             slide(plane, np, a, none);
         }
+    bool limited = permille < 1000;
     uint64_t total = 0;
     uint32_t mi = 0, mo = 0, hits = 0;                   // of the step before (its hits are reduced with the next step's count)
     uint32_t enter[WPL], leave[WPL] = {}, now[WPL];      // rows s + W - 1, s - 1 and s
@@ -288,7 +293,7 @@ lookahead_kernel(const uint32_t* __restrict__ A, const uint32_t* __restrict__ ro
         if (totals && s) total += step_cost(both & 0xFFFFu, mi, mo, __ldg(stepc + s - 1), K);
         const uint32_t want = nC * permille / 1000u;
         if (want) {
-            exchange_units(plane, np, cand, want, cap - nR, H, sum, I, swaps);
+            exchange_units(plane, np, cand, want, cap - nR, H, sum, limited, I, swaps);
             nR += I - swaps;
         }
         mi = s ? I : 0u; mo = s ? swaps : 0u;            // the migrations of step 0 are free
@@ -348,6 +353,7 @@ page_kernel(const uint32_t* __restrict__ planes, int np, uint32_t S, uint32_t EW
         for (int b = 0; b < kPagePlanes; ++b) load_row(planes + ((size_t)s * np + min(b, np - 1)) * EW32, b < np ? EW32 : 0u, w0, next[b]);
     };
     fetch(0);
+    bool limited = false;
     for (uint32_t s = 0; s < S; ++s) {
         uint32_t cand[WPL], I = 0, swaps = 0;
 #pragma unroll
@@ -360,7 +366,7 @@ page_kernel(const uint32_t* __restrict__ planes, int np, uint32_t S, uint32_t EW
         fetch(min(s + 1, S - 1));
         const uint32_t nC = sum(popcn(cand));
         if (nC) {
-            exchange_units(plane, np, cand, nC, cap - nR, H, sum, I, swaps);
+            exchange_units(plane, np, cand, nC, cap - nR, H, sum, limited, I, swaps);
             nR += I - swaps;
         }
         store_row(pages + (size_t)s * EW32, EW32, w0, H);
@@ -385,7 +391,10 @@ page_expand_kernel(const uint32_t* __restrict__ pages, uint32_t page, uint32_t W
 
 // Reactive Scheduling (Section IV-A): promote on miss, evict the least recently used. One CTA walks the steps; row
 // s + 1 follows from row s and the accesses of step s. Keys are the times of last use (step + 1, 0 = never): hits and
-// promoted units get the step's, the evicted are the residents with the smallest (key, index).
+// promoted units get the step's, the evicted are the residents with the smallest (key, index). The smallest key among
+// the residents never falls, so the class of residents that hold it is kept as a set (`oldest`) and moves on to the next
+// key when it is used up: over a whole run no more advances than steps, where a search through the planes cost a
+// reduction per plane and step (4096 units x 512 steps: 0.69 ms with it).
 template <int WPL, bool MULTI>
 __global__ void __launch_bounds__(MULTI ? 32 * kPolicyMaxWarps : 32)
 reactive_kernel(const uint32_t* __restrict__ A, const uint32_t* __restrict__ row0, uint32_t S, uint32_t W32, uint32_t cap,
@@ -398,25 +407,28 @@ reactive_kernel(const uint32_t* __restrict__ A, const uint32_t* __restrict__ row
     }
     CtaSum<MULTI> sum{s_part, 0u};
     const uint32_t w0 = threadIdx.x * WPL;
-    uint32_t H[WPL], plane[kStampPlanes][WPL], a[WPL];
+    uint32_t H[WPL], plane[kStampPlanes][WPL], a[WPL], oldest[WPL];
     initial_row(row0, W32, w0, cap, H);
-    uint32_t nR = sum(popcn(H));
+    uint32_t nR = sum(popcn(H)), tau = 0;                // tau: the key of `oldest`
     store_row(out, W32, w0, H);
 #pragma unroll
-    for (int b = 0; b < kStampPlanes; ++b)
+    for (int j = 0; j < WPL; ++j) {
+        oldest[j] = H[j];
 #pragma unroll
-        for (int j = 0; j < WPL; ++j) plane[b][j] = 0u;
+        for (int b = 0; b < kStampPlanes; ++b) plane[b][j] = 0u;
+    }
     load_row(A, W32, w0, a);
     for (uint32_t s = 0; s + 1 < S; ++s) {
-        const int np = 32 - __clz(s + 1);                // planes of a stamp 0..s+1
+        const int np = 32 - __clz(s + 1);                // planes of a key 0..s+1
         uint32_t a2[WPL], miss[WPL];
         load_row(A + (size_t)(s + 1) * W32, W32, w0, a2);
 #pragma unroll
-        for (int j = 0; j < WPL; ++j) miss[j] = a[j] & ~H[j];
-        const uint32_t nM = sum(popcn(miss));
+        for (int j = 0; j < WPL; ++j) { miss[j] = a[j] & ~H[j]; oldest[j] &= ~a[j]; }
+        const uint32_t both = sum((popcn(miss) << 16) + popcn(oldest));
+        const uint32_t nM = both >> 16;
+        uint32_t n_old = both & 0xFFFFu;
         const uint32_t promoted = min(nM, cap), free_slots = cap - nR;
         if (promoted < nM) first_bits(miss, sum.before(popcn(miss)), promoted);   // CTA-uniform
-        const uint32_t evict = promoted > free_slots ? promoted - free_slots : 0u;
 #pragma unroll
         for (int b = 0; b < kStampPlanes; ++b) {
             if (b >= np) continue;
@@ -427,32 +439,39 @@ reactive_kernel(const uint32_t* __restrict__ A, const uint32_t* __restrict__ row
                 plane[b][j] = (plane[b][j] & ~used) | (v & used);
             }
         }
-        if (evict) {                                     // CTA-uniform
-            uint32_t mr[WPL], gone[WPL], need = evict;
-#pragma unroll
-            for (int j = 0; j < WPL; ++j) { mr[j] = H[j]; gone[j] = 0u; }
-#pragma unroll
-            for (int b = kStampPlanes - 1; b >= 0; --b) {
-                if (b >= np) continue;
-                uint32_t c = 0;
-#pragma unroll
-                for (int j = 0; j < WPL; ++j) c += __popc(mr[j] & ~plane[b][j]);
-                c = sum(c);
-                const uint32_t t = need <= c ? 0xFFFFFFFFu : 0u;
-                if (!t) need -= c;
-#pragma unroll
-                for (int j = 0; j < WPL; ++j) {
-                    gone[j] |= mr[j] & ~plane[b][j] & ~t;
-                    mr[j] &= plane[b][j] ^ t;
-                }
-            }
-            first_bits(mr, sum.before(popcn(mr)), need);
-#pragma unroll
-            for (int j = 0; j < WPL; ++j) H[j] &= ~(gone[j] | mr[j]);
-        }
+        uint32_t evict = promoted > free_slots ? promoted - free_slots : 0u;
         nR += promoted - evict;
+        while (evict > n_old) {                          // CTA-uniform; at most s + 1 keys exist, and nR >= evict units
+            evict -= n_old;
 #pragma unroll
-        for (int j = 0; j < WPL; ++j) { H[j] |= miss[j]; a[j] = a2[j]; }
+            for (int j = 0; j < WPL; ++j) H[j] &= ~oldest[j];
+            ++tau;
+#pragma unroll
+            for (int j = 0; j < WPL; ++j) {
+                uint32_t other = 0;
+#pragma unroll
+                for (int b = 0; b < kStampPlanes; ++b)
+                    if (b < np) other |= plane[b][j] ^ ((tau >> b) & 1u ? 0xFFFFFFFFu : 0u);
+                oldest[j] = H[j] & ~other;
+            }
+            n_old = sum(popcn(oldest));
+            if (tau > s + 1) break;                      // never reached: the keys of the residents end at s + 1
+        }
+        if (evict) {                                     // CTA-uniform
+            uint32_t gone[WPL];
+#pragma unroll
+            for (int j = 0; j < WPL; ++j) gone[j] = oldest[j];
+            first_bits(gone, sum.before(popcn(gone)), evict);
+#pragma unroll
+            for (int j = 0; j < WPL; ++j) { H[j] &= ~gone[j]; oldest[j] &= ~gone[j]; }
+        }
+#pragma unroll
+        for (int j = 0; j < WPL; ++j) {
+            H[j] |= miss[j]; a[j] = a2[j];
+        }
+        if (tau == s + 1)                                // the class of this very step: it grows by the promoted
+#pragma unroll
+            for (int j = 0; j < WPL; ++j) oldest[j] |= miss[j];
         store_row(out + (size_t)(s + 1) * W32, W32, w0, H);
     }
 }
