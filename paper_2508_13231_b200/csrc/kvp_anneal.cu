@@ -1,6 +1,6 @@
 // Annealing kernels. Two of them, chosen per job (see prepare()): the narrow chain kernel described here (one or two
-// warps per chain, one proposal per lane) and the wide one further down (one warp per chain, four proposals per lane,
-// most proposals settled by their placement bits alone).
+// warps per chain, batches of 32 proposals, every one evaluated in full) and the wide one in kvp_chain.cuh (one to four
+// warps per chain, batches of 128 or 256, most proposals settled by their placement bits or a bound alone).
 //
 // State of a chain: the schedule in time-packed form (for every unit a bit string over the steps), either
 // in shared memory (small problems) or in a private slice of global scratch (a plain copy of the initial schedule,
@@ -17,6 +17,7 @@
 #include <stdlib.h>
 #include <string.h>
 
+#include <algorithm>
 #include <type_traits>
 #include <vector>
 
@@ -27,6 +28,18 @@ namespace kvp {
 namespace {
 
 kvp_test_hooks g_hooks = {0u, 0u, 0u, 0u, 0u};   // kvp_set_test_hooks; read once per call
+
+// What an exchange round of neighbouring rungs needs (by pair of rungs).
+struct ExchangeArgs {
+    const uint32_t* always; const uint32_t* table; const uint32_t* shifts;
+    unsigned long long* counts;  // {tried, accepted}
+    uint32_t rungs, seed_lo, seed_hi;
+};
+
+// Byte offsets of the parts of a chain's shared memory (see chain_layout).
+struct ChainLayout {
+    uint32_t occ, full, lead, hb, have, work;
+};
 
 struct ChainParams {
     const uint32_t* Acol;        // [U][S32]
@@ -58,12 +71,11 @@ struct ChainParams {
     uint32_t* cow_out;           // wide kernel, schedules in global scratch: [slots][cow_slots4 * 4] which buckets of
                                  // units a slot's slice holds when its chain ends (the rest is the initial schedule)
     uint32_t cow_shift;          // a bucket is 2^cow_shift consecutive units
-    uint32_t stage_stepc;        // wide kernel without a staged access bitmap: the step constants alone are staged
     unsigned long long* work;    // wide kernel: [3] sums over the chains of {n_again, n_listed, n_items}
     // Replica exchange (wide kernel): the call runs rounds round0 .. round1-1; in round t chain c proposes moves
     // t * exch_every .. (t + 1) * exch_every - 1 (up to `upto`) with the table row of the rung it holds,
     // rung_hist[t * hist_stride + (c - hist_base)].
-    const uint8_t* rung_hist;    // null: the ordinary cooling schedule by temperature levels
+    uint8_t* rung_hist;          // null: the ordinary cooling schedule by temperature levels
     uint64_t exch_every;
     uint32_t round0, round1, hist_stride, hist_base;
     uint4* state;                // if set: [chains][state4] the chain's persistent shared-memory state (and its
@@ -72,12 +84,20 @@ struct ChainParams {
     uint32_t resume;             // 1: start from `state` instead of the initial schedule
     uint32_t cow_slots4;         // schedules in global scratch: uint4 slots of a chain's bucket bitmap; 0 (narrow kernel
                                  // only): plain slices, each a whole copy of the initial schedule
+    // wide kernel: segments seg0 .. seg1 - 1 of seg_len moves (the last one takes what is left up to `upto`), each of
+    // seg_bat batches: the temperature levels of the cooling schedule, or rounds of a replica-exchange run
+    uint32_t seg0, seg1, seg_bat;
+    uint64_t seg_len;
+    ChainLayout lay;
+    uint32_t warps;              // warps per chain
+    uint32_t carry;              // room for accepted proposals: kAccepted (less in tests)
+    const float* bounds;         // [levels] C ln 2: see EvalCtx::bound
+    uint32_t ladder_ctas;        // replica exchange: a CTA holds whole ladders and exchanges between its rounds itself
+    ExchangeArgs ladder;
+    uint32_t* n_exchanged;       // replica exchange in the CTA: by chain
 };
 
 // Batches: every lane of a chain's warp carries kMPL proposals, so a batch is 32 * kMPL consecutive moves.
-// Measured on 256 units x 512 steps, 1024 chains: kMPL = 2 is slower (6.0 ms vs 5.25 ms per 10^8 moves): a move that
-// changes the schedule then costs a re-evaluation pass over twice as many proposals. Serving a chain with two warps
-// that evaluate side by side and commit in turn was tried as well and was no faster (5.9 ms).
 constexpr int kMPL = 1;
 constexpr uint32_t kBatch = 32 * kMPL;
 constexpr uint32_t kWinSlots4 = kBatch * 2;                        // 8 words of windows per proposal
@@ -125,15 +145,17 @@ __device__ __forceinline__ uint32_t window(Ptr col, uint32_t S32, uint32_t s0)
 }
 
 // The same cut for several columns of one proposal: the position is worked out once.
+// The word after the first may lie behind the column (its bits are beyond the horizon then, and masked by every user):
+// columns are followed by at least four readable bytes everywhere.
 struct WinPos {
-    uint32_t w, w2, sh;          // first word, the word after it (clamped), shift
+    uint32_t w, sh;              // first word, shift
     bool first;                  // s0 == 0: bit 0 repeats step 0
 };
-__device__ __forceinline__ WinPos window_pos(uint32_t S32, uint32_t s0)
+__device__ __forceinline__ WinPos window_pos(uint32_t s0)
 {
     WinPos p;
     const uint32_t b0 = s0 ? s0 - 1 : 0u;
-    p.w = b0 >> 5; p.w2 = min(p.w + 1, S32 - 1); p.sh = b0 & 31u; p.first = s0 == 0;
+    p.w = b0 >> 5; p.sh = b0 & 31u; p.first = s0 == 0;
     return p;
 }
 // COLV = 2 or 4: every column is exactly that many words (at most 64 or 128 steps) and comes with one vector load: a
@@ -155,7 +177,7 @@ __device__ __forceinline__ uint32_t window_at(Ptr col, const WinPos p)
         hi = p.w == 0 ? q.y : p.w == 1 ? q.z : q.w;
     } else {
         lo = col[p.w];
-        hi = col[p.w2];
+        hi = col[p.w + 1];
     }
     return p.first ? ((lo << 1) | (lo & 1u)) : __funnelshift_r(lo, hi, p.sh);
 }
@@ -288,26 +310,6 @@ __device__ __forceinline__ int item_delta(const Windows& wn, uint32_t k, const u
     const uint32_t mi = c4.y + (npu & ~nqu) - (pu & ~qu) + (npv & ~nqv) - (pv & ~qv);
     const uint32_t mo = c4.z + (~npu & nqu & 1u) - (~pu & qu & 1u) + (~npv & nqv & 1u) - (~pv & qv & 1u);
     return (int)(step_cost(hr, mi, mo, c, K) - step_cost(c4.x, c4.y, c4.z, c, K));
-}
-
-// Cost of the step at window bit k after the proposal (Eq. 2-4), from its windows and the step's present counters.
-template <bool GROW>
-__device__ __forceinline__ uint32_t item_cost_after(const Windows& wn, uint32_t k, const uint4 c4, uint32_t hb, const StepC c,
-                                                    const CostK K)
-{
-    const uint32_t pu = (wn.Wu >> k) & 1u, qu = (wn.Wu >> (k - 1)) & 1u, npu = (wn.Nu >> k) & 1u, nqu = (wn.Nu >> (k - 1)) & 1u;
-    const uint32_t pv = (wn.Wv >> k) & 1u, qv = (wn.Wv >> (k - 1)) & 1u, npv = (wn.Nv >> k) & 1u, nqv = (wn.Nv >> (k - 1)) & 1u;
-    const uint32_t au = (wn.Au >> k) & 1u, av = (wn.Av >> k) & 1u;
-    const uint32_t hr = c4.x + (au & npu) - (au & pu) + (av & npv) - (av & pv);
-    const uint32_t mo = c4.z + (~npu & nqu & 1u) - (~pu & qu & 1u) + (~npv & nqv & 1u) - (~pv & qv & 1u);
-    if (GROW) {
-        const uint32_t mu = (wn.born & 255u) == k ? 0u : 1u, mw = ((wn.born >> 8) & 255u) == k ? 0u : 1u;
-        const uint32_t mi = c4.y + mu * ((npu & ~nqu) - (pu & ~qu)) + mw * ((npv & ~nqv) - (pv & ~qv));
-        const uint32_t hn = hb + (1u - mu) * (npu - pu) + (1u - mw) * (npv - pv);
-        return step_cost_g(hr, mi, mo, hn, c, K);
-    }
-    const uint32_t mi = c4.y + (npu & ~nqu) - (pu & ~qu) + (npv & ~nqv) - (pv & ~qv);
-    return step_cost(hr, mi, mo, c, K);
 }
 
 __device__ __forceinline__ bool metropolis(int delta, uint32_t w, const uint32_t* __restrict__ trow, uint32_t shift)
@@ -614,7 +616,7 @@ __host__ __device__ inline uint32_t chain_fixed4(uint32_t S, uint32_t S32, bool 
 // plain copy of it (small slices: the copy costs nothing and an applied move is cheaper without the take-over).
 template <bool PSMEM, bool GROW, int W, bool ASMEM, bool COW>
 __global__ void __launch_bounds__(512)
-chain_kernel(const ChainParams prm)
+narrow_chain_kernel(const ChainParams prm)
 {
     static_assert(!COW || !PSMEM, "overlays only for schedules in global scratch");
     static_assert(W >= 1 && W <= kMaxW && (W & (W - 1)) == 0, "warps per chain");
@@ -935,667 +937,15 @@ chain_kernel(const ChainParams prm)
     }
 }
 
-// ---------------------------------------------------------------------------------------------------------------
-// The wide chain kernel: one warp per chain, kRows proposals per lane, so a batch is 32 * kRows consecutive moves.
-//
-// Most proposals are settled by the placement bits alone: a swap of two units with equal placement over the run
-// changes nothing, a flip into a full step is infeasible (Eq. 5). Every lane first classifies its kRows proposals
-// that way (the Philox draws and the window loads of the rows are independent, so the warp has instruction-level
-// parallelism where the narrow kernel has none). Only the rest, typically a tenth to a third, needs the access
-// windows, the set of steps whose cardinalities change and Eq. 2-4 at those steps: their indices are compacted into
-// a list, and the warp works the list off 32 at a time, one proposal per lane, through the shared work queue of
-// (proposal, step) items. The commit walks the batch in move order and applies every accepted, state-changing
-// proposal it meets until it reaches one whose step range meets that of a move applied since it was evaluated;
-// those are evaluated again, all at once, and the walk goes on from there. The outcome is the sequential chain's.
-constexpr int kRows = 4;
-// Largest CTA of the wide kernel with schedules in global scratch; it sets the registers a thread may use (65,536
-// per SM over the resident threads), hence how many chains an SM holds at a time.
-#ifndef KVP_WIDE_GLOBAL_THREADS
-#define KVP_WIDE_GLOBAL_THREADS 512
-#endif
-constexpr int kWideGlobalThreads = KVP_WIDE_GLOBAL_THREADS;
-constexpr uint32_t kWide = 32 * kRows;
-constexpr uint32_t kWideQueueSlots4 = (32 * 31 * 2 + 15) / 16;     // the items of one pass of 32 proposals
+}  // namespace
 
-template <typename CT> __device__ __forceinline__ uint4 ctr_load(const CT* c, uint32_t t);
-template <> __device__ __forceinline__ uint4 ctr_load<uint4>(const uint4* c, uint32_t t) { return c[t]; }
-template <> __device__ __forceinline__ uint4 ctr_load<ushort4>(const ushort4* c, uint32_t t)
-{
-    const ushort4 v = c[t];
-    return make_uint4(v.x, v.y, v.z, v.w);
-}
-template <typename CT> __device__ __forceinline__ void ctr_store(CT* c, uint32_t t, uint4 v);
-template <> __device__ __forceinline__ void ctr_store<uint4>(uint4* c, uint32_t t, uint4 v) { c[t] = v; }
-template <> __device__ __forceinline__ void ctr_store<ushort4>(ushort4* c, uint32_t t, uint4 v)
-{
-    c[t] = make_ushort4((unsigned short)v.x, (unsigned short)v.y, (unsigned short)v.z, (unsigned short)v.w);
-}
+}  // namespace kvp
 
-// Where a chain of the wide kernel keeps its state. CT: the four per-step cardinalities as 16-bit fields when the
-// schedule lives in shared memory (then units < 2^16), as 32-bit fields otherwise. COW: see above.
-template <typename CT, bool COW, int COLV>
-struct WideView {
-    const uint32_t* p0;          // COW: [U][S32] the initial schedule
-    uint32_t* have;              // COW: [cow_slots4 * 4] buckets present in P (shared)
-    uint32_t shift, U, S32;      // COW: bucket size; units; words per unit
-    __device__ __forceinline__ const uint32_t* col(uint32_t u) const
-    {
-        if (COW) {
-            const uint32_t b = u >> shift;
-            return ((have[b >> 5] >> (b & 31u)) & 1u ? P : p0) + (size_t)u * S32;
-        }
-        return P + (size_t)u * S32;
-    }
-    // Before unit u is rewritten: its bucket is copied into the slice if it is not there yet (all lanes, u uniform).
-    __device__ __forceinline__ void own(uint32_t u, uint32_t lane) const
-    {
-        if (!COW) return;
-        const uint32_t b = u >> shift;
-        if ((have[b >> 5] >> (b & 31u)) & 1u) return;
-        const size_t lo = (size_t)(b << shift) * S32, hi = (size_t)min(U, (b + 1u) << shift) * S32;
-        copy_words(P + lo, p0 + lo, hi - lo, lane);
-        __syncwarp();
-        if (lane == 0) have[b >> 5] |= 1u << (b & 31u);
-        __syncwarp();
-    }
-    uint32_t* P;                 // [U][S32] schedule, time-packed (shared or global)
-    CT* ctr;                     // [S] {hr, mi, mo, occ} (shared)
-    uint32_t* full;              // [S32] bit t set iff occ[t] == cap (shared)
-    uint32_t* hb;                // growing cache: [S] units written to HBM at birth (shared)
-    uint32_t* fnow;              // [S] the present cost of every step, Eq. 2 (shared)
-    uint4* win;                  // [kWide][2] by proposal: {pk, u, v, -} until it is evaluated, then its windows
-    int* acc;                    // [kWide] by proposal: its cost change being summed
-    uint8_t* nt;                 // [kWide] the proposals that need a cost evaluation, compacted
-    uint16_t* queue;             // [32 * 31] work items (proposal << 5 | window bit) of one pass
-};
+#include "kvp_chain.cuh"
 
-// The scalars of a chain that only an applied move or a level boundary touches: in shared memory, so that the loop
-// over the batches keeps its registers for the proposals.
-struct WideScalars {
-    uint64_t cur, best, best_move, best_at_boundary, n_chg, hash;
-    uint32_t ulen;               // moves applied since the best state
-    uint32_t snap_dirty;         // the best state is the current one and not saved yet
-    uint32_t qn;                 // items reserved in the work queue during a pass (0 between passes)
-    uint32_t pad;
-    // what the chain's evaluations amounted to (kvp_anneal_stats): proposals evaluated again after an applied move,
-    // proposals that needed a cost evaluation, (proposal, step) items
-    uint64_t n_again, n_listed, n_items;
-    uint64_t n_acc, n_inf;       // accepted / infeasible proposals of earlier calls on this state (replica exchange)
-    uint64_t pad2;
-};
-constexpr uint32_t kWideScalars4 = sizeof(WideScalars) / 16;
+namespace kvp {
 
-// the part of wide_fixed4 that outlives a batch (what a replica-exchange run saves between its rounds)
-// cow4: uint4 slots of the bucket bitmap (schedules in global scratch)
-__host__ __device__ inline uint32_t wide_persist4(uint32_t S, uint32_t S32, bool grow, bool shared, uint32_t cow4)
-{
-    return (shared ? (S + 1) / 2 : S) + (S32 + 3) / 4 + (grow ? (S + 3) / 4 : 0u) + (S + 3) / 4 + (shared ? 0u : cow4) +
-           kWideScalars4;
-}
-
-// shared-memory words (as uint4 slots) of one chain of the wide kernel besides its schedule
-__host__ __device__ inline uint32_t wide_fixed4(uint32_t S, uint32_t S32, bool grow, bool shared, uint32_t cow4)
-{
-    return (shared ? (S + 1) / 2 : S) + (S32 + 3) / 4 + (grow ? (S + 3) / 4 : 0u) + (S + 3) / 4 +
-           (shared ? 0u : cow4) + kWideScalars4 +
-           2 * kWide + kWide / 4 + kWide / 16 + kWideQueueSlots4;
-}
-
-// N queue items per lane, items base + 32 r + lane: the cost change of one step of one proposal each, added to the
-// proposal's sum.
-template <bool GROW, int N, typename CT, bool COW, int COLV>
-__device__ __forceinline__ void wide_items(const WideView<CT, COW, COLV> cv, const StepC* __restrict__ stepc, const CostK K, uint32_t S,
-                                           uint32_t base, uint32_t count, uint32_t lane)
-{
-    int d[N];
-    uint32_t id[N];
-    bool live[N];
-#pragma unroll
-    for (int r = 0; r < N; ++r) {
-        const uint32_t g = base + 32 * r + lane;
-        live[r] = g < count;
-        const uint32_t item = cv.queue[live[r] ? g : 0u];         // a dead lane repeats item 0 and drops the result
-        id[r] = item >> 5;
-        const uint32_t k = item & 31u;
-        const uint4 w0 = cv.win[id[r] * 2], w1 = cv.win[id[r] * 2 + 1];
-        Windows wn;
-        wn.Wu = w0.x; wn.Wv = w0.y; wn.Nu = w0.z; wn.Nv = w0.w; wn.Au = w1.x; wn.Av = w1.y; wn.s0 = w1.z;
-        wn.born = w1.w;
-        const uint32_t t = min(wn.s0 + k - 1, S - 1);
-        const StepC sc = stepc[t];
-        d[r] = (int)(item_cost_after<GROW>(wn, k, ctr_load<CT>(cv.ctr, t), GROW ? cv.hb[t] : 0u, sc, K) - cv.fnow[t]);
-    }
-#pragma unroll
-    for (int r = 0; r < N; ++r)
-        if (live[r] && d[r]) atomicAdd(cv.acc + id[r], d[r]);
-}
-
-// Per-lane record of the kRows proposals a lane owns in the current batch. Row h of lane l is move m + 32 h + l.
-// inf / acc / chg: one bit per row.
-struct WideMoves {
-    uint32_t pk[kRows], u[kRows], v[kRows], w[kRows];
-    int delta[kRows];
-    uint32_t inf, acc, chg;
-};
-
-// Second half of evaluating a proposal that is known to change bits and to be feasible: given its placement windows
-// (Wu; wv = the window of v for a swap), the access windows, the windows after the move and the set of window bits
-// (steps) whose cardinalities, hence cost, change. Same conventions as lane_windows.
-template <bool GROW, int COLV>
-__device__ __forceinline__ uint32_t changed_steps(uint32_t Wu, uint32_t wv, const uint32_t* __restrict__ Acol,
-                                                  const uint32_t* __restrict__ birth, uint32_t S, uint32_t S32,
-                                                  uint32_t pk, uint32_t u, uint32_t v, Windows& wn)
-{
-    const bool swap = pk & 1u;
-    const uint32_t len = (pk >> 1) & 63u, s0 = pk >> 8;
-    const uint32_t run = min(s0 + len, S) - s0;                   // steps whose placement bits change hands
-    const uint32_t nl = min(s0 + len, S - 1) - s0 + 1;            // affected steps: the run and the step after it
-    const uint32_t M = ((1u << run) - 1u) << 1;
-    const uint32_t Sb = ((1u << nl) - 1u) << 1;
-    const WinPos wp = window_pos(S32, s0);
-    const uint32_t Au = window_at<COLV>(Acol + (size_t)u * S32, wp);
-    const uint32_t av = window_at<COLV>(Acol + (size_t)(swap ? v : u) * S32, wp);   // a flip reads unit u twice
-    const uint32_t Av = swap ? av : 0u, Wv = swap ? wv : 0u;
-    uint32_t Bu = 0u, Bv = 0u, live = 0xFFFFFFFFu;
-    if (GROW) {
-        uint32_t Lu, Lv;
-        alive_born(__ldg(birth + u), s0, Lu, Bu);
-        alive_born(__ldg(birth + (swap ? v : u)), s0, Lv, Bv);
-        live = Lu & Lv;
-        if (!swap) Bv = 0u;
-    }
-    const uint32_t D = (swap ? (Wu ^ Wv) : 0xFFFFFFFFu) & M & live;      // bits that toggle
-    uint32_t Nu = Wu ^ D, Nv = swap ? (Wv ^ D) : 0u;
-    if (s0 == 0) {                                                // the virtual step -1 follows step 0
-        Nu = (Nu & ~1u) | ((Nu >> 1) & 1u);
-        Nv = (Nv & ~1u) | ((Nv >> 1) & 1u);
-    }
-    wn.Wu = Wu; wn.Wv = Wv; wn.Nu = Nu; wn.Nv = Nv; wn.Au = Au; wn.Av = Av; wn.s0 = s0;
-    wn.born = GROW ? ((Bu ? 31u - __clz(Bu) : 0u) | ((Bv ? 31u - __clz(Bv) : 0u) << 8)) : 0u;
-    const uint32_t hr = (Au ^ Av) & (Wu ^ Nu);                    // a hit is won or lost (v mirrors u in a swap)
-    const uint32_t euo = (Wu ^ (Wu << 1)) & ~Bu, eun = (Nu ^ (Nu << 1)) & ~Bu;
-    const uint32_t evo = (Wv ^ (Wv << 1)) & ~Bv, evn = (Nv ^ (Nv << 1)) & ~Bv;
-    const uint32_t mg = (euo ^ eun) | (euo & eun & (Wu ^ Nu)) | (evo ^ evn) | (evo & evn & (Wv ^ Nv));
-    const uint32_t wr = ((Wu ^ Nu) & Bu) | ((Wv ^ Nv) & Bv);
-    return (hr | mg | wr) & Sb;
-}
-
-// First half of an evaluation, placement bits only: a swap of equal placements changes nothing, a flip into a full
-// step is infeasible (Eq. 5). The proposals of `need` (per lane: bit h = its row h) that need more are listed in cv.nt
-// with their placement windows parked in their slots. `listed`: how many; `mine`: which of this lane's rows.
-// ALL: nearly every row is named (a fresh batch): the window loads of all rows are issued before any is used, named
-// or not (every row holds a drawn proposal, so every address is good). Otherwise rows without a named proposal are
-// skipped.
-template <bool GROW, bool ALL, typename CT, bool COW, int COLV>
-__device__ __forceinline__ void wide_classify(const WideView<CT, COW, COLV> cv, const uint32_t* __restrict__ birth, uint32_t S,
-                                              uint32_t S32, uint32_t need, uint32_t lane, WideMoves& mv, uint32_t& listed,
-                                              uint32_t& mine)
-{
-    const uint32_t below = (1u << lane) - 1u;
-    uint32_t Wu[kRows], Wv[kRows], Fw[kRows], Lv[kRows];
-    bool skip[kRows];
-#pragma unroll
-    for (int h = 0; h < kRows; ++h) {
-        skip[h] = ALL ? false : !__any_sync(0xFFFFFFFFu, (need >> h) & 1u);
-        Wu[h] = Wv[h] = Fw[h] = 0u; Lv[h] = 0xFFFFFFFFu;
-        if (skip[h]) continue;                                    // warp-uniform
-        const uint32_t pk = mv.pk[h], s0 = pk >> 8;
-        const bool swap = pk & 1u;
-        const WinPos wp = window_pos(S32, s0);
-        Wu[h] = window_at<COLV>(cv.col(mv.u[h]), wp);
-        // the second window: the other unit's placement for a swap, the full-step bitmap for a flip
-        const uint32_t* second = swap ? cv.col(mv.v[h]) : cv.full;
-        const uint32_t w2 = window_at<COLV>(second, wp);
-        Wv[h] = swap ? w2 : Wu[h];
-        Fw[h] = w2;
-        if (GROW) {
-            uint32_t La, Lb, Bu, Bv;
-            alive_born(__ldg(birth + mv.u[h]), s0, La, Bu);
-            alive_born(__ldg(birth + (swap ? mv.v[h] : mv.u[h])), s0, Lb, Bv);
-            Lv[h] = La & Lb;
-        }
-    }
-#pragma unroll
-    for (int h = 0; h < kRows; ++h) {
-        if (skip[h]) continue;
-        const bool named = (need >> h) & 1u;
-        const uint32_t pk = mv.pk[h];
-        const bool swap = pk & 1u;
-        const uint32_t len = (pk >> 1) & 63u, s0 = pk >> 8;
-        const uint32_t run = min(s0 + len, S) - s0;
-        const uint32_t M = ((1u << run) - 1u) << 1;
-        const uint32_t D = (swap ? Wu[h] ^ Wv[h] : 0xFFFFFFFFu) & M & Lv[h];   // a flip toggles every bit of the run
-        const bool chg = D != 0;
-        const bool inf = !swap && (~Wu[h] & D & Fw[h]) != 0;      // a flip may not raise a full step (Eq. 5)
-        if (named) {
-            const uint32_t bit = 1u << h;
-            mv.chg = chg ? mv.chg | bit : mv.chg & ~bit;
-            mv.inf = inf ? mv.inf | bit : mv.inf & ~bit;
-            mv.acc = inf ? mv.acc & ~bit : mv.acc | bit;          // nothing changes: cost change 0, always accepted
-            mv.delta[h] = 0;
-        }
-        const bool more = named && chg && !inf;
-        const uint32_t mb = __ballot_sync(0xFFFFFFFFu, more);
-        const uint32_t id = h * 32 + lane;
-        // the slot of a proposal that is not listed is not looked at again, so a fresh batch parks every row's
-        // windows without a test
-        if (ALL || more) {
-            cv.win[id * 2] = make_uint4(pk, mv.u[h], mv.v[h], Wu[h]);
-            cv.win[id * 2 + 1].x = Wv[h];
-            cv.acc[id] = 0;
-        }
-        if (more) {
-            cv.nt[listed + __popc(mb & below)] = (uint8_t)id;
-            mine |= 1u << h;
-        }
-        listed += __popc(mb);
-    }
-}
-
-// Evaluation of the proposals named by `need` (per lane: bit h = its row h) against the current state.
-// fresh: a new batch, nearly every row named (see wide_classify).
-template <bool GROW, typename CT, bool COW, int COLV>
-__device__ __forceinline__ void wide_evaluate(const WideView<CT, COW, COLV> cv, const uint32_t* __restrict__ Acol,
-                                              const uint32_t* __restrict__ birth, const StepC* __restrict__ stepc,
-                                              const CostK K, uint32_t S, uint32_t S32, const uint32_t* __restrict__ trow,
-                                              uint32_t shift, uint32_t need, bool fresh, uint32_t lane, WideMoves& mv,
-                                              WideScalars* sc)
-{
-    // 1. placement bits only; the proposals that need more are listed
-    uint32_t listed = 0;                                          // proposals listed (warp-uniform)
-    uint32_t mine = 0;                                            // bit h: this lane's row h is listed
-    if (fresh) wide_classify<GROW, true>(cv, birth, S, S32, need, lane, mv, listed, mine);
-    else wide_classify<GROW, false>(cv, birth, S, S32, need, lane, mv, listed, mine);
-    if (!listed) return;                                          // warp-uniform
-    if (lane == 0) sc->n_listed += listed;
-    __syncwarp();
-    // 2. the listed proposals, 32 at a time, one per lane: access windows, the steps whose cost changes, and those
-    //    (proposal, step) items through the shared queue
-    for (uint32_t first = 0; first < listed; first += 32) {
-        const uint32_t g = first + lane;
-        const bool live = g < listed;
-        const uint32_t id = cv.nt[live ? g : first];
-        const uint4 who = cv.win[id * 2];
-        const uint32_t wv = cv.win[id * 2 + 1].x;
-        Windows wn;
-        const uint32_t tm = changed_steps<GROW, COLV>(who.w, wv, Acol, birth, S, S32, who.x, who.y, who.z, wn);
-        __syncwarp();                                             // every lane has read its proposal
-        const uint32_t todo = live ? tm : 0u;
-        if (live) {
-            cv.win[id * 2] = make_uint4(wn.Wu, wn.Wv, wn.Nu, wn.Nv);
-            cv.win[id * 2 + 1] = make_uint4(wn.Au, wn.Av, wn.s0, wn.born);
-        }
-        // every lane reserves room for its items in the queue (the order of the items does not matter)
-        const uint32_t cnt = __popc(todo);
-        uint32_t pos = cnt ? atomicAdd(&sc->qn, cnt) : 0u;
-        __syncwarp();
-        const uint32_t total = sc->qn;
-        __syncwarp();
-        if (total) {
-            if (lane == 0) { sc->n_items += total; sc->qn = 0u; }
-            if (COW) {
-                // many chains per SM, issue slots scarce: every lane peels its own set bits, highest first (the order
-                // of the items in the queue does not matter: their cost changes are summed)
-                for (uint32_t td = todo; td != 0u;) {
-                    const uint32_t k = 31u - __clz(td);
-                    cv.queue[pos++] = (uint16_t)((id << 5) | k);
-                    td ^= 1u << k;
-                }
-            } else {
-                // few chains per SM, latency scarce: all 31 positions tried, no lane waits on a serial bit scan
-#pragma unroll
-                for (uint32_t k = 1; k < 32; ++k) {
-                    const uint32_t bit = (todo >> k) & 1u;
-                    if (bit) cv.queue[pos] = (uint16_t)((id << 5) | k);
-                    pos += bit;
-                }
-            }
-            __syncwarp();
-            for (uint32_t base = 0; base < total; base += 64) {
-                if (base + 32 < total) wide_items<GROW, 2>(cv, stepc, K, S, base, total, lane);
-                else wide_items<GROW, 1>(cv, stepc, K, S, base, total, lane);
-            }
-        }
-        __syncwarp();
-    }
-    // 3. the owners take the sums and decide. Straight-line over the rows (the sums and the thresholds of all rows
-    //    are loaded before any is used); a row that is not listed reads a stale sum and drops the outcome.
-    int d[kRows];
-    uint32_t thr[kRows];
-#pragma unroll
-    for (int h = 0; h < kRows; ++h) d[h] = cv.acc[h * 32 + lane];
-#pragma unroll
-    for (int h = 0; h < kRows; ++h) {
-        const uint32_t q = (uint32_t)max(d[h], 0) >> shift;
-        thr[h] = __ldg(trow + min(q, (uint32_t)KVP_TABLE_Q - 1u));
-        if (q >= KVP_TABLE_Q) thr[h] = 0u;                        // beyond the table: never accepted
-    }
-#pragma unroll
-    for (int h = 0; h < kRows; ++h) {
-        const bool lst = (mine >> h) & 1u;
-        const bool ok = d[h] <= 0 || mv.w[h] < thr[h];            // quantised exp(-delta/C), as in metropolis()
-        const uint32_t bit = 1u << h;
-        if (lst) {
-            mv.delta[h] = d[h];
-            mv.acc = ok ? mv.acc | bit : mv.acc & ~bit;
-        }
-    }
-}
-
-// Apply the proposal whose windows are in slot `id` (pk, u, v given): all lanes take part, lane j updates the
-// counters of window bit j, lanes 0 and 1 rewrite the words of the schedule and of the full-step bitmap.
-template <bool GROW, typename CT, bool COW, int COLV>
-__device__ __forceinline__ void wide_apply(const WideView<CT, COW, COLV> cv, const StepC* __restrict__ stepc, const CostK K,
-                                           uint32_t S, uint32_t S32, uint32_t cap, uint32_t lane,
-                                           uint32_t id, uint32_t pk, uint32_t u, uint32_t v)
-{
-    const uint4 w0 = cv.win[id * 2], w1 = cv.win[id * 2 + 1];
-    const uint32_t Wu = w0.x, Wv = w0.y, Nu = w0.z, Nv = w0.w, Au = w1.x, Av = w1.y;
-    const bool swap = pk & 1u;
-    const uint32_t len = (pk >> 1) & 63u, s0 = pk >> 8;
-    const uint32_t run = min(s0 + len, S) - s0;
-    const uint32_t nl = min(s0 + len, S - 1) - s0 + 1;
-    const bool valid = lane >= 1 && lane <= nl;
-    const uint32_t j = valid ? lane : 1u, t = s0 + j - 1;
-    const uint32_t pu = (Wu >> j) & 1u, qu = (Wu >> (j - 1)) & 1u, npu = (Nu >> j) & 1u, nqu = (Nu >> (j - 1)) & 1u;
-    const uint32_t pv = (Wv >> j) & 1u, qv = (Wv >> (j - 1)) & 1u, npv = (Nv >> j) & 1u, nqv = (Nv >> (j - 1)) & 1u;
-    const uint32_t au = (Au >> j) & 1u, av = (Av >> j) & 1u;
-    uint4 c = ctr_load<CT>(cv.ctr, t);
-    uint32_t hbn = 0u;
-    c.x += (au & npu) - (au & pu) + (av & npv) - (av & pv);
-    if (GROW) {
-        const uint32_t mu = (w1.w & 255u) == j ? 0u : 1u, mw = ((w1.w >> 8) & 255u) == j ? 0u : 1u;
-        c.y += mu * ((npu & ~nqu) - (pu & ~qu)) + mw * ((npv & ~nqv) - (pv & ~qv));
-        const uint32_t dh = (1u - mu) * (npu - pu) + (1u - mw) * (npv - pv);
-        hbn = cv.hb[t] + dh;
-        if (valid && dh) cv.hb[t] = hbn;
-    } else {
-        c.y += (npu & ~nqu) - (pu & ~qu) + (npv & ~nqv) - (pv & ~qv);
-    }
-    c.z += (~npu & nqu & 1u) - (~pu & qu & 1u) + (~npv & nqv & 1u) - (~pv & qv & 1u);
-    c.w += npu - pu + npv - pv;
-    if (valid) {
-        ctr_store<CT>(cv.ctr, t, c);
-        cv.fnow[t] = GROW ? step_cost_g(c.x, c.y, c.z, hbn, stepc[t], K) : step_cost(c.x, c.y, c.z, stepc[t], K);
-    }
-    uint32_t F = __ballot_sync(0xFFFFFFFFu, valid && c.w == cap);   // bit j <-> window bit j
-    uint32_t V = __ballot_sync(0xFFFFFFFFu, valid);
-    cv.own(u, lane);
-    if (swap) cv.own(v, lane);
-    if (lane < 2) {
-        uint32_t M = ((1u << run) - 1u) << 1, NU = Nu, NV = Nv, sbit = s0 - 1;
-        if (s0 == 0) { F >>= 1; V >>= 1; M >>= 1; NU >>= 1; NV >>= 1; sbit = 0; }
-        const uint32_t wj = (sbit >> 5) + lane, sh = sbit & 31u;
-        if (wj < S32 && (lane == 0 || sh != 0)) {
-            // lane 0 holds the part of the window that falls into the first word, lane 1 the spill-over
-            const uint32_t Vx = lane ? V >> (32 - sh) : V << sh, Fx = lane ? F >> (32 - sh) : F << sh;
-            const uint32_t Mx = lane ? M >> (32 - sh) : M << sh;
-            const uint32_t NUx = lane ? NU >> (32 - sh) : NU << sh, NVx = lane ? NV >> (32 - sh) : NV << sh;
-            if (Vx) cv.full[wj] = (cv.full[wj] & ~Vx) | (Fx & Vx);
-            if (Mx) {
-                const size_t iu = (size_t)u * S32 + wj;
-                cv.P[iu] = (cv.P[iu] & ~Mx) | (NUx & Mx);
-                if (swap) {
-                    const size_t iv = (size_t)v * S32 + wj;
-                    cv.P[iv] = (cv.P[iv] & ~Mx) | (NVx & Mx);
-                }
-            }
-        }
-    }
-    __syncwarp();
-}
-
-// PSMEM: the schedule lives in shared memory (16-bit counters); otherwise the chain's slice of global scratch is a
-// copy-on-write overlay of the initial schedule (see kCowBitsMin).
-// ASMEM (only with PSMEM): access bitmap and step constants staged in shared memory once per CTA.
-// COLV (only without PSMEM): 2 or 4 when every column has exactly that many words, else 0 (see window_at).
-template <bool PSMEM, bool GROW, bool ASMEM, int COLV>
-__global__ void __launch_bounds__(PSMEM ? 256 : kWideGlobalThreads, 1)
-wide_chain_kernel(const ChainParams prm)
-{
-    static_assert(PSMEM || !ASMEM, "shared access bitmap only beside shared schedules");
-    static_assert(!PSMEM || COLV == 0, "vector columns only for schedules in global scratch");
-    using CT = typename std::conditional<PSMEM, ushort4, uint4>::type;
-    constexpr bool COW = !PSMEM;
-    extern __shared__ uint4 smem4[];
-    const uint32_t lane = threadIdx.x & 31, cic = threadIdx.x >> 5;
-    const uint32_t cpb = blockDim.x >> 5;                         // chains per CTA
-    const uint32_t slot = blockIdx.x * cpb + cic;
-    const bool active = slot < prm.chain_count;
-    const uint32_t chain = prm.chain_first + slot;
-    const uint32_t S = prm.S, S32 = prm.S32, U = prm.U;
-    const size_t pwords = (size_t)U * S32;
-    const uint32_t c4 = PSMEM ? (S + 1) / 2 : S;                  // uint4 slots of the counters
-    const uint32_t f4 = (S32 + 3) / 4, h4 = GROW ? (S + 3) / 4 : 0u;
-    const uint32_t o4 = COW ? prm.cow_slots4 : 0u;
-    const uint32_t fixed4 = wide_fixed4(S, S32, GROW, PSMEM, o4);
-    uint4* const mine4 = smem4 + (size_t)cic * fixed4;
-    WideView<CT, COW, COLV> cv;
-    cv.ctr = reinterpret_cast<CT*>(mine4);
-    cv.full = reinterpret_cast<uint32_t*>(mine4 + c4);
-    cv.hb = reinterpret_cast<uint32_t*>(mine4 + c4 + f4);
-    const uint32_t n4 = (S + 3) / 4;                              // uint4 slots of the present step costs
-    cv.fnow = reinterpret_cast<uint32_t*>(mine4 + c4 + f4 + h4);
-    cv.have = reinterpret_cast<uint32_t*>(mine4 + c4 + f4 + h4 + n4);
-    WideScalars* const sc = reinterpret_cast<WideScalars*>(mine4 + c4 + f4 + h4 + n4 + o4);
-    cv.win = mine4 + c4 + f4 + h4 + n4 + o4 + kWideScalars4;
-    cv.acc = reinterpret_cast<int*>(cv.win + 2 * kWide);
-    cv.nt = reinterpret_cast<uint8_t*>(cv.win + 2 * kWide + kWide / 4);
-    cv.queue = reinterpret_cast<uint16_t*>(cv.win + 2 * kWide + kWide / 4 + kWide / 16);
-    uint32_t* const pool = reinterpret_cast<uint32_t*>(smem4 + (size_t)cpb * fixed4);   // schedules, then A, then constants
-    cv.P = PSMEM ? pool + (size_t)cic * pwords : prm.ws + (size_t)slot * pwords;
-    cv.p0 = prm.Pcol0; cv.shift = prm.cow_shift; cv.U = U; cv.S32 = S32;
-    const uint32_t* Acol = prm.Acol;
-    const StepC* stepc = prm.stepc;
-    if (ASMEM) {
-        const size_t a_off = ((size_t)cpb * pwords + 3) & ~(size_t)3, c_off = (a_off + pwords + 3) & ~(size_t)3;
-        uint32_t* const a_s = pool + a_off;
-        StepC* const c_s = reinterpret_cast<StepC*>(pool + c_off);
-        copy_words(a_s, prm.Acol, pwords, threadIdx.x, blockDim.x);
-        for (uint32_t i = threadIdx.x; i < S; i += blockDim.x) c_s[i] = __ldg(prm.stepc + i);
-        Acol = a_s;
-        stepc = c_s;
-    } else if (prm.stage_stepc) {                                 // the step constants alone, behind the chains' areas
-        StepC* const c_s = reinterpret_cast<StepC*>(pool + (PSMEM ? (((size_t)cpb * pwords + 3) & ~(size_t)3) : 0));
-        for (uint32_t i = threadIdx.x; i < S; i += blockDim.x) c_s[i] = __ldg(prm.stepc + i);
-        stepc = c_s;
-    }
-    if (active) {
-        for (uint32_t i = lane; i < S; i += 32) {
-            const uint4 c0 = __ldg(prm.counters0 + i);
-            const uint32_t hb0 = GROW ? __ldg(prm.hb0 + i) : 0u;
-            ctr_store<CT>(cv.ctr, i, c0);
-            if (GROW) cv.hb[i] = hb0;
-            cv.fnow[i] = GROW ? step_cost_g(c0.x, c0.y, c0.z, hb0, __ldg(prm.stepc + i), prm.K)
-                              : step_cost(c0.x, c0.y, c0.z, __ldg(prm.stepc + i), prm.K);
-        }
-        for (uint32_t i = lane; i < S32; i += 32) cv.full[i] = __ldg(prm.full0 + i);
-        if (lane == 0) {
-            sc->cur = sc->best = sc->best_at_boundary = prm.init_ticks;
-            sc->best_move = ~0ull; sc->n_chg = 0; sc->hash = 0; sc->ulen = 0u; sc->snap_dirty = 0u; sc->qn = 0u;
-            sc->n_again = sc->n_listed = sc->n_items = 0; sc->n_acc = sc->n_inf = 0;
-        }
-        if (COW) {
-            for (uint32_t i = lane; i < prm.cow_slots4 * 4; i += 32) cv.have[i] = 0u;   // the slice holds nothing yet
-        } else if (!(prm.state && prm.resume)) {
-            copy_words_cold(cv.P, prm.Pcol0, pwords, lane);
-        }
-    }
-    // the persistent part of a chain's shared memory: counters, full-step bitmap, written-to-HBM counts, present step
-    // costs, overlay bitmap, scalars (everything before the per-batch work areas)
-    const uint32_t persist4 = c4 + f4 + h4 + n4 + o4 + kWideScalars4;
-    uint4* const saved = prm.state ? prm.state + (size_t)(chain - prm.hist_base) * prm.state4 : nullptr;
-    if (active && saved && prm.resume) {
-        __syncwarp();
-        for (uint32_t i = lane; i < persist4; i += 32) mine4[i] = saved[i];
-        if (PSMEM) copy_words_cold(cv.P, reinterpret_cast<const uint32_t*>(saved + persist4), pwords, lane);
-    }
-    __syncthreads();
-    if (!active) return;
-    uint32_t* snap = prm.snap ? prm.snap + (size_t)slot * pwords : nullptr;
-    uint64_t* ulog = prm.undo_log ? prm.undo_log + (size_t)slot * prm.undo_cap : nullptr;
-
-    uint64_t n_acc = 0, n_inf = 0;                                // per lane: of the proposals this lane owned
-
-    // A segment of moves at one temperature: a level of the cooling schedule, or a round of a replica-exchange run.
-    const bool exchange = prm.rung_hist != nullptr;
-    uint64_t lvl_start = exchange ? (uint64_t)prm.round0 * prm.exch_every : 0;
-    bool stop = false;
-    for (uint32_t seg = exchange ? prm.round0 : 0u; seg < (exchange ? prm.round1 : prm.levels) && lvl_start < prm.upto; ++seg) {
-        const uint32_t level = exchange ? prm.rung_hist[(size_t)seg * prm.hist_stride + (chain - prm.hist_base)] : seg;
-        const uint64_t lvl_len = exchange ? min(prm.exch_every, prm.upto - lvl_start)
-                                          : (level + 1 < prm.levels ? min(lvl_start + prm.per_level, prm.upto) : prm.upto) - lvl_start;
-        const uint32_t shift = __ldg(prm.shifts + level);
-        const uint32_t* trow = prm.table + (size_t)level * KVP_TABLE_Q;
-        if (!exchange && level > 0) {
-            const uint64_t best = sc->best, before = sc->best_at_boundary;
-            if (prm.early_permille && level >= prm.early_from &&
-                (before - best) * 1000ull < before * (uint64_t)prm.early_permille) {
-                stop = true;
-                break;
-            }
-            __syncwarp();
-            if (lane == 0) sc->best_at_boundary = best;
-            __syncwarp();
-        }
-        for (uint64_t off = 0; off < lvl_len; off += kWide) {
-            const uint64_t m = lvl_start + off;
-            const uint32_t nb = (uint32_t)min((uint64_t)kWide, lvl_len - off);
-            WideMoves mv;
-            mv.inf = mv.acc = mv.chg = 0u;
-            uint32_t pend = 0u;                                   // bit h: this lane's row h is still to be committed
-#pragma unroll
-            for (int h = 0; h < kRows; ++h) {
-                uint32_t r[4];
-                const uint64_t mine = m + 32u * h + lane;
-                philox4x32_10((uint32_t)mine, (uint32_t)(mine >> 32), chain, TAG_MOVE, prm.keys, r);
-                LaneMove lm;
-                decode_move(r, prm.p_swap_256, prm.len_choices, S, U, lm);
-                mv.pk[h] = lm.pk; mv.u[h] = lm.u; mv.v[h] = lm.v; mv.w[h] = lm.w; mv.delta[h] = 0;
-                if (32u * h + lane < nb) pend |= 1u << h;
-            }
-            uint32_t need = pend, stale = 0u;
-            bool first_pass = true;
-            // Evaluate what is named, then commit in move order as far as the evaluations are still good.
-            for (;;) {
-                wide_evaluate<GROW>(cv, Acol, prm.birth, stepc, prm.K, S, S32, trow, shift, need, first_pass, lane, mv, sc);
-                first_pass = false;
-                // Nearly always nothing in the batch changes the schedule: every lane counts its own proposals.
-                if (!__any_sync(0xFFFFFFFFu, (mv.acc & mv.chg & ~mv.inf & pend) != 0u)) {
-                    n_inf += __popc(mv.inf & pend);
-                    n_acc += __popc(mv.acc & ~mv.inf & pend);
-                    break;
-                }
-                bool stopped = false;
-                for (uint32_t h = 0; h < kRows && !stopped; ++h) {
-                    uint32_t rem = __ballot_sync(0xFFFFFFFFu, (pend >> h) & 1u);   // the row's lanes still to commit
-                    if (!rem) continue;
-                    const bool infl = (mv.inf >> h) & 1u, accl = !infl && ((mv.acc >> h) & 1u);
-                    for (;;) {
-                        const uint32_t st = __ballot_sync(0xFFFFFFFFu, (stale >> h) & 1u) & rem;
-                        const uint32_t bl = __ballot_sync(0xFFFFFFFFu, accl && ((mv.chg >> h) & 1u)) & rem;
-                        const uint32_t fst = st ? __ffs(st) - 1u : 32u, fbl = bl ? __ffs(bl) - 1u : 32u;
-                        // the row's moves that are settled now: up to the next state-changing move (included), or up to
-                        // the first proposal whose evaluation is stale (excluded), or all of them
-                        const uint32_t upto_bit = fbl < fst ? fbl + 1u : fst;
-                        const uint32_t done = upto_bit >= 32u ? rem : rem & ((1u << upto_bit) - 1u);
-                        if ((done >> lane) & 1u) {
-                            n_inf += infl ? 1u : 0u;
-                            n_acc += accl ? 1u : 0u;
-                            pend &= ~(1u << h);
-                        }
-                        rem &= ~done;
-                        if (fbl < fst) {
-                            // the next state-changing move, evaluated against the state as it is now: apply it
-                            const uint32_t bb = fbl;
-                            uint32_t pk = 0, bu = 0, bv = 0;
-                            int delta = 0;
-#pragma unroll
-                            for (int k = 0; k < kRows; ++k)
-                                if (h == (uint32_t)k) { pk = mv.pk[k]; bu = mv.u[k]; bv = mv.v[k]; delta = mv.delta[k]; }
-                            pk = __shfl_sync(0xFFFFFFFFu, pk, bb); bu = __shfl_sync(0xFFFFFFFFu, bu, bb);
-                            bv = __shfl_sync(0xFFFFFFFFu, bv, bb); delta = __shfl_sync(0xFFFFFFFFu, delta, bb);
-                            const uint64_t after = (uint64_t)((int64_t)sc->cur + delta);
-                            const bool leaving = snap && sc->snap_dirty && after >= sc->best;
-                            if (leaving) copy_words(snap, cv.P, pwords, lane);   // leaving the best state: save it first
-                            wide_apply<GROW>(cv, stepc, prm.K, S, S32, prm.cap, lane, h * 32 + bb, pk, bu, bv);
-                            if (lane == 0) {
-                                const uint64_t mb = m + 32u * h + bb;
-                                if (leaving) sc->snap_dirty = 0u;
-                                sc->cur = after;
-                                ++sc->n_chg;
-                                sc->hash = (sc->hash ^ mb) * 0x9E3779B97F4A7C15ull + after;
-                                if (after < sc->best) { sc->best = after; sc->best_move = mb; sc->snap_dirty = 1u; sc->ulen = 0u; }
-                                else if (ulog) {                          // every move is its own inverse: remember it
-                                    const uint32_t ulen = sc->ulen;
-                                    if (ulen < prm.undo_cap) ulog[ulen] = mb;
-                                    if (ulen <= prm.undo_cap) sc->ulen = ulen + 1u;
-                                }
-                            }
-                            __syncwarp();
-                            // The applied move rewrote steps s0b .. s0b + len_b (bits, counters, full flags). A pending
-                            // proposal read steps s0 - 1 .. s0 + len: its evaluation is stale iff the two ranges meet.
-                            const uint32_t s0b = pk >> 8, endb = s0b + ((pk >> 1) & 63u);
-#pragma unroll
-                            for (int k = 0; k < kRows; ++k) {
-                                const uint32_t s0 = mv.pk[k] >> 8, end = s0 + ((mv.pk[k] >> 1) & 63u);
-                                if (s0 <= endb + 1 && s0b <= end) stale |= 1u << k;
-                            }
-                            stale &= pend;
-                        } else if (fst < 32u) {
-                            stopped = true;                       // a stale evaluation comes first
-                            break;
-                        } else {
-                            break;                                // the row is done
-                        }
-                    }
-                }
-                if (!stopped) break;
-                need = stale & pend;
-                stale = 0u;
-                const uint32_t again = __reduce_add_sync(0xFFFFFFFFu, __popc(need));
-                if (lane == 0) sc->n_again += again;
-            }
-        }
-        lvl_start += lvl_len;
-    }
-    const uint64_t m_end = stop || exchange ? lvl_start : prm.upto;   // moves done when the call ended
-    // accepted and infeasible proposals were counted by the lanes that owned them
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-        n_acc += __shfl_xor_sync(0xFFFFFFFFu, n_acc, off);
-        n_inf += __shfl_xor_sync(0xFFFFFFFFu, n_inf, off);
-    }
-    n_acc += sc->n_acc; n_inf += sc->n_inf;                       // plus those of earlier calls on this state
-    __syncwarp();
-    if (lane == 0) { sc->n_acc = n_acc; sc->n_inf = n_inf; }
-    __syncwarp();
-    if (saved) {                                                  // the next round goes on from here
-        for (uint32_t i = lane; i < persist4; i += 32) saved[i] = mine4[i];
-        if (PSMEM) copy_words_cold(reinterpret_cast<uint32_t*>(saved + persist4), cv.P, pwords, lane);
-    }
-    if (snap && sc->snap_dirty) copy_words_cold(snap, cv.P, pwords, lane);
-    if (ulog && lane == 0) prm.undo_len[slot] = sc->ulen;
-    if (COW && prm.cow_out)                                       // which buckets the slice holds (for the walk back)
-        for (uint32_t i = lane; i < prm.cow_slots4 * 4; i += 32)
-            prm.cow_out[(size_t)slot * (prm.cow_slots4 * 4) + i] = cv.have[i];
-    if (lane == 0) {
-        kvp_chain_result res;
-        res.best_ticks = sc->best; res.best_move = sc->best_move; res.final_ticks = sc->cur; res.moves_done = m_end;
-        res.n_accepted = n_acc; res.n_changed = sc->n_chg; res.n_infeasible = n_inf; res.traj_hash = sc->hash;
-        prm.results[chain - prm.result_base] = res;
-        if (prm.work) {
-            atomicAdd(prm.work, (unsigned long long)sc->n_again);
-            atomicAdd(prm.work + 1, (unsigned long long)sc->n_listed);
-            atomicAdd(prm.work + 2, (unsigned long long)sc->n_items);
-        }
-    }
-    if (prm.dump && slot == 0) {
-        __syncwarp();
-        if (COW) copy_merged(prm.dump, cv.P, cv.p0, cv.have, cv.shift, U, S32, lane);
-        else copy_words_cold(prm.dump, cv.P, pwords, lane);
-    }
-}
+namespace {
 
 // Takes a finished chain's schedule back to its best state: the moves applied after the best were logged, each
 // swap or flip is its own inverse, so applying them again in reverse order undoes them. One warp; only the
@@ -1741,10 +1091,8 @@ struct ExchangeK {
     uint32_t* holder;
     uint8_t* rung_next;
     uint32_t* n_exchanged;
-    unsigned long long* counts;
-    const uint32_t* xalways; const uint32_t* xtable; const uint32_t* xshifts;
-    uint32_t ladders, rungs, first_ladder;
-    uint32_t seed_lo, seed_hi;
+    ExchangeArgs x;
+    uint32_t ladders, first_ladder;
     uint64_t t;
 };
 
@@ -1753,21 +1101,12 @@ exchange_kernel(const ExchangeK k)
 {
     const uint32_t l = blockIdx.x * blockDim.x + threadIdx.x;
     if (l >= k.ladders) return;
-    uint32_t* hold = k.holder + (size_t)l * k.rungs;
+    uint32_t* hold = k.holder + (size_t)l * k.x.rungs;
     uint32_t tried = 0, done = 0;
-    for (uint32_t j = (uint32_t)(k.t & 1ull); j + 1 < k.rungs; j += 2) {
+    for (uint32_t j = (uint32_t)(k.t & 1ull); j + 1 < k.x.rungs; j += 2) {
         const uint32_t hot = hold[j], cold = hold[j + 1];
-        const uint64_t Eh = k.results[hot].final_ticks, Ec = k.results[cold].final_ticks;
-        bool accept;
-        if (Eh <= Ec || k.xalways[j]) {
-            accept = true;                                // the colder rung holds the worse schedule (or an equal one)
-        } else {
-            uint32_t x[4];
-            philox4x32_10((uint32_t)k.t, (uint32_t)(k.t >> 32), (k.first_ladder + l) * k.rungs + j, TAG_EXCHANGE, k.seed_lo,
-                          k.seed_hi, x);
-            const uint64_t q = (Eh - Ec) >> k.xshifts[j];
-            accept = q < KVP_TABLE_Q && x[3] < k.xtable[(size_t)j * KVP_TABLE_Q + q];
-        }
+        const bool accept = exchange_accepts(k.x, k.t, (k.first_ladder + l) * k.x.rungs, j, k.results[hot].final_ticks,
+                                             k.results[cold].final_ticks);
         ++tried;
         if (accept) {
             hold[j] = cold; hold[j + 1] = hot;
@@ -1775,10 +1114,10 @@ exchange_kernel(const ExchangeK k)
             ++done;
         }
     }
-    for (uint32_t j = 0; j < k.rungs; ++j) k.rung_next[hold[j]] = (uint8_t)j;
+    for (uint32_t j = 0; j < k.x.rungs; ++j) k.rung_next[hold[j]] = (uint8_t)j;
     if (tried) {
-        atomicAdd(k.counts, (unsigned long long)tried);
-        atomicAdd(k.counts + 1, (unsigned long long)done);
+        atomicAdd(k.x.counts, (unsigned long long)tried);
+        atomicAdd(k.x.counts + 1, (unsigned long long)done);
     }
 }
 
@@ -1824,9 +1163,12 @@ struct Ctx {
     size_t smem_per_warp;    // shared memory per chain
     size_t smem_shared;      // shared memory of the CTA beside its chains (access bitmap and step constants)
     bool asmem;              // the access bitmap and the step constants are staged in shared memory
-    bool wide;               // the wide kernel (one warp per chain, four proposals per lane)
+    bool wide;               // the wide kernel
     uint32_t S32;            // words per time-packed column
-    bool stage_stepc;        // wide kernel: the step constants are staged in shared memory without the access bitmap
+    bool ladder_ctas;        // replica exchange: every CTA holds whole ladders (one launch)
+    int rows;                // wide kernel: rows of 32 proposals in a batch
+    bool lin;                // kappa_d >= kappa_k: see kvp_chain.cuh
+    float* bounds;           // [levels]
     std::vector<double> temps;
     uint64_t init_ticks, calib_mean;
     uint32_t launches;
@@ -1847,36 +1189,56 @@ int validate(const kvp_problem* p, const kvp_anneal_params* a)
 typedef void (*ChainKernel)(const ChainParams);
 
 template <bool PSMEM, bool ASMEM, bool COW>
-ChainKernel chain_kernel_pick(bool grow, uint32_t W)
+ChainKernel narrow_kernel_pick(bool grow, uint32_t W)
 {
-    if (W == 2) return grow ? chain_kernel<PSMEM, true, 2, ASMEM, COW> : chain_kernel<PSMEM, false, 2, ASMEM, COW>;
-    return grow ? chain_kernel<PSMEM, true, 1, ASMEM, COW> : chain_kernel<PSMEM, false, 1, ASMEM, COW>;
+    if (W == 2) return grow ? narrow_chain_kernel<PSMEM, true, 2, ASMEM, COW> : narrow_chain_kernel<PSMEM, false, 2, ASMEM, COW>;
+    return grow ? narrow_chain_kernel<PSMEM, true, 1, ASMEM, COW> : narrow_chain_kernel<PSMEM, false, 1, ASMEM, COW>;
 }
 
-ChainKernel chain_kernel_for(bool psmem, bool asmem, bool grow, uint32_t W, bool cow)
+ChainKernel narrow_kernel_for(bool psmem, bool asmem, bool grow, uint32_t W, bool cow)
 {
-    if (!psmem) return cow ? chain_kernel_pick<false, false, true>(grow, W) : chain_kernel_pick<false, false, false>(grow, W);
-    return asmem ? chain_kernel_pick<true, true, false>(grow, W) : chain_kernel_pick<true, false, false>(grow, W);
+    if (!psmem) return cow ? narrow_kernel_pick<false, false, true>(grow, W) : narrow_kernel_pick<false, false, false>(grow, W);
+    return asmem ? narrow_kernel_pick<true, true, false>(grow, W) : narrow_kernel_pick<true, false, false>(grow, W);
 }
 
-ChainKernel wide_kernel_for(bool psmem, bool asmem, bool grow, uint32_t S32)
+template <bool PSMEM, bool ASMEM, bool LIN, int COLV>
+ChainKernel wide_pick(bool grow, int rows)
+{
+    if (!PSMEM && LIN && rows == kRowsOne)
+        return grow ? wide_chain_kernel<PSMEM, true, ASMEM, LIN, COLV, !PSMEM && LIN ? kRowsOne : kRowsMany>
+                    : wide_chain_kernel<PSMEM, false, ASMEM, LIN, COLV, !PSMEM && LIN ? kRowsOne : kRowsMany>;
+    return grow ? wide_chain_kernel<PSMEM, true, ASMEM, LIN, COLV, kRowsMany> : wide_chain_kernel<PSMEM, false, ASMEM, LIN, COLV, kRowsMany>;
+}
+
+ChainKernel wide_kernel_for(bool psmem, bool asmem, bool grow, bool lin, uint32_t S32, int rows)
 {
     if (!psmem) {
-        if (S32 == 2) return grow ? wide_chain_kernel<false, true, false, 2> : wide_chain_kernel<false, false, false, 2>;
-        if (S32 == 4) return grow ? wide_chain_kernel<false, true, false, 4> : wide_chain_kernel<false, false, false, 4>;
-        return grow ? wide_chain_kernel<false, true, false, 0> : wide_chain_kernel<false, false, false, 0>;
+        if (lin && S32 == 2) return wide_pick<false, false, true, 2>(grow, rows);
+        if (lin && S32 == 4) return wide_pick<false, false, true, 4>(grow, rows);
+        return lin ? wide_pick<false, false, true, 0>(grow, rows) : wide_pick<false, false, false, 0>(grow, rows);
     }
-    if (asmem) return grow ? wide_chain_kernel<true, true, true, 0> : wide_chain_kernel<true, false, true, 0>;
-    return grow ? wide_chain_kernel<true, true, false, 0> : wide_chain_kernel<true, false, false, 0>;
+    if (asmem && lin) return wide_pick<true, true, true, 0>(grow, rows);
+    return lin ? wide_pick<true, false, true, 0>(grow, rows) : wide_pick<true, false, false, 0>(grow, rows);
 }
 
 ChainKernel kernel_of(const Ctx& c, bool psmem, bool asmem, uint32_t W)
 {
-    return c.wide ? wide_kernel_for(psmem, asmem, c.grow, c.S32) : chain_kernel_for(psmem, asmem, c.grow, W, c.cow_slots4 != 0);
+    return c.wide ? wide_kernel_for(psmem, asmem, c.grow, c.lin, c.S32, c.rows)
+                  : narrow_kernel_for(psmem, asmem, c.grow, W, c.cow_slots4 != 0);
 }
 
-int launch_chains(const Ctx& c, const ChainParams& prm, uint32_t count)
+int launch_chains(const Ctx& c, ChainParams& prm, uint32_t count)
 {
+    if (c.wide) {
+        const bool rounds = prm.rung_hist != nullptr;
+        prm.lay = chain_layout(prm.S, prm.S32, c.grow, c.psmem, c.lin, c.psmem ? 0u : c.cow_slots4);
+        prm.seg_len = rounds ? prm.exch_every : prm.per_level;
+        prm.seg_bat = (uint32_t)((prm.seg_len + 32 * c.rows - 1) / (32 * c.rows));
+        const uint64_t needed = (prm.upto + prm.seg_len - 1) / prm.seg_len;
+        prm.seg0 = rounds ? prm.round0 : 0u;
+        prm.seg1 = (uint32_t)std::min<uint64_t>(rounds ? prm.round1 : prm.levels, needed);
+        if (rounds && prm.seg1 < needed) prm.upto = prm.seg1 * prm.seg_len;   // the last segment is a whole one
+    }
     const uint32_t grid = (count + c.wpb - 1) / c.wpb;
     const size_t smem = (size_t)c.wpb * c.smem_per_warp + c.smem_shared;
     kernel_of(c, c.psmem, c.asmem, c.wpc)<<<grid, c.wpb * c.wpc * 32, smem, c.st>>>(prm);
@@ -1891,7 +1253,6 @@ int run_chains(Ctx& c, uint32_t first, uint32_t count, uint32_t result_base, kvp
     prm.snap = snap;
     prm.undo_log = with_undo ? c.undo_log : nullptr; prm.undo_len = c.undo_len; prm.undo_cap = c.undo_cap;
     prm.cow_out = c.cow_out; prm.cow_shift = c.cow_shift; prm.cow_slots4 = c.cow_slots4;
-    prm.stage_stepc = c.stage_stepc ? 1u : 0u;
     prm.chain_first = first; prm.chain_count = count; prm.result_base = result_base;
     prm.results = results; prm.upto = upto; prm.dump = dump;
     ++c.launches;
@@ -1899,7 +1260,8 @@ int run_chains(Ctx& c, uint32_t first, uint32_t count, uint32_t result_base, kvp
 }
 
 // Initial schedule, its counters and cost, the temperature ladder and the acceptance table.
-int prepare(kvp_problem* p, const kvp_anneal_params* a, cudaStream_t st, Ctx& c, bool exchange = false)
+// rungs: 0, or the chains of a ladder (replica exchange).
+int prepare(kvp_problem* p, const kvp_anneal_params* a, cudaStream_t st, Ctx& c, uint32_t rungs = 0)
 {
     int rc = validate(p, a);
     if (rc) return rc;
@@ -1918,132 +1280,138 @@ int prepare(kvp_problem* p, const kvp_anneal_params* a, cudaStream_t st, Ctx& c,
     c.grow = p->dL != nullptr;
     const kvp_test_hooks hooks = g_hooks;
     c.S32 = p->S32;
-    // Which kernel. Many chains per SM (more than 8, the jobs that fill the registers of an SM with one warp per
-    // chain; more than 5 when the schedules fit shared memory): the wide kernel, which needs half the instructions
-    // per proposal. Fewer chains per SM: the narrow kernel with two warps per chain, which hides the latency of a
-    // chain's serial parts behind its second warp. A hot start (C_0 from p0 >= 0.5: a fifth of the proposals change
-    // the schedule and the chain is a sequence of applied moves) on few chains: the narrow kernel with one warp per
-    // chain, whose path through an applied move is the shortest.
-    // kvp_set_test_hooks can force either (warps_per_chain 1 or 2: narrow; 3: wide).
+    const bool exchange = rungs != 0;
     const uint32_t chains_per_sm = (a->chains + sms - 1) / sms;
     const size_t pbytes = (size_t)p->U * p->S32 * 4;
     const bool hot = !a->temps && a->p0 >= 0.5;
-    const bool wide_in_smem = p->U < 65536u && (size_t)wide_fixed4(p->S, p->S32, c.grow, true, 0u) * 16 + pbytes <= budget / 2;
-    c.wide = exchange || hooks.warps_per_chain == 3 ||
-             (hooks.warps_per_chain == 0 && (chains_per_sm > 8 || (wide_in_smem && chains_per_sm > 5 && !hot)));
-    // `shared`: the schedule is in shared memory (the wide kernel then keeps 16-bit counters)
-    auto fixed_bytes = [&](uint32_t W, bool halfq = false, bool shared = true) {
-        if (c.wide) return (size_t)wide_fixed4(p->S, p->S32, c.grow, shared, shared ? 0u : c.cow_slots4) * 16;
-        return (size_t)chain_fixed4(p->S, p->S32, c.grow, W, halfq, shared ? 0u : c.cow_slots4) * 16;
-    };
-    c.stage_stepc = false;
+    c.lin = p->K.kd >= p->K.kk;
+    c.ladder_ctas = false;
+    c.rows = kRowsMany;
     c.cow_slots4 = 0;
     c.cow_shift = 0;
-    // Two warps per chain while that leaves an SM at most 16 warps (the registers allow no more): a job of few
-    // chains then keeps twice as many warps in flight. kvp_set_test_hooks can override the choice (tests, tuning).
-    uint32_t W = chains_per_sm <= 8 && !hot ? 2u : 1u;
-    if (hooks.warps_per_chain == 1 || hooks.warps_per_chain == 2) W = hooks.warps_per_chain;
-    if (c.wide) W = 1;
-    c.psmem = fixed_bytes(1) + pbytes <= budget / 2 && (!c.wide || p->U < 65536u);
+    c.smem_shared = 0;
+    c.asmem = false;
+    auto fixed_bytes = [&](uint32_t warps, bool halfq, bool shared) {
+        if (c.wide) return chain_bytes(p->S, p->S32, c.grow, shared, c.lin, shared ? 0u : c.cow_slots4, warps, c.rows);
+        return (size_t)chain_fixed4(p->S, p->S32, c.grow, warps, halfq, shared ? 0u : c.cow_slots4) * 16;
+    };
+    // Which kernel. The wide one, but for two kinds of jobs whose chains apply so many of their moves that evaluations far
+    // ahead of the commits do not last, where the narrow kernel's batches of 32 and its shorter path through an applied
+    // move win: hot starts (C_0 from p0 >= 0.5: a fifth of the proposals change the schedule; 256 units x 512 steps,
+    // 1024 chains x 100,000 moves: 25.5 ms with one narrow warp per chain, 34 on the wide kernel), and few chains on
+    // schedules too large for shared memory (16,384 units x 256 steps, 740 chains: 6.4 against 8.0 ms; 1024 chains:
+    // 15.4 against 14.2) or of hardly any units (16 units, 64 chains: 0.43 against 0.55).
+    // kvp_set_test_hooks can force either (warps_per_chain 1 or 2: narrow; 3 or 16 + w: wide).
+    c.wide = true;
+    c.psmem = fixed_bytes(1, false, true) + pbytes + 16 <= budget / 2 && p->U < 65536u;
+    if (hooks.warps_per_chain) c.wide = hooks.warps_per_chain >= 3;
+    else if (hot) c.wide = false;
+    else c.wide = c.psmem ? p->U >= 64u : chains_per_sm > 6;
+    if (exchange) c.wide = true;
+    if (!c.wide) c.psmem = fixed_bytes(1, false, true) + pbytes <= budget / 2;
+    const uint32_t forced = hooks.warps_per_chain == 3 ? 1u : hooks.warps_per_chain >= 16 ? hooks.warps_per_chain - 16u : hooks.warps_per_chain;
+    const uint32_t full = 16;                                     // warps of a CTA that fills an SM (at 128 registers)
+    uint32_t W = 1;
     if (c.psmem) {
         uint32_t want = chains_per_sm < 1 ? 1 : chains_per_sm;
-        if (W == 2 && (want > 8 || (fixed_bytes(2) + pbytes) * want > budget) && (fixed_bytes(1) + pbytes) * want <= budget)
-            W = 1;                                                 // the second warp's work area does not fit
-        c.smem_per_warp = fixed_bytes(W) + pbytes;
-        uint32_t wmax = (uint32_t)(budget / c.smem_per_warp);
-        if (wmax > (c.wide ? 8u : 16u / W)) wmax = c.wide ? 8u : 16u / W;   // the wide kernel is built for CTAs of up to 256 threads
-        c.wpb = want > wmax ? wmax : want;
+        if (exchange) want = (want + rungs - 1) / rungs * rungs;  // whole ladders
+        // bytes with the access bitmap and (narrow) the step constants staged; wide: columns are followed by readable bytes
+        auto with_a = [&](uint32_t chains, uint32_t warps) {
+            const size_t a_off = ((size_t)chains * (pbytes / 4) + 3) & ~(size_t)3, c_off = (a_off + pbytes / 4 + 3) & ~(size_t)3;
+            return (size_t)chains * fixed_bytes(warps, true, true) + c_off * 4 + (c.wide ? 16 : (size_t)p->S * 16);
+        };
+        if (c.wide) {
+            // two warps per chain, four where an SM has three chains or fewer (256 units x 512 steps, 50,000 moves, 148 and
+            // 740 chains: one warp 1.62 and 1.79 ms, two 1.12 and 1.34, four 1.05 and 2.40)
+            W = chains_per_sm <= 3 ? 4 : 2;
+            while (W > 1 && (want * W > full || with_a(want, W) > budget)) W /= 2;
+        } else if (!hot) {
+            W = 2;                                                // hides the latency of a chain's serial parts
+            if (chains_per_sm > 8 || ((fixed_bytes(2, false, true) + pbytes) * want > budget && (fixed_bytes(1, false, true) + pbytes) * want <= budget))
+                W = 1;
+        }
+        if (forced) W = forced;
         c.wpc = W;
+        c.smem_per_warp = fixed_bytes(W, false, true) + pbytes;
+        uint32_t wmax = (uint32_t)((budget - 16) / c.smem_per_warp);
+        if (wmax > full / W) wmax = full / W;
+        if (wmax < 1) return KVP_ERR_RANGE;
+        c.wpb = want > wmax ? wmax : want;
+        if (exchange && rungs <= wmax) {
+            c.ladder_ctas = true;
+            c.wpb = c.wpb / rungs * rungs;
+        }
         c.resident = a->chains;
-        // the access bitmap and the step constants beside the schedules, if there is room (the offsets are the kernel's)
-        const size_t a_off = ((size_t)c.wpb * (pbytes / 4) + 3) & ~(size_t)3, c_off = (a_off + pbytes / 4 + 3) & ~(size_t)3;
-        const size_t with_a = (size_t)c.wpb * fixed_bytes(W, true) + c_off * 4 + (size_t)p->S * 16;
-        c.asmem = with_a <= budget;
-        if (c.asmem) {                                           // that kernel makes do with half the work queue
-            c.smem_per_warp = fixed_bytes(W, true) + pbytes;
-            c.smem_shared = with_a - (size_t)c.wpb * c.smem_per_warp;
-        } else {
-            c.smem_shared = 0;
-            // the wide kernel stages at least the step constants when they fit
-            const size_t with_c = (size_t)c.wpb * c.smem_per_warp + 16 + (size_t)p->S * 16;
-            if (c.wide && with_c <= budget) {
-                c.stage_stepc = true;
-                c.smem_shared = with_c - (size_t)c.wpb * c.smem_per_warp;
-            }
+        c.smem_shared = c.wide ? 16 : 0;
+        c.asmem = with_a(c.wpb, W) <= budget && (!c.wide || c.lin);
+        if (c.asmem) {                                            // (the narrow kernel then makes do with half the work queue)
+            c.smem_per_warp = fixed_bytes(W, true, true) + pbytes;
+            c.smem_shared = with_a(c.wpb, W) - (size_t)c.wpb * c.smem_per_warp;
         }
         KVP_CUDA(cudaFuncSetAttribute(kernel_of(c, true, c.asmem, W), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)budget));
     } else {
-        {
-            // Copy-on-write slices: always for the wide kernel; for the narrow kernel where whole copies of the initial
-            // schedule would add up to gigabytes (growing_8b: 1024 x 17 MB, a third of the kernel's time), not where
-            // they are small (layer_8b: 1024 x 512 KB), because a take-over lengthens the path through an applied move
-            // (layer_8b 14.0 -> 16.0 ms with it).
-            const size_t per_sm_max = c.wide ? kWideGlobalThreads / 32 : 16 / W;
-            const size_t most = a->chains < per_sm_max * sms ? a->chains : per_sm_max * sms;
-            const bool overlay = c.wide || (hooks.overlay ? hooks.overlay == 1 : most * col_bytes >= ((size_t)4 << 30));
-            c.cow_slots4 = 0;
-            c.cow_shift = 0;
-            if (overlay) {
-                // The bucket bitmap takes what a full CTA of chains leaves of the shared memory: the smaller the
-                // buckets, the fewer reads of a long chain go to its private slice.
-                const size_t bare = fixed_bytes(W, false, false);
-                const size_t stepc_bytes = c.wide && (size_t)p->S * 16 <= 32768 ? (size_t)p->S * 16 : 0;
-                uint32_t per_cta = c.wide ? kWideGlobalThreads / 32 : 16 / W;     // chains of a full CTA
-                if (chains_per_sm < per_cta) per_cta = chains_per_sm ? chains_per_sm : 1u;
-                if ((budget - stepc_bytes) / bare < per_cta) per_cta = (uint32_t)((budget - stepc_bytes) / bare);
-                if (per_cta < 1) return KVP_ERR_RANGE;
-                const size_t share = (budget - stepc_bytes) / per_cta;
-                size_t bits = share > bare ? (share - bare) / 16 * 128 : 0;
-                if (bits < kCowBitsMin) bits = kCowBitsMin;
-                if (bits > kCowBitsMax) bits = kCowBitsMax;
-                c.cow_shift = 0;
-                while (((uint64_t)p->U + (1ull << c.cow_shift) - 1) >> c.cow_shift > bits) ++c.cow_shift;
-                const uint64_t buckets = ((uint64_t)p->U + (1ull << c.cow_shift) - 1) >> c.cow_shift;
-                c.cow_slots4 = (uint32_t)((buckets + 127) / 128);
-            }
-            const size_t ctr_bytes = fixed_bytes(W, false, false);
-            if (ctr_bytes > budget) return KVP_ERR_RANGE;
-            c.smem_per_warp = ctr_bytes;
-            c.smem_shared = 0;
-            c.asmem = false;
-            c.wpc = W;
-            // the wide kernel stages the step constants once per CTA when they are small
-            c.stage_stepc = c.wide && (size_t)p->S * 16 <= 32768 && ctr_bytes + (size_t)p->S * 16 <= budget;
-            if (c.stage_stepc) c.smem_shared = (size_t)p->S * 16;
-            uint32_t wcap = (uint32_t)((budget - c.smem_shared) / ctr_bytes);   // chains per CTA at most
-            if (wcap > 16 / W) wcap = 16 / W;
-            if (c.wide && wcap > kWideGlobalThreads / 32) wcap = kWideGlobalThreads / 32;
-            KVP_CUDA(cudaFuncSetAttribute(kernel_of(c, false, false, W), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)budget));
-            int ctas = 0;
-            KVP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ctas, kernel_of(c, false, false, W), (int)(wcap * W * 32),
-                                                                   wcap * c.smem_per_warp + c.smem_shared));
-            if (ctas < 1) return KVP_ERR_RANGE;
-            uint32_t per_sm = (uint32_t)ctas * wcap;                   // resident chains per SM, at most 32 warps
-            if (per_sm * W > 32) per_sm = 32 / W / wcap ? 32 / W / wcap * wcap : wcap;
-            size_t free_b = 0, total_b = 0;
-            KVP_CUDA(cudaMemGetInfo(&free_b, &total_b));
-            free_b += p->chain_ws_bytes;                               // what we already hold can be reused
-            {                                                          // and so can what the pool holds in reserve
-                cudaMemPool_t pool; uint64_t reserved = 0, used = 0;
-                if (cudaDeviceGetDefaultMemPool(&pool, dev) == cudaSuccess &&
-                    cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReservedMemCurrent, &reserved) == cudaSuccess &&
-                    cudaMemPoolGetAttribute(pool, cudaMemPoolAttrUsedMemCurrent, &used) == cudaSuccess && reserved > used)
-                    free_b += (size_t)(reserved - used);
-            }
-            const size_t usable = free_b / 10 * 7;
-            size_t fit = usable / col_bytes;
-            if (fit < 1) return KVP_ERR_NOMEM;
-            size_t cap_r = (size_t)per_sm * sms;
-            size_t r = a->chains < cap_r ? a->chains : cap_r;
-            if (r > fit) r = fit;
-            // test hook: at most n chains at a time, so that small jobs come in several waves
-            if (hooks.resident >= 1 && (size_t)hooks.resident < r) r = hooks.resident;
-            const uint32_t waves = (uint32_t)((a->chains + r - 1) / r);
-            c.resident = (a->chains + waves - 1) / waves;              // equal waves
-            // a wave is spread over all SMs: CTAs of ceil(resident / SMs) chains where one CTA per SM holds them
-            const uint32_t even = (c.resident + sms - 1) / sms;
-            c.wpb = even < wcap ? even : wcap;
+        // Two warps per chain while that leaves an SM at most 16 warps (the registers allow no more). More per chain are no
+        // faster (16,384 units x 256 steps, 148 chains: 6.76 ms with two and with four, 7.5 with one).
+        if (!exchange && chains_per_sm <= 8 && !(hot && !c.wide)) W = 2;
+        if (forced) W = forced;
+        if (W == 1 && c.wide && c.lin) c.rows = kRowsOne;
+        uint32_t per_cta = full / W;                              // chains of a full CTA
+        if (chains_per_sm < per_cta) per_cta = chains_per_sm ? chains_per_sm : 1u;
+        // Copy-on-write slices: always for the wide kernel; for the narrow kernel where whole copies of the initial
+        // schedule would add up to gigabytes (growing_8b: 1024 x 17 MB, a third of the kernel's time), not where they are
+        // small (layer_8b: 1024 x 512 KB), because a take-over lengthens the path through an applied move (layer_8b
+        // 14.0 -> 16.0 ms with it).
+        const size_t most = a->chains < (size_t)full / W * sms ? a->chains : (size_t)full / W * sms;
+        const bool overlay = c.wide || (hooks.overlay ? hooks.overlay == 1 : most * col_bytes >= ((size_t)4 << 30));
+        if (overlay) {
+            // The bucket bitmap takes what a full CTA of chains leaves of the shared memory: the smaller the buckets, the
+            // fewer reads of a long chain go to its private slice.
+            const size_t bare = fixed_bytes(W, false, false);
+            if (budget / bare < per_cta) per_cta = (uint32_t)(budget / bare);
+            if (per_cta < 1) return KVP_ERR_RANGE;
+            const size_t share = budget / per_cta;
+            size_t bits = share > bare ? (share - bare) / 16 * 128 : 0;
+            if (bits < kCowBitsMin) bits = kCowBitsMin;
+            if (bits > kCowBitsMax) bits = kCowBitsMax;
+            while (((uint64_t)p->U + (1ull << c.cow_shift) - 1) >> c.cow_shift > bits) ++c.cow_shift;
+            const uint64_t buckets = ((uint64_t)p->U + (1ull << c.cow_shift) - 1) >> c.cow_shift;
+            c.cow_slots4 = (uint32_t)((buckets + 127) / 128);
         }
+        c.smem_per_warp = fixed_bytes(W, false, false);
+        if (c.smem_per_warp > budget) return KVP_ERR_RANGE;
+        c.wpc = W;
+        uint32_t wcap = (uint32_t)(budget / c.smem_per_warp);     // chains per CTA at most
+        if (wcap > full / W) wcap = full / W;
+        KVP_CUDA(cudaFuncSetAttribute(kernel_of(c, false, false, W), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)budget));
+        int ctas = 0;
+        KVP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ctas, kernel_of(c, false, false, W), (int)(wcap * W * 32),
+                                                               wcap * c.smem_per_warp));
+        if (ctas < 1) return KVP_ERR_RANGE;
+        uint32_t per_sm = (uint32_t)ctas * wcap;                   // resident chains per SM, at most 32 warps
+        if (per_sm * W > 32) per_sm = 32 / W / wcap ? 32 / W / wcap * wcap : wcap;
+        size_t free_b = 0, total_b = 0;
+        KVP_CUDA(cudaMemGetInfo(&free_b, &total_b));
+        free_b += p->chain_ws_bytes;                               // what we already hold can be reused
+        {                                                          // and so can what the pool holds in reserve
+            cudaMemPool_t pool; uint64_t reserved = 0, used = 0;
+            if (cudaDeviceGetDefaultMemPool(&pool, dev) == cudaSuccess &&
+                cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReservedMemCurrent, &reserved) == cudaSuccess &&
+                cudaMemPoolGetAttribute(pool, cudaMemPoolAttrUsedMemCurrent, &used) == cudaSuccess && reserved > used)
+                free_b += (size_t)(reserved - used);
+        }
+        const size_t usable = free_b / 10 * 7;
+        size_t fit = usable / col_bytes;
+        if (fit < 1) return KVP_ERR_NOMEM;
+        size_t cap_r = (size_t)per_sm * sms;
+        size_t r = a->chains < cap_r ? a->chains : cap_r;
+        if (r > fit) r = fit;
+        // test hook: at most n chains at a time, so that small jobs come in several waves
+        if (hooks.resident >= 1 && (size_t)hooks.resident < r) r = hooks.resident;
+        const uint32_t waves = (uint32_t)((a->chains + r - 1) / r);
+        c.resident = (a->chains + waves - 1) / waves;              // equal waves
+        // a wave is spread over all SMs: CTAs of ceil(resident / SMs) chains where one CTA per SM holds them
+        const uint32_t even = (c.resident + sms - 1) / sms;
+        c.wpb = even < wcap ? even : wcap;
     }
     // a replica-exchange run keeps every chain's slice between its rounds: all chains have to be resident at once
     if (exchange && !c.psmem && a->chains > c.resident) return KVP_ERR_RANGE;
@@ -2052,7 +1420,7 @@ int prepare(kvp_problem* p, const kvp_anneal_params* a, cudaStream_t st, Ctx& c,
     size_t off = 0;
     auto take = [&](size_t bytes) { size_t o = off; off += align256(bytes); return o; };
     const size_t o_P0 = take(sched_bytes), o_col0 = take(col_bytes), o_cnt = take((size_t)p->S * 16);
-    const size_t o_small = take(256), o_table = take((size_t)a->levels * KVP_TABLE_Q * 4), o_shift = take((size_t)a->levels * 4);
+    const size_t o_small = take(256), o_table = take((size_t)a->levels * KVP_TABLE_Q * 4), o_shift = take((size_t)a->levels * 4), o_bound = take((size_t)a->levels * 4);
     const size_t o_res = take((size_t)(a->chains + 1) * sizeof(kvp_chain_result));
     const size_t o_dump = take(col_bytes), o_sched = take(sched_bytes);
     const size_t o_slots = take(c.psmem ? 0 : (size_t)c.resident * col_bytes);
@@ -2076,6 +1444,7 @@ int prepare(kvp_problem* p, const kvp_anneal_params* a, cudaStream_t st, Ctx& c,
     char* base = static_cast<char*>(p->d_chain_ws);
     c.P0 = (uint32_t*)(base + o_P0); c.Pcol0 = (uint32_t*)(base + o_col0); c.counts0 = (uint32_t*)(base + o_cnt);
     c.small = (uint64_t*)(base + o_small); c.table = (uint32_t*)(base + o_table); c.shifts = (uint32_t*)(base + o_shift);
+    c.bounds = (float*)(base + o_bound);
     c.results = (kvp_chain_result*)(base + o_res); c.dumpcol = (uint32_t*)(base + o_dump);
     c.sched = (uint32_t*)(base + o_sched); c.slots = (uint32_t*)(base + o_slots);
     c.hb0 = c.grow ? (uint32_t*)(base + o_hb0) : nullptr; c.hb_tmp = c.grow ? (uint32_t*)(base + o_hbt) : nullptr;
@@ -2117,7 +1486,7 @@ int prepare(kvp_problem* p, const kvp_anneal_params* a, cudaStream_t st, Ctx& c,
     ChainParams& prm = c.prm;
     memset(&prm, 0, sizeof prm);
     prm.Acol = p->dAcol; prm.stepc = p->d_stepc; prm.counters0 = (const uint4*)c.counts0; prm.Pcol0 = c.Pcol0;
-    prm.table = c.table; prm.shifts = c.shifts; prm.ws = c.slots; prm.K = p->K; prm.full0 = c.full0;
+    prm.table = c.table; prm.shifts = c.shifts; prm.bounds = c.bounds; prm.warps = c.wpc; prm.ws = c.slots; prm.K = p->K; prm.full0 = c.full0;
     prm.birth = p->d_birth; prm.hb0 = c.hb0;
     prm.err = reinterpret_cast<uint32_t*>(c.small + 16);
     prm.work = nullptr;                                   // set by kvp_anneal for the chains of the search proper
@@ -2127,7 +1496,9 @@ int prepare(kvp_problem* p, const kvp_anneal_params* a, cudaStream_t st, Ctx& c,
     // test hook: batches with more than n < 496 queue items already take the two-halves path of the half-size work
     // queue, which ordinary inputs almost never reach
     prm.split_at = kQueueCap / 2;
+    prm.carry = kAccepted;
     if (hooks.split_queue_plus1 >= 1 && hooks.split_queue_plus1 - 1 < kQueueCap / 2) prm.split_at = hooks.split_queue_plus1 - 1;
+    if (hooks.split_queue_plus1 >= 1 && hooks.split_queue_plus1 <= kAccepted) prm.carry = hooks.split_queue_plus1;
     KVP_CUDA(cudaMemsetAsync(prm.err, 0, 4, st));
     prm.U = p->U; prm.S = p->S; prm.S32 = p->S32; prm.cap = p->cap;
     prm.levels = a->levels; prm.p_swap_256 = a->p_swap_256; prm.len_choices = a->max_len_log2 + 1;
@@ -2165,6 +1536,12 @@ int prepare(kvp_problem* p, const kvp_anneal_params* a, cudaStream_t st, Ctx& c,
     if ((rc = kvp_accept_table(c.temps.data(), a->levels, table.data(), shifts.data()))) return rc;
     KVP_CUDA(cudaMemcpyAsync(c.table, table.data(), table.size() * 4, cudaMemcpyHostToDevice, st));
     KVP_CUDA(cudaMemcpyAsync(c.shifts, shifts.data(), shifts.size() * 4, cudaMemcpyHostToDevice, st));
+    // the lower bounds of kvp_chain.cuh are sums of at most 31 steps' changes in 32 bits
+    const uint64_t step_max = 4ull * std::max(p->K.khF, p->K.kdF) + std::max(p->K.kh, p->K.ke) + 2ull * std::max(p->K.kh, p->K.kd);
+    std::vector<float> bounds(a->levels, INFINITY);
+    if (31 * step_max < (1ull << 30))
+        for (uint32_t j = 0; j < a->levels; ++j) bounds[j] = (float)((c.temps[j] >= 1.0 ? c.temps[j] : 1.0) * 0.69314718);
+    KVP_CUDA(cudaMemcpyAsync(c.bounds, bounds.data(), bounds.size() * 4, cudaMemcpyHostToDevice, st));
     KVP_CUDA(cudaStreamSynchronize(st));           // the host vectors go out of scope
     return KVP_OK;
 }
@@ -2382,7 +1759,7 @@ extern "C" int kvp_anneal_exchange(kvp_problem* p, const kvp_anneal_params* a, c
     } ev;
     for (; ev.n < 4; ++ev.n) KVP_CUDA(cudaEventCreate(&ev.e[ev.n]));
     KVP_CUDA(cudaEventRecord(ev[0], st));
-    if ((rc = prepare(p, a, st, c, true))) return rc;
+    if ((rc = prepare(p, a, st, c, xp->rungs))) return rc;
 
     // exchange thresholds of the pairs of neighbouring rungs: the move table's form at the pair temperatures
     const uint32_t pairs = rungs > 1 ? rungs - 1 : 1;
@@ -2392,7 +1769,7 @@ extern "C" int kvp_anneal_exchange(kvp_problem* p, const kvp_anneal_params* a, c
     if ((rc = kvp_accept_table(pair_temps.data(), pairs, xtable.data(), xshifts.data()))) return rc;
 
     // workspace of the run: rung history, holders, exchange counts, thresholds, the chains' saved states
-    const uint32_t persist4 = wide_persist4(p->S, p->S32, c.grow, c.psmem, c.cow_slots4);
+    const uint32_t persist4 = chain_layout(p->S, p->S32, c.grow, c.psmem, c.lin, c.psmem ? 0u : c.cow_slots4).work / 16;
     const size_t pwords = (size_t)p->U * p->S32;
     const uint32_t state4 = persist4 + (c.psmem ? (uint32_t)((pwords + 3) / 4) : 0u);
     size_t off = 0;
@@ -2422,7 +1799,6 @@ extern "C" int kvp_anneal_exchange(kvp_problem* p, const kvp_anneal_params* a, c
     ChainParams prm = c.prm;
     prm.snap = c.snap; prm.undo_log = nullptr;
     prm.cow_out = nullptr; prm.cow_shift = c.cow_shift; prm.cow_slots4 = c.cow_slots4;
-    prm.stage_stepc = c.stage_stepc ? 1u : 0u;
     prm.chain_first = a->first_chain; prm.chain_count = chains; prm.result_base = a->first_chain;
     prm.results = c.results; prm.upto = a->moves; prm.dump = nullptr;
     prm.rung_hist = hist; prm.exch_every = xp->exchange_every; prm.hist_stride = chains; prm.hist_base = a->first_chain;
@@ -2430,12 +1806,20 @@ extern "C" int kvp_anneal_exchange(kvp_problem* p, const kvp_anneal_params* a, c
     unsigned long long* work_dev = reinterpret_cast<unsigned long long*>(c.small + 24);
     KVP_CUDA(cudaMemsetAsync(work_dev, 0, 24, st));
     ExchangeK xk;
-    xk.results = c.results; xk.holder = holder; xk.n_exchanged = nex; xk.counts = counts;
-    xk.xalways = (const uint32_t*)(xw + o_alw); xk.xtable = (const uint32_t*)(xw + o_xt); xk.xshifts = (const uint32_t*)(xw + o_xsh);
-    xk.ladders = chains / rungs; xk.rungs = rungs; xk.first_ladder = a->first_chain / rungs;
-    xk.seed_lo = (uint32_t)a->seed; xk.seed_hi = (uint32_t)(a->seed >> 32);
-    for (uint32_t t = 0; t < rounds; ++t) {
-        prm.round0 = t; prm.round1 = t + 1; prm.resume = t > 0 ? 1u : 0u;
+    xk.results = c.results; xk.holder = holder; xk.n_exchanged = nex; xk.x.counts = counts;
+    xk.x.always = (const uint32_t*)(xw + o_alw); xk.x.table = (const uint32_t*)(xw + o_xt); xk.x.shifts = (const uint32_t*)(xw + o_xsh);
+    xk.ladders = chains / rungs; xk.x.rungs = rungs; xk.first_ladder = a->first_chain / rungs;
+    xk.x.seed_lo = (uint32_t)a->seed; xk.x.seed_hi = (uint32_t)(a->seed >> 32);
+    if (c.ladder_ctas) {
+        // every CTA holds whole ladders: one launch, the rounds end in a CTA barrier
+        prm.round0 = 0; prm.round1 = rounds; prm.state = nullptr;
+        prm.ladder_ctas = 1u; prm.ladder = xk.x; prm.n_exchanged = nex; prm.work = work_dev;
+        if ((rc = launch_chains(c, prm, chains))) return rc;
+        ++c.launches;
+        prm.ladder_ctas = 0u; prm.n_exchanged = nullptr;
+    }
+    for (uint32_t t = 0; t < rounds && !c.ladder_ctas; ++t) {
+        prm.round0 = t; prm.round1 = t + 1; prm.resume = t > 0 ? 1u : 0u; prm.upto = a->moves;
         prm.work = t + 1 == rounds ? work_dev : nullptr;   // the counts travel with the saved state; the last round reports
         if ((rc = launch_chains(c, prm, chains))) return rc;
         ++c.launches;
