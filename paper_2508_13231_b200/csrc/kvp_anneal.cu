@@ -942,6 +942,7 @@ narrow_chain_kernel(const ChainParams prm)
 }  // namespace kvp
 
 #include "kvp_chain.cuh"
+#include "kvp_hot.cuh"
 
 namespace kvp {
 
@@ -1165,6 +1166,7 @@ struct Ctx {
     bool asmem;              // the access bitmap and the step constants are staged in shared memory
     bool wide;               // the wide kernel
     uint32_t S32;            // words per time-packed column
+    bool hot;                // the sequential kernel (kvp_hot.cuh)
     bool ladder_ctas;        // replica exchange: every CTA holds whole ladders (one launch)
     int rows;                // wide kernel: rows of 32 proposals in a batch
     bool lin;                // kappa_d >= kappa_k: see kvp_chain.cuh
@@ -1223,13 +1225,14 @@ ChainKernel wide_kernel_for(bool psmem, bool asmem, bool grow, bool lin, uint32_
 
 ChainKernel kernel_of(const Ctx& c, bool psmem, bool asmem, uint32_t W)
 {
+    if (c.hot) return asmem ? hot_chain_kernel<true> : hot_chain_kernel<false>;
     return c.wide ? wide_kernel_for(psmem, asmem, c.grow, c.lin, c.S32, c.rows)
                   : narrow_kernel_for(psmem, asmem, c.grow, W, c.cow_slots4 != 0);
 }
 
 int launch_chains(const Ctx& c, ChainParams& prm, uint32_t count)
 {
-    if (c.wide) {
+    if (c.wide || c.hot) {
         const bool rounds = prm.rung_hist != nullptr;
         prm.lay = chain_layout(prm.S, prm.S32, c.grow, c.psmem, c.lin, c.psmem ? 0u : c.cow_slots4);
         prm.seg_len = rounds ? prm.exch_every : prm.per_level;
@@ -1291,7 +1294,9 @@ int prepare(kvp_problem* p, const kvp_anneal_params* a, cudaStream_t st, Ctx& c,
     c.cow_shift = 0;
     c.smem_shared = 0;
     c.asmem = false;
+    c.hot = false;
     auto fixed_bytes = [&](uint32_t warps, bool halfq, bool shared) {
+        if (c.hot) return (size_t)hot_stride(p->S, p->S32);
         if (c.wide) return chain_bytes(p->S, p->S32, c.grow, shared, c.lin, shared ? 0u : c.cow_slots4, warps, c.rows);
         return (size_t)chain_fixed4(p->S, p->S32, c.grow, warps, halfq, shared ? 0u : c.cow_slots4) * 16;
     };
@@ -1304,12 +1309,14 @@ int prepare(kvp_problem* p, const kvp_anneal_params* a, cudaStream_t st, Ctx& c,
     // kvp_set_test_hooks can force either (warps_per_chain 1 or 2: narrow; 3 or 16 + w: wide).
     c.wide = true;
     c.psmem = fixed_bytes(1, false, true) + pbytes + 16 <= budget / 2 && p->U < 65536u;
-    if (hooks.warps_per_chain) c.wide = hooks.warps_per_chain >= 3;
+    if (hooks.warps_per_chain) c.wide = hooks.warps_per_chain == 3 || hooks.warps_per_chain >= 16;
     else if (hot) c.wide = false;
-    else c.wide = c.psmem ? p->U >= 64u : chains_per_sm > 6;
+    else c.wide = c.psmem ? (uint64_t)p->U * p->S >= 4096u : p->U >= 32768u || chains_per_sm > 6;
     if (exchange) c.wide = true;
+    c.hot = !c.wide && (hooks.warps_per_chain ? hooks.warps_per_chain == 4 : hot) && c.lin && !c.grow && p->U < 65536u &&
+            hot_stride(p->S, p->S32) + pbytes + 16 <= budget / 2;
     if (!c.wide) c.psmem = fixed_bytes(1, false, true) + pbytes <= budget / 2;
-    const uint32_t forced = hooks.warps_per_chain == 3 ? 1u : hooks.warps_per_chain >= 16 ? hooks.warps_per_chain - 16u : hooks.warps_per_chain;
+    const uint32_t forced = hooks.warps_per_chain == 3 || hooks.warps_per_chain == 4 ? 1u : hooks.warps_per_chain >= 16 ? hooks.warps_per_chain - 16u : hooks.warps_per_chain;
     const uint32_t full = 16;                                     // warps of a CTA that fills an SM (at 128 registers)
     uint32_t W = 1;
     if (c.psmem) {
@@ -1318,7 +1325,7 @@ int prepare(kvp_problem* p, const kvp_anneal_params* a, cudaStream_t st, Ctx& c,
         // bytes with the access bitmap and (narrow) the step constants staged; wide: columns are followed by readable bytes
         auto with_a = [&](uint32_t chains, uint32_t warps) {
             const size_t a_off = ((size_t)chains * (pbytes / 4) + 3) & ~(size_t)3, c_off = (a_off + pbytes / 4 + 3) & ~(size_t)3;
-            return (size_t)chains * fixed_bytes(warps, true, true) + c_off * 4 + (c.wide ? 16 : (size_t)p->S * 16);
+            return (size_t)chains * fixed_bytes(warps, true, true) + c_off * 4 + (c.wide || c.hot ? 16 : (size_t)p->S * 16);
         };
         if (c.wide) {
             // two warps per chain, four where an SM has three chains or fewer (256 units x 512 steps, 50,000 moves, 148 and
@@ -1335,6 +1342,7 @@ int prepare(kvp_problem* p, const kvp_anneal_params* a, cudaStream_t st, Ctx& c,
         c.smem_per_warp = fixed_bytes(W, false, true) + pbytes;
         uint32_t wmax = (uint32_t)((budget - 16) / c.smem_per_warp);
         if (wmax > full / W) wmax = full / W;
+        if (c.hot && wmax > 8u) wmax = 8u;                        // the sequential kernel is built for CTAs of up to 256 threads
         if (wmax < 1) return KVP_ERR_RANGE;
         c.wpb = want > wmax ? wmax : want;
         if (exchange && rungs <= wmax) {
@@ -1342,7 +1350,7 @@ int prepare(kvp_problem* p, const kvp_anneal_params* a, cudaStream_t st, Ctx& c,
             c.wpb = c.wpb / rungs * rungs;
         }
         c.resident = a->chains;
-        c.smem_shared = c.wide ? 16 : 0;
+        c.smem_shared = c.wide || c.hot ? 16 : 0;
         c.asmem = with_a(c.wpb, W) <= budget && (!c.wide || c.lin);
         if (c.asmem) {                                            // (the narrow kernel then makes do with half the work queue)
             c.smem_per_warp = fixed_bytes(W, true, true) + pbytes;
