@@ -7,7 +7,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libkvp.so")
 SOURCES = ["kvp_api.cu", "kvp_cost.cu", "kvp_layout.cu", "kvp_anneal.cu", "kvp_trace.cu", "kvp_policy.cu", "kvp_table.cpp"]
-HEADERS = ["kvp_common.cuh", "kvp_chain.cuh", "kvp_hot.cuh"]
+HEADERS = ["kvp_common.cuh", "kvp_chain.cuh", "kvp_narrow.cuh"]
 
 
 def _nvcc():

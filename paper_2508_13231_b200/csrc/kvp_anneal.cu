@@ -58,7 +58,6 @@ struct ChainParams {
     uint32_t undo_cap;
     uint32_t* err;               // set to 1 by a warp that gave up waiting for its turn
     uint32_t drop_first_turn;    // test hook: the owner of batch 0 never passes the turn on, so the next wait runs out
-    uint32_t split_at;           // a batch with more queue items than this goes in two halves (kQueueCap / 2; less in tests)
     const uint32_t* birth;       // growing cache: [U] step at which a unit is written (0 = there from the start)
     const uint32_t* hb0;         // growing cache: [S] units written to HBM at birth under the initial schedule
     CostK K;
@@ -96,17 +95,6 @@ struct ChainParams {
     ExchangeArgs ladder;
     uint32_t* n_exchanged;       // replica exchange in the CTA: by chain
 };
-
-// Batches: every lane of a chain's warp carries kMPL proposals, so a batch is 32 * kMPL consecutive moves.
-constexpr int kMPL = 1;
-constexpr uint32_t kBatch = 32 * kMPL;
-constexpr uint32_t kWinSlots4 = kBatch * 2;                        // 8 words of windows per proposal
-constexpr uint32_t kAccSlots4 = kBatch / 4;                        // one int per proposal
-// uint16 work items, 31 per proposal in the worst case. Where shared memory is short (HALFQ) the queue holds the worst
-// case of half a warp's proposals and a batch with more items than that is worked off in two halves.
-constexpr uint32_t kQueueCap = kBatch * 31;
-constexpr uint32_t kQueueSlots4 = (kQueueCap * 2 + 15) / 16;
-constexpr uint32_t kHalfQueueSlots4 = (kQueueCap / 2 * 2 + 15) / 16;
 
 // A proposal as its lane keeps it in registers: the Philox words and, after evaluation, the verdict.
 // The placement windows live in shared memory (ChainView::win), 8 words per proposal:
@@ -181,49 +169,6 @@ __device__ __forceinline__ uint32_t window_at(Ptr col, const WinPos p)
     }
     return p.first ? ((lo << 1) | (lo & 1u)) : __funnelshift_r(lo, hi, p.sh);
 }
-
-struct ChainView {               // where a chain's state lives
-    uint32_t* P;                 // [U][S32] schedule, time-packed (shared, or the chain's slice of global scratch)
-    // COW (a compile-time choice of the kernel): the slice of global scratch is a copy-on-write overlay of the initial
-    // schedule p0 (see kCowBitsMin) and `have` says which buckets of 2^shift units it holds. Otherwise the schedule is
-    // all in P.
-    const uint32_t* p0;
-    uint32_t* have;
-    uint32_t shift, U, S32;
-    bool shared_chain;           // a second warp of the chain reads while this one commits
-    template <bool COW>
-    __device__ __forceinline__ const uint32_t* col(uint32_t u) const
-    {
-        if (COW) {
-            const uint32_t b = u >> shift;
-            // volatile: another warp of the chain may be taking the bucket over meanwhile (it sets the bit after the
-            // copy); a select, not a branch, so that the loads of a batch stay in one straight-line block
-            const uint32_t w = reinterpret_cast<const volatile uint32_t*>(have)[b >> 5];
-            return ((w >> (b & 31u)) & 1u ? P : p0) + (size_t)u * S32;
-        }
-        return P + (size_t)u * S32;
-    }
-    // Before unit u is rewritten (all lanes of the committing warp, u uniform): its bucket is copied into the slice.
-    template <bool COW>
-    __device__ __forceinline__ void own(uint32_t u, uint32_t lane) const
-    {
-        if (!COW) return;
-        const uint32_t b = u >> shift;
-        if ((have[b >> 5] >> (b & 31u)) & 1u) return;
-        const size_t lo = (size_t)(b << shift) * S32, hi = (size_t)min(U, (b + 1u) << shift) * S32;
-        for (size_t i = lo + lane; i < hi; i += 32) P[i] = p0[i];
-        if (shared_chain) __threadfence_block();                  // the copy before the bit, for the chain's other warp
-        __syncwarp();
-        if (lane == 0) have[b >> 5] |= 1u << (b & 31u);
-        __syncwarp();
-    }
-    uint4* ctr;                  // [S] {hr, mi, mo, occ} (shared)
-    uint32_t* full;              // [S32] bit t set iff occ[t] == cap (shared)
-    uint4* win;                  // [kBatch][2] windows of the batch's proposals (shared)
-    int* acc;                    // [kBatch] cost change of each proposal being summed (shared)
-    uint16_t* queue;             // [kBatch * 31] work items (proposal slot << 5 | window bit) (shared)
-    uint32_t* hb;                // growing cache: [S] units written to HBM at birth (shared)
-};
 
 // born: window bit of the step in which u (low byte) and v (next byte) are written, 0 = not among bits 1..31
 struct Windows { uint32_t Wu, Wv, Nu, Nv, Au, Av, s0, born; };
@@ -342,180 +287,6 @@ __device__ __forceinline__ void eval_lane(PPtr P, const uint32_t* __restrict__ A
     mv.acc = metropolis(delta, mv.w, trow, shift);
 }
 
-// N queue items per lane, items base + 32 r + lane: the cost change of one step of one proposal each, added to the
-// proposal's sum.
-template <bool GROW, bool ASMEM, int N>
-__device__ __forceinline__ void eval_items(const ChainView cv, const StepC* __restrict__ stepc, const CostK K, uint32_t S,
-                                           uint32_t base, uint32_t count, uint32_t lane)
-{
-    int d[N];
-    uint32_t slot[N];
-    bool live[N];
-#pragma unroll
-    for (int r = 0; r < N; ++r) {
-        const uint32_t g = base + 32 * r + lane;
-        live[r] = g < count;
-        const uint32_t item = live[r] ? cv.queue[g] : 1u;         // a dead lane works on (proposal 0, bit 1) and drops it
-        slot[r] = item >> 5;
-        const uint32_t k = item & 31u;
-        const uint4 w0 = cv.win[slot[r] * 2], w1 = cv.win[slot[r] * 2 + 1];
-        Windows wn;
-        wn.Wu = w0.x; wn.Wv = w0.y; wn.Nu = w0.z; wn.Nv = w0.w; wn.Au = w1.x; wn.Av = w1.y; wn.s0 = w1.z;
-        wn.born = w1.w;
-        const uint32_t t = min(wn.s0 + k - 1, S - 1);
-        const StepC sc = ASMEM ? stepc[t] : __ldg(stepc + t);
-        d[r] = item_delta<GROW>(wn, k, cv.ctr[t], GROW ? cv.hb[t] : 0u, sc, K);
-    }
-#pragma unroll
-    for (int r = 0; r < N; ++r)
-        if (live[r] && d[r]) atomicAdd(cv.acc + slot[r], d[r]);
-}
-
-// Evaluation of the proposals named by `need` (one mask per proposal row), shared by the warp: every lane
-// prepares its own proposals, the (proposal, step) pairs whose cost changes are queued in shared memory, and
-// the warp works the queue off 32 pairs at a time, so that lanes with short and long proposals carry the
-// same load.
-// ALL: every lane prepares its proposal whether `need` names it or not (its items are dropped if not), so that this
-// part is straight-line code; `side_work` is then scheduled into it by the compiler (the draw of the next batch: a
-// long chain of dependent integer operations that fills the issue slots the window loads leave empty).
-template <bool GROW, bool ASMEM, bool ALL, bool COW, typename SideWork>
-__device__ __forceinline__ void eval_batch(const ChainView cv, const uint32_t* __restrict__ Acol,
-                                           const uint32_t* __restrict__ birth,
-                                           const StepC* __restrict__ stepc, const CostK K, uint32_t S, uint32_t S32,
-                                           const uint32_t* __restrict__ trow, uint32_t shift, uint32_t split_at,
-                                           const uint32_t (&need)[kMPL], uint32_t lane, LaneMove (&mv)[kMPL],
-                                           SideWork&& side_work)
-{
-    uint32_t todo[kMPL], cnt = 0;
-#pragma unroll
-    for (int h = 0; h < kMPL; ++h) {
-        todo[h] = 0;
-        const bool named = (need[h] >> lane) & 1u;
-        if (ALL || named) {
-            const uint32_t slot = h * 32 + lane;
-            Windows wn;
-            const uint32_t tm = lane_windows<GROW>(cv.col<COW>(mv[h].u), cv.col<COW>((mv[h].pk & 1u) ? mv[h].v : mv[h].u), Acol, cv.full,
-                                                   birth, S, S32, mv[h], wn);
-            todo[h] = named ? tm : 0u;
-            cv.win[slot * 2] = make_uint4(wn.Wu, wn.Wv, wn.Nu, wn.Nv);
-            cv.win[slot * 2 + 1] = make_uint4(wn.Au, wn.Av, wn.s0, wn.born);
-            cv.acc[slot] = 0;
-        }
-        cnt += __popc(todo[h]);
-    }
-    side_work();
-    // exclusive prefix sum of cnt over the lanes, bit-sliced: the five ballots do not depend on one another
-    uint32_t pos = 0, total = 0;
-    const uint32_t below = (1u << lane) - 1u;
-#pragma unroll
-    for (int bit = 0; bit < 5 + (kMPL > 1 ? 1 : 0) + (kMPL > 2 ? 1 : 0); ++bit) {
-        const uint32_t has = __ballot_sync(0xFFFFFFFFu, (cnt >> bit) & 1u);
-        pos += __popc(has & below) << bit;
-        total += __popc(has) << bit;
-    }
-    // queue the set bits of every mask of the lanes named by `pushing`; all 31 positions are tried so that no lane
-    // waits on a serial bit scan. Item `first` goes to queue position 0.
-    auto push = [&](bool pushing, uint32_t first) {
-#pragma unroll
-        for (int h = 0; h < kMPL; ++h) {
-            const uint32_t td = pushing ? todo[h] : 0u;
-            if (__any_sync(0xFFFFFFFFu, td != 0)) {
-#pragma unroll
-                for (uint32_t k = 1; k < 32; ++k) {
-                    const uint32_t bit = (td >> k) & 1u;
-                    if (bit) cv.queue[pos - first] = (uint16_t)(((h * 32 + lane) << 5) | k);
-                    pos += bit;
-                }
-            }
-        }
-        __syncwarp();
-    };
-    // two items per lane and trip (the two evaluations are independent and overlap), one where 32 or fewer are left
-    auto work_off = [&](uint32_t count) {
-        for (uint32_t base = 0; base < count; base += 64) {
-            if (base + 32 < count) eval_items<GROW, ASMEM, 2>(cv, stepc, K, S, base, count, lane);
-            else eval_items<GROW, ASMEM, 1>(cv, stepc, K, S, base, count, lane);
-        }
-    };
-    if (!ASMEM || total <= split_at) {
-        push(true, 0u);
-        work_off(total);
-    } else {
-        // ASMEM: the queue holds kQueueCap / 2 items, the worst case of 16 lanes. A batch with more (rare) goes in two
-        // halves, lanes 0..15 first.
-        const uint32_t mid = __shfl_sync(0xFFFFFFFFu, pos, 16);   // items of lanes 0..15
-        push(lane < 16, 0u);
-        work_off(mid);
-        __syncwarp();
-        push(lane >= 16, mid);
-        work_off(total - mid);
-    }
-    __syncwarp();
-#pragma unroll
-    for (int h = 0; h < kMPL; ++h)
-        if ((need[h] >> lane) & 1u) {
-            mv[h].delta = cv.acc[h * 32 + lane];
-            mv[h].acc = metropolis(mv[h].delta, mv[h].w, trow, shift);
-        }
-}
-
-// Apply the proposal in window slot `slot` (pk, u, v given): all lanes take part, lane j updates the counters
-// of window bit j, lanes 0 and 1 rewrite the words of the schedule and of the full-step bitmap.
-template <bool GROW, bool COW>
-__device__ __forceinline__ void apply_move(const ChainView cv, uint32_t S, uint32_t S32, uint32_t cap, uint32_t lane,
-                                           uint32_t slot, uint32_t pk, uint32_t u, uint32_t v)
-{
-    const uint4 w0 = cv.win[slot * 2], w1 = cv.win[slot * 2 + 1];
-    const uint32_t Wu = w0.x, Wv = w0.y, Nu = w0.z, Nv = w0.w, Au = w1.x, Av = w1.y;
-    const bool swap = pk & 1u;
-    const uint32_t len = (pk >> 1) & 63u, s0 = pk >> 8;
-    const uint32_t run = min(s0 + len, S) - s0;
-    const uint32_t nl = min(s0 + len, S - 1) - s0 + 1;
-    const bool valid = lane >= 1 && lane <= nl;
-    const uint32_t j = valid ? lane : 1u, t = s0 + j - 1;
-    const uint32_t pu = (Wu >> j) & 1u, qu = (Wu >> (j - 1)) & 1u, npu = (Nu >> j) & 1u, nqu = (Nu >> (j - 1)) & 1u;
-    const uint32_t pv = (Wv >> j) & 1u, qv = (Wv >> (j - 1)) & 1u, npv = (Nv >> j) & 1u, nqv = (Nv >> (j - 1)) & 1u;
-    const uint32_t au = (Au >> j) & 1u, av = (Av >> j) & 1u;
-    uint4 c = cv.ctr[t];
-    c.x += (au & npu) - (au & pu) + (av & npv) - (av & pv);
-    if (GROW) {
-        const uint32_t mu = (w1.w & 255u) == j ? 0u : 1u, mw = ((w1.w >> 8) & 255u) == j ? 0u : 1u;
-        c.y += mu * ((npu & ~nqu) - (pu & ~qu)) + mw * ((npv & ~nqv) - (pv & ~qv));
-        const uint32_t dh = (1u - mu) * (npu - pu) + (1u - mw) * (npv - pv);
-        if (valid && dh) cv.hb[t] += dh;
-    } else {
-        c.y += (npu & ~nqu) - (pu & ~qu) + (npv & ~nqv) - (pv & ~qv);
-    }
-    c.z += (~npu & nqu & 1u) - (~pu & qu & 1u) + (~npv & nqv & 1u) - (~pv & qv & 1u);
-    c.w += npu - pu + npv - pv;
-    if (valid) cv.ctr[t] = c;
-    uint32_t F = __ballot_sync(0xFFFFFFFFu, valid && c.w == cap);   // bit j <-> window bit j
-    uint32_t V = __ballot_sync(0xFFFFFFFFu, valid);
-    cv.own<COW>(u, lane);
-    if (swap) cv.own<COW>(v, lane);
-    if (lane < 2) {
-        uint32_t M = ((1u << run) - 1u) << 1, NU = Nu, NV = Nv, sbit = s0 - 1;
-        if (s0 == 0) { F >>= 1; V >>= 1; M >>= 1; NU >>= 1; NV >>= 1; sbit = 0; }
-        const uint32_t wj = (sbit >> 5) + lane, sh = sbit & 31u;
-        if (wj < S32 && (lane == 0 || sh != 0)) {
-            // lane 0 holds the part of the window that falls into the first word, lane 1 the spill-over
-            const uint32_t Vx = lane ? V >> (32 - sh) : V << sh, Fx = lane ? F >> (32 - sh) : F << sh;
-            const uint32_t Mx = lane ? M >> (32 - sh) : M << sh;
-            const uint32_t NUx = lane ? NU >> (32 - sh) : NU << sh, NVx = lane ? NV >> (32 - sh) : NV << sh;
-            if (Vx) cv.full[wj] = (cv.full[wj] & ~Vx) | (Fx & Vx);
-            if (Mx) {
-                const size_t iu = (size_t)u * S32 + wj;
-                cv.P[iu] = (cv.P[iu] & ~Mx) | (NUx & Mx);
-                if (swap) {
-                    const size_t iv = (size_t)v * S32 + wj;
-                    cv.P[iv] = (cv.P[iv] & ~Mx) | (NVx & Mx);
-                }
-            }
-        }
-    }
-    __syncwarp();
-}
-
 // A group of nthr threads (one or more whole warps, this thread being number tid) copies n words. A chain in global
 // scratch starts by copying tens of megabytes this way, so eight 16-byte loads per thread are in flight before the
 // first store.
@@ -571,29 +342,7 @@ __device__ __forceinline__ void copy_merged(uint32_t* __restrict__ dst, const ui
     }
 }
 
-// Hand-over block of a chain that is served by more than one warp (shared memory, one per chain).
-// The warps of a chain take the batches in turn: warp w owns batches w, w + W, w + 2W, ... It evaluates a batch
-// against whatever state it finds (another warp may be committing an earlier batch meanwhile), then waits for its
-// turn, evaluates again the proposals that a move applied in the meantime could have touched, and commits. `turn`
-// is the index of the batch whose owner may commit; `napplied` counts the state-changing moves of the chain and
-// `applog` keeps the step ranges of the latest kLog of them. The chain-wide scalars are read and written back only
-// in a turn that applies a move, starts a temperature level or ends the chain; the two counters that change in
-// nearly every batch are kept per warp and added up at the end.
-constexpr uint32_t kLog = 16;
-constexpr int kMaxW = 2;
-struct ChainShare {
-    uint64_t cur, best, best_move, best_at_boundary, n_chg, hash;
-    uint64_t n_acc[kMaxW], n_inf[kMaxW];
-    uint32_t ulen, snap_dirty, stopped, pad;
-    uint32_t turn, napplied, pad2[2];
-    uint32_t applog[kLog];       // s0 | (s0 + len) << 16 of an applied move
-};
-constexpr uint32_t kShareSlots4 = (sizeof(ChainShare) + 15) / 16;
-// per warp: windows, sums, work queue
-__host__ __device__ constexpr uint32_t priv_slots4(bool halfq)
-{
-    return kWinSlots4 + kAccSlots4 + (halfq ? kHalfQueueSlots4 : kQueueSlots4);
-}
+constexpr uint32_t kLog = 16;    // applied moves a chain's log keeps
 // A wait for the turn gives up after this many polls (each at least some tens of nanoseconds apart): the chain then
 // reports KVP_ERR_TIMEOUT instead of holding the GPU. A turn lasts microseconds.
 constexpr uint32_t kTurnPolls = 1u << 24;
@@ -601,348 +350,12 @@ constexpr uint32_t kTurnPolls = 1u << 24;
 __device__ __forceinline__ uint32_t ld_volatile_u32(const uint32_t* p) { return *reinterpret_cast<const volatile uint32_t*>(p); }
 __device__ __forceinline__ void st_volatile_u32(uint32_t* p, uint32_t v) { *reinterpret_cast<volatile uint32_t*>(p) = v; }
 
-// shared-memory words (as uint4 slots) of one chain besides its schedule
-// cow4: uint4 slots of the bucket bitmap of a copy-on-write slice (schedules in global scratch), else 0
-__host__ __device__ inline uint32_t chain_fixed4(uint32_t S, uint32_t S32, bool grow, uint32_t W, bool halfq, uint32_t cow4)
-{
-    return S + (S32 + 3) / 4 + (grow ? (S + 3) / 4 : 0u) + cow4 + (W > 1 ? kShareSlots4 : 0u) + W * priv_slots4(halfq);
-}
-
-// ASMEM (only with PSMEM): the access bitmap and the per-step constants, which every chain of the CTA reads, are
-// staged in shared memory once per CTA. With the schedules in shared memory the L1 cache is down to its minimum and
-// cannot hold them.
-// Without PSMEM the chain's slice of global scratch is a copy-on-write overlay of the initial schedule when
-// prm.cow_slots4 is set (jobs whose slices add up to gigabytes: the chains then start without copying anything), else a
-// plain copy of it (small slices: the copy costs nothing and an applied move is cheaper without the take-over).
-template <bool PSMEM, bool GROW, int W, bool ASMEM, bool COW>
-__global__ void __launch_bounds__(512)
-narrow_chain_kernel(const ChainParams prm)
-{
-    static_assert(!COW || !PSMEM, "overlays only for schedules in global scratch");
-    static_assert(W >= 1 && W <= kMaxW && (W & (W - 1)) == 0, "warps per chain");
-    static_assert(PSMEM || !ASMEM, "shared access bitmap only beside shared schedules");
-    extern __shared__ uint4 smem4[];
-    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const uint32_t cpb = (blockDim.x >> 5) / W;                   // chains per CTA
-    const uint32_t cic = warp / W, sub = warp % W;                // chain within the CTA, warp within the chain
-    const uint32_t tid = sub * 32 + lane;                         // thread within the chain
-    const uint32_t slot = blockIdx.x * cpb + cic;
-    const bool active = slot < prm.chain_count;
-    if (W == 1 && !ASMEM && !active) return;
-    const uint32_t chain = prm.chain_first + slot;
-    const uint32_t S = prm.S, S32 = prm.S32, U = prm.U;
-    const size_t pwords = (size_t)U * S32;
-    const uint32_t f4 = (S32 + 3) / 4;                            // uint4 slots of the full-step bitmap
-    const uint32_t h4 = GROW ? (S + 3) / 4 : 0u;                  // uint4 slots of the written-to-HBM counts
-    const uint32_t o4 = COW ? prm.cow_slots4 : 0u;                 // the slice is a copy-on-write overlay
-    const uint32_t fixed4 = chain_fixed4(S, S32, GROW, W, ASMEM, o4);
-    uint4* const mine4 = smem4 + (size_t)cic * fixed4;
-    ChainView cv;
-    cv.ctr = mine4;
-    cv.full = reinterpret_cast<uint32_t*>(mine4 + S);
-    cv.hb = reinterpret_cast<uint32_t*>(mine4 + S + f4);
-    uint32_t* const cowmap = reinterpret_cast<uint32_t*>(mine4 + S + f4 + h4);   // buckets the slice holds
-    ChainShare* const sh = reinterpret_cast<ChainShare*>(mine4 + S + f4 + h4 + o4);
-    uint4* const priv4 = mine4 + S + f4 + h4 + o4 + (W > 1 ? kShareSlots4 : 0u) + sub * priv_slots4(ASMEM);
-    cv.win = priv4;
-    cv.acc = reinterpret_cast<int*>(priv4 + kWinSlots4);
-    cv.queue = reinterpret_cast<uint16_t*>(priv4 + kWinSlots4 + kAccSlots4);
-    uint32_t* const pool = reinterpret_cast<uint32_t*>(smem4 + (size_t)cpb * fixed4);   // schedules, then A, then constants
-    cv.P = PSMEM ? pool + (size_t)cic * pwords : prm.ws + (size_t)slot * pwords;
-    cv.p0 = prm.Pcol0; cv.have = COW ? cowmap : nullptr; cv.shared_chain = W > 1; cv.shift = prm.cow_shift; cv.U = U; cv.S32 = S32;
-    const uint32_t* Acol = prm.Acol;
-    const StepC* stepc = prm.stepc;
-    if (ASMEM) {
-        const size_t a_off = ((size_t)cpb * pwords + 3) & ~(size_t)3, c_off = (a_off + pwords + 3) & ~(size_t)3;
-        uint32_t* const a_s = pool + a_off;
-        StepC* const c_s = reinterpret_cast<StepC*>(pool + c_off);
-        copy_words(a_s, prm.Acol, pwords, threadIdx.x, blockDim.x);
-        for (uint32_t i = threadIdx.x; i < S; i += blockDim.x) c_s[i] = __ldg(prm.stepc + i);
-        Acol = a_s;
-        stepc = c_s;
-    }
-    if (active) {
-        for (uint32_t i = tid; i < S; i += 32 * W) cv.ctr[i] = __ldg(prm.counters0 + i);
-        for (uint32_t i = tid; i < S32; i += 32 * W) cv.full[i] = __ldg(prm.full0 + i);
-        if (GROW)
-            for (uint32_t i = tid; i < S; i += 32 * W) cv.hb[i] = __ldg(prm.hb0 + i);
-        for (uint32_t i = lane; i < kWinSlots4; i += 32) cv.win[i] = make_uint4(0u, 0u, 0u, 0u);
-        if (!COW) copy_words(cv.P, prm.Pcol0, pwords, tid, 32 * W);
-        else
-            for (uint32_t i = tid; i < prm.cow_slots4 * 4; i += 32 * W) cowmap[i] = 0u;   // the slice holds nothing yet
-        if (W > 1 && tid == 0) {
-            sh->cur = sh->best = sh->best_at_boundary = prm.init_ticks;
-            sh->best_move = ~0ull; sh->n_chg = 0; sh->hash = 0;
-            for (int w = 0; w < kMaxW; ++w) { sh->n_acc[w] = 0; sh->n_inf[w] = 0; }
-            sh->ulen = 0u; sh->snap_dirty = 0u; sh->stopped = 0u; sh->turn = 0u; sh->napplied = 0u;
-        }
-    }
-    if (W > 1 || ASMEM) {
-        __syncthreads();
-        if (!active) return;
-    } else {
-        __syncwarp();
-    }
-    uint32_t* snap = prm.snap ? prm.snap + (size_t)slot * pwords : nullptr;
-    uint64_t* ulog = prm.undo_log ? prm.undo_log + (size_t)slot * prm.undo_cap : nullptr;
-
-    // Chain-wide scalars. One warp: they live in registers. Several warps: the master copy is in `sh`; a warp
-    // fetches it (`have`) in a turn that needs it and writes it back before it passes the turn on.
-    uint64_t cur = prm.init_ticks, best = cur, best_move = ~0ull, best_at_boundary = cur;
-    uint64_t n_chg = 0, hash = 0;
-    bool snap_dirty = false;                                      // the best state is the current one, not yet saved
-    uint32_t ulen = 0;                                            // moves applied since the best state
-    uint64_t n_acc = 0, n_inf = 0;                                // this warp's share of the two counters
-    uint32_t napp = 0;                                            // state-changing moves so far (W > 1)
-    bool have = W == 1;
-    auto fetch = [&]() {
-        if (W > 1 && !have) {
-            cur = sh->cur; best = sh->best; best_move = sh->best_move; best_at_boundary = sh->best_at_boundary;
-            n_chg = sh->n_chg; hash = sh->hash; ulen = sh->ulen; snap_dirty = sh->snap_dirty != 0;
-            have = true;
-        }
-    };
-    // Ends this warp's turn for batch b: scalars back to `sh` if they were fetched, then the next batch may commit.
-    auto pass_turn = [&](uint32_t b) {
-        __syncwarp();
-        if (lane == 0) {
-            if (have) {
-                sh->cur = cur; sh->best = best; sh->best_move = best_move; sh->best_at_boundary = best_at_boundary;
-                sh->n_chg = n_chg; sh->hash = hash; sh->ulen = ulen; sh->snap_dirty = snap_dirty ? 1u : 0u;
-            }
-            sh->n_acc[sub] = n_acc; sh->n_inf[sub] = n_inf;
-            __threadfence_block();
-            if (!(prm.drop_first_turn && b == 0)) st_volatile_u32(&sh->turn, b + 1u);
-        }
-        have = false;
-    };
-
-    uint64_t lvl_start = 0;                                       // first move of the level
-    uint32_t base = 0;                                            // index of the level's first batch (mod 2^32)
-    bool stop = false;
-    for (uint32_t level = 0; level < prm.levels && lvl_start < prm.upto; ++level) {
-        // a temperature level: its moves in batches of up to 32 * kMPL consecutive moves (fewer than 2^32 batches:
-        // the host refuses longer levels)
-        const uint64_t lvl_len = (level + 1 < prm.levels ? min(lvl_start + prm.per_level, prm.upto) : prm.upto) - lvl_start;
-        const uint32_t nbat = (uint32_t)((lvl_len + kBatch - 1) / kBatch);
-        const uint32_t last_nb = (uint32_t)(lvl_len - (uint64_t)(nbat - 1) * kBatch);
-        const bool last_level = lvl_start + lvl_len >= prm.upto;
-        const uint32_t shift = __ldg(prm.shifts + level);
-        const uint32_t* trow = prm.table + (size_t)level * KVP_TABLE_Q;
-        if (W == 1 && level > 0) {
-            if (prm.early_permille && level >= prm.early_from &&
-                (best_at_boundary - best) * 1000ull < best_at_boundary * (uint64_t)prm.early_permille) {
-                stop = true;
-                break;
-            }
-            best_at_boundary = best;
-        }
-        // A batch: move m + 32 h + lane in row h of its lane. Every lane draws and evaluates its own proposals
-        // against the current state; the warp then commits them in move order. A move that changes the schedule
-        // invalidates only later moves whose step windows overlap its own; those are evaluated again before their
-        // turn comes, so the outcome is that of the sequential chain.
-        bool have_next = false;                                   // `next` holds the draw of the batch about to start
-        LaneMove next;
-        next.pk = next.u = next.v = next.w = 0u; next.delta = 0; next.inf = next.acc = next.chg = false;
-        for (uint32_t bi = (sub - base) & (W - 1); bi < nbat; bi += W) {
-            const uint64_t m = lvl_start + (uint64_t)bi * kBatch;
-            const uint32_t nb = bi + 1 < nbat ? kBatch : last_nb;
-            const uint32_t b = base + bi;
-            uint32_t n0 = 0;
-            if (W > 1) {
-                // Moves applied from now on may be half visible to the reads below: they are checked for at the turn.
-                n0 = __shfl_sync(0xFFFFFFFFu, ld_volatile_u32(&sh->napplied), 0);
-                __threadfence_block();
-            }
-            static_assert(kMPL == 1, "the draw of the next batch is carried in one LaneMove");
-            LaneMove mv[kMPL];
-            uint32_t todo[kMPL], need[kMPL];
-            if (have_next) {
-                mv[0] = next;
-            } else {
-                uint32_t r[4];
-                const uint64_t mine = m + lane;
-                philox4x32_10((uint32_t)mine, (uint32_t)(mine >> 32), chain, TAG_MOVE, prm.keys, r);
-                decode_move(r, prm.p_swap_256, prm.len_choices, S, U, mv[0]);
-            }
-            mv[0].inf = false; mv[0].acc = false; mv[0].chg = false; mv[0].delta = 0;
-            todo[0] = nb >= 32 ? 0xFFFFFFFFu : (1u << nb) - 1u;
-            need[0] = todo[0];
-            // the proposals of this warp's next batch of the level are drawn while this batch's windows are loaded
-            // (drawn, and dropped, even where the level has no further batch for this warp)
-            eval_batch<GROW, ASMEM, true, COW>(cv, Acol, prm.birth, stepc, prm.K, S, S32, trow, shift, prm.split_at, need, lane, mv,
-                                          [&]() {
-                                              uint32_t r[4];
-                                              const uint64_t mine = m + (uint64_t)W * kBatch + lane;
-                                              philox4x32_10((uint32_t)mine, (uint32_t)(mine >> 32), chain, TAG_MOVE, prm.keys, r);
-                                              decode_move(r, prm.p_swap_256, prm.len_choices, S, U, next);
-                                          });
-            have_next = bi + W < nbat;
-#pragma unroll
-            for (int h = 0; h < kMPL; ++h) need[h] = 0;
-            if (W > 1) {
-                // wait for the turn
-                uint32_t polls = 0, t;
-                for (;;) {
-                    t = __shfl_sync(0xFFFFFFFFu, ld_volatile_u32(&sh->turn), 0);
-                    if (t == b || ++polls > kTurnPolls) break;
-                    __nanosleep(64);
-                }
-                __threadfence_block();
-                if (t != b) {                                     // gave up: flag it, let the others pass, leave
-                    if (lane == 0) {
-                        atomicExch(prm.err, 1u);
-                        st_volatile_u32(&sh->stopped, 2u);
-                        __threadfence_block();
-                        st_volatile_u32(&sh->turn, b + 1u);
-                    }
-                    return;
-                }
-                if (ld_volatile_u32(&sh->stopped)) {              // the chain has ended: pass the turn on and leave
-                    __syncwarp();
-                    if (lane == 0) st_volatile_u32(&sh->turn, b + 1u);
-                    return;
-                }
-                napp = sh->napplied;
-                // proposals whose steps meet those of a move applied since this batch was evaluated
-                if (napp - n0 > kLog) {
-#pragma unroll
-                    for (int h = 0; h < kMPL; ++h) need[h] = todo[h];
-                } else {
-                    for (uint32_t k = n0; k != napp; ++k) {
-                        const uint32_t e = sh->applog[k % kLog], s0b = e & 0xFFFFu, endb = e >> 16;
-#pragma unroll
-                        for (int h = 0; h < kMPL; ++h) {
-                            const uint32_t s0 = mv[h].pk >> 8, end = s0 + ((mv[h].pk >> 1) & 63u);
-                            need[h] |= __ballot_sync(0xFFFFFFFFu, s0 <= endb + 1 && s0b <= end) & todo[h];
-                        }
-                    }
-                }
-                if (bi == 0 && level > 0) {                       // the level's first batch: stop rule, new reference
-                    fetch();
-                    if (prm.early_permille && level >= prm.early_from &&
-                        (best_at_boundary - best) * 1000ull < best_at_boundary * (uint64_t)prm.early_permille) {
-                        stop = true;
-                        break;
-                    }
-                    best_at_boundary = best;
-                }
-            }
-            for (;;) {
-                uint32_t any_need = 0;
-#pragma unroll
-                for (int h = 0; h < kMPL; ++h) any_need |= need[h];
-                if (any_need)
-                    eval_batch<GROW, ASMEM, false, COW>(cv, Acol, prm.birth, stepc, prm.K, S, S32, trow, shift, prm.split_at, need, lane, mv,
-                                                   []() {});
-                bool applied = false;
-#pragma unroll
-                for (int h = 0; h < kMPL; ++h) need[h] = 0;
-#pragma unroll
-                for (int h = 0; h < kMPL; ++h) {
-                    if (applied || !todo[h]) continue;
-                    const uint32_t infb = __ballot_sync(0xFFFFFFFFu, mv[h].inf);
-                    const uint32_t accb = __ballot_sync(0xFFFFFFFFu, !mv[h].inf && mv[h].acc);
-                    const uint32_t blk = __ballot_sync(0xFFFFFFFFu, !mv[h].inf && mv[h].acc && mv[h].chg) & todo[h];
-                    if (!blk) {                                   // nothing in this row changes the schedule
-                        n_inf += __popc(infb & todo[h]);
-                        n_acc += __popc(accb & todo[h]);
-                        todo[h] = 0;
-                        continue;
-                    }
-                    const uint32_t bb = __ffs(blk) - 1;
-                    const uint32_t done = todo[h] & (0xFFFFFFFFu >> (31 - bb));  // the row's moves up to and including bb
-                    n_inf += __popc(infb & done);
-                    n_acc += __popc(accb & done);
-                    fetch();
-                    ++n_chg;
-                    const int delta = __shfl_sync(0xFFFFFFFFu, mv[h].delta, bb);
-                    const uint32_t pk = __shfl_sync(0xFFFFFFFFu, mv[h].pk, bb);
-                    const uint32_t bu = __shfl_sync(0xFFFFFFFFu, mv[h].u, bb), bv = __shfl_sync(0xFFFFFFFFu, mv[h].v, bb);
-                    const uint64_t after = (uint64_t)((int64_t)cur + delta);
-                    if (snap && snap_dirty && after >= best) {    // leaving the best state: save it first
-                        copy_words(snap, cv.P, pwords, lane);
-                        snap_dirty = false;
-                    }
-                    apply_move<GROW, COW>(cv, S, S32, prm.cap, lane, h * 32 + bb, pk, bu, bv);
-                    // The applied move rewrote steps s0b .. s0b + len_b (bits, counters, full flags). A later
-                    // proposal read steps s0 - 1 .. s0 + len: it has to be evaluated again iff the two ranges meet.
-                    const uint32_t s0b = pk >> 8, endb = s0b + ((pk >> 1) & 63u);
-                    if (W > 1) {                                  // tell the warps that are evaluating later batches
-                        if (lane == 0) {
-                            sh->applog[napp % kLog] = s0b | (endb << 16);
-                            __threadfence_block();
-                            st_volatile_u32(&sh->napplied, napp + 1u);
-                        }
-                        ++napp;
-                    }
-                    cur = after;
-                    const uint64_t mb = m + 32u * h + bb;
-                    hash = (hash ^ mb) * 0x9E3779B97F4A7C15ull + cur;
-                    if (cur < best) { best = cur; best_move = mb; snap_dirty = true; ulen = 0; }
-                    else if (ulog) {                              // every move is its own inverse: remember it
-                        if (ulen < prm.undo_cap && lane == 0) ulog[ulen] = mb;
-                        if (ulen <= prm.undo_cap) ++ulen;
-                    }
-                    todo[h] &= ~done;
-#pragma unroll
-                    for (int h2 = 0; h2 < kMPL; ++h2) {
-                        const uint32_t s0 = mv[h2].pk >> 8, end = s0 + ((mv[h2].pk >> 1) & 63u);
-                        need[h2] = __ballot_sync(0xFFFFFFFFu, s0 <= endb + 1 && s0b <= end) & todo[h2];
-                    }
-                    applied = true;
-                }
-                if (!applied) break;
-            }
-            if (W > 1 && !(last_level && bi + 1 == nbat)) pass_turn(b);   // hand the chain to the owner of the next batch
-        }
-        if (stop) break;                                          // `base` stays the index of the batch that stopped
-        base += nbat;
-        lvl_start += lvl_len;
-    }
-    const uint64_t m_end = stop ? lvl_start : prm.upto;           // moves done when the chain ended
-    // The warp that committed the last batch, or that ended the chain by the stop rule, reports.
-    if (W > 1) {
-        const bool writer = stop || (base ? ((base - 1u) & (W - 1)) == sub : sub == 0);
-        if (!writer) return;
-        fetch();
-        sh->n_acc[sub] = n_acc; sh->n_inf[sub] = n_inf;           // all lanes write the same values
-        __syncwarp();
-        n_acc = 0; n_inf = 0;
-        for (int w = 0; w < W; ++w) { n_acc += sh->n_acc[w]; n_inf += sh->n_inf[w]; }
-    }
-    if (snap && snap_dirty) copy_words(snap, cv.P, pwords, lane);
-    if (ulog && lane == 0) prm.undo_len[slot] = ulen;
-    if (COW && prm.cow_out)                                    // which buckets the slice holds (for the walk back)
-        for (uint32_t i = lane; i < prm.cow_slots4 * 4; i += 32)
-            prm.cow_out[(size_t)slot * (prm.cow_slots4 * 4) + i] = cowmap[i];
-    if (lane == 0) {
-        kvp_chain_result res;
-        res.best_ticks = best; res.best_move = best_move; res.final_ticks = cur; res.moves_done = m_end;
-        res.n_accepted = n_acc; res.n_changed = n_chg; res.n_infeasible = n_inf; res.traj_hash = hash;
-        prm.results[chain - prm.result_base] = res;
-    }
-    if (prm.dump && slot == 0) {
-        __syncwarp();
-        if (!COW) copy_words(prm.dump, cv.P, pwords, lane);
-        else copy_merged(prm.dump, cv.P, prm.Pcol0, cowmap, prm.cow_shift, U, S32, lane);
-    }
-    if (W > 1 && stop) {                                          // ended by the stop rule: release the next owner
-        __syncwarp();
-        if (lane == 0) {
-            st_volatile_u32(&sh->stopped, 1u);
-            __threadfence_block();
-            st_volatile_u32(&sh->turn, base + 1u);
-        }
-    }
-}
-
 }  // namespace
 
 }  // namespace kvp
 
 #include "kvp_chain.cuh"
-#include "kvp_hot.cuh"
+#include "kvp_narrow.cuh"
 
 namespace kvp {
 
@@ -1166,7 +579,6 @@ struct Ctx {
     bool asmem;              // the access bitmap and the step constants are staged in shared memory
     bool wide;               // the wide kernel
     uint32_t S32;            // words per time-packed column
-    bool hot;                // the sequential kernel (kvp_hot.cuh)
     bool ladder_ctas;        // replica exchange: every CTA holds whole ladders (one launch)
     int rows;                // wide kernel: rows of 32 proposals in a batch
     bool lin;                // kappa_d >= kappa_k: see kvp_chain.cuh
@@ -1190,17 +602,12 @@ int validate(const kvp_problem* p, const kvp_anneal_params* a)
 
 typedef void (*ChainKernel)(const ChainParams);
 
-template <bool PSMEM, bool ASMEM, bool COW>
-ChainKernel narrow_kernel_pick(bool grow, uint32_t W)
+ChainKernel narrow_kernel_for(bool psmem, bool asmem, uint32_t S32, uint32_t W)
 {
-    if (W == 2) return grow ? narrow_chain_kernel<PSMEM, true, 2, ASMEM, COW> : narrow_chain_kernel<PSMEM, false, 2, ASMEM, COW>;
-    return grow ? narrow_chain_kernel<PSMEM, true, 1, ASMEM, COW> : narrow_chain_kernel<PSMEM, false, 1, ASMEM, COW>;
-}
-
-ChainKernel narrow_kernel_for(bool psmem, bool asmem, bool grow, uint32_t W, bool cow)
-{
-    if (!psmem) return cow ? narrow_kernel_pick<false, false, true>(grow, W) : narrow_kernel_pick<false, false, false>(grow, W);
-    return asmem ? narrow_kernel_pick<true, true, false>(grow, W) : narrow_kernel_pick<true, false, false>(grow, W);
+    if (psmem && W == 1) return asmem ? narrow_chain_kernel<true, true, true, 0> : narrow_chain_kernel<true, true, false, 0>;
+    if (psmem) return asmem ? narrow_chain_kernel<false, true, true, 0> : narrow_chain_kernel<false, true, false, 0>;
+    return S32 == 2 ? narrow_chain_kernel<false, false, false, 2> : S32 == 4 ? narrow_chain_kernel<false, false, false, 4>
+                                                                             : narrow_chain_kernel<false, false, false, 0>;
 }
 
 template <bool PSMEM, bool ASMEM, bool LIN, int COLV>
@@ -1225,18 +632,18 @@ ChainKernel wide_kernel_for(bool psmem, bool asmem, bool grow, bool lin, uint32_
 
 ChainKernel kernel_of(const Ctx& c, bool psmem, bool asmem, uint32_t W)
 {
-    if (c.hot) return asmem ? hot_chain_kernel<true> : hot_chain_kernel<false>;
     return c.wide ? wide_kernel_for(psmem, asmem, c.grow, c.lin, c.S32, c.rows)
-                  : narrow_kernel_for(psmem, asmem, c.grow, W, c.cow_slots4 != 0);
+                  : narrow_kernel_for(psmem, asmem, c.S32, W);
 }
 
 int launch_chains(const Ctx& c, ChainParams& prm, uint32_t count)
 {
-    if (c.wide || c.hot) {
+    {
         const bool rounds = prm.rung_hist != nullptr;
-        prm.lay = chain_layout(prm.S, prm.S32, c.grow, c.psmem, c.lin, c.psmem ? 0u : c.cow_slots4);
+        prm.lay = !c.wide ? narrow_layout(prm.S, prm.S32, c.psmem, c.psmem ? 0u : c.cow_slots4) : chain_layout(prm.S, prm.S32, c.grow, c.psmem, c.lin, c.psmem ? 0u : c.cow_slots4);
         prm.seg_len = rounds ? prm.exch_every : prm.per_level;
-        prm.seg_bat = (uint32_t)((prm.seg_len + 32 * c.rows - 1) / (32 * c.rows));
+        const uint32_t batch = c.wide ? 32u * c.rows : 32u;
+        prm.seg_bat = (uint32_t)((prm.seg_len + batch - 1) / batch);
         const uint64_t needed = (prm.upto + prm.seg_len - 1) / prm.seg_len;
         prm.seg0 = rounds ? prm.round0 : 0u;
         prm.seg1 = (uint32_t)std::min<uint64_t>(rounds ? prm.round1 : prm.levels, needed);
@@ -1279,7 +686,6 @@ int prepare(kvp_problem* p, const kvp_anneal_params* a, cudaStream_t st, Ctx& c,
     KVP_CUDA(cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
     KVP_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     const size_t budget = (size_t)smem_max - 1024;
-    // per chain: counters, full-step bitmap and, per warp, the batch's windows, accumulators and work queue
     c.grow = p->dL != nullptr;
     const kvp_test_hooks hooks = g_hooks;
     c.S32 = p->S32;
@@ -1294,55 +700,40 @@ int prepare(kvp_problem* p, const kvp_anneal_params* a, cudaStream_t st, Ctx& c,
     c.cow_shift = 0;
     c.smem_shared = 0;
     c.asmem = false;
-    c.hot = false;
-    auto fixed_bytes = [&](uint32_t warps, bool halfq, bool shared) {
-        if (c.hot) return (size_t)hot_stride(p->S, p->S32);
+    auto fixed_bytes = [&](uint32_t warps, bool shared) {
         if (c.wide) return chain_bytes(p->S, p->S32, c.grow, shared, c.lin, shared ? 0u : c.cow_slots4, warps, c.rows);
-        return (size_t)chain_fixed4(p->S, p->S32, c.grow, warps, halfq, shared ? 0u : c.cow_slots4) * 16;
+        return narrow_bytes(p->S, p->S32, shared, shared ? 0u : c.cow_slots4, warps);
     };
-    // Which kernel. The wide one, but for two kinds of jobs whose chains apply so many of their moves that evaluations far
-    // ahead of the commits do not last, where the narrow kernel's batches of 32 and its shorter path through an applied
-    // move win: hot starts (C_0 from p0 >= 0.5: a fifth of the proposals change the schedule; 256 units x 512 steps,
-    // 1024 chains x 100,000 moves: 25.5 ms with one narrow warp per chain, 34 on the wide kernel), and few chains on
-    // schedules too large for shared memory (16,384 units x 256 steps, 740 chains: 6.4 against 8.0 ms; 1024 chains:
-    // 15.4 against 14.2) or of hardly any units (16 units, 64 chains: 0.43 against 0.55).
-    // kvp_set_test_hooks can force either (warps_per_chain 1 or 2: narrow; 3 or 16 + w: wide).
-    c.wide = true;
-    c.psmem = fixed_bytes(1, false, true) + pbytes + 16 <= budget / 2 && p->U < 65536u;
-    if (hooks.warps_per_chain) c.wide = hooks.warps_per_chain == 3 || hooks.warps_per_chain >= 16;
+    c.psmem = true;
+    if (hooks.warps_per_chain) c.wide = hooks.warps_per_chain == 3 || (hooks.warps_per_chain >= 16 && hooks.warps_per_chain < 32);
     else if (hot) c.wide = false;
-    else c.wide = c.psmem ? (uint64_t)p->U * p->S >= 4096u : p->U >= 32768u || chains_per_sm > 6;
-    if (exchange) c.wide = true;
-    c.hot = !c.wide && (hooks.warps_per_chain ? hooks.warps_per_chain == 4 : hot) && c.lin && !c.grow && p->U < 65536u &&
-            hot_stride(p->S, p->S32) + pbytes + 16 <= budget / 2;
-    if (!c.wide) c.psmem = fixed_bytes(1, false, true) + pbytes <= budget / 2;
-    const uint32_t forced = hooks.warps_per_chain == 3 || hooks.warps_per_chain == 4 ? 1u : hooks.warps_per_chain >= 16 ? hooks.warps_per_chain - 16u : hooks.warps_per_chain;
-    const uint32_t full = 16;                                     // warps of a CTA that fills an SM (at 128 registers)
+    else c.wide = (uint64_t)p->U * p->S >= 4096u;
+    if (exchange || !c.lin || c.grow) c.wide = true;              // the narrow kernel does not serve these
+    c.psmem = fixed_bytes(1, true) + pbytes + 16 <= budget / 2 && p->U < 65536u;
+    const uint32_t forced = hooks.warps_per_chain == 3 ? 1u : hooks.warps_per_chain >= 16 ? hooks.warps_per_chain & 15u : hooks.warps_per_chain;
+#ifndef NTHR
+#define NTHR 512
+#endif
+    const uint32_t full = !c.wide && !c.psmem ? NTHR / 32 : 16;                                     // warps of a CTA that fills an SM (at 128 registers)
     uint32_t W = 1;
     if (c.psmem) {
         uint32_t want = chains_per_sm < 1 ? 1 : chains_per_sm;
         if (exchange) want = (want + rungs - 1) / rungs * rungs;  // whole ladders
-        // bytes with the access bitmap and (narrow) the step constants staged; wide: columns are followed by readable bytes
+        // bytes with the access bitmap staged; columns are followed by readable bytes
         auto with_a = [&](uint32_t chains, uint32_t warps) {
             const size_t a_off = ((size_t)chains * (pbytes / 4) + 3) & ~(size_t)3, c_off = (a_off + pbytes / 4 + 3) & ~(size_t)3;
-            return (size_t)chains * fixed_bytes(warps, true, true) + c_off * 4 + (c.wide || c.hot ? 16 : (size_t)p->S * 16);
+            return (size_t)chains * fixed_bytes(warps, true) + c_off * 4 + 16;
         };
-        if (c.wide) {
-            // two warps per chain, four where an SM has three chains or fewer (256 units x 512 steps, 50,000 moves, 148 and
-            // 740 chains: one warp 1.62 and 1.79 ms, two 1.12 and 1.34, four 1.05 and 2.40)
-            W = chains_per_sm <= 3 ? 4 : 2;
-            while (W > 1 && (want * W > full || with_a(want, W) > budget)) W /= 2;
-        } else if (!hot) {
-            W = 2;                                                // hides the latency of a chain's serial parts
-            if (chains_per_sm > 8 || ((fixed_bytes(2, false, true) + pbytes) * want > budget && (fixed_bytes(1, false, true) + pbytes) * want <= budget))
-                W = 1;
-        }
+        // two warps per chain, four where an SM has three chains or fewer (256 units x 512 steps, 50,000 moves, 148 and
+        // 740 chains: one warp 1.62 and 1.79 ms, two 1.12 and 1.34, four 1.05 and 2.40)
+        W = chains_per_sm <= 3 ? 4 : 2;
+        while (W > 1 && (want * W > full || with_a(want, W) > budget)) W /= 2;
         if (forced) W = forced;
         c.wpc = W;
-        c.smem_per_warp = fixed_bytes(W, false, true) + pbytes;
+        c.smem_per_warp = fixed_bytes(W, true) + pbytes;
         uint32_t wmax = (uint32_t)((budget - 16) / c.smem_per_warp);
         if (wmax > full / W) wmax = full / W;
-        if (c.hot && wmax > 8u) wmax = 8u;                        // the sequential kernel is built for CTAs of up to 256 threads
+        if (!c.wide && W == 1 && wmax > 8u) wmax = 8u;            // that variant is built for CTAs of up to 256 threads
         if (wmax < 1) return KVP_ERR_RANGE;
         c.wpb = want > wmax ? wmax : want;
         if (exchange && rungs <= wmax) {
@@ -1350,31 +741,24 @@ int prepare(kvp_problem* p, const kvp_anneal_params* a, cudaStream_t st, Ctx& c,
             c.wpb = c.wpb / rungs * rungs;
         }
         c.resident = a->chains;
-        c.smem_shared = c.wide || c.hot ? 16 : 0;
+        c.smem_shared = 16;
         c.asmem = with_a(c.wpb, W) <= budget && (!c.wide || c.lin);
-        if (c.asmem) {                                            // (the narrow kernel then makes do with half the work queue)
-            c.smem_per_warp = fixed_bytes(W, true, true) + pbytes;
+        if (c.asmem) {
             c.smem_shared = with_a(c.wpb, W) - (size_t)c.wpb * c.smem_per_warp;
         }
         KVP_CUDA(cudaFuncSetAttribute(kernel_of(c, true, c.asmem, W), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)budget));
     } else {
         // Two warps per chain while that leaves an SM at most 16 warps (the registers allow no more). More per chain are no
         // faster (16,384 units x 256 steps, 148 chains: 6.76 ms with two and with four, 7.5 with one).
-        if (!exchange && chains_per_sm <= 8 && !(hot && !c.wide)) W = 2;
+        if (!exchange && chains_per_sm <= 8) W = 2;
         if (forced) W = forced;
         if (W == 1 && c.wide && c.lin) c.rows = kRowsOne;
         uint32_t per_cta = full / W;                              // chains of a full CTA
         if (chains_per_sm < per_cta) per_cta = chains_per_sm ? chains_per_sm : 1u;
-        // Copy-on-write slices: always for the wide kernel; for the narrow kernel where whole copies of the initial
-        // schedule would add up to gigabytes (growing_8b: 1024 x 17 MB, a third of the kernel's time), not where they are
-        // small (layer_8b: 1024 x 512 KB), because a take-over lengthens the path through an applied move (layer_8b
-        // 14.0 -> 16.0 ms with it).
-        const size_t most = a->chains < (size_t)full / W * sms ? a->chains : (size_t)full / W * sms;
-        const bool overlay = c.wide || (hooks.overlay ? hooks.overlay == 1 : most * col_bytes >= ((size_t)4 << 30));
-        if (overlay) {
+        {
             // The bucket bitmap takes what a full CTA of chains leaves of the shared memory: the smaller the buckets, the
             // fewer reads of a long chain go to its private slice.
-            const size_t bare = fixed_bytes(W, false, false);
+            const size_t bare = fixed_bytes(W, false);
             if (budget / bare < per_cta) per_cta = (uint32_t)(budget / bare);
             if (per_cta < 1) return KVP_ERR_RANGE;
             const size_t share = budget / per_cta;
@@ -1385,7 +769,7 @@ int prepare(kvp_problem* p, const kvp_anneal_params* a, cudaStream_t st, Ctx& c,
             const uint64_t buckets = ((uint64_t)p->U + (1ull << c.cow_shift) - 1) >> c.cow_shift;
             c.cow_slots4 = (uint32_t)((buckets + 127) / 128);
         }
-        c.smem_per_warp = fixed_bytes(W, false, false);
+        c.smem_per_warp = fixed_bytes(W, false);
         if (c.smem_per_warp > budget) return KVP_ERR_RANGE;
         c.wpc = W;
         uint32_t wcap = (uint32_t)(budget / c.smem_per_warp);     // chains per CTA at most
@@ -1501,11 +885,8 @@ int prepare(kvp_problem* p, const kvp_anneal_params* a, cudaStream_t st, Ctx& c,
     // test hook (tests of the bounded wait only): one hand-over per chain is withheld, the waiting warp gives up
     // after its poll limit (about a second) and the call returns KVP_ERR_TIMEOUT
     prm.drop_first_turn = hooks.drop_turn ? 1u : 0u;
-    // test hook: batches with more than n < 496 queue items already take the two-halves path of the half-size work
-    // queue, which ordinary inputs almost never reach
-    prm.split_at = kQueueCap / 2;
+    // test hook: less room for accepted proposals, so that a batch stops to commit more often
     prm.carry = kAccepted;
-    if (hooks.split_queue_plus1 >= 1 && hooks.split_queue_plus1 - 1 < kQueueCap / 2) prm.split_at = hooks.split_queue_plus1 - 1;
     if (hooks.split_queue_plus1 >= 1 && hooks.split_queue_plus1 <= kAccepted) prm.carry = hooks.split_queue_plus1;
     KVP_CUDA(cudaMemsetAsync(prm.err, 0, 4, st));
     prm.U = p->U; prm.S = p->S; prm.S32 = p->S32; prm.cap = p->cap;

@@ -43,9 +43,9 @@ constexpr uint32_t kNone = 256;                           // no proposal (the id
 // the two step bitmaps turned; its units.
 struct Applied {
     uint32_t steps;              // s0 | (s0 + len) << 16
-    uint32_t bits;               // first | last << 16; first > last: none
+    uint32_t bits;               // first | last << 16; first > last: none (narrow kernel: of the bitmap "te >= th")
     uint32_t units;              // low halves of u | v << 16 (u twice for a flip)
-    uint32_t pad;
+    uint32_t fulls;              // narrow kernel: likewise of the bitmap "HBM is full"
 };
 
 // The scalars of a chain, its hand-over block when several warps serve it, and the log of its latest applied moves.
@@ -799,7 +799,7 @@ wide_chain_kernel(const __grid_constant__ ChainParams prm)
                     Applied g;
                     g.steps = s0b | (s0b + ((a.x >> 1) & 31u)) << 16;
                     g.units = (a.y & 0xFFFFu) | ((a.x & 1u) ? a.z : a.y) << 16;
-                    g.pad = 0u;
+                    g.fulls = 0u;
                     g.bits = apply(c, lane, a, w);
                     if (lane == 0) record(prm, sc, m + id, after, leaving, g, slot);
                     __syncwarp();
