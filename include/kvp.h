@@ -275,11 +275,11 @@ int kvp_accept_table(const double* temps, uint32_t levels, uint32_t* table, uint
  *   stats (host) or NULL; stats->per_chain must be NULL or a host array [chains]
  *   (entry i belongs to chain first_chain + i)
  * Synchronises `stream` before returning.
- * Two chain kernels serve a job, chosen by its size (chains per SM, units, whether the schedules fit shared memory) and
- * start temperature: the wide one evaluates batches of 128 or 256 proposals, rejecting most of them by a lower bound of
- * their cost change, with one to four warps per chain; the narrow one batches of 32, with one or two. Chains whose
- * schedules do not fit shared memory keep them as copy-on-write overlays of the one initial schedule (or, small ones on the
- * narrow kernel, as copies of it). The
+ * Two chain kernels serve a job, chosen by its size (chains per SM, units, steps, whether the schedules fit shared memory)
+ * and start temperature: the wide one evaluates batches of 128 or 256 proposals ahead, rejecting most of them by a lower
+ * bound of their cost change; the narrow one prepares batches of 32 and evaluates what is left of them in move order.
+ * Either serves a chain with one to four warps. Chains whose schedules do not fit shared memory keep them as copy-on-write
+ * overlays of the one initial schedule. The
  * results are those of the sequential chain either way. The only device-side wait of the library is a warp's wait
  * for its turn where several serve a chain; it is bounded, and a chain whose wait runs out makes the call return
  * KVP_ERR_TIMEOUT (the outputs are then undefined). The library reads no environment variable; the switches that
@@ -468,18 +468,16 @@ void kvp_philox4x32_10(const uint32_t ctr[4], const uint32_t key[2], uint32_t ou
  * kvp_anneal_chain_state. No production caller needs them. All zero = the library's normal behaviour; NULL resets.
  */
 typedef struct {
-    uint32_t warps_per_chain;   /* 1 or 2: the narrow chain kernel with that many warps per chain; 3: the wide
-                                   chain kernel with one; 16 + w: the wide one with w (a power of two up to 8);
-                                   whatever the job size                                                         */
+    uint32_t warps_per_chain;   /* 1, 2 or 32 + w: the narrow chain kernel with 1, 2 or w (up to 4) warps per
+                                   chain; 3 or 16 + w: the wide one with 1 or w (1, 2, 4 or 8); whatever the job
+                                   size (jobs the narrow kernel does not serve go to the wide one)                */
     uint32_t drop_turn;         /* 1: withhold one hand-over per chain so that the bounded wait for the turn
                                    runs out (about a second) and the call returns KVP_ERR_TIMEOUT               */
-    uint32_t split_queue_plus1; /* n + 1: batches with more than n work items take the rarely reached two-halves
-                                   path of the half-size work queue; wide kernel, n < 6: a batch stops to commit
-                                   when it has n + 1 accepted moves instead of 6                                  */
+    uint32_t split_queue_plus1; /* n + 1, n < 6: a batch of the wide kernel stops to commit when it has n + 1
+                                   accepted moves instead of 6                                                    */
     uint32_t resident;          /* n: at most n chains whose schedules live in global memory run at a time, so
                                    that a small job comes in several waves                                       */
-    uint32_t overlay;           /* narrow chain kernel, schedules in global memory: 1 = copy-on-write slices, 2 =
-                                   plain slices, whatever the size of the job (0: by size)                       */
+    uint32_t overlay;           /* without effect: schedules in global memory are always copy-on-write slices     */
 } kvp_test_hooks;
 void kvp_set_test_hooks(const kvp_test_hooks* hooks);
 

@@ -579,6 +579,7 @@ struct Ctx {
     bool asmem;              // the access bitmap and the step constants are staged in shared memory
     bool wide;               // the wide kernel
     uint32_t S32;            // words per time-packed column
+    bool solo;               // narrow kernel, schedules in shared memory: the variant for one warp per chain
     bool ladder_ctas;        // replica exchange: every CTA holds whole ladders (one launch)
     int rows;                // wide kernel: rows of 32 proposals in a batch
     bool lin;                // kappa_d >= kappa_k: see kvp_chain.cuh
@@ -602,9 +603,9 @@ int validate(const kvp_problem* p, const kvp_anneal_params* a)
 
 typedef void (*ChainKernel)(const ChainParams);
 
-ChainKernel narrow_kernel_for(bool psmem, bool asmem, uint32_t S32, uint32_t W)
+ChainKernel narrow_kernel_for(bool psmem, bool asmem, uint32_t S32, bool solo)
 {
-    if (psmem && W == 1) return asmem ? narrow_chain_kernel<true, true, true, 0> : narrow_chain_kernel<true, true, false, 0>;
+    if (psmem && solo) return asmem ? narrow_chain_kernel<true, true, true, 0> : narrow_chain_kernel<true, true, false, 0>;
     if (psmem) return asmem ? narrow_chain_kernel<false, true, true, 0> : narrow_chain_kernel<false, true, false, 0>;
     return S32 == 2 ? narrow_chain_kernel<false, false, false, 2> : S32 == 4 ? narrow_chain_kernel<false, false, false, 4>
                                                                              : narrow_chain_kernel<false, false, false, 0>;
@@ -633,7 +634,7 @@ ChainKernel wide_kernel_for(bool psmem, bool asmem, bool grow, bool lin, uint32_
 ChainKernel kernel_of(const Ctx& c, bool psmem, bool asmem, uint32_t W)
 {
     return c.wide ? wide_kernel_for(psmem, asmem, c.grow, c.lin, c.S32, c.rows)
-                  : narrow_kernel_for(psmem, asmem, c.S32, W);
+                  : narrow_kernel_for(psmem, asmem, c.S32, c.solo);
 }
 
 int launch_chains(const Ctx& c, ChainParams& prm, uint32_t count)
@@ -694,7 +695,7 @@ int prepare(kvp_problem* p, const kvp_anneal_params* a, cudaStream_t st, Ctx& c,
     const size_t pbytes = (size_t)p->U * p->S32 * 4;
     const bool hot = !a->temps && a->p0 >= 0.5;
     c.lin = p->K.kd >= p->K.kk;
-    c.ladder_ctas = false;
+    c.ladder_ctas = c.solo = false;
     c.rows = kRowsMany;
     c.cow_slots4 = 0;
     c.cow_shift = 0;
@@ -704,17 +705,41 @@ int prepare(kvp_problem* p, const kvp_anneal_params* a, cudaStream_t st, Ctx& c,
         if (c.wide) return chain_bytes(p->S, p->S32, c.grow, shared, c.lin, shared ? 0u : c.cow_slots4, warps, c.rows);
         return narrow_bytes(p->S, p->S32, shared, shared ? 0u : c.cow_slots4, warps);
     };
-    c.psmem = true;
-    if (hooks.warps_per_chain) c.wide = hooks.warps_per_chain == 3 || (hooks.warps_per_chain >= 16 && hooks.warps_per_chain < 32);
-    else if (hot) c.wide = false;
-    else c.wide = (uint64_t)p->U * p->S >= 4096u;
-    if (exchange || !c.lin || c.grow) c.wide = true;              // the narrow kernel does not serve these
+    // Which kernel, and how many warps per chain (W; an SM holds 16). The lines are where the two cross over in measurements
+    // on 1 to 640 groups, 16 to 2.6M units, 32 to 512 steps and 64 to 4096 chains of 8,000 to 200,000 moves.
+    //  - Hot starts (C_0 from p0 >= 0.5: a fifth of the proposals change the schedule): the narrow kernel. Schedules in
+    //    shared memory: one warp, 13.5 ms on 256 units x 512 steps, 1024 chains x 100,000 moves (two: 22, hand-overs are
+    //    too many; wide kernel: 32). In global memory two warps while an SM has at most 8 chains (equal or 5% better).
+    //  - Otherwise, at most 8 chains per SM: the narrow kernel with as many warps as fit, four at most, two at most on
+    //    short horizons, where moves meet more often (16,384 units x 256 steps, 1024 chains x 200,000 moves: 11.5 against
+    //    14.3 ms; 65,536 x 128, 64 chains x 20,000: 0.48 with four warps, 0.76 with two). But where a batch has few
+    //    proposals to judge, that is with many units, the wide kernel's compaction pays off as soon as an SM has more than
+    //    5 chains (262,144 x 64, 1036 chains x 50,000: 1.33 against 1.77 ms).
+    //  - More chains per SM: the wide kernel with one warp per chain; but the narrow one on schedules in global memory of
+    //    few units, whose chains apply many moves (16,384 x 256, 1480 chains x 20,000: 2.2 against 3.7 ms), and on short
+    //    horizons in shared memory (64 x 64: 0.89 against 1.04 ms; 64 x 512: 0.82 against 0.77).
+    // What counts as chains of an SM is how many it holds at a time, when their schedules take its shared memory.
+    // kvp_set_test_hooks can force the choice (warps_per_chain 1, 2 or 32 + w: narrow; 3 or 16 + w: wide).
+    const bool many_units = p->U >= 32768u;
+    c.wide = false;
     c.psmem = fixed_bytes(1, true) + pbytes + 16 <= budget / 2 && p->U < 65536u;
+    uint32_t held = chains_per_sm;
+    if (c.psmem) {
+        const uint32_t fit = (uint32_t)((budget - 16) / (fixed_bytes(1, true) + pbytes));
+        if (held > fit) held = fit > 8 && fit < 12 ? 8u : fit;    // eight with two warps each do more than eleven with one
+    }
+    const bool few = held <= 8;
+    if (!hot) c.wide = c.psmem ? !few && p->S >= 256u : many_units && held > 5;
+    if (hooks.warps_per_chain) c.wide = hooks.warps_per_chain == 3 || (hooks.warps_per_chain >= 16 && hooks.warps_per_chain < 32);
+    if (exchange || !c.lin || c.grow) c.wide = true;              // the narrow kernel does not serve these
+    if (c.wide) c.psmem = fixed_bytes(1, true) + pbytes + 16 <= budget / 2 && p->U < 65536u;
     const uint32_t forced = hooks.warps_per_chain == 3 ? 1u : hooks.warps_per_chain >= 16 ? hooks.warps_per_chain & 15u : hooks.warps_per_chain;
-#ifndef NTHR
-#define NTHR 512
-#endif
-    const uint32_t full = !c.wide && !c.psmem ? NTHR / 32 : 16;                                     // warps of a CTA that fills an SM (at 128 registers)
+    const uint32_t full = 16;
+    auto narrow_warps = [&]() {
+        if (hot) return !c.psmem && few ? 2u : 1u;
+        const uint32_t most = held <= 4 ? 4u : held == 5 ? 3u : held <= 8 ? 2u : 1u;
+        return p->S < 128u && (c.psmem || !many_units) ? std::min(most, 2u) : most;
+    };
     uint32_t W = 1;
     if (c.psmem) {
         uint32_t want = chains_per_sm < 1 ? 1 : chains_per_sm;
@@ -724,18 +749,23 @@ int prepare(kvp_problem* p, const kvp_anneal_params* a, cudaStream_t st, Ctx& c,
             const size_t a_off = ((size_t)chains * (pbytes / 4) + 3) & ~(size_t)3, c_off = (a_off + pbytes / 4 + 3) & ~(size_t)3;
             return (size_t)chains * fixed_bytes(warps, true) + c_off * 4 + 16;
         };
-        // two warps per chain, four where an SM has three chains or fewer (256 units x 512 steps, 50,000 moves, 148 and
-        // 740 chains: one warp 1.62 and 1.79 ms, two 1.12 and 1.34, four 1.05 and 2.40)
-        W = chains_per_sm <= 3 ? 4 : 2;
-        while (W > 1 && (want * W > full || with_a(want, W) > budget)) W /= 2;
+        if (c.wide) {
+            // two warps per chain, four where an SM has three chains or fewer (256 units x 512 steps, 50,000 moves, 148 and
+            // 740 chains: one warp 1.62 and 1.79 ms, two 1.12 and 1.34, four 1.05 and 2.40)
+            W = chains_per_sm <= 3 ? 4 : 2;
+            while (W > 1 && (want * W > full || with_a(want, W) > budget)) W /= 2;
+        } else {
+            W = narrow_warps();
+            while (W > 1 && (fixed_bytes(W, true) + pbytes) * held + 16 > budget) --W;
+        }
         if (forced) W = forced;
         c.wpc = W;
         c.smem_per_warp = fixed_bytes(W, true) + pbytes;
         uint32_t wmax = (uint32_t)((budget - 16) / c.smem_per_warp);
         if (wmax > full / W) wmax = full / W;
-        if (!c.wide && W == 1 && wmax > 8u) wmax = 8u;            // that variant is built for CTAs of up to 256 threads
         if (wmax < 1) return KVP_ERR_RANGE;
         c.wpb = want > wmax ? wmax : want;
+        c.solo = !c.wide && W == 1 && c.wpb <= 8u;                // that variant is built for CTAs of up to 256 threads
         if (exchange && rungs <= wmax) {
             c.ladder_ctas = true;
             c.wpb = c.wpb / rungs * rungs;
@@ -748,9 +778,9 @@ int prepare(kvp_problem* p, const kvp_anneal_params* a, cudaStream_t st, Ctx& c,
         }
         KVP_CUDA(cudaFuncSetAttribute(kernel_of(c, true, c.asmem, W), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)budget));
     } else {
-        // Two warps per chain while that leaves an SM at most 16 warps (the registers allow no more). More per chain are no
-        // faster (16,384 units x 256 steps, 148 chains: 6.76 ms with two and with four, 7.5 with one).
-        if (!exchange && chains_per_sm <= 8) W = 2;
+        // wide: two warps per chain while an SM has at most 8 (more per chain are no faster)
+        if (!c.wide) W = narrow_warps();
+        else if (!exchange && few) W = 2;
         if (forced) W = forced;
         if (W == 1 && c.wide && c.lin) c.rows = kRowsOne;
         uint32_t per_cta = full / W;                              // chains of a full CTA

@@ -7,24 +7,18 @@
 // lower bound of kvp_chain.cuh, which rejects most of the rest. An applied move spoils a later preparation only if both name
 // a unit and have steps in common; a flip is checked again if one of its steps became full or free, a bounded rejection if
 // the leading side of one of its steps changed. The proposals that are left are evaluated in move order, against the state
-// as it is, a lane per step of the window; kSide of them side by side, since their steps seldom meet those of one another,
-// and what bounds a chain is the latency of these dependent steps (votes, sums over the warp, shared-memory loads).
+// as it is, a lane per step of the window (two side by side where the registers allow it: their steps seldom meet); what
+// bounds a chain is the latency of these dependent steps (votes, sums over the warp, shared-memory loads).
 // W warps may serve a chain: they take its batches in turn and prepare ahead of each other's commits (see ChainShared).
 //
 // The kernel before evaluated its 32 proposals in full, ahead of the commits, through a work queue of (proposal, step)
-// items, one move applied per pass. Measured (B200), before and now: KVP_NARROW_MEASURED
+// items, one move applied per pass. Measured (B200), before and now: 256 units x 512 steps at p0 = 0.8, 1024
+// chains x 100,000 moves: 25.5 -> 13.6 ms; 16 x 32, 64 x 10,000: 0.43 -> 0.35; 16,384 x 256, 1024 x 200,000: 15.4 -> 11.5.
 #pragma once
 
 namespace kvp {
 
 namespace {
-
-#ifndef NSIDE
-#define NSIDE 1
-#endif
-#ifndef NTHR
-#define NTHR 512
-#endif
 
 constexpr uint32_t kPrepared4 = 4 * 32;                   // uint4 slots of a warp's prepared proposals
 
@@ -69,11 +63,11 @@ struct Narrow {
 // PSMEM: schedules in shared memory; otherwise a chain's slice of global scratch is a copy-on-write overlay of the initial
 // schedule. ASMEM: the access bitmap staged there, too. SOLO: one warp per chain (W == 1).
 template <bool SOLO, bool PSMEM, bool ASMEM, int COLV>
-__global__ void __launch_bounds__(SOLO ? 256 : PSMEM ? 512 : NTHR, 1)
+__global__ void __launch_bounds__(SOLO ? 256 : 512, 1)
 narrow_chain_kernel(const __grid_constant__ ChainParams prm)
 {
     static_assert(PSMEM ? COLV == 0 : !ASMEM && !SOLO, "vector columns only for schedules in global scratch");
-    constexpr int kSide = SOLO ? 2 : NSIDE;
+    constexpr int kSide = SOLO ? 2 : 1;                           // (registers: 157; two in the other variants spill)
     using Occ = typename Narrow<PSMEM>::Occ;
     const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5, W = SOLO ? 1u : prm.warps;
     const uint32_t cpb = (blockDim.x >> 5) / W, cic = warp / W, sub = warp % W;   // chains per CTA; chain; warp of the chain

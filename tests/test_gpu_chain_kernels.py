@@ -1,0 +1,71 @@
+"""The chain kernels' variants at the sizes where they can go wrong, against the oracle bit for bit: every number of warps
+per chain, window edges (steps around multiples of 32), vector columns (two and four words), columns longer than half a
+warp, schedules in shared and in global memory, weights for which the narrow kernel is not built, replica exchange inside
+CTAs and in launches."""
+import numpy as np
+import pytest
+
+from paper_2508_13231_b200 import workloads as wl
+from gpu_util import both_problems, to_np
+
+pytestmark = pytest.mark.gpu
+GB = 10 ** 9
+NARROW, WIDE = (1, 2, 35, 36), (3, 18, 20)       # kvp_test_hooks.warps_per_chain
+
+
+@pytest.fixture(scope="module")
+def kvp():
+    from paper_2508_13231_b200 import kvp
+    return kvp
+
+
+def _same(g, o, **kw):
+    out = g.anneal(g.make_params(**kw), want_per_chain=True)
+    ref = o.anneal(o.make_params(**kw))
+    assert [r.astuple() for r in out["per_chain"]] == [r.astuple() for r in ref["per_chain"]]
+    assert np.array_equal(to_np(out["best_schedule"]), ref["best_schedule"])
+
+
+@pytest.mark.parametrize("warps", NARROW + WIDE)
+@pytest.mark.parametrize("U,S,cap", [
+    (2, 2, 1), (31, 32, 9), (40, 31, 0), (40, 33, 40), (65, 64, 20), (33, 97, 10),   # schedules in shared memory
+    (7000, 64, 2000), (5000, 128, 900), (3000, 257, 700), (300, 2050, 90),           # in global memory: 2, 4, 9, 65 words
+])
+def test_shapes(kvp, oracle, hooks, warps, U, S, cap):
+    hooks(warps_per_chain=warps)
+    A = wl.random_access(U, S, 0.2, seed=U + S)
+    g, o = both_problems(kvp, oracle, U, 8192, S, A, cap, (4900 * GB, 900 * GB, 500 * GB))
+    for p0 in (0.8, 1e-4):
+        _same(g, o, chains=5, moves=1500, seed=U, levels=6, p0=p0, early_stop_permille=1, early_stop_from_level=4)
+
+
+@pytest.mark.parametrize("bw,flags", [((4900, 500, 900), 3), ((4900, 500, 900), 1), ((3, 1, 1), 0)])
+def test_weights(kvp, oracle, hooks, bw, flags):
+    """A link slower than the DRAM channels (the cost is not linear in migrations), migrations free on a side or both."""
+    A = wl.random_access(90, 70, 0.3, seed=1)
+    g, o = both_problems(kvp, oracle, 90, 8192, 70, A, 30, tuple(b * GB for b in bw), mig_flags=flags)
+    for warps in (2, 18):
+        hooks(warps_per_chain=warps)
+        _same(g, o, chains=6, moves=2000, seed=4, levels=4, p0=0.3)
+
+
+@pytest.mark.parametrize("chains,rungs", [(24, 3), (40, 8), (36, 12), (40, 20)])
+def test_exchange_rounds(kvp, oracle, chains, rungs):
+    """Ladders that fill a CTA exactly, leave chains of it idle, or do not fit one (a launch per round)."""
+    A = wl.random_access(120, 90, 0.25, seed=2)
+    g, o = both_problems(kvp, oracle, 120, 8192, 90, A, 30, (8000 * GB, 900 * GB, 900 * GB))
+    kw = dict(chains=chains, moves=701, seed=9, levels=rungs, p0=1e-2, alpha=0.7)
+    out = g.anneal_exchange(g.make_params(**kw), rungs, 100)
+    ref = o.anneal_exchange(o.make_params(**kw), rungs, 100, want_best=True)
+    assert [r.astuple() for r in out["per_chain"]] == [r.astuple() for r in ref["per_chain"]]
+    assert out["final_rung"] == ref["final_rung"].tolist() and out["n_exchanged"] == ref["n_exchanged"].tolist()
+    assert np.array_equal(to_np(out["best_schedule"]), ref["best_schedule"])
+
+
+@pytest.mark.parametrize("scale", [1, 2 ** 10, 2 ** 20])
+def test_accept_table_rows(kvp, oracle, scale):
+    """Rows built as geometric sequences against exp() for every entry, at temperatures around powers of two."""
+    temps = np.sort(np.concatenate([[0.3, 1.0, 1.0, 44.5, 44.6], scale * np.geomspace(1.0, 1000.0, 300)]))[::-1].copy()
+    table, shifts = kvp.accept_table(temps)
+    want, wshifts = oracle.accept_table(temps)
+    assert np.array_equal(to_np(table), np.asarray(want, dtype=np.uint32)) and np.array_equal(to_np(shifts), np.asarray(wshifts, dtype=np.uint32))
