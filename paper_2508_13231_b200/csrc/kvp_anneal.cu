@@ -561,7 +561,6 @@ struct Ctx {
     uint32_t* slots;         // chain state slices (global variant)
     uint32_t* full0;         // [S32]
     uint32_t* hb0;           // growing cache: [S] written-to-HBM counts of the initial schedule
-    uint32_t* hb_tmp;        // growing cache: [S] the same for the winner's re-score
     bool grow;
     uint32_t* snap;          // best-state snapshots (shared-memory variant), or null
     uint64_t* undo_log;      // undo logs (global variant), or null
@@ -841,13 +840,12 @@ int prepare(kvp_problem* p, const kvp_anneal_params* a, cudaStream_t st, Ctx& c,
     // workspace layout
     size_t off = 0;
     auto take = [&](size_t bytes) { size_t o = off; off += align256(bytes); return o; };
-    const size_t o_P0 = take(sched_bytes), o_col0 = take(col_bytes), o_cnt = take((size_t)p->S * 16);
+    const size_t o_P0 = take(sched_bytes), o_col0 = take(col_bytes), o_cnt = take((size_t)p->S * 20 + 4);   // counts, births, ticket
     const size_t o_small = take(256), o_table = take((size_t)a->levels * KVP_TABLE_Q * 4), o_shift = take((size_t)a->levels * 4), o_bound = take((size_t)a->levels * 4);
     const size_t o_res = take((size_t)(a->chains + 1) * sizeof(kvp_chain_result));
     const size_t o_dump = take(col_bytes), o_sched = take(sched_bytes);
     const size_t o_slots = take(c.psmem ? 0 : (size_t)c.resident * col_bytes);
     const size_t o_full = take((size_t)p->S32 * 4);
-    const size_t o_hb0 = take(c.grow ? (size_t)p->S * 4 : 0), o_hbt = take(c.grow ? (size_t)p->S * 4 : 0);
     // Chains whose schedule lives in shared memory save it to global memory whenever they leave their best state;
     // chains in global scratch do not (a copy would cost as much as thousands of moves): their winner is replayed.
     const size_t snap_bytes = (size_t)a->chains * p->U * p->S32 * 4;
@@ -869,7 +867,7 @@ int prepare(kvp_problem* p, const kvp_anneal_params* a, cudaStream_t st, Ctx& c,
     c.bounds = (float*)(base + o_bound);
     c.results = (kvp_chain_result*)(base + o_res); c.dumpcol = (uint32_t*)(base + o_dump);
     c.sched = (uint32_t*)(base + o_sched); c.slots = (uint32_t*)(base + o_slots);
-    c.hb0 = c.grow ? (uint32_t*)(base + o_hb0) : nullptr; c.hb_tmp = c.grow ? (uint32_t*)(base + o_hbt) : nullptr;
+    c.hb0 = c.grow ? c.counts0 + (size_t)p->S * 4 : nullptr;
     c.full0 = (uint32_t*)(base + o_full); c.snap = snapshots ? (uint32_t*)(base + o_snap) : nullptr;
     c.undo_log = c.psmem ? nullptr : (uint64_t*)(base + o_ulog); c.undo_len = c.psmem ? nullptr : (uint32_t*)(base + o_ulen);
     c.cow_out = cow ? (uint32_t*)(base + o_cow) : nullptr;
@@ -896,11 +894,9 @@ int prepare(kvp_problem* p, const kvp_anneal_params* a, cudaStream_t st, Ctx& c,
         if ((rc = launch_bit_transpose(c.P0, p->S, p->W32, p->U, c.Pcol0, p->S32, st))) return rc;
         c.launches += a->init_mode == KVP_INIT_USER ? 2 : 1;
     }
-    if ((rc = launch_counts(p, c.P0, 1, c.counts0, c.hb0, st, &c.launches))) return rc;
-    if ((rc = launch_finish(p, c.counts0, c.hb0, 1, nullptr, c.small, nullptr, nullptr, (int32_t*)(c.small + 2), c.small + 1,
-                            st)))
+    if ((rc = launch_score(p, c.P0, 1, c.counts0, c.counts0, c.hb0, nullptr, c.small, nullptr, nullptr, (int32_t*)(c.small + 2),
+                           c.small + 1, st, &c.launches)))
         return rc;
-    ++c.launches;
     full_mask_kernel<<<(p->S32 * 32 + 255) / 256, 256, 0, st>>>((const uint4*)c.counts0, p->S, p->cap, c.full0);
     KVP_CUDA(cudaGetLastError());
     ++c.launches;
@@ -1075,11 +1071,9 @@ extern "C" int kvp_anneal(kvp_problem* p, const kvp_anneal_params* a, uint32_t* 
         red.best_chain += a->first_chain;
         if ((rc = replay_to_sched(p, c, red.best_chain, upto, c.results + a->chains))) return rc;
     }
-    if ((rc = launch_counts(p, c.sched, 1, c.counts0, c.hb_tmp, st, &c.launches))) return rc;
-    if ((rc = launch_finish(p, c.counts0, c.hb_tmp, 1, nullptr, c.small, nullptr, nullptr, (int32_t*)(c.small + 2),
-                            c.small + 1, st)))
+    if ((rc = launch_score(p, c.sched, 1, c.counts0, nullptr, nullptr, nullptr, c.small, nullptr, nullptr, (int32_t*)(c.small + 2),
+                           c.small + 1, st, &c.launches)))
         return rc;
-    ++c.launches;
     if (best_schedule)
         KVP_CUDA(cudaMemcpyAsync(best_schedule, c.sched, (size_t)p->S * p->W32 * 4, cudaMemcpyDeviceToDevice, st));
     uint64_t host_small[4];
@@ -1279,11 +1273,9 @@ extern "C" int kvp_anneal_exchange(kvp_problem* p, const kvp_anneal_params* a, c
         c.launches += 2;
     }
     red.best_chain += a->first_chain;
-    if ((rc = launch_counts(p, c.sched, 1, c.counts0, c.hb_tmp, st, &c.launches))) return rc;
-    if ((rc = launch_finish(p, c.counts0, c.hb_tmp, 1, nullptr, c.small, nullptr, nullptr, (int32_t*)(c.small + 2),
-                            c.small + 1, st)))
+    if ((rc = launch_score(p, c.sched, 1, c.counts0, nullptr, nullptr, nullptr, c.small, nullptr, nullptr, (int32_t*)(c.small + 2),
+                           c.small + 1, st, &c.launches)))
         return rc;
-    ++c.launches;
     if (best_schedule)
         KVP_CUDA(cudaMemcpyAsync(best_schedule, c.sched, (size_t)p->S * p->W32 * 4, cudaMemcpyDeviceToDevice, st));
     uint64_t host_small[4];

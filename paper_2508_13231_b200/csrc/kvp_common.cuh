@@ -151,12 +151,13 @@ int ensure_chain_ws(kvp_problem* p, size_t bytes, cudaStream_t st);
 
 // kvp_cost.cu
 int launch_row_popcount(const uint32_t* rows, uint32_t S, uint32_t W32, uint32_t* out, cudaStream_t st);
-// hbc: [n][S] units written to HBM at birth; needed (and only used) when the problem has births
-int launch_counts(const kvp_problem* p, const uint32_t* schedules, uint32_t n, uint32_t* counts, uint32_t* hbc,
-                  cudaStream_t st, uint32_t* launches);
-int launch_finish(const kvp_problem* p, const uint32_t* counts, const uint32_t* hbc, uint32_t n, uint64_t* step_ticks,
-                  uint64_t* total_ticks, double* step_seconds, double* total_seconds, int32_t* bad_step, uint64_t* hits,
-                  cudaStream_t st);
+// Scores n schedules (Eq. 1-5). scratch: score_scratch_bytes(p, n) bytes, null if that is 0. counts_out [n][S][4] = {hr, mi,
+// mo, occ} and hbc_out [n][S] (problems with births: units written to HBM at birth): copies of the counts, or null.
+size_t score_scratch_bytes(const kvp_problem* p, uint32_t n);
+int launch_score(const kvp_problem* p, const uint32_t* schedules, uint32_t n, void* scratch, uint32_t* counts_out, uint32_t* hbc_out,
+                 uint64_t* step_ticks, uint64_t* total_ticks, double* step_seconds, double* total_seconds, int32_t* bad_step,
+                 uint64_t* hits, cudaStream_t st, uint32_t* launches);
+int launch_counts(const kvp_problem* p, const uint32_t* schedules, uint32_t n, uint32_t* counts, cudaStream_t st);
 
 // kvp_layout.cu
 int launch_bit_transpose(const uint32_t* in, uint32_t rows, uint32_t in_words, uint32_t cols, uint32_t* out,

@@ -1,11 +1,13 @@
 // Cost kernels: per-step cardinalities of a schedule (popc over mask AND placement words) and Eq. 1-5.
 //
-// The counting pass is the HBM-bound part: every word of A and of P is read once, P[s-1] is carried
-// in registers from the previous iteration. Two shapes:
-//   wide rows   (>= 17 vectors per row): a warp owns 64 consecutive 16-byte vectors of every row of a
-//               step chunk; a CTA of 8 warps therefore reads 8 KB contiguous per row and array.
-//   narrow rows (<= 16 vectors per row): a sub-warp group of LPR lanes owns whole rows, consecutive
-//               groups own consecutive rows, so a warp still reads contiguous memory.
+// Two forms. Small schedules, where launches and latency are all there is: score_kernel, one CTA per schedule, groups of
+// lanes own whole rows, everything in one launch. Large ones, HBM-bound: count_wide_kernel, in which a warp owns 64
+// consecutive 16-byte vectors of every row of a step chunk, carries P[s-1] in registers (every word of A and P is read once)
+// and adds its per-step counts to global counters; the last CTA of a schedule turns them into ticks.
+#include <string.h>
+
+#include <algorithm>
+
 #include "kvp_common.cuh"
 
 namespace kvp {
@@ -56,6 +58,57 @@ __device__ __forceinline__ uint2 vec_counts(uint4 a, uint4 p, uint4 prev)
     return make_uint2(hr | (mi << 16), mo | (occ << 16));
 }
 
+// Where the results of a scoring go; every pointer but stepc may be null.
+struct ScoreOut {
+    const StepC* stepc;
+    CostK K;
+    uint32_t cap;
+    double spt;
+    uint64_t* step_ticks; uint64_t* total_ticks;
+    double* step_seconds; double* total_seconds;
+    int32_t* bad_step;
+    uint64_t* hits;
+};
+
+// One step's counts c = {hr, mi, mo, occ} (and hb, growing cache) of schedule i into its outputs and the running sums.
+struct ScoreSum {
+    uint64_t ticks = 0, hits = 0;
+    uint32_t bad = 0xFFFFFFFFu;
+};
+template <bool GROW>
+__device__ __forceinline__ void score_step(const ScoreOut& o, uint32_t i, uint32_t S, uint32_t s, uint4 c, uint32_t hb, ScoreSum& sum)
+{
+    const uint32_t f = GROW ? step_cost_g(c.x, c.y, c.z, hb, __ldg(&o.stepc[s]), o.K) : step_cost(c.x, c.y, c.z, __ldg(&o.stepc[s]), o.K);
+    if (o.step_ticks) o.step_ticks[(size_t)i * S + s] = f;
+    if (o.step_seconds) o.step_seconds[(size_t)i * S + s] = (double)f * o.spt;
+    sum.ticks += f;
+    sum.hits += c.x;
+    if (c.w > o.cap) sum.bad = min(sum.bad, s);
+}
+// the CTA's sums into the totals of schedule i; all threads call it
+__device__ __forceinline__ void score_total(const ScoreOut& o, uint32_t i, ScoreSum sum)
+{
+    __shared__ uint64_t s_sum[32], s_hit[32];
+    __shared__ uint32_t s_bad[32];
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+        sum.ticks += __shfl_xor_sync(0xFFFFFFFFu, sum.ticks, off);
+        sum.hits += __shfl_xor_sync(0xFFFFFFFFu, sum.hits, off);
+    }
+    sum.bad = __reduce_min_sync(0xFFFFFFFFu, sum.bad);
+    const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (lane == 0) { s_sum[warp] = sum.ticks; s_hit[warp] = sum.hits; s_bad[warp] = sum.bad; }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (uint32_t w = 1; w < blockDim.x / 32; ++w) { sum.ticks += s_sum[w]; sum.hits += s_hit[w]; sum.bad = min(sum.bad, s_bad[w]); }
+        if (o.total_ticks) o.total_ticks[i] = sum.ticks;
+        if (o.total_seconds) o.total_seconds[i] = (double)sum.ticks * o.spt;
+        if (o.bad_step) o.bad_step[i] = sum.bad == 0xFFFFFFFFu ? -1 : (int32_t)sum.bad;
+        if (o.hits) o.hits[i] = sum.hits;
+    }
+    __syncthreads();
+}
+
 constexpr int WIDE_WARPS = 8;
 constexpr int WIDE_VEC = 2;              // 16-byte vectors per lane and row
 
@@ -93,7 +146,7 @@ template <int VEC, bool GROW, int NS>
 __global__ void __launch_bounds__(WIDE_WARPS * 32)
 count_wide_kernel(const uint32_t* __restrict__ A, const uint32_t* __restrict__ Ps, uint32_t S, uint32_t W32,
                   uint32_t WV, uint32_t pad_mask, uint32_t SC, uint32_t n, uint32_t* __restrict__ counts,
-                  const uint32_t* __restrict__ L, uint32_t* __restrict__ hbc)
+                  const uint32_t* __restrict__ L, uint32_t* __restrict__ hbc, uint32_t* __restrict__ tickets, const ScoreOut out)
 {
     extern __shared__ uint2 acc[];                       // [NS][WIDE_WARPS][SC], then GROW: uint32 [NS][WIDE_WARPS][SC]
     uint32_t* acc_hb = reinterpret_cast<uint32_t*>(acc + NS * WIDE_WARPS * SC);
@@ -199,90 +252,70 @@ count_wide_kernel(const uint32_t* __restrict__ A, const uint32_t* __restrict__ P
             }
         }
     }
+    if (!tickets) return;
+    // the last CTA of these schedules scores them
+    __shared__ uint32_t s_last;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) s_last = atomicAdd(tickets + blockIdx.z, 1u) + 1u == gridDim.x * gridDim.y ? 1u : 0u;
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+#pragma unroll 1
+    for (uint32_t i = blockIdx.z * NS; i < min(n, (blockIdx.z + 1) * NS); ++i) {
+        ScoreSum sum;
+        for (uint32_t s = threadIdx.x; s < S; s += blockDim.x)
+            score_step<GROW>(out, i, S, s, __ldcg(reinterpret_cast<const uint4*>(counts) + (size_t)i * S + s),
+                             GROW ? __ldcg(hbc + (size_t)i * S + s) : 0u, sum);
+        score_total(out, i, sum);
+    }
 }
 
-constexpr int NARROW_ITERS = 8;
-
-template <int VEC, int LPR, bool GROW>
-__global__ void __launch_bounds__(256)
-count_narrow_kernel(const uint32_t* __restrict__ A, const uint32_t* __restrict__ Ps, uint32_t S, uint32_t W32,
-                    uint32_t WV, uint32_t pad_mask, uint32_t* __restrict__ counts, const uint32_t* __restrict__ L,
-                    uint32_t* __restrict__ hbc)
+// Small schedules: CTA i scores schedule i. LPR lanes own a row (a power of two; more than 32 vectors: the lanes go round),
+// consecutive groups consecutive rows. counts: the four cardinalities, if wanted.
+template <int VEC, bool GROW>
+__global__ void __launch_bounds__(1024)
+score_kernel(const uint32_t* __restrict__ A, const uint32_t* __restrict__ Ps, uint32_t S, uint32_t W32, uint32_t WV, uint32_t LPR,
+             uint32_t pad_mask, const uint32_t* __restrict__ L, uint32_t* __restrict__ counts, uint32_t* __restrict__ hbc, const ScoreOut out)
 {
-    constexpr uint32_t GROUPS = 256 / LPR;               // rows in flight per CTA
-    const uint32_t g = threadIdx.x / LPR, cv = threadIdx.x % LPR;
-    const bool col_ok = cv < WV;
-    const uint32_t* __restrict__ P = Ps + (size_t)blockIdx.y * S * W32;
-    const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
+    const uint32_t groups = blockDim.x / LPR, g = threadIdx.x / LPR, l = threadIdx.x % LPR, i = blockIdx.x;
+    const uint32_t* __restrict__ P = Ps + (size_t)i * S * W32;
+    ScoreSum sum;
 #pragma unroll 2
-    for (int it = 0; it < NARROW_ITERS; ++it) {
-        const uint32_t s = (blockIdx.x * NARROW_ITERS + it) * GROUPS + g;
-        const bool ok = col_ok && s < S;
-        const uint4 a = ok ? load_vec<VEC>(A, W32, s, cv) : zero;
-        uint4 p = ok ? mask_last<VEC>(load_vec<VEC>(P, W32, s, cv), cv, WV, pad_mask) : zero;
-        uint4 q = ok ? mask_last<VEC>(load_vec<VEC>(P, W32, s ? s - 1 : 0, cv), cv, WV, pad_mask) : zero;
-        uint32_t hb = 0;
-        if (GROW) {                                      // see count_wide_kernel
-            const uint4 l = ok ? load_vec<VEC>(L, W32, s, cv) : zero;
-            const uint4 lq = ok ? load_vec<VEC>(L, W32, s ? s - 1 : 0, cv) : zero;
-            p = and4(p, l);
-            q = and4(q, lq);
-            hb = popc4(andn4(p, lq));
-        }
-        uint2 c = vec_counts(a, p, q);
-        if (GROW) c.x -= hb << 16;                       // born in HBM: written, not migrated in
-#pragma unroll
-        for (int off = LPR / 2; off > 0; off >>= 1) {
-            c.x += __shfl_xor_sync(0xFFFFFFFFu, c.x, off);
-            c.y += __shfl_xor_sync(0xFFFFFFFFu, c.y, off);
+    for (uint32_t s0 = 0; s0 < S; s0 += groups) {                 // (all lanes of a warp go through the votes)
+        const uint32_t s = s0 + g, sp = s ? s - 1 : 0;
+        uint32_t hr = 0, mi = 0, mo = 0, occ = 0, hb = 0;
+        if (s < S)
+            for (uint32_t cv = l; cv < WV; cv += LPR) {
+                const uint4 a = load_vec<VEC>(A, W32, s, cv);
+                uint4 p = mask_last<VEC>(load_vec<VEC>(P, W32, s, cv), cv, WV, pad_mask);
+                uint4 q = mask_last<VEC>(load_vec<VEC>(P, W32, sp, cv), cv, WV, pad_mask);
+                if (GROW) {                                       // see count_wide_kernel
+                    const uint4 lq = load_vec<VEC>(L, W32, sp, cv);
+                    p = and4(p, load_vec<VEC>(L, W32, s, cv));
+                    q = and4(q, lq);
+                    const uint32_t born = popc4(andn4(p, lq));
+                    hb += born;
+                    mi -= born;                                   // written, not migrated in
+                }
+                const uint2 c = vec_counts(a, p, q);
+                hr += c.x & 0xFFFFu; mi += c.x >> 16; mo += c.y & 0xFFFFu; occ += c.y >> 16;
+            }
+        for (uint32_t off = LPR / 2; off > 0; off >>= 1) {
+            hr += __shfl_xor_sync(0xFFFFFFFFu, hr, off);
+            mi += __shfl_xor_sync(0xFFFFFFFFu, mi, off);
+            mo += __shfl_xor_sync(0xFFFFFFFFu, mo, off);
+            occ += __shfl_xor_sync(0xFFFFFFFFu, occ, off);
             if (GROW) hb += __shfl_xor_sync(0xFFFFFFFFu, hb, off);
         }
-        if (cv == 0 && s < S) {
-            reinterpret_cast<uint4*>(counts)[(size_t)blockIdx.y * S + s] =
-                make_uint4(c.x & 0xFFFFu, c.x >> 16, c.y & 0xFFFFu, c.y >> 16);
-            if (GROW) hbc[(size_t)blockIdx.y * S + s] = hb;
+        if (l == 0 && s < S) {
+            const uint4 c = make_uint4(hr, mi, mo, occ);
+            if (counts) reinterpret_cast<uint4*>(counts)[(size_t)i * S + s] = c;
+            if (GROW && hbc) hbc[(size_t)i * S + s] = hb;
+            if (out.stepc) score_step<GROW>(out, i, S, s, c, hb, sum);
         }
     }
-}
-
-__global__ void __launch_bounds__(256)
-finish_kernel(const uint4* __restrict__ counts, const uint32_t* __restrict__ hbc, const StepC* __restrict__ stepc, CostK K,
-              uint32_t S, uint32_t cap,
-              double spt, uint64_t* __restrict__ step_ticks, uint64_t* __restrict__ total_ticks,
-              double* __restrict__ step_seconds, double* __restrict__ total_seconds, int32_t* __restrict__ bad_step,
-              uint64_t* __restrict__ hits)
-{
-    __shared__ uint64_t s_sum[8], s_hit[8];
-    __shared__ uint32_t s_bad[8];
-    const uint32_t i = blockIdx.x;
-    uint64_t sum = 0, hit = 0;
-    uint32_t bad = 0xFFFFFFFFu;
-    for (uint32_t s = threadIdx.x; s < S; s += blockDim.x) {
-        const uint4 c = counts[(size_t)i * S + s];
-        const uint32_t f = hbc ? step_cost_g(c.x, c.y, c.z, hbc[(size_t)i * S + s], __ldg(&stepc[s]), K)
-                               : step_cost(c.x, c.y, c.z, __ldg(&stepc[s]), K);
-        if (step_ticks) step_ticks[(size_t)i * S + s] = f;
-        if (step_seconds) step_seconds[(size_t)i * S + s] = (double)f * spt;
-        sum += f;
-        hit += c.x;
-        if (c.w > cap) bad = min(bad, s);
-    }
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-        sum += __shfl_xor_sync(0xFFFFFFFFu, sum, off);
-        hit += __shfl_xor_sync(0xFFFFFFFFu, hit, off);
-        bad = min(bad, __shfl_xor_sync(0xFFFFFFFFu, bad, off));
-    }
-    const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (lane == 0) { s_sum[warp] = sum; s_hit[warp] = hit; s_bad[warp] = bad; }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int w = 1; w < 8; ++w) { sum += s_sum[w]; hit += s_hit[w]; bad = min(bad, s_bad[w]); }
-        if (total_ticks) total_ticks[i] = sum;
-        if (total_seconds) total_seconds[i] = (double)sum * spt;
-        if (bad_step) bad_step[i] = bad == 0xFFFFFFFFu ? -1 : (int32_t)bad;
-        if (hits) hits[i] = hit;
-    }
+    if (out.stepc) score_total(out, i, sum);
 }
 
 __global__ void __launch_bounds__(256)
@@ -296,26 +329,6 @@ row_popcount_kernel(const uint32_t* __restrict__ rows, uint32_t S, uint32_t W32,
     if (lane == 0) out[warp] = c;
 }
 
-template <int VEC, bool GROW>
-int launch_narrow(uint32_t WV, uint32_t n, const uint32_t* A, const uint32_t* P, uint32_t S, uint32_t W32,
-                  uint32_t pad_mask, uint32_t* counts, const uint32_t* L, uint32_t* hbc, cudaStream_t st)
-{
-#define KVP_NARROW(LPR)                                                                                          \
-    {                                                                                                            \
-        const uint32_t rows_per_cta = (256 / LPR) * NARROW_ITERS;                                                \
-        dim3 grid((S + rows_per_cta - 1) / rows_per_cta, n);                                                     \
-        count_narrow_kernel<VEC, LPR, GROW><<<grid, 256, 0, st>>>(A, P, S, W32, WV, pad_mask, counts, L, hbc);   \
-    }
-    if (WV <= 1) KVP_NARROW(1)
-    else if (WV <= 2) KVP_NARROW(2)
-    else if (WV <= 4) KVP_NARROW(4)
-    else if (WV <= 8) KVP_NARROW(8)
-    else KVP_NARROW(16)
-#undef KVP_NARROW
-    KVP_CUDA(cudaGetLastError());
-    return KVP_OK;
-}
-
 }  // namespace
 
 int launch_row_popcount(const uint32_t* rows, uint32_t S, uint32_t W32, uint32_t* out, cudaStream_t st)
@@ -325,24 +338,45 @@ int launch_row_popcount(const uint32_t* rows, uint32_t S, uint32_t W32, uint32_t
     return KVP_OK;
 }
 
-// counts [n][S][4] = {hr, mi, mo, occ}; hbc [n][S] for a problem with births
-int launch_counts(const kvp_problem* p, const uint32_t* schedules, uint32_t n, uint32_t* counts, uint32_t* hbc,
-                  cudaStream_t st, uint32_t* launches)
+// A schedule is small when one CTA is done with it before a grid of CTAs would have started: up to 512 KB (of one SM's some
+// 200 GB/s, beside a second and a third launch). Many of them with long rows go to the streaming kernel, which reads P once.
+static bool is_small(const kvp_problem* p, uint32_t n)
+{
+    const size_t bytes = (size_t)p->S * p->W32 * 4;
+    return (bytes <= (512u << 10) && (p->W32 <= 64 || n * bytes <= ((size_t)16 << 20))) || (p->W32 <= 64 && n >= 148);
+}
+
+size_t score_scratch_bytes(const kvp_problem* p, uint32_t n)
+{
+    return is_small(p, n) ? 0 : (size_t)n * p->S * (p->dL ? 20 : 16) + (size_t)n * 4;
+}
+
+// counts [n][S][4] = {hr, mi, mo, occ}, or null if score_scratch_bytes(p, n) is 0; hbc [n][S] for a problem with births,
+// likewise; tickets [n] behind counts and hbc, or null. out.stepc null: only the counts are wanted.
+static int launch_score_impl(const kvp_problem* p, const uint32_t* schedules, uint32_t n, uint32_t* counts, uint32_t* hbc,
+                             uint32_t* tickets, const ScoreOut& out, cudaStream_t st, uint32_t* launches)
 {
     const bool grow = p->dL != nullptr;
-    if (grow && !hbc) return KVP_ERR_ARG;
     const bool vec4 = (p->W32 % 4 == 0) && ((reinterpret_cast<uintptr_t>(schedules) & 15) == 0);
     const uint32_t WV = vec4 ? p->W32 / 4 : p->W32;
-    if (WV <= 16) {
-        if (launches) *launches += 1;
-        if (grow)
-            return vec4 ? launch_narrow<4, true>(WV, n, p->dA, schedules, p->S, p->W32, p->pad_mask, counts, p->dL, hbc, st)
-                        : launch_narrow<1, true>(WV, n, p->dA, schedules, p->S, p->W32, p->pad_mask, counts, p->dL, hbc, st);
-        return vec4 ? launch_narrow<4, false>(WV, n, p->dA, schedules, p->S, p->W32, p->pad_mask, counts, nullptr, nullptr, st)
-                    : launch_narrow<1, false>(WV, n, p->dA, schedules, p->S, p->W32, p->pad_mask, counts, nullptr, nullptr, st);
+    if (launches) *launches += 1;
+    if (is_small(p, n)) {
+        uint32_t LPR = 1;
+        while (LPR < 32 && LPR < WV) LPR *= 2;
+        // one CTA per SM or fewer: as many rows side by side as there are; many CTAs: smaller ones
+        uint32_t T = (uint32_t)std::min<uint64_t>(n <= 148 ? 1024 : 256, ((uint64_t)p->S * LPR + 31) / 32 * 32);
+#define KVP_SCORE(VEC, GROW) \
+        score_kernel<VEC, GROW><<<n, T, 0, st>>>(p->dA, schedules, p->S, p->W32, WV, LPR, p->pad_mask, p->dL, counts, hbc, out)
+        if (grow) { if (vec4) KVP_SCORE(4, true); else KVP_SCORE(1, true); }
+        else { if (vec4) KVP_SCORE(4, false); else KVP_SCORE(1, false); }
+#undef KVP_SCORE
+        KVP_CUDA(cudaGetLastError());
+        return KVP_OK;
     }
-    KVP_CUDA(cudaMemsetAsync(counts, 0, (size_t)n * p->S * 16, st));
-    if (grow) KVP_CUDA(cudaMemsetAsync(hbc, 0, (size_t)n * p->S * 4, st));
+    // one call clears counts, hbc and tickets where they follow one another
+    const size_t cbytes = (size_t)n * p->S * 16, hbytes = grow ? (size_t)n * p->S * 4 : 0, tbytes = tickets ? (size_t)n * 4 : 0;
+    KVP_CUDA(cudaMemsetAsync(counts, 0, cbytes + ((char*)hbc == (char*)counts + cbytes || !grow ? hbytes + tbytes : 0), st));
+    if (grow && (char*)hbc != (char*)counts + cbytes) KVP_CUDA(cudaMemsetAsync(hbc, 0, hbytes, st));
     const uint32_t col_ctas = (WV + WIDE_WARPS * 32 * WIDE_VEC - 1) / (WIDE_WARPS * 32 * WIDE_VEC);
     // two schedules per thread once a batch is large enough to fill the GPU that way
     const uint32_t NS = n >= 8 ? 2u : 1u;
@@ -353,14 +387,14 @@ int launch_counts(const kvp_problem* p, const uint32_t* schedules, uint32_t n, u
     while (SC > 8 && (uint64_t)col_ctas * ((p->S + SC - 1) / SC) * nz < 148u * 8u * 4u) SC = (SC + 1) / 2;
     // the per-step accumulators of a chunk live in dynamic shared memory: keep them within the 48 KB a kernel gets
     // without opting in (NS * WIDE_WARPS * SC entries of 8 bytes, 12 with births)
-    const uint32_t sc_max = (uint32_t)((48u * 1024u) / (NS * WIDE_WARPS * (sizeof(uint2) + (grow ? 4 : 0))));
+    const uint32_t sc_max = (uint32_t)((47u * 1024u) / (NS * WIDE_WARPS * (sizeof(uint2) + (grow ? 4 : 0))));
     if (SC > sc_max) SC = sc_max;
     dim3 grid(col_ctas, (p->S + SC - 1) / SC, nz);
     const size_t smem = (size_t)NS * WIDE_WARPS * SC * (sizeof(uint2) + (grow ? 4 : 0));
     const int T = WIDE_WARPS * 32;
 #define KVP_WIDE(VEC, GROW, NSCH)                                                                                  \
     count_wide_kernel<VEC, GROW, NSCH><<<grid, T, smem, st>>>(p->dA, schedules, p->S, p->W32, WV, p->pad_mask, SC, n, \
-                                                              counts, GROW ? p->dL : nullptr, GROW ? hbc : nullptr)
+                                                              counts, GROW ? p->dL : nullptr, GROW ? hbc : nullptr, tickets, out)
     if (NS == 2) {
         if (grow) { if (vec4) KVP_WIDE(4, true, 2); else KVP_WIDE(1, true, 2); }
         else { if (vec4) KVP_WIDE(4, false, 2); else KVP_WIDE(1, false, 2); }
@@ -370,19 +404,34 @@ int launch_counts(const kvp_problem* p, const uint32_t* schedules, uint32_t n, u
     }
 #undef KVP_WIDE
     KVP_CUDA(cudaGetLastError());
-    if (launches) *launches += 1;
     return KVP_OK;
 }
 
-int launch_finish(const kvp_problem* p, const uint32_t* counts, const uint32_t* hbc, uint32_t n, uint64_t* step_ticks,
-                  uint64_t* total_ticks, double* step_seconds, double* total_seconds, int32_t* bad_step, uint64_t* hits,
-                  cudaStream_t st)
+int launch_score(const kvp_problem* p, const uint32_t* schedules, uint32_t n, void* scratch, uint32_t* counts_out, uint32_t* hbc_out,
+                 uint64_t* step_ticks, uint64_t* total_ticks, double* step_seconds, double* total_seconds, int32_t* bad_step,
+                 uint64_t* hits, cudaStream_t st, uint32_t* launches)
 {
-    if (p->dL && !hbc) return KVP_ERR_ARG;
-    finish_kernel<<<n, 256, 0, st>>>(reinterpret_cast<const uint4*>(counts), p->dL ? hbc : nullptr, p->d_stepc, p->K, p->S,
-                                      p->cap, p->spt, step_ticks, total_ticks, step_seconds, total_seconds, bad_step, hits);
-    KVP_CUDA(cudaGetLastError());
+    ScoreOut o;
+    o.stepc = p->d_stepc; o.K = p->K; o.cap = p->cap; o.spt = p->spt;
+    o.step_ticks = step_ticks; o.total_ticks = total_ticks; o.step_seconds = step_seconds; o.total_seconds = total_seconds;
+    o.bad_step = bad_step; o.hits = hits;
+    // scratch: counts, hbc (births), tickets
+    uint32_t* counts = static_cast<uint32_t*>(scratch);
+    uint32_t* hbc = counts && p->dL ? counts + (size_t)n * p->S * 4 : nullptr;
+    uint32_t* tickets = counts ? counts + (size_t)n * p->S * (p->dL ? 5 : 4) : nullptr;
+    if (is_small(p, n)) { counts = counts_out; hbc = hbc_out; }
+    int rc = launch_score_impl(p, schedules, n, counts, hbc, tickets, o, st, launches);
+    if (rc || is_small(p, n)) return rc;
+    if (counts_out && counts_out != counts) KVP_CUDA(cudaMemcpyAsync(counts_out, counts, (size_t)n * p->S * 16, cudaMemcpyDeviceToDevice, st));
+    if (hbc_out && hbc && hbc_out != hbc) KVP_CUDA(cudaMemcpyAsync(hbc_out, hbc, (size_t)n * p->S * 4, cudaMemcpyDeviceToDevice, st));
     return KVP_OK;
+}
+
+int launch_counts(const kvp_problem* p, const uint32_t* schedules, uint32_t n, uint32_t* counts, cudaStream_t st)
+{
+    ScoreOut none;
+    memset(&none, 0, sizeof none);
+    return launch_score_impl(p, schedules, n, counts, nullptr, nullptr, none, st, nullptr);
 }
 
 }  // namespace kvp
@@ -400,8 +449,7 @@ extern "C" int kvp_eval_counts(kvp_problem* p, const uint32_t* schedules, uint32
     const size_t sched_words = (size_t)p->S * p->W32;
     for (uint32_t i = 0; i < n; i += kBatchSlice) {
         const uint32_t m = n - i < kBatchSlice ? n - i : kBatchSlice;
-        int rc = kvp::launch_counts(p, schedules + i * sched_words, m, counts + (size_t)i * p->S * 4, nullptr,
-                                    static_cast<cudaStream_t>(stream), nullptr);
+        int rc = kvp::launch_counts(p, schedules + i * sched_words, m, counts + (size_t)i * p->S * 4, static_cast<cudaStream_t>(stream));
         if (rc) return rc;
     }
     return KVP_OK;
@@ -413,20 +461,16 @@ extern "C" int kvp_eval(kvp_problem* p, const uint32_t* schedules, uint32_t n, u
     if (!p || !schedules || !total_ticks || !n) return KVP_ERR_ARG;
     KVP_CUDA(cudaSetDevice(p->device));
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    const uint32_t slice = n < kBatchSlice ? n : kBatchSlice;
-    int rc = kvp::ensure_scratch(p, (size_t)slice * p->S * 20, st);
-    if (rc) return rc;
-    uint32_t* counts = static_cast<uint32_t*>(p->d_scratch);
-    uint32_t* hbc = counts + (size_t)slice * p->S * 4;   // used by problems with births only
     const size_t sched_words = (size_t)p->S * p->W32;
     for (uint32_t i = 0; i < n; i += kBatchSlice) {
         const uint32_t m = n - i < kBatchSlice ? n - i : kBatchSlice;
-        if ((rc = kvp::launch_counts(p, schedules + i * sched_words, m, counts, hbc, st, nullptr))) return rc;
-        const size_t so = (size_t)i * p->S;
-        if ((rc = kvp::launch_finish(p, counts, hbc, m, step_ticks ? step_ticks + so : nullptr, total_ticks + i,
-                                     step_seconds ? step_seconds + so : nullptr,
-                                     total_seconds ? total_seconds + i : nullptr, bad_step ? bad_step + i : nullptr,
-                                     nullptr, st)))
+        const size_t so = (size_t)i * p->S, need = kvp::score_scratch_bytes(p, m);
+        int rc = need ? kvp::ensure_scratch(p, need, st) : KVP_OK;
+        if (rc) return rc;
+        p->last_stream = st;
+        if ((rc = kvp::launch_score(p, schedules + i * sched_words, m, need ? p->d_scratch : nullptr, nullptr, nullptr,
+                                    step_ticks ? step_ticks + so : nullptr, total_ticks + i, step_seconds ? step_seconds + so : nullptr,
+                                    total_seconds ? total_seconds + i : nullptr, bad_step ? bad_step + i : nullptr, nullptr, st, nullptr)))
             return rc;
     }
     return KVP_OK;
@@ -436,7 +480,8 @@ extern "C" int kvp_eval(kvp_problem* p, const uint32_t* schedules, uint32_t n, u
 // kvp_eval without any allocation: the per-step cardinalities go to a fixed array in the library image.
 // Meant for callers that cannot afford or are not allowed a cudaMalloc at this point (a latency-bound
 // loop, a process whose memory pool owns the whole device, allocator-free code). See include/kvp.h.
-static __device__ __align__(256) uint32_t g_noalloc_counts[KVP_NOALLOC_SCRATCH_BYTES / 4];
+// Behind the counters of n schedules, at most 65,536 of one step, are their tickets.
+static __device__ __align__(256) uint32_t g_noalloc_counts[KVP_NOALLOC_SCRATCH_BYTES / 4 + 65536];
 
 namespace {
 constexpr int kMaxDevices = 64;
@@ -470,20 +515,16 @@ extern "C" int kvp_eval_noalloc(kvp_problem* p, const uint32_t* schedules, uint3
     if (rc) return rc;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     p->last_stream = st;
-    // The array still holds the previous call's numbers. launch_counts either overwrites every entry it
-    // owns (narrow rows) or clears them on the stream before accumulating (wide rows). The schedule index is a
-    // grid dimension, so a batch of more than kBatchSlice schedules (possible within the limit only for one or two
-    // steps) goes in slices, each with its own part of the array.
+    // The array still holds the previous call's numbers: what has to start from zero is cleared on the stream by
+    // launch_score. The schedule index is a grid dimension, so a batch of more than kBatchSlice schedules (possible
+    // within the limit only for one or two steps) goes in slices.
     const size_t sched_words = (size_t)p->S * p->W32;
     for (uint32_t i = 0; i < n; i += kBatchSlice) {
         const uint32_t m = n - i < kBatchSlice ? n - i : kBatchSlice;
         const size_t so = (size_t)i * p->S;
-        uint32_t* part = counts + so * 4;
-        if ((rc = kvp::launch_counts(p, schedules + i * sched_words, m, part, nullptr, st, nullptr))) return rc;
-        if ((rc = kvp::launch_finish(p, part, nullptr, m, step_ticks ? step_ticks + so : nullptr, total_ticks + i,
-                                     step_seconds ? step_seconds + so : nullptr,
-                                     total_seconds ? total_seconds + i : nullptr, bad_step ? bad_step + i : nullptr,
-                                     nullptr, st)))
+        if ((rc = kvp::launch_score(p, schedules + i * sched_words, m, counts, nullptr, nullptr, step_ticks ? step_ticks + so : nullptr,
+                                    total_ticks + i, step_seconds ? step_seconds + so : nullptr,
+                                    total_seconds ? total_seconds + i : nullptr, bad_step ? bad_step + i : nullptr, nullptr, st, nullptr)))
             return rc;
     }
     return KVP_OK;
