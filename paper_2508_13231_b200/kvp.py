@@ -1,10 +1,12 @@
-"""Thin ctypes binding of libkvp.so (include/kvp.h): argument marshalling only.
+"""Thin binding of libkvp.so (include/kvp.h): argument marshalling only, through ctypes; the calls that score schedules,
+whose host time would be mostly Python's, through a small extension module (csrc/kvp_torch.cpp).
 
 Bulk data are torch CUDA tensors (device memory and streams come from PyTorch); every step of the
 computation runs in the library's CUDA kernels. There is no CPU path: if the shared library is
 missing or no CUDA device is usable, calls raise.
 """
 import ctypes as C
+import importlib.util
 import os
 
 import torch
@@ -122,7 +124,7 @@ def _lib():
         if not os.path.exists(LIB_PATH):
             raise ImportError(f"{LIB_PATH} is missing: build it with `python -m paper_2508_13231_b200.build` "
                               "(there is no CPU fallback)")
-        h = C.CDLL(LIB_PATH)
+        h = C.CDLL(LIB_PATH, mode=C.RTLD_GLOBAL)
         h.kvp_strerror.restype = C.c_char_p
         h.kvp_last_cuda_error.restype = C.c_char_p
         h.kvp_destroy.restype = None
@@ -130,6 +132,24 @@ def _lib():
         h.kvp_set_test_hooks.restype = None
         _handle = h
     return _handle
+
+
+_native_module = None
+
+
+def _native():
+    """The extension module; it links against libkvp.so, so both see one library."""
+    global _native_module
+    if _native_module is None:
+        _lib()
+        path = os.path.join(_HERE, "_kvp_torch.so")
+        if not os.path.exists(path):
+            raise ImportError(f"{path} is missing: build it with `python -m paper_2508_13231_b200.build`")
+        spec = importlib.util.spec_from_file_location("_kvp_torch", path)
+        module = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(module)
+        _native_module = module
+    return _native_module
 
 
 def _chk(rc, what):
@@ -148,8 +168,7 @@ def _ptr(t, dtype=None):
 
 
 def _stream(stream=None):
-    s = torch.cuda.current_stream() if stream is None else stream
-    return C.c_void_p(s.cuda_stream)
+    return C.c_void_p(_native().current_stream() if stream is None else stream.cuda_stream)
 
 
 def set_test_hooks(warps_per_chain=0, drop_turn=0, split_queue=None, resident=0, overlay=0):
@@ -220,6 +239,7 @@ class Problem:
         _chk(_lib().kvp_create(C.byref(self._h), C.c_uint32(units), C.c_uint64(bytes_per_unit), C.c_uint32(steps),
                                _ptr(access, torch.int32), C.c_uint32(cap), C.byref(ms), hw_a, ew_a, _stream(stream)),
              "kvp_create")
+        self._address = self._h.value                         # for the extension module; 0 once closed
         if birth is not None:                                # growing cache (kvp_set_births)
             if birth.numel() != self.units:
                 self.close()
@@ -239,6 +259,7 @@ class Problem:
         if getattr(self, "_h", None):
             _lib().kvp_destroy(self._h)
             self._h = None
+            self._address = 0
 
     def __del__(self):
         try:
@@ -246,24 +267,13 @@ class Problem:
         except Exception:
             pass
 
-    def _n(self, schedules):
-        per = self.steps * self.w32
-        if schedules.numel() % per:
-            raise ValueError("schedules must be [n][steps][W32]")
-        return schedules.numel() // per
-
     def eval(self, schedules, want_steps=True, want_seconds=True, stream=None):
         """kvp_eval -> dict of CUDA tensors (step_ticks int64 [n][S], total_ticks int64 [n], seconds, bad_step)."""
-        n = self._n(schedules)
-        dev = schedules.device
-        st = torch.empty((n, self.steps), dtype=torch.int64, device=dev) if want_steps else None
-        tt = torch.empty(n, dtype=torch.int64, device=dev)
-        ss = torch.empty((n, self.steps), dtype=torch.float64, device=dev) if (want_steps and want_seconds) else None
-        ts = torch.empty(n, dtype=torch.float64, device=dev) if want_seconds else None
-        bad = torch.empty(n, dtype=torch.int32, device=dev)
-        _chk(_lib().kvp_eval(self._h, _ptr(schedules, torch.int32), C.c_uint32(n), _ptr(st), _ptr(tt), _ptr(ss),
-                             _ptr(ts), _ptr(bad), _stream(stream)), "kvp_eval")
-        return dict(step_ticks=st, total_ticks=tt, step_seconds=ss, total_seconds=ts, bad_step=bad)
+        out = _native().eval(self._address, self.steps, self.w32, schedules, want_steps, want_seconds,
+                             None if stream is None else stream.cuda_stream)
+        if out.__class__ is int:
+            _chk(out, "kvp_eval")
+        return out
 
     def eval_noalloc(self, schedules, step_ticks, total_ticks, step_seconds, total_seconds, bad_step, stream=None):
         """kvp_eval_noalloc: like eval(), but the library allocates nothing. The caller passes every output
@@ -271,16 +281,16 @@ class Problem:
         For code that cannot call the allocator here: a latency-bound loop, or a process whose memory pool
         owns the device. Batches are limited to n * steps <= 65536; calls share one scratch array per GPU,
         so do not let two of them run concurrently."""
-        n = self._n(schedules)
-        _chk(_lib().kvp_eval_noalloc(self._h, _ptr(schedules, torch.int32), C.c_uint32(n), _ptr(step_ticks),
-                                     _ptr(total_ticks), _ptr(step_seconds), _ptr(total_seconds), _ptr(bad_step),
-                                     _stream(stream)), "kvp_eval_noalloc")
+        rc = _native().eval_noalloc(self._address, self.steps, self.w32, schedules, step_ticks, total_ticks, step_seconds,
+                                    total_seconds, bad_step, None if stream is None else stream.cuda_stream)
+        if rc:
+            _chk(rc, "kvp_eval_noalloc")
 
     def eval_counts(self, schedules, stream=None):
-        n = self._n(schedules)
-        cnt = torch.empty((n, self.steps, 4), dtype=torch.int32, device=schedules.device)
-        _chk(_lib().kvp_eval_counts(self._h, _ptr(schedules, torch.int32), C.c_uint32(n), _ptr(cnt), _stream(stream)),
-             "kvp_eval_counts")
+        """kvp_eval_counts -> CUDA int32 [n][S][4] = {hr, mi, mo, occ}."""
+        cnt = _native().eval_counts(self._address, self.steps, self.w32, schedules, None if stream is None else stream.cuda_stream)
+        if cnt.__class__ is int:
+            _chk(cnt, "kvp_eval_counts")
         return cnt
 
     def make_params(self, chains, moves, seed=0, levels=64, p0=0.8, alpha=0.9, temps=None, early_stop_permille=0,
