@@ -875,8 +875,10 @@ int prepare(kvp_problem* p, const kvp_anneal_params* a, cudaStream_t st, Ctx& c,
     // initial schedule in both layouts
     if (a->init_mode == KVP_INIT_USER) {
         if ((rc = launch_clean_copy(a->init_schedule, c.P0, p->S, p->W32, p->pad_mask, st))) return rc;
+        // a unit of the initial placement enters HBM when it is written; the chains keep the bits before that clear
+        if (c.grow && (rc = launch_and_rows(c.P0, p->dL, (size_t)p->S * p->W32, st))) return rc;
         if ((rc = launch_bit_transpose(c.P0, p->S, p->W32, p->U, c.Pcol0, p->S32, st))) return rc;
-        c.launches += 2;
+        c.launches += c.grow ? 3 : 2;
     } else {
         const uint32_t* row = p->d_row_freq;
         if (a->init_mode == KVP_INIT_STATIC_FIRST) {
@@ -884,15 +886,9 @@ int prepare(kvp_problem* p, const kvp_anneal_params* a, cudaStream_t st, Ctx& c,
             row = c.sched;
             ++c.launches;
         }
-        if ((rc = launch_broadcast_row(row, p->S, p->W32, c.P0, st))) return rc;
-        if (!c.grow && (rc = launch_row_to_columns(row, p->U, p->S, p->S32, c.Pcol0, st))) return rc;
+        if ((rc = launch_broadcast_row(row, p->S, p->W32, p->dL, c.P0, st))) return rc;
+        if ((rc = launch_row_to_columns(row, p->U, p->S, p->S32, p->d_birth, c.Pcol0, st))) return rc;
         c.launches += 2;
-    }
-    if (c.grow) {
-        // a unit of the initial placement enters HBM when it is written; the chains keep the bits before that clear
-        if ((rc = launch_and_rows(c.P0, p->dL, (size_t)p->S * p->W32, st))) return rc;
-        if ((rc = launch_bit_transpose(c.P0, p->S, p->W32, p->U, c.Pcol0, p->S32, st))) return rc;
-        c.launches += a->init_mode == KVP_INIT_USER ? 2 : 1;
     }
     if ((rc = launch_score(p, c.P0, 1, c.counts0, c.counts0, c.hb0, nullptr, c.small, nullptr, nullptr, (int32_t*)(c.small + 2),
                            c.small + 1, st, &c.launches)))

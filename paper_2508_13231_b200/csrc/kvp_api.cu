@@ -109,30 +109,7 @@ extern "C" void kvp_destroy(kvp_problem* p)
 static int create_impl(kvp_problem* p, const uint32_t* access, const uint32_t* hw, const uint32_t* ew, cudaStream_t st)
 {
     const size_t nw = (size_t)p->S * p->W32;
-    int rc = prepare_pool(p->device);
-    if (rc) return rc;
-    p->last_stream = st;
-    // one block for everything the problem keeps
-    size_t off = 0;
-    auto take = [&](size_t bytes) { size_t o = off; off += (bytes + 255) & ~(size_t)255; return o; };
-    const size_t oA = take(nw * 4), oAcol = take((size_t)p->U * p->S32 * 4), oa = take((size_t)p->S * 4);
-    const size_t osc = take((size_t)p->S * sizeof(StepC)), ouc = take((size_t)p->U * 4), orf = take((size_t)p->W32 * 4);
-    KVP_CUDA(cudaMallocAsync(&p->d_block, off, st));
-    char* base = static_cast<char*>(p->d_block);
-    p->dA = (uint32_t*)(base + oA); p->dAcol = (uint32_t*)(base + oAcol); p->d_a = (uint32_t*)(base + oa);
-    p->d_stepc = (StepC*)(base + osc); p->d_ucnt = (uint32_t*)(base + ouc); p->d_row_freq = (uint32_t*)(base + orf);
-    // what launch_static_freq_row needs: histogram, selection, tie counts of the chunks of 1024 units
-    if ((rc = ensure_scratch(p, (size_t)(p->S + 8) * 16 + ((size_t)p->W32 / 32 + 2) * 4, st))) return rc;
-    if ((rc = launch_clean_copy(access, p->dA, p->S, p->W32, p->pad_mask, st))) return rc;
-    if ((rc = launch_row_popcount(p->dA, p->S, p->W32, p->d_a, st))) return rc;
-    if ((rc = launch_bit_transpose(p->dA, p->S, p->W32, p->U, p->dAcol, p->S32, st))) return rc;
-    if ((rc = launch_unit_counts(p->dAcol, p->U, p->S32, p->d_ucnt, st))) return rc;
-    if ((rc = launch_static_freq_row(p, p->d_row_freq, st))) return rc;
-    std::vector<uint32_t> a(p->S);
-    KVP_CUDA(cudaMemcpyAsync(a.data(), p->d_a, (size_t)p->S * 4, cudaMemcpyDeviceToHost, st));
-    KVP_CUDA(cudaStreamSynchronize(st));
-    // Per-step constants of the cost function; everything must stay below 2^31 so that the
-    // annealer can work in 32-bit arithmetic.
+    // Everything the cost function adds up must stay below 2^31 so that the annealer can work in 32-bit arithmetic.
     uint64_t wmax = 0;
     p->h_writes = static_cast<uint32_t*>(malloc((size_t)p->S * 4));
     if (!p->h_writes) return KVP_ERR_NOMEM;
@@ -144,15 +121,36 @@ static int create_impl(kvp_problem* p, const uint32_t* access, const uint32_t* h
     }
     const uint64_t kmax = p->kh > p->ke ? p->kh : p->ke;
     if (kmax * (2ull * p->U + wmax) >= (1ull << 31)) return KVP_ERR_RANGE;
-    std::vector<StepC> sc(p->S);
-    p->total_accessed = 0;
-    for (uint32_t s = 0; s < p->S; ++s) {
-        const uint64_t h = hw ? hw[s] : 0, e = ew ? ew[s] : 0;
-        sc[s] = make_uint4((uint32_t)(p->kh * h), (uint32_t)(p->kk * e), (uint32_t)(p->kd * e), (uint32_t)(p->ke * a[s]));
-        p->total_accessed += a[s];
+    int rc = prepare_pool(p->device);
+    if (rc) return rc;
+    p->last_stream = st;
+    // One block for everything the problem keeps; what has to start at zero (the access counts of steps and units, the
+    // scratch of the static row) lies together.
+    size_t off = 0;
+    auto take = [&](size_t bytes) { size_t o = off; off += (bytes + 255) & ~(size_t)255; return o; };
+    const size_t oA = take(nw * 4), oAcol = take((size_t)p->U * p->S32 * 4);
+    const size_t osc = take((size_t)p->S * sizeof(StepC)), orf = take((size_t)p->W32 * 4);
+    const size_t oa = take((size_t)p->S * 4), ouc = take((size_t)p->U * 4), ofr = take(static_freq_words(p) * 4);
+    const size_t owr = take(hw || ew ? (size_t)p->S * 8 : 0);
+    KVP_CUDA(cudaMallocAsync(&p->d_block, off, st));
+    char* base = static_cast<char*>(p->d_block);
+    p->dA = (uint32_t*)(base + oA); p->dAcol = (uint32_t*)(base + oAcol); p->d_a = (uint32_t*)(base + oa);
+    p->d_stepc = (StepC*)(base + osc); p->d_ucnt = (uint32_t*)(base + ouc); p->d_row_freq = (uint32_t*)(base + orf);
+    uint32_t* writes = hw || ew ? (uint32_t*)(base + owr) : nullptr;
+    KVP_CUDA(cudaMemsetAsync(base + oa, 0, owr - oa, st));
+    std::vector<uint32_t> host(writes ? (size_t)p->S * 2 : 0);
+    if (writes) {
+        for (uint32_t s = 0; s < p->S; ++s) { host[s] = hw ? hw[s] : 0u; host[p->S + s] = ew ? ew[s] : 0u; }
+        KVP_CUDA(cudaMemcpyAsync(writes, host.data(), (size_t)p->S * 8, cudaMemcpyHostToDevice, st));
     }
-    KVP_CUDA(cudaMemcpyAsync(p->d_stepc, sc.data(), (size_t)p->S * sizeof(StepC), cudaMemcpyHostToDevice, st));
-    KVP_CUDA(cudaStreamSynchronize(st));
+    if ((rc = launch_open(p, access, st))) return rc;
+    if ((rc = launch_stepc(p->d_stepc, writes, p->d_a, p->S, p->K, st))) return rc;
+    if ((rc = launch_static_freq_row(p, (uint32_t*)(base + ofr), p->d_row_freq, st))) return rc;
+    std::vector<uint32_t> a(p->S);
+    KVP_CUDA(cudaMemcpyAsync(a.data(), p->d_a, (size_t)p->S * 4, cudaMemcpyDeviceToHost, st));
+    KVP_CUDA(cudaStreamSynchronize(st));                 // the host vectors go out of scope
+    p->total_accessed = 0;
+    for (uint32_t s = 0; s < p->S; ++s) p->total_accessed += a[s];
     return KVP_OK;
 }
 

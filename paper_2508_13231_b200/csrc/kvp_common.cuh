@@ -150,7 +150,6 @@ int ensure_scratch(kvp_problem* p, size_t bytes, cudaStream_t st);
 int ensure_chain_ws(kvp_problem* p, size_t bytes, cudaStream_t st);
 
 // kvp_cost.cu
-int launch_row_popcount(const uint32_t* rows, uint32_t S, uint32_t W32, uint32_t* out, cudaStream_t st);
 // Scores n schedules (Eq. 1-5). scratch: score_scratch_bytes(p, n) bytes, null if that is 0. counts_out [n][S][4] = {hr, mi,
 // mo, occ} and hbc_out [n][S] (problems with births: units written to HBM at birth): copies of the counts, or null.
 size_t score_scratch_bytes(const kvp_problem* p, uint32_t n);
@@ -163,11 +162,14 @@ int launch_counts(const kvp_problem* p, const uint32_t* schedules, uint32_t n, u
 int launch_bit_transpose(const uint32_t* in, uint32_t rows, uint32_t in_words, uint32_t cols, uint32_t* out,
                          uint32_t out_words, cudaStream_t st);
 int launch_clean_copy(const uint32_t* in, uint32_t* out, uint32_t S, uint32_t W32, uint32_t pad_mask, cudaStream_t st);
-int launch_unit_counts(const uint32_t* Acol, uint32_t U, uint32_t S32, uint32_t* ucnt, cudaStream_t st);
-int launch_static_freq_row(const kvp_problem* p, uint32_t* row, cudaStream_t st);
+int launch_open(const kvp_problem* p, const uint32_t* access, cudaStream_t st);
+int launch_stepc(StepC* stepc, const uint32_t* writes, const uint32_t* a, uint32_t S, const CostK& K, cudaStream_t st);
+size_t static_freq_words(const kvp_problem* p);
+int launch_static_freq_row(const kvp_problem* p, uint32_t* scratch, uint32_t* row, cudaStream_t st);
 int launch_static_first_row(const kvp_problem* p, uint32_t* row, cudaStream_t st);
-int launch_broadcast_row(const uint32_t* row, uint32_t S, uint32_t W32, uint32_t* sched, cudaStream_t st);
-int launch_row_to_columns(const uint32_t* row, uint32_t U, uint32_t S, uint32_t S32, uint32_t* Pcol, cudaStream_t st);
+int launch_broadcast_row(const uint32_t* row, uint32_t S, uint32_t W32, const uint32_t* L, uint32_t* sched, cudaStream_t st);
+int launch_row_to_columns(const uint32_t* row, uint32_t U, uint32_t S, uint32_t S32, const uint32_t* birth, uint32_t* Pcol,
+                          cudaStream_t st);
 int launch_alive_rows(const uint32_t* birth, uint32_t U, uint32_t S, uint32_t W32, uint32_t* L, cudaStream_t st);
 int launch_birth_stats(const uint32_t* birth, uint32_t U, uint32_t S, const uint32_t* Acol, uint32_t S32, uint32_t* nb,
                        uint32_t* flag, cudaStream_t st);

@@ -318,25 +318,7 @@ score_kernel(const uint32_t* __restrict__ A, const uint32_t* __restrict__ Ps, ui
     if (out.stepc) score_total(out, i, sum);
 }
 
-__global__ void __launch_bounds__(256)
-row_popcount_kernel(const uint32_t* __restrict__ rows, uint32_t S, uint32_t W32, uint32_t* __restrict__ out)
-{
-    const uint32_t warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-    if (warp >= S) return;
-    uint32_t c = 0;
-    for (uint32_t w = lane; w < W32; w += 32) c += __popc(__ldg(rows + (size_t)warp * W32 + w));
-    c = __reduce_add_sync(0xFFFFFFFFu, c);
-    if (lane == 0) out[warp] = c;
-}
-
 }  // namespace
-
-int launch_row_popcount(const uint32_t* rows, uint32_t S, uint32_t W32, uint32_t* out, cudaStream_t st)
-{
-    row_popcount_kernel<<<(S + 7) / 8, 256, 0, st>>>(rows, S, W32, out);
-    KVP_CUDA(cudaGetLastError());
-    return KVP_OK;
-}
 
 // A schedule is small when one CTA is done with it before a grid of CTAs would have started: up to 512 KB (of one SM's some
 // 200 GB/s, beside a second and a third launch). Many of them with long rows go to the streaming kernel, which reads P once.
