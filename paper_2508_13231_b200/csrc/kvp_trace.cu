@@ -25,7 +25,9 @@ struct TraceK {
 };
 
 // Irwin-Hall(8) noise with unit variance in Q16.16: the sum of the eight 16-bit halves of one Philox block, centred
-// and scaled by floor(). |result| <= 321,057, so 32 bits hold it; only the product needs 64.
+// and scaled by floor(sum * 80265 / 2^16). |result| <= 321,057. The operands are shifted up by 12 and 4 bits so that the
+// floor is the high word of a 32-bit product: a 64-bit product and a shift take twice the multiplier's time, which is
+// what the score kernels wait for.
 __device__ __forceinline__ int32_t noise_q16(const PhiloxKeys& keys, uint32_t u, uint32_t t)
 {
     uint32_t r[4];
@@ -33,8 +35,7 @@ __device__ __forceinline__ int32_t noise_q16(const PhiloxKeys& keys, uint32_t u,
     uint32_t sum = 0;
 #pragma unroll
     for (int i = 0; i < 4; ++i) sum = __dp2a_lo(r[i], 0x0101u, sum);      // + low half + high half
-    const int64_t scaled = (int64_t)((int32_t)sum - 262140) * 80265;
-    return (int32_t)(scaled >> 16);                                       // arithmetic shift = floor
+    return __mulhi(((int32_t)sum - 262140) * 4096, 80265 * 16);
 }
 
 // Sum of a per-thread value over the CTA; every thread gets the result. slot: one of 32 shared counters.
@@ -48,79 +49,97 @@ __device__ __forceinline__ uint32_t block_sum(uint32_t v, uint32_t* slot)
 
 constexpr int kDigitBits = 8;                        // the search fixes this many bits of the threshold per pass
 constexpr int kBins = 1 << kDigitBits;
-constexpr int kPasses = 32 / kDigitBits;
 constexpr uint32_t kListCap = 256;                   // a threshold bin of up to this many keys is finished by ranking
+constexpr int32_t kNoKey = INT32_MIN;                // a slot without a unit; no score has this value
 
 struct SelectSmem {
-    uint32_t hist[kPasses][kBins];   // per pass: how many keys with the threshold's higher bits have each digit
+    alignas(16) uint32_t hist[kBins];            // how many keys with the threshold's higher bits have each digit
     uint32_t cnt[4];                 // block-wide counts beside the search ([1]: keys in `list`)
-    uint32_t list[kListCap];         // the keys of the threshold's bin after the first pass
+    int32_t list[kListCap];          // the keys of the threshold's bin after the first pass
     uint32_t warp[32];
     uint32_t run;
-    uint32_t hi, lo;                 // largest and smallest key of the step
-    uint32_t K, need, equal;         // threshold so far, how many keys are still to find at or below it, ties at it
+    int32_t hi, lo;                  // largest key of the step, and a lower bound of the k-th largest
+    int32_t K;                       // lower edge of the threshold's bin, at last the threshold
+    uint32_t need, equal;            // how many keys are still to find in that bin, and how many it holds
 };
 
 // State of one selection; a barrier must follow before select_step.
 __device__ __forceinline__ void select_reset(SelectSmem& sm)
 {
-    for (uint32_t i = threadIdx.x; i < kPasses * kBins; i += blockDim.x) (&sm.hist[0][0])[i] = 0;
+    for (uint32_t i = threadIdx.x; i < kBins; i += blockDim.x) sm.hist[i] = 0;
     if (threadIdx.x < 4) sm.cnt[threadIdx.x] = 0;
-    if (threadIdx.x == 0) { sm.hi = 0u; sm.lo = ~0u; }
+    if (threadIdx.x == 0) { sm.hi = INT32_MIN; sm.lo = INT32_MAX; }
 }
 
-// Top-k of one (group, step): the CTA holds the n keys (UPT per thread, unit i = j*T + tid, 0 past n) and sets the
+// Top-k of one (group, step): the CTA holds the n keys (UPT per thread, unit i = j*T + tid, kNoKey past n) and sets the
 // bits of the k largest, ties to the lower unit index. select_reset and a barrier come first.
-// topk: how many to pick (at most the number of non-zero keys when zero marks a unit that is not there yet).
+// topk: how many to pick (at most the number of keys other than kNoKey).
 //
-// The threshold K (the k-th largest key) is found digit by digit from the top, eight bits per pass: the keys that
-// agree with K in the bits fixed so far are counted per digit in a shared-memory histogram, and one warp walks
-// the histogram from the top until the counts reach what is still needed. The search works on the keys minus the
-// smallest one, so only the bits of (largest - smallest) need a pass: three passes on these scores.
+// What bounds it: instructions per key, then the latency of the barriers. So keys that cannot be picked are dropped first.
+// Every warp looks at the largest key of each lane and finds, by six ballots, a value that `want` = ceil(k / warps) of them
+// reach; the smallest such value over the warps is reached by at least k keys of the step, so the k-th largest is not
+// below it. (Where that would take more than 24 of the 32 lanes, `want` is 0 and the bound is the smallest key.) Keys from
+// the bound up, about 9% of them at k = 5%, are counted per digit of (key - bound) in a shared-memory histogram, one
+// warp walks it from the top until the counts reach what is needed, and the keys of the bin found there, a few, are
+// ranked against each other. A bin with many keys (ties) takes more histogram passes, eight bits each.
+// 640 groups of 4096 units x 64 steps, 205 picked: 323 us with every key in the histogram and eight keys per thread, 240 now.
 // FULL: the CTA's UPT * T slots are exactly the n units, so no slot needs a bounds test.
 template <int UPT, bool FULL = false>
-__device__ __forceinline__ void select_step(const uint32_t (&key)[UPT], const TraceK& k, uint32_t topk, uint32_t gbase,
+__device__ __forceinline__ void select_step(const int32_t (&key)[UPT], const TraceK& k, uint32_t want, uint32_t topk, uint32_t gbase,
                                             uint32_t t, SelectSmem& sm)
 {
     const uint32_t T = blockDim.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    uint32_t mx = 0u, mn = ~0u;
+    {
+        int32_t mine = key[0];
 #pragma unroll
-    for (int j = 0; j < UPT; ++j)
-        if (FULL || j * T + tid < k.n) { mx = max(mx, key[j]); mn = min(mn, key[j]); }
-    mx = __reduce_max_sync(0xFFFFFFFFu, mx);
-    mn = __reduce_min_sync(0xFFFFFFFFu, mn);
-    if (lane == 0) { atomicMax(&sm.hi, mx); atomicMin(&sm.lo, mn); }
-    __syncthreads();
-    // The search runs on key - smallest key: the same order, and the digits then spread over the range the keys
-    // really cover (scores on both sides of zero differ in every leading bit, although they span twenty bits or so:
-    // as raw keys they would need four passes, the first two with nearly all keys in two or three bins).
-    const uint32_t lo = sm.lo;
-    uint32_t kk[UPT];
+        for (int j = 1; j < UPT; ++j) mine = max(mine, key[j]);
+        const int32_t mx = __reduce_max_sync(0xFFFFFFFFu, mine);
+        int32_t bound;
+        if (UPT >= 4 && want) {
+            const int32_t mn = __reduce_min_sync(0xFFFFFFFFu, mine);
+            const uint32_t d = (uint32_t)mine - (uint32_t)mn;
+            const int shift = max(26 - __clz((uint32_t)mx - (uint32_t)mn), 0);
+            uint32_t x = 0;
 #pragma unroll
-    for (int j = 0; j < UPT; ++j) kk[j] = key[j] - lo;
-    int rem = 32 - __clz(sm.hi - lo);                        // bits still open; 0 when all keys are equal
-    uint32_t K = 0u;                                         // the bits above them are zero in every reduced key
-    uint32_t need = topk, equal = k.n;                       // all keys equal: every one ties at K
-    for (int pass = 0; rem > 0; ++pass) {
-        const int w = rem < kDigitBits ? rem : kDigitBits, sh = rem - w;
-        uint32_t* hist = sm.hist[pass];
-        if (pass == 0) {                                     // no reduced key has a bit above the open ones: all count
+            for (int i = 5; i >= 0; --i) {
+                const uint32_t trial = x + (1u << (i + shift));
+                if (__popc(__ballot_sync(0xFFFFFFFFu, d >= trial)) >= want) x = trial;
+            }
+            bound = (int32_t)((uint32_t)mn + x);
+        } else {
+            bound = INT32_MAX;
 #pragma unroll
             for (int j = 0; j < UPT; ++j)
-                if (FULL || j * T + tid < k.n) atomicAdd(hist + (kk[j] >> sh), 1u);
-        } else {
+                if (FULL || j * T + tid < k.n) bound = min(bound, key[j]);
+            bound = __reduce_min_sync(0xFFFFFFFFu, bound);
+        }
+        if (lane == 0) { atomicMax(&sm.hi, mx); atomicMin(&sm.lo, bound); }
+    }
+    __syncthreads();
+    int32_t K = sm.lo;
+    int rem = 32 - __clz((uint32_t)sm.hi - (uint32_t)K);     // bits still open; 0 when all these keys are equal
+    uint32_t need = topk, equal = ~0u;                        // one value only: ties, if there is any key
+    for (int pass = 0; rem > 0; ++pass) {
+        const int sh = rem < kDigitBits ? 0 : rem - kDigitBits;
+        if (pass) {
+            for (uint32_t i = tid; i < kBins; i += T) sm.hist[i] = 0;
+            __syncthreads();
+        }
+        // one predicated instruction per key, no branch: d >> sh stays inside the histogram for the keys that count
+        const uint32_t hist = (uint32_t)__cvta_generic_to_shared(sm.hist), span = rem < 32 ? (1u << rem) - 1u : ~0u;
 #pragma unroll
-            for (int j = 0; j < UPT; ++j) {
-                const bool in = (FULL || j * T + tid < k.n) && (kk[j] >> rem) == (K >> rem);
-                if (in) atomicAdd(hist + ((kk[j] >> sh) & ((1u << w) - 1u)), 1u);
-            }
+        for (int j = 0; j < UPT; ++j) {
+            const uint32_t d = (uint32_t)key[j] - (uint32_t)K;   // keys below K wrap; the pass's range is cut at span
+            const uint32_t in = (FULL || j * T + tid < k.n) && key[j] >= K && d <= span;
+            asm volatile("{ .reg .pred p; setp.ne.u32 p, %0, 0; @p red.shared.add.u32 [%1], 1; }" :: "r"(in), "r"(hist + (d >> sh) * 4u) : "memory");
         }
         __syncthreads();
         if (warp == 0) {
-            // lane l owns digits 8l .. 8l+7; suffix sums over the lanes, then over the owner's eight bins
-            uint32_t h[8], s = 0;
+            // a lane owns kOwn neighbouring digits; suffix sums over the lanes, then over the owner's bins
+            constexpr uint32_t kOwn = kBins / 32;
+            uint32_t h[kOwn], s = 0;
 #pragma unroll
-            for (int i = 0; i < 8; ++i) { h[i] = hist[8 * lane + i]; s += h[i]; }
+            for (uint32_t i = 0; i < kOwn; ++i) { h[i] = sm.hist[kOwn * lane + i]; s += h[i]; }
             uint32_t suf = s;
 #pragma unroll
             for (int off = 1; off < 32; off <<= 1) {
@@ -131,9 +150,9 @@ __device__ __forceinline__ void select_step(const uint32_t (&key)[UPT], const Tr
             if (lane == 31u - __clz(reach)) {
                 uint32_t higher = suf - s;
 #pragma unroll
-                for (int i = 7; i >= 0; --i) {
+                for (int i = kOwn - 1; i >= 0; --i) {
                     if (higher + h[i] >= need) {
-                        sm.K = K | ((uint32_t)(8 * lane + i) << sh);
+                        sm.K = (int32_t)((uint32_t)K + ((kOwn * lane + i) << sh));
                         sm.need = need - higher;
                         sm.equal = h[i];
                         break;
@@ -146,18 +165,24 @@ __device__ __forceinline__ void select_step(const uint32_t (&key)[UPT], const Tr
         K = sm.K; need = sm.need; equal = sm.equal;
         rem = sh;
         if (pass == 0 && rem > 0 && equal <= kListCap) {
-            // The first digit's bin usually holds a few dozen keys: they go to a shared list and each is ranked against
-            // the others, which settles the remaining bits at once; further histogram passes, in which every thread
-            // tests all of its keys again, are left to bins with many keys (ties).
+            // The first digit's bin usually holds a few keys: they go to a shared list and each is ranked against
+            // the others, which settles the remaining bits at once.
+            uint32_t least = ~0u;
 #pragma unroll
             for (int j = 0; j < UPT; ++j)
-                if ((FULL || j * T + tid < k.n) && (kk[j] >> rem) == (K >> rem)) sm.list[atomicAdd(&sm.cnt[1], 1u)] = kk[j];
+                if (FULL || j * T + tid < k.n) least = min(least, (uint32_t)key[j] - (uint32_t)K);
+            if (least >> rem == 0u) {
+#pragma unroll
+                for (int j = 0; j < UPT; ++j)
+                    if ((FULL || j * T + tid < k.n) && ((uint32_t)key[j] - (uint32_t)K) >> rem == 0u)
+                        sm.list[atomicAdd(&sm.cnt[1], 1u)] = key[j];
+            }
             __syncthreads();
             for (uint32_t c = tid; c < equal; c += T) {
-                const uint32_t v = sm.list[c];
+                const int32_t v = sm.list[c];
                 uint32_t above = 0, same = 0;
                 for (uint32_t i = 0; i < equal; ++i) {
-                    const uint32_t x = sm.list[i];
+                    const int32_t x = sm.list[i];
                     above += x > v ? 1u : 0u;
                     same += x == v ? 1u : 0u;
                 }
@@ -171,20 +196,17 @@ __device__ __forceinline__ void select_step(const uint32_t (&key)[UPT], const Tr
         }
     }
     const uint32_t take = need;                              // ties to admit, lowest unit index first
-    const bool rank_ties = equal != take;
+    const bool rank_ties = equal != take;                    // and when all keys from the bound up are equal
     uint32_t* row = k.out + (size_t)t * k.W32;
-    auto emit = [&](int j, bool pick) {
-        const uint32_t i = j * T + tid;
-        if (k.aligned) {
-            const uint32_t bits = __ballot_sync(0xFFFFFFFFu, pick);
-            if (lane == 0 && (FULL || j * T + (tid & ~31u) < k.n)) row[(gbase + j * T + tid) >> 5] = bits;
-        } else if (pick) {
-            atomicOr(row + ((gbase + i) >> 5), 1u << ((gbase + i) & 31));
-        }
-    };
-    if (!rank_ties) {                                        // the usual case, kept apart so that its loop stays small
+    if (!rank_ties && k.aligned) {                           // the usual case, kept apart so that its loop stays small
+        uint32_t word = 0;                                   // lane j keeps and stores round j's word
 #pragma unroll
-        for (int j = 0; j < UPT; ++j) emit(j, (FULL || j * T + tid < k.n) && kk[j] >= K);
+        for (int j = 0; j < UPT; ++j) {
+            const uint32_t bits = __ballot_sync(0xFFFFFFFFu, (FULL || j * T + tid < k.n) && key[j] >= K);
+            if (lane == (uint32_t)j) word = bits;
+        }
+        const uint32_t i = lane * T + (tid & ~31u);
+        if (lane < UPT && (FULL || i < k.n)) row[(gbase + i) >> 5] = word;
         return;
     }
     if (tid == 0) sm.run = 0;
@@ -193,7 +215,7 @@ __device__ __forceinline__ void select_step(const uint32_t (&key)[UPT], const Tr
     for (int j = 0; j < UPT; ++j) {
         const uint32_t i = j * T + tid;
         const bool ok = FULL || i < k.n;
-        const bool tie = ok && kk[j] == K;
+        const bool tie = ok && key[j] == K;
         // units of round j are consecutive over the CTA, so index order = (round, thread) order
         const uint32_t tb = __ballot_sync(0xFFFFFFFFu, tie);
         if (lane == 0) sm.warp[warp] = __popc(tb);
@@ -201,22 +223,36 @@ __device__ __forceinline__ void select_step(const uint32_t (&key)[UPT], const Tr
         uint32_t before = sm.run;
         for (uint32_t w = 0; w < warp; ++w) before += sm.warp[w];
         before += __popc(tb & ((1u << lane) - 1u));
-        const bool pick = (ok && kk[j] > K) || (tie && before < take);
+        const bool pick = (ok && key[j] > K) || (tie && before < take);
         __syncthreads();
         if (tid == 0) { uint32_t s = 0; for (uint32_t w = 0; w < (T >> 5); ++w) s += sm.warp[w]; sm.run += s; }
         __syncthreads();
-        emit(j, pick);
+        if (k.aligned) {
+            const uint32_t bits = __ballot_sync(0xFFFFFFFFu, pick);
+            if (lane == 0 && (FULL || j * T + (tid & ~31u) < k.n)) row[(gbase + j * T + tid) >> 5] = bits;
+        } else if (pick) {
+            atomicOr(row + ((gbase + i) >> 5), 1u << ((gbase + i) & 31));
+        }
     }
+}
+
+// ceil(k / warps), if the lanes' largest keys can bound the k-th largest that way, else 0. From 25 of 32 lanes on the
+// bound lies so low that it would keep a third of the keys.
+__host__ __device__ __forceinline__ uint32_t select_want(uint32_t topk, uint32_t threads)
+{
+    const uint32_t warps = threads / 32, want = (topk + warps - 1) / warps;
+    return want <= 24u ? want : 0u;
 }
 
 // importance of unit u at step t given its state at t-1 (Q16.16). The 64-bit sum of the two 32x32 products is
 // shifted and then cut to 32 bits (the range check on the host keeps the true value inside them).
+template <bool BURST>
 __device__ __forceinline__ int32_t next_state(const TraceK& k, uint32_t u, uint32_t t, int32_t x)
 {
     const int32_t e = noise_q16(k.keys, u, t);
     const int64_t acc = t == 0 ? (int64_t)k.sigma_q * e : (int64_t)k.rho_q * x + (int64_t)k.c_q * e;
     int32_t xn = (int32_t)(acc >> 16);
-    if (k.burst_thr) {
+    if (BURST && k.burst_thr) {
         uint32_t r[4];
         philox4x32_10(u, t, 0u, TAG_BURST, k.keys, r);
         if (r[0] < k.burst_thr) xn += k.burst_jump;
@@ -226,7 +262,7 @@ __device__ __forceinline__ int32_t next_state(const TraceK& k, uint32_t u, uint3
 
 // Fused form: one CTA per group walks the steps; used when the score matrix would not fit the scratch budget.
 // Two CTAs per SM (at most 32 registers per thread): one CTA's barriers in the search hide behind the other's work.
-// GROW: units have birth steps; one that is not there yet gets key 0 and is never picked.
+// GROW: units have birth steps; one that is not there yet gets kNoKey and is never picked.
 template <int UPT, bool GROW>
 __global__ void __launch_bounds__(1024, 2)
 trace_kernel(const TraceK k)
@@ -251,17 +287,19 @@ trace_kernel(const TraceK k)
             born[j] = i < k.n ? __ldg(k.birth + gbase + i) : 0u;
         }
     }
+    const uint32_t want = UPT >= 4 ? select_want(k.topk, T) : 0u;
     for (uint32_t tok = 0, t = layer; t < k.steps; ++tok, t += k.layers) {
         select_reset(sm);
-        uint32_t key[UPT], here = 0;
+        int32_t key[UPT];
+        uint32_t here = 0;
 #pragma unroll
         for (int j = 0; j < UPT; ++j) {
             const uint32_t i = j * T + tid;
-            key[j] = 0;
+            key[j] = kNoKey;
             if (i < k.n) {
-                x[j] = next_state(k, gbase + i, tok, x[j]);
+                x[j] = next_state<true>(k, gbase + i, tok, x[j]);
                 if (!GROW || born[GROW ? j : 0] <= t) {
-                    key[j] = (uint32_t)(x[j] + b[j]) ^ 0x80000000u;   // order-preserving map int32 -> uint32, never 0
+                    key[j] = x[j] + b[j];
                     ++here;
                 }
             }
@@ -269,7 +307,7 @@ trace_kernel(const TraceK k)
         __syncthreads();
         uint32_t topk = k.topk;
         if (GROW) topk = min(topk, block_sum(here, &sm.cnt[0]));
-        select_step<UPT>(key, k, topk, gbase, t, sm);
+        select_step<UPT>(key, k, want, topk, gbase, t, sm);
         __syncthreads();
     }
 }
@@ -319,9 +357,10 @@ trace_scores_kernel(const TraceK k, uint32_t U, int32_t* __restrict__ scores)
 
 // Pass 1 for traces of many units: a thread per unit walks the steps, draws and recurrence together, and the threads
 // of a warp write 128 contiguous bytes per step. No shared memory and no barrier; the draws of later steps do not
-// depend on the state, so the loop, unrolled eight times (3% faster than four), overlaps their Philox chains with the
+// depend on the state, so the loop, unrolled four times, overlaps their Philox chains with the
 // recurrence. It needs about a
 // thousand units per SM to fill the machine, which is why fewer units take the segmented kernel above.
+template <bool BURST>
 __global__ void __launch_bounds__(256)
 trace_scores_unit_kernel(const TraceK k, uint32_t U, int32_t* __restrict__ scores)
 {
@@ -329,30 +368,28 @@ trace_scores_unit_kernel(const TraceK k, uint32_t U, int32_t* __restrict__ score
     if (u >= U) return;
     const int32_t b = k.base ? __ldg(k.base + u) : 0;
     int32_t x = 0;
-#pragma unroll 8
+#pragma unroll 4
     for (uint32_t t = 0; t < k.steps; ++t) {
-        x = next_state(k, u, t, x);
+        x = next_state<BURST>(k, u, t, x);
         scores[(size_t)t * U + u] = x + b;
     }
 }
 
 // Two-pass form, pass 2: the top-k selections of different steps are independent: one CTA per (group, step).
 template <int UPT, bool FULL>
-__global__ void __launch_bounds__(1024)
-trace_select_kernel(const TraceK k, uint32_t U, const int32_t* __restrict__ scores)
+__global__ void __launch_bounds__(512, 3)
+trace_select_kernel(const TraceK k, uint32_t want, uint32_t U, const int32_t* __restrict__ scores)
 {
     __shared__ SelectSmem sm;
     const uint32_t g = blockIdx.x, t = blockIdx.y, T = blockDim.x, tid = threadIdx.x;
     const uint32_t gbase = g * k.n;
     select_reset(sm);
-    uint32_t key[UPT];
+    int32_t key[UPT];
+    const int32_t* from = scores + (size_t)t * U + gbase + tid;
 #pragma unroll
-    for (int j = 0; j < UPT; ++j) {
-        const uint32_t i = j * T + tid;
-        key[j] = (FULL || i < k.n) ? (uint32_t)__ldg(scores + (size_t)t * U + gbase + i) ^ 0x80000000u : 0u;
-    }
+    for (int j = 0; j < UPT; ++j) key[j] = (FULL || j * T + tid < k.n) ? __ldcs(from + j * T) : kNoKey;
     __syncthreads();
-    select_step<UPT, FULL>(key, k, k.topk, gbase, t, sm);
+    select_step<UPT, FULL>(key, k, want, k.topk, gbase, t, sm);
 }
 
 }  // namespace
@@ -401,7 +438,9 @@ extern "C" int kvp_trace_generate(const kvp_trace_params* tp, uint32_t* access_b
     // Two passes (scores, then one CTA per (group, step)) whenever the score matrix fits a 1 GiB scratch: the work
     // then comes in tens of thousands of equal pieces, while the fused kernel has only `groups` CTAs that walk the
     // steps one after the other (measured: 0.84 vs 0.89 ms on 256 groups of 2048, 1.85 vs 2.11 ms on 640 of 4096,
-    // 0.05 vs 2.1 ms on one group of 256).
+    // 0.05 vs 2.1 ms on one group of 256). One launch with CTAs of both kinds, selecting from the chunk of steps before, was
+    // slower than two after each other (1.10 against 0.99 ms on 640 of 4096): the kinds crowd each other out of registers and
+    // instruction cache.
     const size_t score_bytes = (size_t)U64 * tp->steps * 4;
     if (score_bytes <= ((size_t)1 << 30) && !(tp->flags & KVP_TRACE_SINGLE_PASS) && !layered) {
         int32_t* scores = nullptr;
@@ -410,26 +449,30 @@ extern "C" int kvp_trace_generate(const kvp_trace_params* tp, uint32_t* access_b
         int prc = retain_in_pool(dev, score_bytes);          // the next call gets the block back from the pool
         if (prc) return prc;
         KVP_CUDA(cudaMallocAsync(&scores, score_bytes, st));
-        if (U64 >= 148u * 1024u) trace_scores_unit_kernel<<<(uint32_t)((U64 + 255) / 256), 256, 0, st>>>(k, (uint32_t)U64, scores);
-        else trace_scores_kernel<<<(uint32_t)((U64 + 31) / 32), kScoreThreads, 0, st>>>(k, (uint32_t)U64, scores);
+        const uint32_t U = (uint32_t)U64;
+        if (U >= 148u * 1024u) {
+            if (k.burst_thr) trace_scores_unit_kernel<true><<<(U + 255) / 256, 256, 0, st>>>(k, U, scores);
+            else trace_scores_unit_kernel<false><<<(U + 255) / 256, 256, 0, st>>>(k, U, scores);
+        } else {
+            trace_scores_kernel<<<(U + 31) / 32, kScoreThreads, 0, st>>>(k, U, scores);
+        }
         dim3 grid(tp->groups, tp->steps);
         // Small CTAs with many units per thread: a selection is a chain of barriers and a serial histogram walk, so
-        // what counts is how many of them an SM overlaps (whole call, 640 groups of 4096 units x 64 steps: 1.85 ms
-        // with 1024 threads, 1.70 ms with 256; 256 groups of 2048 x 128 steps: 0.84 against 0.61 ms with 128). Since the
-        // search needs one histogram pass only, eight units per thread are a little faster than sixteen (1.05 against
-        // 1.07 ms and 0.359 against 0.363 ms on these two shapes).
+        // what counts is how many of them an SM overlaps, and a key has little to do (with sixteen keys per thread 294 us, with
+        // eight 330 on 640 groups of 4096 units x 64 steps; 240 with sixteen and registers for three times 512 threads).
         int su = 1;
-        while (su < 8 && (n + su - 1) / su > 128) su *= 2;
-        const uint32_t ST = ((n + su - 1) / su + 31) / 32 * 32;
+        while (su < 16 && (n + su - 1) / su > 128) su *= 2;
+        const uint32_t ST = ((n + su - 1) / su + 31) / 32 * 32, want = select_want(k.topk, ST);
         const bool full = (uint64_t)su * ST == n;             // every slot of the CTA holds a unit
-#define KVP_SELECT(UPT)                                                                              \
-    if (full) trace_select_kernel<UPT, true><<<grid, ST, 0, st>>>(k, (uint32_t)U64, scores);         \
-    else trace_select_kernel<UPT, false><<<grid, ST, 0, st>>>(k, (uint32_t)U64, scores)
+#define KVP_SELECT(UPT)                                                                     \
+    if (full) trace_select_kernel<UPT, true><<<grid, ST, 0, st>>>(k, want, U, scores);      \
+    else trace_select_kernel<UPT, false><<<grid, ST, 0, st>>>(k, want, U, scores)
         switch (su) {
             case 1: KVP_SELECT(1); break;
             case 2: KVP_SELECT(2); break;
             case 4: KVP_SELECT(4); break;
-            default: KVP_SELECT(8); break;
+            case 8: KVP_SELECT(8); break;
+            default: KVP_SELECT(16); break;
         }
 #undef KVP_SELECT
         cudaError_t le = cudaGetLastError();
