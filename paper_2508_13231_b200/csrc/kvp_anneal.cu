@@ -720,7 +720,7 @@ int prepare(kvp_problem* p, const kvp_anneal_params* a, cudaStream_t st, Ctx& c,
     // What counts as chains of an SM is how many it holds at a time, when their schedules take its shared memory.
     // kvp_set_test_hooks can force the choice (warps_per_chain 1, 2 or 32 + w: narrow; 3 or 16 + w: wide).
     const bool many_units = p->U >= 32768u;
-    c.wide = false;
+    c.wide = false;                                               // (for the bytes of a chain)
     c.psmem = fixed_bytes(1, true) + pbytes + 16 <= budget / 2 && p->U < 65536u;
     uint32_t held = chains_per_sm;
     if (c.psmem) {
@@ -730,7 +730,14 @@ int prepare(kvp_problem* p, const kvp_anneal_params* a, cudaStream_t st, Ctx& c,
     const bool few = held <= 8;
     if (!hot) c.wide = c.psmem ? !few && p->S >= 256u : many_units && held > 5;
     if (hooks.warps_per_chain) c.wide = hooks.warps_per_chain == 3 || (hooks.warps_per_chain >= 16 && hooks.warps_per_chain < 32);
-    if (exchange || !c.lin || c.grow) c.wide = true;              // the narrow kernel does not serve these
+    if (exchange) {
+        // Whole ladders in a CTA: every round waits for the hottest rungs, which apply the most moves, and one warp per chain
+        // is fastest there (128 ladders of 8 on 256 units x 512 steps, 100,000 moves: 4.5 ms, two warps 5.1, wide kernel 7.5;
+        // 7 of 4 on 46 x 61, 38,619 moves: 3.5, 5.4, 11.2).
+        const bool ladders = c.psmem && rungs <= 16 && rungs * (fixed_bytes(1, true) + pbytes) + 16 <= budget;
+        c.wide = !ladders || hooks.warps_per_chain == 3 || (hooks.warps_per_chain >= 16 && hooks.warps_per_chain < 32);
+    }
+    if (!c.lin || c.grow) c.wide = true;                          // the narrow kernel does not serve these
     if (c.wide) c.psmem = fixed_bytes(1, true) + pbytes + 16 <= budget / 2 && p->U < 65536u;
     const uint32_t forced = hooks.warps_per_chain == 3 ? 1u : hooks.warps_per_chain >= 16 ? hooks.warps_per_chain & 15u : hooks.warps_per_chain;
     const uint32_t full = 16;
@@ -754,10 +761,11 @@ int prepare(kvp_problem* p, const kvp_anneal_params* a, cudaStream_t st, Ctx& c,
             W = chains_per_sm <= 3 ? 4 : 2;
             while (W > 1 && (want * W > full || with_a(want, W) > budget)) W /= 2;
         } else {
-            W = narrow_warps();
+            W = exchange ? 1u : narrow_warps();
             while (W > 1 && (fixed_bytes(W, true) + pbytes) * held + 16 > budget) --W;
         }
         if (forced) W = forced;
+        if (exchange && !c.wide && (rungs * W > full || rungs * (fixed_bytes(W, true) + pbytes) + 16 > budget)) W = 1;
         c.wpc = W;
         c.smem_per_warp = fixed_bytes(W, true) + pbytes;
         uint32_t wmax = (uint32_t)((budget - 16) / c.smem_per_warp);
@@ -1222,7 +1230,7 @@ extern "C" int kvp_anneal_exchange(kvp_problem* p, const kvp_anneal_params* a, c
     if (c.ladder_ctas) {
         // every CTA holds whole ladders: one launch, the rounds end in a CTA barrier
         prm.round0 = 0; prm.round1 = rounds; prm.state = nullptr;
-        prm.ladder_ctas = 1u; prm.ladder = xk.x; prm.n_exchanged = nex; prm.work = work_dev;
+        prm.ladder_ctas = 1u; prm.ladder = xk.x; prm.n_exchanged = nex; prm.work = c.wide ? work_dev : nullptr;
         if ((rc = launch_chains(c, prm, chains))) return rc;
         ++c.launches;
         prm.ladder_ctas = 0u; prm.n_exchanged = nullptr;
@@ -1301,7 +1309,7 @@ extern "C" int kvp_anneal_exchange(kvp_problem* p, const kvp_anneal_params* a, c
         cudaEventElapsedTime(&stats->ms_chains, ev[1], ev[2]);
         cudaEventElapsedTime(&stats->ms_finish, ev[2], ev[3]);
         stats->kernel_launches = c.launches;
-        stats->chain_launches = rounds; stats->resident_chains = chains; stats->wide_kernel = 1u;
+        stats->chain_launches = rounds; stats->resident_chains = chains; stats->wide_kernel = c.wide ? 1u : 0u;
         stats->work_again = work[0]; stats->work_listed = work[1]; stats->work_items = work[2];
         stats->exchange_rounds = rounds; stats->exchanges_tried = xcounts[0]; stats->exchanges_accepted = xcounts[1];
     }

@@ -1,5 +1,6 @@
 // The narrow chain kernel (included by kvp_anneal.cu only): for jobs of few chains per SM and for chains that apply many of
-// their moves, such as hot starts, where a fifth to a quarter of the proposals change the schedule.
+// their moves, such as hot starts, where a fifth to a quarter of the proposals change the schedule, and the hot rungs of
+// replica exchange (whole ladders in a CTA).
 //
 // There, evaluations of cost changes ahead of the commits do not last. What lasts is what depends on a proposal's own units:
 // a warp takes 32 consecutive proposals, one per lane, and prepares them word-parallel: the windows, what the placement bits
@@ -109,7 +110,14 @@ narrow_chain_kernel(const __grid_constant__ ChainParams prm)
             copy_words(P, prm.Pcol0, pwords, sub * 32 + lane, W * 32);
     }
     __syncthreads();
-    if (!active) return;
+    const bool fused = PSMEM && prm.ladder_ctas != 0u;            // whole ladders in this CTA: exchange between segments
+    if (!active && !fused) return;
+    __shared__ uint8_t s_holder[PSMEM ? 16 : 1];                  // fused: the chain (within the CTA) on each rung
+    if (fused) {
+        if (threadIdx.x < 16) s_holder[threadIdx.x] = (uint8_t)threadIdx.x;
+        if (active && sub == 0 && lane == 0) c.sc()->rung = cic % prm.ladder.rungs;
+        __syncthreads();
+    }
     auto column = [&](uint32_t u) -> const uint32_t* {
         if (PSMEM) return P + u * S32;
         const uint32_t b = u >> prm.cow_shift, w = ld_volatile_u32(c.have() + (b >> 5));   // (another warp may be taking it over)
@@ -134,17 +142,21 @@ narrow_chain_kernel(const __grid_constant__ ChainParams prm)
 
     uint32_t n_same = 0, n_inf = 0;                               // per lane
     const int kh = (int)prm.K.kh, ke = (int)prm.K.ke, khF = (int)prm.K.khF, kdF = (int)prm.K.kdF;
-    bool over = false, silent = false;                            // this warp is done with its chain; because a wait ran out
-    for (uint32_t level = 0; level < prm.seg1 && !over; ++level) {
+    const bool exchange = prm.rung_hist != nullptr;               // a level is a round of a replica-exchange run
+    bool over = !active, silent = false;                          // this warp is done with its chain; because a wait ran out
+    for (uint32_t level = 0; level < prm.seg1; ++level) {
+        if (over && !fused) break;
         const uint64_t lvl_start = level * prm.seg_len, lvl_len = min(level + 1 == prm.seg1 ? ~(uint64_t)0 : prm.seg_len, prm.upto - lvl_start);
         const uint32_t nbat = (uint32_t)((lvl_len + 31) / 32), last_nb = (uint32_t)(lvl_len - (uint64_t)(nbat - 1) * 32);
         const uint32_t base = level * prm.seg_bat;                // index of the level's first batch (mod 2^32)
-        const uint32_t shift = __ldg(prm.shifts + level);
-        const uint32_t* const row = prm.table + (size_t)level * KVP_TABLE_Q;
-        const float scale = __ldg(prm.bounds + level) * __uint_as_float((127u - shift) << 23);   // C ln 2 in bins
+        // row of the acceptance table
+        const uint32_t rank = over ? 0u : !exchange ? level : fused ? c.sc()->rung : prm.rung_hist[(size_t)level * prm.hist_stride + (chain - prm.hist_base)];
+        const uint32_t shift = __ldg(prm.shifts + rank);
+        const uint32_t* const row = prm.table + (size_t)rank * KVP_TABLE_Q;
+        const float scale = __ldg(prm.bounds + rank) * __uint_as_float((127u - shift) << 23);   // C ln 2 in bins
         const bool bounded = scale < 1e30f;                       // the lower bounds fit 32 bits
 #pragma unroll 1
-        for (uint32_t bi = (sub + W - base % W) % W; bi < nbat; bi += W) {
+        for (uint32_t bi = (sub + W - base % W) % W; bi < nbat && !over; bi += W) {
             const uint64_t m = lvl_start + (uint64_t)bi * 32;
             const uint32_t nb = bi + 1 < nbat ? 32u : last_nb;
             uint32_t n0 = 0;
@@ -269,7 +281,7 @@ narrow_chain_kernel(const __grid_constant__ ChainParams prm)
                             break;
                         }
                     }
-                    if (bi == 0 && level > 0) {                   // the level's first batch: stop rule, new reference
+                    if (!exchange && bi == 0 && level > 0) {                   // the level's first batch: stop rule, new reference
                         if (!SOLO) best = c.sc()->best;
                         const uint64_t before = c.sc()->best_at_boundary;
                         if (prm.early_permille && level >= prm.early_from &&
@@ -422,8 +434,16 @@ narrow_chain_kernel(const __grid_constant__ ChainParams prm)
             atomicAdd(reinterpret_cast<unsigned long long*>(&c.sc()->n_inf), (unsigned long long)n_inf);
             n_same = n_inf = 0u;
         }
+        if (fused && level + 1 < prm.seg1) {
+            if (SOLO && active && lane == 0) c.sc()->cur = cur;
+            __syncthreads();                                      // every chain of the CTA has done its round
+            exchange_round(c, s_holder, stride, cpb, level);
+            __syncthreads();
+            if (active && sub == 0 && lane == 0)
+                prm.rung_hist[(size_t)(level + 1) * prm.hist_stride + (chain - prm.hist_base)] = (uint8_t)c.sc()->rung;
+        }
     }
-    if (silent) return;
+    if (!active || silent) return;
     // every warp adds what it counted; the last one to leave reports for the chain
     atomicAdd(reinterpret_cast<unsigned long long*>(&c.sc()->n_same), (unsigned long long)n_same);
     atomicAdd(reinterpret_cast<unsigned long long*>(&c.sc()->n_inf), (unsigned long long)n_inf);
@@ -439,9 +459,10 @@ narrow_chain_kernel(const __grid_constant__ ChainParams prm)
     if (lane == 0) {
         kvp_chain_result res;
         res.best_ticks = c.sc()->best; res.best_move = c.sc()->best_move; res.final_ticks = c.sc()->cur;
-        res.moves_done = c.sc()->m_end ? c.sc()->m_end : prm.upto;
+        res.moves_done = c.sc()->m_end ? c.sc()->m_end : min(prm.upto, exchange ? prm.seg1 * prm.seg_len : ~(uint64_t)0);
         res.n_accepted = c.sc()->n_same + c.sc()->n_chg; res.n_changed = c.sc()->n_chg; res.n_infeasible = c.sc()->n_inf; res.traj_hash = c.sc()->hash;
         prm.results[chain - prm.result_base] = res;
+        if (prm.n_exchanged) prm.n_exchanged[chain - prm.hist_base] = c.sc()->n_exchanged;
     }
     if (prm.snap && c.sc()->snap_dirty) copy_words_cold(prm.snap + (size_t)slot * pwords, P, pwords, lane);
     if (prm.undo_log && lane == 0) prm.undo_len[slot] = c.sc()->ulen;

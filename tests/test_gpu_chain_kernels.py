@@ -49,9 +49,11 @@ def test_weights(kvp, oracle, hooks, bw, flags):
         _same(g, o, chains=6, moves=2000, seed=4, levels=4, p0=0.3)
 
 
+@pytest.mark.parametrize("warps", [0, 2, 3, 18])
 @pytest.mark.parametrize("chains,rungs", [(24, 3), (40, 8), (36, 12), (40, 20)])
-def test_exchange_rounds(kvp, oracle, chains, rungs):
-    """Ladders that fill a CTA exactly, leave chains of it idle, or do not fit one (a launch per round)."""
+def test_exchange_rounds(kvp, oracle, hooks, warps, chains, rungs):
+    """Ladders that fill a CTA exactly, leave chains of it idle, or do not fit one (a launch per round); both kernels."""
+    hooks(warps_per_chain=warps)
     A = wl.random_access(120, 90, 0.25, seed=2)
     g, o = both_problems(kvp, oracle, 120, 8192, 90, A, 30, (8000 * GB, 900 * GB, 900 * GB))
     kw = dict(chains=chains, moves=701, seed=9, levels=rungs, p0=1e-2, alpha=0.7)
