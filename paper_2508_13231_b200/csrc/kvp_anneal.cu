@@ -553,7 +553,11 @@ struct Ctx {
     uint32_t* P0;            // [S][W32] initial schedule, step-major
     uint32_t* Pcol0;         // [U][S32]
     uint32_t* counts0;       // [S][4]
-    uint64_t* small;         // [0] total ticks, [1] hits, [2] bad step (int32), [4..5] calibration, [8..] reduce out
+    uint64_t* small;         // [0] total ticks, [1] hits, [2] bad step (int32), [4..5] calibration, [8..] reduce out, [16] err, [24..] work
+    char* host;              // host side of the copies: 256 bytes for `small`, then the tables
+    size_t host_bytes;
+    std::vector<char> host_own;
+    uint64_t* host_small() const { return reinterpret_cast<uint64_t*>(host); }
     uint32_t* table; uint32_t* shifts;
     kvp_chain_result* results;
     uint32_t* dumpcol;       // [U][S32]
@@ -669,6 +673,37 @@ int run_chains(Ctx& c, uint32_t first, uint32_t count, uint32_t result_base, kvp
     return launch_chains(c, prm, count);
 }
 
+// bytes of an acceptance table with its shifts and bounds
+size_t table_bytes(uint32_t levels) { return (size_t)levels * (KVP_TABLE_Q + 2) * 4; }
+
+// Host side of a call's copies: page-locked, so that a copy neither waits for a staging copy nor holds the host up (the
+// tables of 64 levels, 262 KB in three pageable copies: 40 us of a call of 540). Every call ends with a synchronisation,
+// so one block per thread is enough; it is kept up to 1 MB and freed with the thread. Larger calls use ordinary memory.
+struct Staging {
+    char* p = nullptr;
+    size_t bytes = 0;
+    ~Staging() { if (p) cudaFreeHost(p); }
+};
+
+char* staging(size_t bytes, std::vector<char>& otherwise)
+{
+    static thread_local Staging mine;
+    if (mine.bytes >= bytes) return mine.p;
+    if (bytes <= ((size_t)1 << 20)) {
+        if (mine.p) cudaFreeHost(mine.p);
+        mine = Staging();
+        const size_t want = bytes <= ((size_t)512 << 10) ? (size_t)512 << 10 : (size_t)1 << 20;
+        if (cudaHostAlloc(reinterpret_cast<void**>(&mine.p), want, cudaHostAllocPortable) == cudaSuccess) {
+            mine.bytes = want;
+            return mine.p;
+        }
+        cudaGetLastError();                                       // ordinary memory does as well
+        mine.p = nullptr;
+    }
+    otherwise.resize(bytes);
+    return otherwise.data();
+}
+
 // Initial schedule, its counters and cost, the temperature ladder and the acceptance table.
 // rungs: 0, or the chains of a ladder (replica exchange).
 int prepare(kvp_problem* p, const kvp_anneal_params* a, cudaStream_t st, Ctx& c, uint32_t rungs = 0)
@@ -678,6 +713,9 @@ int prepare(kvp_problem* p, const kvp_anneal_params* a, cudaStream_t st, Ctx& c,
     KVP_CUDA(cudaSetDevice(p->device));
     c.st = st;
     c.launches = 0;
+    // the small block, the table of the levels; replica exchange: the table of the pairs of rungs, the last rungs
+    c.host_bytes = 256 + table_bytes(a->levels) + (rungs ? table_bytes(rungs) + a->chains : 0);
+    c.host = staging(c.host_bytes, c.host_own);
     const size_t sched_bytes = align256((size_t)p->S * p->W32 * 4);
     const size_t col_bytes = align256((size_t)p->U * p->S32 * 4);
 
@@ -818,22 +856,25 @@ int prepare(kvp_problem* p, const kvp_anneal_params* a, cudaStream_t st, Ctx& c,
         if (ctas < 1) return KVP_ERR_RANGE;
         uint32_t per_sm = (uint32_t)ctas * wcap;                   // resident chains per SM, at most 32 warps
         if (per_sm * W > 32) per_sm = 32 / W / wcap ? 32 / W / wcap * wcap : wcap;
-        size_t free_b = 0, total_b = 0;
-        KVP_CUDA(cudaMemGetInfo(&free_b, &total_b));
-        free_b += p->chain_ws_bytes;                               // what we already hold can be reused
-        {                                                          // and so can what the pool holds in reserve
+        size_t cap_r = (size_t)per_sm * sms;
+        size_t r = a->chains < cap_r ? a->chains : cap_r;
+        // How many slices fit. What the problem holds and what the pool has in reserve is known without asking the driver
+        // for the device's free memory, which takes 90 us.
+        size_t have = p->chain_ws_bytes;
+        {
             cudaMemPool_t pool; uint64_t reserved = 0, used = 0;
             if (cudaDeviceGetDefaultMemPool(&pool, dev) == cudaSuccess &&
                 cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReservedMemCurrent, &reserved) == cudaSuccess &&
                 cudaMemPoolGetAttribute(pool, cudaMemPoolAttrUsedMemCurrent, &used) == cudaSuccess && reserved > used)
-                free_b += (size_t)(reserved - used);
+                have += (size_t)(reserved - used);
         }
-        const size_t usable = free_b / 10 * 7;
-        size_t fit = usable / col_bytes;
-        if (fit < 1) return KVP_ERR_NOMEM;
-        size_t cap_r = (size_t)per_sm * sms;
-        size_t r = a->chains < cap_r ? a->chains : cap_r;
-        if (r > fit) r = fit;
+        if (have / 10 * 7 < r * col_bytes) {
+            size_t free_b = 0, total_b = 0;
+            KVP_CUDA(cudaMemGetInfo(&free_b, &total_b));
+            const size_t fit = (have + free_b) / 10 * 7 / col_bytes;
+            if (fit < 1) return KVP_ERR_NOMEM;
+            if (r > fit) r = fit;
+        }
         // test hook: at most n chains at a time, so that small jobs come in several waves
         if (hooks.resident >= 1 && (size_t)hooks.resident < r) r = hooks.resident;
         const uint32_t waves = (uint32_t)((a->chains + r - 1) / r);
@@ -849,7 +890,7 @@ int prepare(kvp_problem* p, const kvp_anneal_params* a, cudaStream_t st, Ctx& c,
     size_t off = 0;
     auto take = [&](size_t bytes) { size_t o = off; off += align256(bytes); return o; };
     const size_t o_P0 = take(sched_bytes), o_col0 = take(col_bytes), o_cnt = take((size_t)p->S * 20 + 4);   // counts, births, ticket
-    const size_t o_small = take(256), o_table = take((size_t)a->levels * KVP_TABLE_Q * 4), o_shift = take((size_t)a->levels * 4), o_bound = take((size_t)a->levels * 4);
+    const size_t o_small = take(256), o_table = take(table_bytes(a->levels));
     const size_t o_res = take((size_t)(a->chains + 1) * sizeof(kvp_chain_result));
     const size_t o_dump = take(col_bytes), o_sched = take(sched_bytes);
     const size_t o_slots = take(c.psmem ? 0 : (size_t)c.resident * col_bytes);
@@ -871,8 +912,8 @@ int prepare(kvp_problem* p, const kvp_anneal_params* a, cudaStream_t st, Ctx& c,
     if (rc) return rc;
     char* base = static_cast<char*>(p->d_chain_ws);
     c.P0 = (uint32_t*)(base + o_P0); c.Pcol0 = (uint32_t*)(base + o_col0); c.counts0 = (uint32_t*)(base + o_cnt);
-    c.small = (uint64_t*)(base + o_small); c.table = (uint32_t*)(base + o_table); c.shifts = (uint32_t*)(base + o_shift);
-    c.bounds = (float*)(base + o_bound);
+    c.small = (uint64_t*)(base + o_small); c.table = (uint32_t*)(base + o_table);
+    c.shifts = c.table + (size_t)a->levels * KVP_TABLE_Q; c.bounds = (float*)(c.shifts + a->levels);
     c.results = (kvp_chain_result*)(base + o_res); c.dumpcol = (uint32_t*)(base + o_dump);
     c.sched = (uint32_t*)(base + o_sched); c.slots = (uint32_t*)(base + o_slots);
     c.hb0 = c.grow ? c.counts0 + (size_t)p->S * 4 : nullptr;
@@ -881,6 +922,7 @@ int prepare(kvp_problem* p, const kvp_anneal_params* a, cudaStream_t st, Ctx& c,
     c.cow_out = cow ? (uint32_t*)(base + o_cow) : nullptr;
 
     // initial schedule in both layouts
+    KVP_CUDA(cudaMemsetAsync(c.small, 0, 256, st));
     if (a->init_mode == KVP_INIT_USER) {
         if ((rc = launch_clean_copy(a->init_schedule, c.P0, p->S, p->W32, p->pad_mask, st))) return rc;
         // a unit of the initial placement enters HBM when it is written; the chains keep the bits before that clear
@@ -894,9 +936,8 @@ int prepare(kvp_problem* p, const kvp_anneal_params* a, cudaStream_t st, Ctx& c,
             row = c.sched;
             ++c.launches;
         }
-        if ((rc = launch_broadcast_row(row, p->S, p->W32, p->dL, c.P0, st))) return rc;
-        if ((rc = launch_row_to_columns(row, p->U, p->S, p->S32, p->d_birth, c.Pcol0, st))) return rc;
-        c.launches += 2;
+        if ((rc = launch_initial_schedule(p, row, c.P0, c.Pcol0, st))) return rc;
+        ++c.launches;
     }
     if ((rc = launch_score(p, c.P0, 1, c.counts0, c.counts0, c.hb0, nullptr, c.small, nullptr, nullptr, (int32_t*)(c.small + 2),
                            c.small + 1, st, &c.launches)))
@@ -918,7 +959,6 @@ int prepare(kvp_problem* p, const kvp_anneal_params* a, cudaStream_t st, Ctx& c,
     // test hook: less room for accepted proposals, so that a batch stops to commit more often
     prm.carry = kAccepted;
     if (hooks.split_queue_plus1 >= 1 && hooks.split_queue_plus1 <= kAccepted) prm.carry = hooks.split_queue_plus1;
-    KVP_CUDA(cudaMemsetAsync(prm.err, 0, 4, st));
     prm.U = p->U; prm.S = p->S; prm.S32 = p->S32; prm.cap = p->cap;
     prm.levels = a->levels; prm.p_swap_256 = a->p_swap_256; prm.len_choices = a->max_len_log2 + 1;
     prm.early_permille = a->early_stop_permille; prm.early_from = a->early_stop_from_level;
@@ -930,14 +970,13 @@ int prepare(kvp_problem* p, const kvp_anneal_params* a, cudaStream_t st, Ctx& c,
     c.calib_mean = 0;
     const bool calibrate = a->temps == nullptr;
     if (calibrate) {
-        KVP_CUDA(cudaMemsetAsync(c.small + 4, 0, 16, st));
         if (c.grow) calib_kernel<true><<<CALIB_N / 256, 256, 0, st>>>(prm, (unsigned long long*)(c.small + 4));
         else calib_kernel<false><<<CALIB_N / 256, 256, 0, st>>>(prm, (unsigned long long*)(c.small + 4));
         KVP_CUDA(cudaGetLastError());
         ++c.launches;
     }
-    uint64_t host_small[8];
-    KVP_CUDA(cudaMemcpyAsync(host_small, c.small, sizeof host_small, cudaMemcpyDeviceToHost, st));
+    uint64_t* const host_small = c.host_small();
+    KVP_CUDA(cudaMemcpyAsync(host_small, c.small, 64, cudaMemcpyDeviceToHost, st));
     KVP_CUDA(cudaStreamSynchronize(st));
     if ((int32_t)(host_small[2] & 0xFFFFFFFFu) >= 0) return KVP_ERR_CAPACITY;   // Eq. 5 on the initial schedule
     c.init_ticks = host_small[0];
@@ -951,30 +990,28 @@ int prepare(kvp_problem* p, const kvp_anneal_params* a, cudaStream_t st, Ctx& c,
     } else {
         for (uint32_t j = 0; j < a->levels; ++j) c.temps[j] = a->temps[j];
     }
-    std::vector<uint32_t> table((size_t)a->levels * KVP_TABLE_Q), shifts(a->levels);
-    if ((rc = kvp_accept_table(c.temps.data(), a->levels, table.data(), shifts.data()))) return rc;
-    KVP_CUDA(cudaMemcpyAsync(c.table, table.data(), table.size() * 4, cudaMemcpyHostToDevice, st));
-    KVP_CUDA(cudaMemcpyAsync(c.shifts, shifts.data(), shifts.size() * 4, cudaMemcpyHostToDevice, st));
+    uint32_t* const table = reinterpret_cast<uint32_t*>(c.host + 256);
+    uint32_t* const shifts = table + (size_t)a->levels * KVP_TABLE_Q;
+    float* const bounds = reinterpret_cast<float*>(shifts + a->levels);
+    if ((rc = kvp_accept_table(c.temps.data(), a->levels, table, shifts))) return rc;
     // the lower bounds of kvp_chain.cuh are sums of at most 31 steps' changes in 32 bits
     const uint64_t step_max = 4ull * std::max(p->K.khF, p->K.kdF) + std::max(p->K.kh, p->K.ke) + 2ull * std::max(p->K.kh, p->K.kd);
-    std::vector<float> bounds(a->levels, INFINITY);
-    if (31 * step_max < (1ull << 30))
-        for (uint32_t j = 0; j < a->levels; ++j) bounds[j] = (float)((c.temps[j] >= 1.0 ? c.temps[j] : 1.0) * 0.69314718);
-    KVP_CUDA(cudaMemcpyAsync(c.bounds, bounds.data(), bounds.size() * 4, cudaMemcpyHostToDevice, st));
-    KVP_CUDA(cudaStreamSynchronize(st));           // the host vectors go out of scope
+    const bool bounded = 31 * step_max < (1ull << 30);
+    for (uint32_t j = 0; j < a->levels; ++j) bounds[j] = bounded ? (float)((c.temps[j] >= 1.0 ? c.temps[j] : 1.0) * 0.69314718) : INFINITY;
+    KVP_CUDA(cudaMemcpyAsync(c.table, table, table_bytes(a->levels), cudaMemcpyHostToDevice, st));
     return KVP_OK;
 }
 
-// Replay `chain` for `upto` proposals and leave its schedule, step-major, in c.sched.
-int replay_to_sched(kvp_problem* p, Ctx& c, uint32_t chain, uint64_t upto, kvp_chain_result* result_dev)
+// Replay `chain` for `upto` proposals and leave its schedule, step-major, in `sched`.
+int replay_to_sched(kvp_problem* p, Ctx& c, uint32_t chain, uint64_t upto, kvp_chain_result* result_dev, uint32_t* sched)
 {
     int rc;
     if (upto == 0) {
-        KVP_CUDA(cudaMemcpyAsync(c.sched, c.P0, (size_t)p->S * p->W32 * 4, cudaMemcpyDeviceToDevice, c.st));
+        KVP_CUDA(cudaMemcpyAsync(sched, c.P0, (size_t)p->S * p->W32 * 4, cudaMemcpyDeviceToDevice, c.st));
         return KVP_OK;
     }
     if ((rc = run_chains(c, chain, 1, chain, result_dev, upto, c.dumpcol, nullptr))) return rc;
-    if ((rc = launch_bit_transpose(c.dumpcol, p->U, p->S32, p->S, c.sched, p->W32, c.st))) return rc;
+    if ((rc = launch_bit_transpose(c.dumpcol, p->U, p->S32, p->S, sched, p->W32, c.st))) return rc;
     ++c.launches;
     return KVP_OK;
 }
@@ -1011,7 +1048,6 @@ extern "C" int kvp_anneal(kvp_problem* p, const kvp_anneal_params* a, uint32_t* 
     uint32_t dumped_chain = 0xFFFFFFFFu;                  // call-local index of the chain whose best state is in dumpcol
     uint32_t waves = 0;
     unsigned long long* work_dev = reinterpret_cast<unsigned long long*>(c.small + 24);
-    KVP_CUDA(cudaMemsetAsync(work_dev, 0, 24, st));
     c.prm.work = c.wide ? work_dev : nullptr;
     for (uint32_t first = 0; first < a->chains; first += c.resident, ++waves) {
         const uint32_t count = a->chains - first < c.resident ? a->chains - first : c.resident;
@@ -1052,41 +1088,48 @@ extern "C" int kvp_anneal(kvp_problem* p, const kvp_anneal_params* a, uint32_t* 
     }
     KVP_CUDA(cudaEventRecord(ev[2], st));
     c.prm.work = nullptr;                                 // a replay of the winner is not part of the count
-    unsigned long long work[3] = {0, 0, 0};
-    KVP_CUDA(cudaMemcpyAsync(work, work_dev, sizeof work, cudaMemcpyDeviceToHost, st));
 
     // cross-chain reduction, then the winner's schedule (its own snapshot, its walked-back state, or a replay) and a
     // re-score
+    uint32_t* const sched = best_schedule ? best_schedule : c.sched;
+    uint64_t* const host_small = c.host_small();
     if (!c.undo_log) {
         reduce_kernel<<<1, 1024, 0, st>>>(c.results, a->chains, c.prm.err, red_dev);
         KVP_CUDA(cudaGetLastError());
         ++c.launches;
-        KVP_CUDA(cudaMemcpyAsync(&red, red_dev, sizeof red, cudaMemcpyDeviceToHost, st));
-        KVP_CUDA(cudaStreamSynchronize(st));
-        if (red.pad) return KVP_ERR_TIMEOUT;
     }
-    const uint64_t upto = red.best_move == ~0ull ? 0 : red.best_move + 1;
-    if (upto && (c.snap || dumped_chain == red.best_chain)) {
-        const uint32_t* col = c.snap ? c.snap + (size_t)red.best_chain * p->U * p->S32 : c.dumpcol;
-        if ((rc = launch_bit_transpose(col, p->U, p->S32, p->S, c.sched, p->W32, st))) return rc;
+    if (c.snap) {                                          // the device knows which snapshot: no wait in between
+        ChosenInput winner;
+        winner.otherwise = c.Pcol0; winner.valid = &red_dev->best_move; winner.index = &red_dev->best_chain;
+        if ((rc = launch_bit_transpose(c.snap, p->U, p->S32, p->S, sched, p->W32, st, winner))) return rc;
         ++c.launches;
-        red.best_chain += a->first_chain;                  // the reduction works on call-local indices
     } else {
-        red.best_chain += a->first_chain;
-        if ((rc = replay_to_sched(p, c, red.best_chain, upto, c.results + a->chains))) return rc;
+        if (!c.undo_log) {
+            KVP_CUDA(cudaMemcpyAsync(&red, red_dev, sizeof red, cudaMemcpyDeviceToHost, st));
+            KVP_CUDA(cudaStreamSynchronize(st));
+            if (red.pad) return KVP_ERR_TIMEOUT;
+        }
+        const uint64_t upto = red.best_move == ~0ull ? 0 : red.best_move + 1;
+        if (upto && dumped_chain == red.best_chain) {
+            if ((rc = launch_bit_transpose(c.dumpcol, p->U, p->S32, p->S, sched, p->W32, st))) return rc;
+            ++c.launches;
+        } else if ((rc = replay_to_sched(p, c, a->first_chain + red.best_chain, upto, c.results + a->chains, sched))) {
+            return rc;
+        }
     }
-    if ((rc = launch_score(p, c.sched, 1, c.counts0, nullptr, nullptr, nullptr, c.small, nullptr, nullptr, (int32_t*)(c.small + 2),
+    if ((rc = launch_score(p, sched, 1, c.counts0, nullptr, nullptr, nullptr, c.small, nullptr, nullptr, (int32_t*)(c.small + 2),
                            c.small + 1, st, &c.launches)))
         return rc;
-    if (best_schedule)
-        KVP_CUDA(cudaMemcpyAsync(best_schedule, c.sched, (size_t)p->S * p->W32 * 4, cudaMemcpyDeviceToDevice, st));
-    uint64_t host_small[4];
-    KVP_CUDA(cudaMemcpyAsync(host_small, c.small, sizeof host_small, cudaMemcpyDeviceToHost, st));
+    KVP_CUDA(cudaMemcpyAsync(host_small, c.small, 256, cudaMemcpyDeviceToHost, st));
     if (stats && stats->per_chain)
         KVP_CUDA(cudaMemcpyAsync(stats->per_chain, c.results, (size_t)a->chains * sizeof(kvp_chain_result),
                                  cudaMemcpyDeviceToHost, st));
     KVP_CUDA(cudaEventRecord(ev[3], st));
     KVP_CUDA(cudaStreamSynchronize(st));
+    memcpy(&red, host_small + 8, sizeof red);
+    if (red.pad) return KVP_ERR_TIMEOUT;
+    red.best_chain += a->first_chain;                      // the reduction works on call-local indices
+    const uint64_t* const work = host_small + 24;
     const bool ok = host_small[0] == red.best_ticks && (int32_t)(host_small[2] & 0xFFFFFFFFu) < 0;
     if (best_ticks) *best_ticks = red.best_ticks;
     if (best_seconds) *best_seconds = (double)red.best_ticks * p->spt;
@@ -1125,8 +1168,7 @@ extern "C" int kvp_anneal_chain_state(kvp_problem* p, const kvp_anneal_params* a
         r0.best_ticks = r0.final_ticks = c.init_ticks; r0.best_move = ~0ull;
         KVP_CUDA(cudaMemcpyAsync(res_dev, &r0, sizeof r0, cudaMemcpyHostToDevice, st));
     }
-    if ((rc = replay_to_sched(p, c, chain, upto_moves, res_dev))) return rc;
-    KVP_CUDA(cudaMemcpyAsync(schedule, c.sched, (size_t)p->S * p->W32 * 4, cudaMemcpyDeviceToDevice, st));
+    if ((rc = replay_to_sched(p, c, chain, upto_moves, res_dev, schedule))) return rc;
     if (result) KVP_CUDA(cudaMemcpyAsync(result, res_dev, sizeof *result, cudaMemcpyDeviceToHost, st));
     uint32_t gave_up = 0;
     KVP_CUDA(cudaMemcpyAsync(&gave_up, c.prm.err, 4, cudaMemcpyDeviceToHost, st));
@@ -1181,9 +1223,13 @@ extern "C" int kvp_anneal_exchange(kvp_problem* p, const kvp_anneal_params* a, c
     // exchange thresholds of the pairs of neighbouring rungs: the move table's form at the pair temperatures
     const uint32_t pairs = rungs > 1 ? rungs - 1 : 1;
     std::vector<double> pair_temps(pairs, 1.0);
-    std::vector<uint32_t> always(pairs, 0u), xtable((size_t)pairs * KVP_TABLE_Q), xshifts(pairs);
-    if ((rc = kvp_exchange_temps(c.temps.data(), rungs, pair_temps.data(), always.data()))) return rc;
-    if ((rc = kvp_accept_table(pair_temps.data(), pairs, xtable.data(), xshifts.data()))) return rc;
+    uint32_t* const xtable = reinterpret_cast<uint32_t*>(c.host + 256 + table_bytes(rungs));
+    uint32_t* const xshifts = xtable + (size_t)pairs * KVP_TABLE_Q;
+    uint32_t* const always = xshifts + pairs;
+    uint8_t* const last_row = reinterpret_cast<uint8_t*>(c.host + 256 + 2 * table_bytes(rungs));
+    memset(always, 0, (size_t)pairs * 4);
+    if ((rc = kvp_exchange_temps(c.temps.data(), rungs, pair_temps.data(), always))) return rc;
+    if ((rc = kvp_accept_table(pair_temps.data(), pairs, xtable, xshifts))) return rc;
 
     // workspace of the run: rung history, holders, exchange counts, thresholds, the chains' saved states
     const uint32_t persist4 = chain_layout(p->S, p->S32, c.grow, c.psmem, c.lin, c.psmem ? 0u : c.cow_slots4).work / 16;
@@ -1192,8 +1238,7 @@ extern "C" int kvp_anneal_exchange(kvp_problem* p, const kvp_anneal_params* a, c
     size_t off = 0;
     auto take = [&](size_t bytes) { size_t o = off; off += align256(bytes); return o; };
     const size_t o_hist = take((size_t)rounds * chains), o_hold = take((size_t)chains * 4), o_nex = take((size_t)chains * 4);
-    const size_t o_cnt = take(16), o_alw = take((size_t)pairs * 4), o_xsh = take((size_t)pairs * 4);
-    const size_t o_xt = take((size_t)pairs * KVP_TABLE_Q * 4), o_state = take((size_t)chains * state4 * 16);
+    const size_t o_xt = take(table_bytes(pairs)), o_state = take(c.ladder_ctas ? 0 : (size_t)chains * state4 * 16);
     char* xw = nullptr;
     KVP_CUDA(cudaMallocAsync(&xw, off, st));
     struct Free {                                          // in stream order, on every way out
@@ -1203,11 +1248,9 @@ extern "C" int kvp_anneal_exchange(kvp_problem* p, const kvp_anneal_params* a, c
     uint8_t* hist = (uint8_t*)(xw + o_hist);
     uint32_t* holder = (uint32_t*)(xw + o_hold);
     uint32_t* nex = (uint32_t*)(xw + o_nex);
-    unsigned long long* counts = (unsigned long long*)(xw + o_cnt);
-    KVP_CUDA(cudaMemsetAsync(counts, 0, 16, st));
-    KVP_CUDA(cudaMemcpyAsync(xw + o_alw, always.data(), (size_t)pairs * 4, cudaMemcpyHostToDevice, st));
-    KVP_CUDA(cudaMemcpyAsync(xw + o_xsh, xshifts.data(), (size_t)pairs * 4, cudaMemcpyHostToDevice, st));
-    KVP_CUDA(cudaMemcpyAsync(xw + o_xt, xtable.data(), xtable.size() * 4, cudaMemcpyHostToDevice, st));
+    unsigned long long* counts = (unsigned long long*)(c.small + 28);   // zero since prepare()
+    const uint32_t* const xtable_dev = (const uint32_t*)(xw + o_xt);
+    KVP_CUDA(cudaMemcpyAsync(xw + o_xt, xtable, table_bytes(pairs), cudaMemcpyHostToDevice, st));
     exchange_init_kernel<<<(chains + 255) / 256, 256, 0, st>>>(holder, hist, nex, chains, rungs);
     KVP_CUDA(cudaGetLastError());
     ++c.launches;
@@ -1221,10 +1264,9 @@ extern "C" int kvp_anneal_exchange(kvp_problem* p, const kvp_anneal_params* a, c
     prm.rung_hist = hist; prm.exch_every = xp->exchange_every; prm.hist_stride = chains; prm.hist_base = a->first_chain;
     prm.state = (uint4*)(xw + o_state); prm.state4 = state4;
     unsigned long long* work_dev = reinterpret_cast<unsigned long long*>(c.small + 24);
-    KVP_CUDA(cudaMemsetAsync(work_dev, 0, 24, st));
     ExchangeK xk;
     xk.results = c.results; xk.holder = holder; xk.n_exchanged = nex; xk.x.counts = counts;
-    xk.x.always = (const uint32_t*)(xw + o_alw); xk.x.table = (const uint32_t*)(xw + o_xt); xk.x.shifts = (const uint32_t*)(xw + o_xsh);
+    xk.x.table = xtable_dev; xk.x.shifts = xtable_dev + (size_t)pairs * KVP_TABLE_Q; xk.x.always = xk.x.shifts + pairs;
     xk.ladders = chains / rungs; xk.x.rungs = rungs; xk.first_ladder = a->first_chain / rungs;
     xk.x.seed_lo = (uint32_t)a->seed; xk.x.seed_hi = (uint32_t)(a->seed >> 32);
     if (c.ladder_ctas) {
@@ -1254,46 +1296,48 @@ extern "C" int kvp_anneal_exchange(kvp_problem* p, const kvp_anneal_params* a, c
     reduce_kernel<<<1, 1024, 0, st>>>(c.results, chains, c.prm.err, red_dev);
     KVP_CUDA(cudaGetLastError());
     ++c.launches;
-    unsigned long long work[3] = {0, 0, 0}, xcounts[2] = {0, 0};
-    KVP_CUDA(cudaMemcpyAsync(&red, red_dev, sizeof red, cudaMemcpyDeviceToHost, st));
-    KVP_CUDA(cudaMemcpyAsync(work, work_dev, sizeof work, cudaMemcpyDeviceToHost, st));
-    KVP_CUDA(cudaMemcpyAsync(xcounts, counts, sizeof xcounts, cudaMemcpyDeviceToHost, st));
-    KVP_CUDA(cudaStreamSynchronize(st));
     // the winner's schedule: its snapshot, or a replay of that one chain through the rungs it held
-    const uint64_t upto = red.best_move == ~0ull ? 0 : red.best_move + 1;
-    if (upto == 0) {
-        KVP_CUDA(cudaMemcpyAsync(c.sched, c.P0, (size_t)p->S * p->W32 * 4, cudaMemcpyDeviceToDevice, st));
-    } else if (c.snap) {
-        if ((rc = launch_bit_transpose(c.snap + (size_t)red.best_chain * pwords, p->U, p->S32, p->S, c.sched, p->W32, st))) return rc;
+    uint32_t* const sched = best_schedule ? best_schedule : c.sched;
+    uint64_t* const host_small = c.host_small();
+    if (c.snap) {                                          // the device knows which snapshot: no wait in between
+        ChosenInput winner;
+        winner.otherwise = c.Pcol0; winner.valid = &red_dev->best_move; winner.index = &red_dev->best_chain;
+        if ((rc = launch_bit_transpose(c.snap, p->U, p->S32, p->S, sched, p->W32, st, winner))) return rc;
         ++c.launches;
     } else {
-        ChainParams rp = prm;
-        rp.snap = nullptr; rp.state = nullptr; rp.resume = 0u; rp.work = nullptr;
-        rp.chain_first = a->first_chain + red.best_chain; rp.chain_count = 1; rp.result_base = rp.chain_first;
-        rp.results = c.results + chains; rp.upto = upto; rp.dump = c.dumpcol;
-        rp.round0 = 0; rp.round1 = rounds;
-        if ((rc = launch_chains(c, rp, 1))) return rc;
-        if ((rc = launch_bit_transpose(c.dumpcol, p->U, p->S32, p->S, c.sched, p->W32, st))) return rc;
-        c.launches += 2;
+        KVP_CUDA(cudaMemcpyAsync(&red, red_dev, sizeof red, cudaMemcpyDeviceToHost, st));
+        KVP_CUDA(cudaStreamSynchronize(st));
+        if (red.pad) return KVP_ERR_TIMEOUT;
+        const uint64_t upto = red.best_move == ~0ull ? 0 : red.best_move + 1;
+        if (upto == 0) {
+            KVP_CUDA(cudaMemcpyAsync(sched, c.P0, (size_t)p->S * p->W32 * 4, cudaMemcpyDeviceToDevice, st));
+        } else {
+            ChainParams rp = prm;
+            rp.snap = nullptr; rp.state = nullptr; rp.resume = 0u; rp.work = nullptr;
+            rp.chain_first = a->first_chain + red.best_chain; rp.chain_count = 1; rp.result_base = rp.chain_first;
+            rp.results = c.results + chains; rp.upto = upto; rp.dump = c.dumpcol;
+            rp.round0 = 0; rp.round1 = rounds;
+            if ((rc = launch_chains(c, rp, 1))) return rc;
+            if ((rc = launch_bit_transpose(c.dumpcol, p->U, p->S32, p->S, sched, p->W32, st))) return rc;
+            c.launches += 2;
+        }
     }
-    red.best_chain += a->first_chain;
-    if ((rc = launch_score(p, c.sched, 1, c.counts0, nullptr, nullptr, nullptr, c.small, nullptr, nullptr, (int32_t*)(c.small + 2),
+    if ((rc = launch_score(p, sched, 1, c.counts0, nullptr, nullptr, nullptr, c.small, nullptr, nullptr, (int32_t*)(c.small + 2),
                            c.small + 1, st, &c.launches)))
         return rc;
-    if (best_schedule)
-        KVP_CUDA(cudaMemcpyAsync(best_schedule, c.sched, (size_t)p->S * p->W32 * 4, cudaMemcpyDeviceToDevice, st));
-    uint64_t host_small[4];
-    KVP_CUDA(cudaMemcpyAsync(host_small, c.small, sizeof host_small, cudaMemcpyDeviceToHost, st));
+    KVP_CUDA(cudaMemcpyAsync(host_small, c.small, 256, cudaMemcpyDeviceToHost, st));
     if (stats && stats->per_chain)
         KVP_CUDA(cudaMemcpyAsync(stats->per_chain, c.results, (size_t)chains * sizeof(kvp_chain_result), cudaMemcpyDeviceToHost, st));
-    std::vector<uint8_t> last_row(final_rung ? chains : 0);
-    if (final_rung)
-        KVP_CUDA(cudaMemcpyAsync(last_row.data(), hist + (size_t)(rounds - 1) * chains, chains, cudaMemcpyDeviceToHost, st));
+    if (final_rung) KVP_CUDA(cudaMemcpyAsync(last_row, hist + (size_t)(rounds - 1) * chains, chains, cudaMemcpyDeviceToHost, st));
     if (n_exchanged) KVP_CUDA(cudaMemcpyAsync(n_exchanged, nex, (size_t)chains * 4, cudaMemcpyDeviceToHost, st));
     KVP_CUDA(cudaEventRecord(ev[3], st));
     KVP_CUDA(cudaStreamSynchronize(st));
     if (final_rung)
         for (uint32_t i = 0; i < chains; ++i) final_rung[i] = last_row[i];
+    memcpy(&red, host_small + 8, sizeof red);
+    if (red.pad) return KVP_ERR_TIMEOUT;
+    red.best_chain += a->first_chain;
+    const uint64_t *const work = host_small + 24, *const xcounts = host_small + 28;
     const bool ok = host_small[0] == red.best_ticks && (int32_t)(host_small[2] & 0xFFFFFFFFu) < 0;
     if (best_ticks) *best_ticks = red.best_ticks;
     if (best_seconds) *best_seconds = (double)red.best_ticks * p->spt;

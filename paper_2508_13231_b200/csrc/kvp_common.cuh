@@ -159,17 +159,22 @@ int launch_score(const kvp_problem* p, const uint32_t* schedules, uint32_t n, vo
 int launch_counts(const kvp_problem* p, const uint32_t* schedules, uint32_t n, uint32_t* counts, cudaStream_t st);
 
 // kvp_layout.cu
+// Input that a kernel before has chosen: number *index of the matrices that start at `in`, or `otherwise` if *valid is ~0.
+struct ChosenInput {
+    const uint32_t* otherwise;
+    const uint64_t* valid;
+    const uint32_t* index;
+};
 int launch_bit_transpose(const uint32_t* in, uint32_t rows, uint32_t in_words, uint32_t cols, uint32_t* out,
-                         uint32_t out_words, cudaStream_t st);
+                         uint32_t out_words, cudaStream_t st, const ChosenInput& chosen = ChosenInput());
 int launch_clean_copy(const uint32_t* in, uint32_t* out, uint32_t S, uint32_t W32, uint32_t pad_mask, cudaStream_t st);
 int launch_open(const kvp_problem* p, const uint32_t* access, cudaStream_t st);
 int launch_stepc(StepC* stepc, const uint32_t* writes, const uint32_t* a, uint32_t S, const CostK& K, cudaStream_t st);
 size_t static_freq_words(const kvp_problem* p);
 int launch_static_freq_row(const kvp_problem* p, uint32_t* scratch, uint32_t* row, cudaStream_t st);
 int launch_static_first_row(const kvp_problem* p, uint32_t* row, cudaStream_t st);
-int launch_broadcast_row(const uint32_t* row, uint32_t S, uint32_t W32, const uint32_t* L, uint32_t* sched, cudaStream_t st);
-int launch_row_to_columns(const uint32_t* row, uint32_t U, uint32_t S, uint32_t S32, const uint32_t* birth, uint32_t* Pcol,
-                          cudaStream_t st);
+int launch_broadcast_row(const uint32_t* row, uint32_t S, uint32_t W32, uint32_t* sched, cudaStream_t st);
+int launch_initial_schedule(const kvp_problem* p, const uint32_t* row, uint32_t* sched, uint32_t* Pcol, cudaStream_t st);
 int launch_alive_rows(const uint32_t* birth, uint32_t U, uint32_t S, uint32_t W32, uint32_t* L, cudaStream_t st);
 int launch_birth_stats(const uint32_t* birth, uint32_t U, uint32_t S, const uint32_t* Acol, uint32_t S32, uint32_t* nb,
                        uint32_t* flag, cudaStream_t st);

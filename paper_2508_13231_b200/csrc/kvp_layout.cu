@@ -55,9 +55,10 @@ struct OpenArgs {
 
 template <int LRB, int LWB, bool OPEN>
 __global__ void __launch_bounds__(256)
-bit_transpose_kernel(const uint32_t* __restrict__ in, uint32_t rows, uint32_t in_words, uint32_t cols,
-                     uint32_t* __restrict__ out, uint32_t out_words, const OpenArgs open)
+bit_transpose_kernel(const uint32_t* in, uint32_t rows, uint32_t in_words, uint32_t cols,
+                     uint32_t* __restrict__ out, uint32_t out_words, const OpenArgs open, const ChosenInput chosen)
 {
+    if (chosen.index) in = *chosen.valid == ~0ull ? chosen.otherwise : in + (size_t)*chosen.index * rows * in_words;
     constexpr uint32_t RB = 1u << LRB, WB = 1u << LWB, IS = WB | 1u, OS = RB | 1u;
     __shared__ uint32_t tin[RB * 32 * IS], tout[WB * 32 * OS];
     __shared__ uint32_t s_rows[OPEN ? RB * 32 : 1];
@@ -266,17 +267,23 @@ __global__ void static_first_kernel(uint32_t* __restrict__ row, uint32_t W32, ui
 }
 
 // every row of sched equals `row`; with births (L not null) cut to the units that exist at the step
-__global__ void broadcast_row_kernel(const uint32_t* __restrict__ row, uint32_t W32, size_t total, const uint32_t* __restrict__ L,
-                                     uint32_t* __restrict__ sched)
+__device__ __forceinline__ void broadcast_row(const uint32_t* __restrict__ row, uint32_t W32, size_t total, const uint32_t* __restrict__ L,
+                                              uint32_t* __restrict__ sched)
 {
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x)
         sched[i] = __ldg(row + i % W32) & (L ? __ldg(L + i) : ~0u);
 }
-
-// time-packed columns of a schedule whose every row equals `row`, from the step on at which the unit exists
-__global__ void row_to_columns_kernel(const uint32_t* __restrict__ row, uint32_t U, uint32_t S, uint32_t S32,
-                                      const uint32_t* __restrict__ birth, uint32_t* __restrict__ Pcol)
+__global__ void broadcast_row_kernel(const uint32_t* __restrict__ row, uint32_t W32, size_t total, uint32_t* __restrict__ sched)
 {
+    broadcast_row(row, W32, total, nullptr, sched);
+}
+
+// The same and its time-packed columns: a unit's bits are set from the step on at which it exists.
+__global__ void initial_schedule_kernel(const uint32_t* __restrict__ row, uint32_t U, uint32_t S, uint32_t W32, uint32_t S32,
+                                        const uint32_t* __restrict__ L, const uint32_t* __restrict__ birth,
+                                        uint32_t* __restrict__ sched, uint32_t* __restrict__ Pcol)
+{
+    broadcast_row(row, W32, (size_t)S * W32, L, sched);
     const size_t total = (size_t)U * S32;
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
         const uint32_t u = (uint32_t)(i / S32), j = (uint32_t)(i % S32);
@@ -357,26 +364,27 @@ inline uint32_t grid_for(size_t total, uint32_t block)
 
 template <int LRB, int LWB, bool OPEN>
 static int launch_transpose(const uint32_t* in, uint32_t rows, uint32_t in_words, uint32_t cols, uint32_t* out, uint32_t out_words,
-                            const OpenArgs& open, uint32_t most_y, cudaStream_t st)
+                            const OpenArgs& open, const ChosenInput& chosen, uint32_t most_y, cudaStream_t st)
 {
     uint32_t y = (in_words + (1u << LWB) - 1) >> LWB;
     if (y > most_y) y = most_y;
     dim3 grid((out_words + (1u << LRB) - 1) >> LRB, y);
-    bit_transpose_kernel<LRB, LWB, OPEN><<<grid, 256, 0, st>>>(in, rows, in_words, cols, out, out_words, open);
+    bit_transpose_kernel<LRB, LWB, OPEN><<<grid, 256, 0, st>>>(in, rows, in_words, cols, out, out_words, open, chosen);
     KVP_CUDA(cudaGetLastError());
     return KVP_OK;
 }
 
 // Tiles follow the short side: short rows in (a few steps' words per unit) take many rows, short rows out many words.
 int launch_bit_transpose(const uint32_t* in, uint32_t rows, uint32_t in_words, uint32_t cols, uint32_t* out,
-                         uint32_t out_words, cudaStream_t st)
+                         uint32_t out_words, cudaStream_t st, const ChosenInput& chosen)
 {
-    const OpenArgs none = {};
-    if (in_words <= 2) return launch_transpose<5, 1, false>(in, rows, in_words, cols, out, out_words, none, 32768, st);
-    if (in_words <= 4) return launch_transpose<4, 2, false>(in, rows, in_words, cols, out, out_words, none, 32768, st);
-    if (out_words <= 2) return launch_transpose<1, 5, false>(in, rows, in_words, cols, out, out_words, none, 32768, st);
-    if (out_words <= 4) return launch_transpose<2, 4, false>(in, rows, in_words, cols, out, out_words, none, 32768, st);
-    return launch_transpose<3, 3, false>(in, rows, in_words, cols, out, out_words, none, 32768, st);
+#define KVP_TRANSPOSE(LRB, LWB) launch_transpose<LRB, LWB, false>(in, rows, in_words, cols, out, out_words, OpenArgs(), chosen, 32768, st)
+    if (in_words <= 2) return KVP_TRANSPOSE(5, 1);
+    if (in_words <= 4) return KVP_TRANSPOSE(4, 2);
+    if (out_words <= 2) return KVP_TRANSPOSE(1, 5);
+    if (out_words <= 4) return KVP_TRANSPOSE(2, 4);
+    return KVP_TRANSPOSE(3, 3);
+#undef KVP_TRANSPOSE
 }
 
 // p->dA, p->dAcol, p->d_a and p->d_ucnt from the caller's access bitmap; d_a and d_ucnt come zeroed.
@@ -386,7 +394,7 @@ int launch_open(const kvp_problem* p, const uint32_t* access, cudaStream_t st)
     open.copy = p->dA; open.row_count = p->d_a; open.ucnt = p->d_ucnt; open.pad_mask = p->pad_mask;
     open.ucnt_add = p->S32 > 8;
     const uint32_t fill = 148 * 8;                       // CTAs that fill the machine: eight of 256 threads per SM
-#define KVP_OPEN(LRB, LWB, most) launch_transpose<LRB, LWB, true>(access, p->S, p->W32, p->U, p->dAcol, p->S32, open, most, st)
+#define KVP_OPEN(LRB, LWB, most) launch_transpose<LRB, LWB, true>(access, p->S, p->W32, p->U, p->dAcol, p->S32, open, ChosenInput(), most, st)
     if (p->S32 <= 2) return KVP_OPEN(1, 5, fill);
     if (p->S32 <= 4) return KVP_OPEN(2, 4, fill);
     const uint32_t tiles = (p->S32 + 7) / 8;
@@ -444,19 +452,18 @@ int launch_static_first_row(const kvp_problem* p, uint32_t* row, cudaStream_t st
     return KVP_OK;
 }
 
-int launch_broadcast_row(const uint32_t* row, uint32_t S, uint32_t W32, const uint32_t* L, uint32_t* sched, cudaStream_t st)
+int launch_broadcast_row(const uint32_t* row, uint32_t S, uint32_t W32, uint32_t* sched, cudaStream_t st)
 {
     const size_t total = (size_t)S * W32;
-    broadcast_row_kernel<<<grid_for(total, 256), 256, 0, st>>>(row, W32, total, L, sched);
+    broadcast_row_kernel<<<grid_for(total, 256), 256, 0, st>>>(row, W32, total, sched);
     KVP_CUDA(cudaGetLastError());
     return KVP_OK;
 }
 
-int launch_row_to_columns(const uint32_t* row, uint32_t U, uint32_t S, uint32_t S32, const uint32_t* birth, uint32_t* Pcol,
-                          cudaStream_t st)
+int launch_initial_schedule(const kvp_problem* p, const uint32_t* row, uint32_t* sched, uint32_t* Pcol, cudaStream_t st)
 {
-    const size_t total = (size_t)U * S32;
-    row_to_columns_kernel<<<grid_for(total, 256), 256, 0, st>>>(row, U, S, S32, birth, Pcol);
+    initial_schedule_kernel<<<grid_for((size_t)p->U * p->S32, 256), 256, 0, st>>>(row, p->U, p->S, p->W32, p->S32, p->dL, p->d_birth,
+                                                                                 sched, Pcol);
     KVP_CUDA(cudaGetLastError());
     return KVP_OK;
 }

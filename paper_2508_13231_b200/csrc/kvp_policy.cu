@@ -632,7 +632,7 @@ extern "C" int kvp_policy_lookahead(kvp_problem* p, uint32_t init_mode, const ui
                 if ((rc = ensure_scratch(p, (size_t)p->W32 * 4, st))) return rc;
                 if ((rc = launch_static_first_row(p, static_cast<uint32_t*>(p->d_scratch), st))) return rc;
             }
-            if ((rc = launch_broadcast_row(row ? row : static_cast<uint32_t*>(p->d_scratch), p->S, p->W32, nullptr,
+            if ((rc = launch_broadcast_row(row ? row : static_cast<uint32_t*>(p->d_scratch), p->S, p->W32,
                                            schedules + (size_t)i * p->S * p->W32, st)))
                 return rc;
             continue;
