@@ -868,7 +868,7 @@ int prepare(kvp_problem* p, const kvp_anneal_params* a, cudaStream_t st, Ctx& c,
                 cudaMemPoolGetAttribute(pool, cudaMemPoolAttrUsedMemCurrent, &used) == cudaSuccess && reserved > used)
                 have += (size_t)(reserved - used);
         }
-        if (have / 10 * 7 < r * col_bytes) {
+        if (p->chain_ws_bytes < r * col_bytes && have / 10 * 9 < r * col_bytes) {
             size_t free_b = 0, total_b = 0;
             KVP_CUDA(cudaMemGetInfo(&free_b, &total_b));
             const size_t fit = (have + free_b) / 10 * 7 / col_bytes;
