@@ -3,7 +3,7 @@
 // Two forms. Small schedules, where launches and latency are all there is: score_kernel, one CTA per schedule, groups of
 // lanes own whole rows, everything in one launch. Large ones, HBM-bound: count_wide_kernel, in which a warp owns 64
 // consecutive 16-byte vectors of every row of a step chunk, carries P[s-1] in registers (every word of A and P is read once)
-// and adds its per-step counts to global counters; the last CTA of a schedule turns them into ticks.
+// and adds its per-step counts to global counters; the last CTA of a schedule, or a second launch, turns them into ticks.
 #include <string.h>
 
 #include <algorithm>
@@ -109,6 +109,17 @@ __device__ __forceinline__ void score_total(const ScoreOut& o, uint32_t i, Score
     __syncthreads();
 }
 
+// schedule i from its counts in global memory, by a CTA
+template <bool GROW>
+__device__ __forceinline__ void score_counts(const ScoreOut& o, uint32_t i, uint32_t S, const uint32_t* counts, const uint32_t* hbc)
+{
+    ScoreSum sum;
+    for (uint32_t s = threadIdx.x; s < S; s += blockDim.x)
+        score_step<GROW>(o, i, S, s, __ldcg(reinterpret_cast<const uint4*>(counts) + (size_t)i * S + s),
+                         GROW ? __ldcg(hbc + (size_t)i * S + s) : 0u, sum);
+    score_total(o, i, sum);
+}
+
 constexpr int WIDE_WARPS = 8;
 constexpr int WIDE_VEC = 2;              // 16-byte vectors per lane and row
 
@@ -142,7 +153,9 @@ __device__ __forceinline__ uint32_t popc8(const uint32_t (&w)[8])
 // hb: they were written there, not migrated, so mi = occ - stay - hb.
 // NS schedules of a batch share a thread: the access words are loaded once and used for all of them, which halves
 // the L2 traffic of a batch (A is the half of the bytes that comes from L2, not DRAM).
-template <int VEC, bool GROW, int NS>
+// LAST: the last CTA of a group of schedules scores them. (Two kernels: with the scoring behind a test of a parameter the
+// loads of the loop are scheduled worse, 419 against 346 us on 96 schedules of 640 x 4096 units x 64 steps.)
+template <int VEC, bool GROW, int NS, bool LAST>
 __global__ void __launch_bounds__(WIDE_WARPS * 32)
 count_wide_kernel(const uint32_t* __restrict__ A, const uint32_t* __restrict__ Ps, uint32_t S, uint32_t W32,
                   uint32_t WV, uint32_t pad_mask, uint32_t SC, uint32_t n, uint32_t* __restrict__ counts,
@@ -252,8 +265,7 @@ count_wide_kernel(const uint32_t* __restrict__ A, const uint32_t* __restrict__ P
             }
         }
     }
-    if (!tickets) return;
-    // the last CTA of these schedules scores them
+    if (!LAST) return;
     __shared__ uint32_t s_last;
     __threadfence();
     __syncthreads();
@@ -262,13 +274,15 @@ count_wide_kernel(const uint32_t* __restrict__ A, const uint32_t* __restrict__ P
     if (!s_last) return;
     __threadfence();
 #pragma unroll 1
-    for (uint32_t i = blockIdx.z * NS; i < min(n, (blockIdx.z + 1) * NS); ++i) {
-        ScoreSum sum;
-        for (uint32_t s = threadIdx.x; s < S; s += blockDim.x)
-            score_step<GROW>(out, i, S, s, __ldcg(reinterpret_cast<const uint4*>(counts) + (size_t)i * S + s),
-                             GROW ? __ldcg(hbc + (size_t)i * S + s) : 0u, sum);
-        score_total(out, i, sum);
-    }
+    for (uint32_t i = blockIdx.z * NS; i < min(n, (blockIdx.z + 1) * NS); ++i) score_counts<GROW>(out, i, S, counts, hbc);
+}
+
+// Large batches: the counts of schedule i by CTA i, in a launch of its own.
+template <bool GROW>
+__global__ void __launch_bounds__(256)
+score_counts_kernel(const uint32_t* __restrict__ counts, const uint32_t* __restrict__ hbc, uint32_t S, const ScoreOut out)
+{
+    score_counts<GROW>(out, blockIdx.x, S, counts, hbc);
 }
 
 // Small schedules: CTA i scores schedule i. LPR lanes own a row (a power of two; more than 32 vectors: the lanes go round),
@@ -374,9 +388,14 @@ static int launch_score_impl(const kvp_problem* p, const uint32_t* schedules, ui
     dim3 grid(col_ctas, (p->S + SC - 1) / SC, nz);
     const size_t smem = (size_t)NS * WIDE_WARPS * SC * (sizeof(uint2) + (grow ? 4 : 0));
     const int T = WIDE_WARPS * 32;
-#define KVP_WIDE(VEC, GROW, NSCH)                                                                                  \
-    count_wide_kernel<VEC, GROW, NSCH><<<grid, T, smem, st>>>(p->dA, schedules, p->S, p->W32, WV, p->pad_mask, SC, n, \
-                                                              counts, GROW ? p->dL : nullptr, GROW ? hbc : nullptr, tickets, out)
+    // A CTA that takes a ticket waits until its counts have arrived, one or two microseconds. Up to one wave of CTAs that is
+    // less than another launch; a large batch pays it in every wave (256 schedules of 65,536 units x 256 steps: 136 us with
+    // tickets, 116 with the second launch).
+    const bool apart = tickets && (uint64_t)grid.x * grid.y * grid.z > 148u * 8u;
+    if (apart) tickets = nullptr;
+#define KVP_WIDE(VEC, GROW, NSCH)                                                                                         \
+    (tickets ? count_wide_kernel<VEC, GROW, NSCH, true> : count_wide_kernel<VEC, GROW, NSCH, false>)<<<grid, T, smem, st>>>( \
+        p->dA, schedules, p->S, p->W32, WV, p->pad_mask, SC, n, counts, GROW ? p->dL : nullptr, GROW ? hbc : nullptr, tickets, out)
     if (NS == 2) {
         if (grow) { if (vec4) KVP_WIDE(4, true, 2); else KVP_WIDE(1, true, 2); }
         else { if (vec4) KVP_WIDE(4, false, 2); else KVP_WIDE(1, false, 2); }
@@ -386,6 +405,12 @@ static int launch_score_impl(const kvp_problem* p, const uint32_t* schedules, ui
     }
 #undef KVP_WIDE
     KVP_CUDA(cudaGetLastError());
+    if (apart) {
+        if (grow) score_counts_kernel<true><<<n, 256, 0, st>>>(counts, hbc, p->S, out);
+        else score_counts_kernel<false><<<n, 256, 0, st>>>(counts, hbc, p->S, out);
+        KVP_CUDA(cudaGetLastError());
+        if (launches) *launches += 1;
+    }
     return KVP_OK;
 }
 
