@@ -1,18 +1,18 @@
-// Annealing kernels. Two of them, chosen per job (see prepare()): the narrow chain kernel described here (one or two
-// warps per chain, batches of 32 proposals, every one evaluated in full) and the wide one in kvp_chain.cuh (one to four
-// warps per chain, batches of 128 or 256, most proposals settled by their placement bits or a bound alone).
+// Annealing: the host side, calibration, reduction and the winner's way back. The chains run on one of two kernels, chosen
+// per job (see prepare()): the narrow one in kvp_narrow.cuh (one to four warps per chain, 32 proposals prepared at a time
+// and evaluated in move order) and the wide one in kvp_chain.cuh (one to four warps per chain, batches of 128 or 256
+// proposals, most of them settled by their placement bits or by a lower bound of the cost change).
 //
 // State of a chain: the schedule in time-packed form (for every unit a bit string over the steps), either
-// in shared memory (small problems) or in a private slice of global scratch (a plain copy of the initial schedule,
-// or a copy-on-write overlay of the one all chains share), plus the four per-step cardinalities {hr, mi, mo, occ}
-// in shared memory and the running total T.
+// in shared memory (small problems) or in a private slice of global scratch (a copy-on-write overlay of the initial
+// schedule all chains share), and in shared memory per step the two sides {th, te} of Eq. 2 and the occupancy, the
+// bitmaps of full steps and of steps where te leads, and the running total T.
 //
 // A proposal (one Philox4x32-10 block, a pure function of seed, chain and move index) names a run of at most
-// 30 consecutive steps and one or two units. Only the run's steps and the step after it change cost. Proposals
-// are drawn and evaluated 32 at a time, one per lane, against the state the batch starts from; the (proposal,
-// step) pairs whose cost changes go through a work queue shared by the warp; the warp then commits the batch in
-// move order with a Metropolis test against the quantised exp(-delta/C) table, evaluating again only what an
-// applied move could have touched. With two warps per chain the warps take the batches in turn (see ChainShare).
+// 30 consecutive steps and one or two units. Only the run's steps and the step after it change cost. Both kernels leave
+// the sequential chain's results: moves are committed in move order with a Metropolis test against the quantised
+// exp(-delta/C) table, and what an applied move could have touched is evaluated again. Several warps of a chain take its
+// batches in turn (see ChainShared).
 #include <math.h>
 #include <stdlib.h>
 #include <string.h>
@@ -904,8 +904,7 @@ int prepare(kvp_problem* p, const kvp_anneal_params* a, cudaStream_t st, Ctx& c,
     // the winner can be walked back instead of replayed from its first move.
     c.undo_cap = c.psmem ? 0u : 4096u;
     const size_t o_ulog = take((size_t)c.resident * c.undo_cap * 8), o_ulen = take(c.psmem ? 0 : (size_t)c.resident * 4);
-    // Where the chains come in several waves they also log the units they rewrite (4 bytes each, up to 16384): the
-    // chain that takes over the slice in the next wave copies only those from the initial schedule again, not all of it.
+    // Which buckets of its slice a chain has taken over, for the walk back of the winner.
     const bool cow = !c.psmem && c.cow_slots4 != 0;
     const size_t o_cow = take(cow ? (size_t)c.resident * c.cow_slots4 * 16 : 0);
     rc = ensure_chain_ws(p, off, st);

@@ -1,9 +1,10 @@
 // Cost kernels: per-step cardinalities of a schedule (popc over mask AND placement words) and Eq. 1-5.
 //
-// Two forms. Small schedules, where launches and latency are all there is: score_kernel, one CTA per schedule, groups of
+// Three forms. Small schedules, where launches and latency are all there is: score_kernel, one CTA per schedule, groups of
 // lanes own whole rows, everything in one launch. Large ones, HBM-bound: count_wide_kernel, in which a warp owns 64
 // consecutive 16-byte vectors of every row of a step chunk, carries P[s-1] in registers (every word of A and P is read once)
 // and adds its per-step counts to global counters; the last CTA of a schedule, or a second launch, turns them into ticks.
+// Large batches: count_staged_kernel, the same with rows fetched ahead into shared memory.
 #include <string.h>
 
 #include <algorithm>
@@ -277,6 +278,127 @@ count_wide_kernel(const uint32_t* __restrict__ A, const uint32_t* __restrict__ P
     for (uint32_t i = blockIdx.z * NS; i < min(n, (blockIdx.z + 1) * NS); ++i) score_counts<GROW>(out, i, S, counts, hbc);
 }
 
+// Large batches of rows of whole 16-byte vectors, no births: count_wide_kernel for pairs of schedules, with the rows of the
+// next steps on their way into shared memory by asynchronous copies. Every lane copies its own vectors into slots of its own,
+// so there is no barrier, and what is in flight takes no registers: the loads of the other kernel are as far ahead of their
+// use as the compiler's schedule happens to put them. Three CTAs per SM (72 KB of rows each, two of three stages in
+// flight). Bound by DRAM: 96 schedules of 640 x 4096 units x 64 steps 348 -> 326 us, 6.2 TB/s; the logic pipe is next (66%),
+// hence the cheaper population count, without which this form took 372 us.
+constexpr int kStages = 3;
+
+__device__ __forceinline__ void copy_async(uint4* to, const uint4* from)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"((uint32_t)__cvta_generic_to_shared(to)), "l"(from) : "memory");
+}
+
+// Number of set bits in eight words with four popc: seven of the words are added bit-position-wise into ones, twos and
+// fours; the eighth is counted as it is, which is cheaper than carrying it through (8 logic instructions, popc8 has 14).
+__device__ __forceinline__ uint32_t popc7_1(const uint32_t (&w)[8])
+{
+    uint32_t ones, other, twos, fours, ta, tb, tc;
+    csa(ta, ones, w[0], w[1], w[2]);
+    csa(tb, other, w[3], w[4], w[5]);
+    csa(tc, ones, ones, other, w[6]);
+    csa(fours, twos, ta, tb, tc);
+    return __popc(ones) + __popc(w[7]) + 2 * __popc(twos) + 4 * __popc(fours);
+}
+
+__global__ void __launch_bounds__(WIDE_WARPS * 32, 3)
+count_staged_kernel(const uint32_t* __restrict__ A, const uint32_t* __restrict__ Ps, uint32_t S, uint32_t W32, uint32_t WV,
+                    uint32_t pad_mask, uint32_t SC, uint32_t n, uint32_t* __restrict__ counts)
+{
+    constexpr int NS = 2, kRows = (1 + NS) * WIDE_VEC;
+    extern __shared__ uint4 smem4[];
+    const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    uint4* const ring = smem4 + (size_t)warp * (kStages * kRows * 32) + lane;    // slot (stage, row, vector) of this lane: stride 32
+    uint2* const acc = reinterpret_cast<uint2*>(smem4 + WIDE_WARPS * kStages * kRows * 32);   // [NS][WIDE_WARPS][SC]
+    const uint32_t cv0 = (blockIdx.x * WIDE_WARPS + warp) * (32 * WIDE_VEC) + lane;
+    const uint32_t sb = blockIdx.y * SC, se = min(S, sb + SC);
+    const uint32_t* __restrict__ P[NS];
+#pragma unroll
+    for (int q = 0; q < NS; ++q)                         // a schedule past the batch re-reads the last one; its counts are dropped
+        P[q] = Ps + (size_t)min(blockIdx.z * NS + q, n - 1) * S * W32;
+    const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
+    for (int i = 0; i < kStages * kRows; ++i) ring[i * 32] = zero;               // vectors beyond the row stay zero
+    auto fetch = [&](uint32_t s, uint32_t stage) {
+        if (s < se) {
+#pragma unroll
+            for (int j = 0; j < WIDE_VEC; ++j) {
+                const uint32_t cv = cv0 + 32 * j;
+                if (cv >= WV) continue;
+                copy_async(ring + (stage * kRows + j) * 32, reinterpret_cast<const uint4*>(A + (size_t)s * W32) + cv);
+#pragma unroll
+                for (int q = 0; q < NS; ++q)
+                    copy_async(ring + (stage * kRows + (1 + q) * WIDE_VEC + j) * 32, reinterpret_cast<const uint4*>(P[q] + (size_t)s * W32) + cv);
+            }
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+#pragma unroll
+    for (int k = 0; k + 1 < kStages; ++k) fetch(sb + k, k);
+    uint4 prev[NS][WIDE_VEC];
+    uint32_t occ_prev[NS];
+#pragma unroll
+    for (int q = 0; q < NS; ++q) {
+        uint32_t w[8];
+#pragma unroll
+        for (int j = 0; j < WIDE_VEC; ++j) {
+            const uint32_t cv = cv0 + 32 * j;
+            prev[q][j] = cv < WV ? mask_last<4>(load_vec<4>(P[q], W32, sb ? sb - 1 : 0, cv), cv, WV, pad_mask) : zero;
+            w[4 * j] = prev[q][j].x; w[4 * j + 1] = prev[q][j].y; w[4 * j + 2] = prev[q][j].z; w[4 * j + 3] = prev[q][j].w;
+        }
+        occ_prev[q] = popc7_1(w);
+    }
+    uint32_t stage = 0;
+#pragma unroll 1
+    for (uint32_t s = sb; s < se; ++s) {
+        fetch(s + kStages - 1, stage ? stage - 1 : kStages - 1);   // into the slots read in the step before
+        asm volatile("cp.async.wait_group %0;" :: "n"(kStages - 1) : "memory");
+        uint4 a[WIDE_VEC];
+#pragma unroll
+        for (int j = 0; j < WIDE_VEC; ++j) a[j] = ring[(stage * kRows + j) * 32];
+#pragma unroll
+        for (int q = 0; q < NS; ++q) {
+            uint32_t wp[8], wh[8], ws[8];
+#pragma unroll
+            for (int j = 0; j < WIDE_VEC; ++j) {
+                const uint4 pj = mask_last<4>(ring[(stage * kRows + (1 + q) * WIDE_VEC + j) * 32], cv0 + 32 * j, WV, pad_mask);
+                const uint4 hj = and4(a[j], pj), sj = and4(pj, prev[q][j]);
+                wp[4 * j] = pj.x; wp[4 * j + 1] = pj.y; wp[4 * j + 2] = pj.z; wp[4 * j + 3] = pj.w;
+                wh[4 * j] = hj.x; wh[4 * j + 1] = hj.y; wh[4 * j + 2] = hj.z; wh[4 * j + 3] = hj.w;
+                ws[4 * j] = sj.x; ws[4 * j + 1] = sj.y; ws[4 * j + 2] = sj.z; ws[4 * j + 3] = sj.w;
+                prev[q][j] = pj;
+            }
+            const uint32_t occ = popc7_1(wp), hr = popc7_1(wh), stay = popc7_1(ws);
+            uint2 c = make_uint2(hr | ((occ - stay) << 16), (occ_prev[q] - stay) | (occ << 16));
+            occ_prev[q] = occ;
+            c.x = __reduce_add_sync(0xFFFFFFFFu, c.x);   // 16-bit fields: 32 lanes * 256 < 65536
+            c.y = __reduce_add_sync(0xFFFFFFFFu, c.y);
+            if (lane == 0) acc[(q * WIDE_WARPS + warp) * SC + (s - sb)] = c;
+        }
+        stage = stage + 1 < kStages ? stage + 1 : 0;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < NS; ++q) {
+        const uint32_t sched = blockIdx.z * NS + q;
+        if (sched >= n) break;
+        for (uint32_t i = threadIdx.x; i < se - sb; i += blockDim.x) {
+            uint32_t hr = 0, mi = 0, mo = 0, occ = 0;
+#pragma unroll
+            for (int w = 0; w < WIDE_WARPS; ++w) {
+                const uint2 c = acc[(q * WIDE_WARPS + w) * SC + i];
+                hr += c.x & 0xFFFFu; mi += c.x >> 16; mo += c.y & 0xFFFFu; occ += c.y >> 16;
+            }
+            uint32_t* dst = counts + ((size_t)sched * S + sb + i) * 4;
+            if (hr) atomicAdd(dst + 0, hr);
+            if (mi) atomicAdd(dst + 1, mi);
+            if (mo) atomicAdd(dst + 2, mo);
+            if (occ) atomicAdd(dst + 3, occ);
+        }
+    }
+}
+
 // Large batches: the counts of schedule i by CTA i, in a launch of its own.
 template <bool GROW>
 __global__ void __launch_bounds__(256)
@@ -381,6 +503,10 @@ static int launch_score_impl(const kvp_problem* p, const uint32_t* schedules, ui
     // partial wave costs little; every chunk re-reads one halo row (1/SC more traffic, mostly from L2).
     uint32_t SC = p->S;
     while (SC > 8 && (uint64_t)col_ctas * ((p->S + SC - 1) / SC) * nz < 148u * 8u * 4u) SC = (SC + 1) / 2;
+    // Pairs of schedules with rows of whole vectors can take count_staged_kernel, whose three CTAs per SM leave 3 KB each for
+    // the accumulators.
+    const bool pairs = NS == 2 && !grow && vec4;
+    if (pairs && SC > 24) SC = 24;
     // the per-step accumulators of a chunk live in dynamic shared memory: keep them within the 48 KB a kernel gets
     // without opting in (NS * WIDE_WARPS * SC entries of 8 bytes, 12 with births)
     const uint32_t sc_max = (uint32_t)((47u * 1024u) / (NS * WIDE_WARPS * (sizeof(uint2) + (grow ? 4 : 0))));
@@ -396,7 +522,11 @@ static int launch_score_impl(const kvp_problem* p, const uint32_t* schedules, ui
 #define KVP_WIDE(VEC, GROW, NSCH)                                                                                         \
     (tickets ? count_wide_kernel<VEC, GROW, NSCH, true> : count_wide_kernel<VEC, GROW, NSCH, false>)<<<grid, T, smem, st>>>( \
         p->dA, schedules, p->S, p->W32, WV, p->pad_mask, SC, n, counts, GROW ? p->dL : nullptr, GROW ? hbc : nullptr, tickets, out)
-    if (NS == 2) {
+    if (pairs && !tickets) {
+        const size_t bytes = smem + (size_t)WIDE_WARPS * kStages * (1 + 2) * WIDE_VEC * 32 * sizeof(uint4);
+        KVP_CUDA(cudaFuncSetAttribute(count_staged_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 80 << 10));
+        count_staged_kernel<<<grid, T, bytes, st>>>(p->dA, schedules, p->S, p->W32, WV, p->pad_mask, SC, n, counts);
+    } else if (NS == 2) {
         if (grow) { if (vec4) KVP_WIDE(4, true, 2); else KVP_WIDE(1, true, 2); }
         else { if (vec4) KVP_WIDE(4, false, 2); else KVP_WIDE(1, false, 2); }
     } else {
