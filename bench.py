@@ -30,32 +30,40 @@ if ROOT not in sys.path:
 WORKLOAD = "long_70b"
 METRIC = "sa_move_evals_per_sec"
 UNIT = "move-evals/s"
-# Issue-slot roofline of the chain kernel: 148 SMs x 4 warp schedulers x 1.965 GHz, one warp instruction per
-# scheduler and cycle. Algorithmic work per move evaluation: 16 warp instructions (per 32 moves: Philox and decode
-# ~105, window extraction and word-parallel bit logic ~100, work-queue scan and push ~100, about 35 (lane, step)
-# cost evaluations of ~70 thread instructions each in two warp rounds ~150, Metropolis and in-order commit ~50).
+# Issue-slot roofline of the chain kernels: 148 SMs x 4 warp schedulers x 1.965 GHz, one warp instruction per scheduler
+# and cycle.
 ISSUE_PEAK_GWIPS = 148 * 4 * 1.965
-ALG_WARP_INSTR_PER_MOVE = 16.0          # the narrow chain kernel: every proposal is evaluated in full
-# The wide chain kernel settles most proposals by their placement bits alone, so its algorithmic work depends on the
-# workload; the kernel counts what its evaluations amounted to (kvp_anneal_stats) and the numerator is, in warp
+# Work per move of a formulation that evaluates every proposal in full (Philox and decoding, windows and bit logic, Eq. 2-4
+# at every step that changes, commit), in warp instructions; only the yardstick of frac_against_16_per_move.
+ALG_FULL_EVALUATION = 16.0
+# The narrow chain kernel: what every proposal needs, thread instructions / 32: Philox and decoding 63, four windows 40,
+# masks of hits and migration edges 40, lower bound (14 popcounts, sums and products) 38, largest accepted change 10, record
+# 8. The evaluations of the proposals that are left (a lane per step) and the applied moves are not counted.
+ALG_WARP_INSTR_PER_MOVE = 199 / 32
+# The wide chain kernel settles most proposals by their placement bits or by a lower bound, so its algorithmic work depends
+# on the workload; the kernel counts what its evaluations amounted to (kvp_anneal_stats) and the numerator is, in warp
 # instructions (thread instructions / 32 of the formulation, counted by hand from the steps it needs):
 #   per move          2.06 : Philox4x32-10 (10 rounds of 2 wide multiplies and 2 three-input XORs) 40, counter 3,
 #                            decoding of swap / run length / first step / two units 18, its share of the commit vote 2
 #   per evaluation    1.65 : unpacking 4, run mask 5, window position 5, two placement columns (overlay lookup, address,
 #                            load, funnel shift) 22, toggled bits, Eq. 5 test, verdict bits 13, listing 4
-#   per listed one    1.47 : slot 2, two access columns 10, windows after the move 6, the steps whose cardinalities
-#                            change 18, window store 2, room in the queue 3, sum and Metropolis test 6
-#   per (proposal, step) item 1.45 : queue 3, windows, counters, constants, present cost 5 loads, bit extraction 10,
-#                            new cardinalities 12, Eq. 2-4 once 13, difference and accumulation 3
+#   per listed one    2.25 : slot 2, two access columns 10, windows after the move 6, masks of hits and migration edges 18,
+#                            lower bound of the cost change (window of the leading side 2, 14 popcounts, 14 sums and
+#                            products, its limit 6)
+#   per (proposal, step) item of those not rejected by the bound 0.75 : bit extraction 10, th and te 1 load, their change
+#                            6, maxima and difference 4, its share of the sum 3
 # evaluations = moves + proposals evaluated again after an applied move.
-ALG_WIDE = {"move": 2.06, "evaluation": 1.65, "listed": 1.47, "item": 1.45}
+ALG_WIDE = {"move": 2.06, "evaluation": 1.65, "listed": 2.25, "item": 0.75}
+
+
+def wide_alg(st):
+    """Warp instructions per move of the wide chain kernel, from the counts of kvp_anneal_stats."""
+    moves = float(st.moves_total)
+    return (ALG_WIDE["move"] * moves + ALG_WIDE["evaluation"] * (moves + st.work_again) + ALG_WIDE["listed"] * st.work_listed +
+            ALG_WIDE["item"] * st.work_items) / moves
+
+
 PEAK_SOURCE_ALU = "148 SMs x 4 issue slots x 1.965 GHz (unit counts and clocks)"
-# DRAM bytes (read + written) of one chain-kernel launch, from a one-pass profiler capture of the very launches this
-# benchmark times (2048 chains x 1,000,000 moves of long_70b); not measured in the run that prints it, and labelled so.
-# To be taken again whenever the chain kernel or the copy-on-write layout changes.
-PROFILED_DRAM_BYTES_PER_LAUNCH = {("long_70b", 2048, 1_000_000): 15.68e9}
-PROFILED_NOTE = ("dram__bytes_read.sum + dram__bytes_write.sum of one launch (13.26 + 2.42 GB), one-pass ncu capture of "
-                 "the benchmark command; a profile figure, not measured in this run")
 FLUSH_NOTE = "flushed with a 256 MB write between timed iterations"
 
 
@@ -296,7 +304,7 @@ def cost_kernel_record(steps, warmup):
     alg_bytes = (n + 1) * S * W32 * 4
     peak, src = _hbm_peak()
     achieved = alg_bytes / (ms * 1e-3) / 1e9
-    return {"kernel": "count_wide_kernel+finish_kernel (kvp_eval)", "metric": "schedules_scored_per_sec",
+    return {"kernel": "count_wide_kernel + score_counts_kernel (kvp_eval)", "metric": "schedules_scored_per_sec",
             "value": n / (ms * 1e-3), "unit": "schedules/s", "ms_per_call": ms, "steps": steps,
             "config": {"workload": name, "batch": n, "words_per_row": W32, "rows": S, "l2": FLUSH_NOTE},
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
@@ -306,15 +314,15 @@ def cost_kernel_record(steps, warmup):
 # Algorithmic thread instructions of the trace kernels per (unit, step): one Philox4x32-10 for the noise (10 rounds
 # of two wide multiplies, four xors and two key additions: 60 with 3-input logic ops), the 8-term Irwin-Hall sum
 # and the AR(1) update 22, a second Philox and a compare for the burst draw 62 when bursts are on, and the top-k
-# search: the range reduction (2), three histogram passes of a prefix compare, a digit and a shared-memory add per
-# unit (12) and the selection compares (4): 18.
+# search: the lanes' largest keys (1), a compare, a digit and a predicated shared-memory add (5), membership of the
+# threshold's bin (2) and the selection compare, vote and select (3): 11.
 # Multiplier pipe: 148 SMs x 4 schedulers x 1.965 GHz, a warp-wide 32 x 32 -> 64 bit multiply every four cycles
 # (measured: ncu's pipe-busy cycles of the score pass divided by its multiply instructions) = 9.3e12 multiplies/s.
 WIDE_MUL_PEAK_T = 148 * 4 * 1.965e9 / 4 * 32 / 1e12
 
 
 def trace_alg_thread_instr(bursts):
-    return 60 + 22 + (62 if bursts else 0) + 18
+    return 60 + 22 + (62 if bursts else 0) + 11
 
 
 def trace_kernel_record(steps, warmup):
@@ -396,7 +404,8 @@ def run_growing(args):
         total_ms += e0.elapsed_time(e1)
         chain_ms += out["stats"].ms_chains
     ms, cms = total_ms / args.steps, chain_ms / args.steps
-    achieved = ALG_WARP_INSTR_PER_MOVE * chains * moves / (cms * 1e-3) / 1e9
+    st = out["stats"]
+    achieved = (wide_alg(st) if st.wide_kernel else ALG_WARP_INSTR_PER_MOVE) * chains * moves / (cms * 1e-3) / 1e9
     line = {"metric": METRIC, "value": chains * moves / (ms * 1e-3), "unit": UNIT, "ms_per_step": ms, "steps": args.steps,
             "config": {"workload": name, "units": U, "steps": S, "layers": cfg["layers"], "chains": chains, "moves": moves,
                        "p0": cfg["p0"], "l2": FLUSH_NOTE},
@@ -514,7 +523,7 @@ class PathBench:
             out["global_best"] = self.sharding.combine_best(dist, out["best_ticks"], out["stats"].best_chain, device="cuda")
         # kernels: 2 trace (scores, select) + 6 create (clean, popcount, transpose, unit counts, histogram,
         #          static row) + 2 eval (count, finish) + those kvp_anneal reports
-        self.launches = 2 + 6 + 2 + out["stats"].kernel_launches
+        self.launches = 2 + 5 + 1 + out["stats"].kernel_launches
         prob.close()
         return out
 
@@ -559,27 +568,23 @@ class PathBench:
         per_launch_ms = chain_ms / max(1, chain_launches)
         moves = float(st.moves_total)                        # of the last step; every step does the same number
         if st.wide_kernel:
-            alg = (ALG_WIDE["move"] * moves + ALG_WIDE["evaluation"] * (moves + st.work_again) +
-                   ALG_WIDE["listed"] * st.work_listed + ALG_WIDE["item"] * st.work_items) / moves
-            form = {"kernel_form": "wide (one warp per chain, four proposals per lane, placement bits first)",
+            alg = wide_alg(st)
+            form = {"kernel_form": "wide (batches of 128 or 256 proposals, settled by placement bits, then by a lower bound, the rest step by step)",
                     "work_per_move": {"evaluated_again": st.work_again / moves, "listed": st.work_listed / moves,
                                       "items": st.work_items / moves},
                     "frac_against_16_per_move": None}
         else:
             alg = ALG_WARP_INSTR_PER_MOVE
-            form = {"kernel_form": "narrow (one proposal per lane, every proposal evaluated in full)"}
+            form = {"kernel_form": "narrow (32 proposals prepared at a time, evaluated in move order where the bound does not reject them)"}
         moves_per_launch = moves * n_steps / max(1, chain_launches)
         achieved = alg * moves_per_launch / (per_launch_ms * 1e-3) / 1e9
         if st.wide_kernel:   # the same time against the work of the full-evaluation formulation, for comparison only
-            form["frac_against_16_per_move"] = (ALG_WARP_INSTR_PER_MOVE * moves_per_launch / (per_launch_ms * 1e-3) / 1e9 /
+            form["frac_against_16_per_move"] = (ALG_FULL_EVALUATION * moves_per_launch / (per_launch_ms * 1e-3) / 1e9 /
                                                 ISSUE_PEAK_GWIPS)
-        traffic = PROFILED_DRAM_BYTES_PER_LAUNCH.get((self.name, int(st.resident_chains), int(self.moves))) if st.wide_kernel else None
-        if traffic is not None:
-            form["traffic_source"] = PROFILED_NOTE
         return {"bound": "alu", "kernel": "chain kernel (%s)" % ("schedules in shared memory" if self.U * self.S <= (1 << 18)
                                                                   else "schedules in global memory"),
                 "achieved": achieved, "peak": ISSUE_PEAK_GWIPS, "unit": "Gwarp-inst/s", "frac": achieved / ISSUE_PEAK_GWIPS,
-                "traffic": traffic, "ms_per_launch": per_launch_ms, "launches_per_step": chain_launches / max(1, n_steps),
+                "traffic": None, "ms_per_launch": per_launch_ms, "launches_per_step": chain_launches / max(1, n_steps),
                 "chains_per_launch": int(st.resident_chains), "algorithmic_warp_instr_per_move": alg,
                 "peak_source": PEAK_SOURCE_ALU, **form}
 
