@@ -56,6 +56,13 @@ bool stream_of(PyObject* o, int device, void** st)
     return !PyErr_Occurred();
 }
 
+// Other Python threads run meanwhile: a call into the library launches, may allocate, and waits when the stream's launch
+// queue is full. (Arguments stay alive: the caller's frame holds them.)
+struct Unlocked {
+    PyThreadState* state = PyEval_SaveThread();
+    ~Unlocked() { PyEval_RestoreThread(state); }
+};
+
 at::Tensor make(at::IntArrayRef size, at::ScalarType dtype, c10::Device dev) { return at::detail::empty_cuda(size, dtype, dev, std::nullopt); }
 
 PyObject* k_step_ticks; PyObject* k_total_ticks; PyObject* k_step_seconds; PyObject* k_total_seconds; PyObject* k_bad_step;
@@ -85,14 +92,18 @@ PyObject* eval(PyObject*, PyObject* const* args, Py_ssize_t nargs)
     try {
         at::Tensor a, b, c, d, e;
         const int64_t rows[2] = {(int64_t)n, (int64_t)S}, one[1] = {(int64_t)n};
-        if (steps) a = make(rows, at::kLong, dev);
-        b = make(one, at::kLong, dev);
-        if (steps && seconds) c = make(rows, at::kDouble, dev);
-        if (seconds) d = make(one, at::kDouble, dev);
-        e = make(one, at::kInt, dev);
-        const int rc = kvp_eval(p, static_cast<uint32_t*>(sched), n, steps ? static_cast<uint64_t*>(a.data_ptr()) : nullptr,
-                                static_cast<uint64_t*>(b.data_ptr()), c.defined() ? static_cast<double*>(c.data_ptr()) : nullptr,
-                                seconds ? static_cast<double*>(d.data_ptr()) : nullptr, static_cast<int32_t*>(e.data_ptr()), st);
+        int rc;
+        {
+            Unlocked unlocked;
+            if (steps) a = make(rows, at::kLong, dev);
+            b = make(one, at::kLong, dev);
+            if (steps && seconds) c = make(rows, at::kDouble, dev);
+            if (seconds) d = make(one, at::kDouble, dev);
+            e = make(one, at::kInt, dev);
+            rc = kvp_eval(p, static_cast<uint32_t*>(sched), n, steps ? static_cast<uint64_t*>(a.data_ptr()) : nullptr,
+                          static_cast<uint64_t*>(b.data_ptr()), c.defined() ? static_cast<double*>(c.data_ptr()) : nullptr,
+                          seconds ? static_cast<double*>(d.data_ptr()) : nullptr, static_cast<int32_t*>(e.data_ptr()), st);
+        }
         if (rc) return PyLong_FromLong(rc);
         PyObject* out = PyDict_New();
         if (!out || !put(out, k_step_ticks, a) || !put(out, k_total_ticks, b) || !put(out, k_step_seconds, c) ||
@@ -120,8 +131,13 @@ PyObject* eval_noalloc(PyObject*, PyObject* const* args, Py_ssize_t nargs)
     for (int i = 0; i < 5; ++i)
         if (!device_ptr(args[4 + i], at::kInt, false, &o[i])) return nullptr;
     if (!stream_of(args[9], THPVariable_Unpack(args[3]).device().index(), &st)) return nullptr;
-    return PyLong_FromLong(kvp_eval_noalloc(p, static_cast<uint32_t*>(sched), n, static_cast<uint64_t*>(o[0]), static_cast<uint64_t*>(o[1]),
-                                            static_cast<double*>(o[2]), static_cast<double*>(o[3]), static_cast<int32_t*>(o[4]), st));
+    int rc;
+    {
+        Unlocked unlocked;
+        rc = kvp_eval_noalloc(p, static_cast<uint32_t*>(sched), n, static_cast<uint64_t*>(o[0]), static_cast<uint64_t*>(o[1]),
+                              static_cast<double*>(o[2]), static_cast<double*>(o[3]), static_cast<int32_t*>(o[4]), st);
+    }
+    return PyLong_FromLong(rc);
 }
 
 // eval_counts(problem, steps, w32, schedules, stream or None) -> tensor, or an error code
@@ -137,8 +153,13 @@ PyObject* eval_counts(PyObject*, PyObject* const* args, Py_ssize_t nargs)
     if (!stream_of(args[4], dev.index(), &st)) return nullptr;
     try {
         const int64_t shape[3] = {(int64_t)n, (int64_t)S, 4};
-        const at::Tensor t = make(shape, at::kInt, dev);
-        const int rc = kvp_eval_counts(p, static_cast<uint32_t*>(sched), n, static_cast<uint32_t*>(t.data_ptr()), st);
+        at::Tensor t;
+        int rc;
+        {
+            Unlocked unlocked;
+            t = make(shape, at::kInt, dev);
+            rc = kvp_eval_counts(p, static_cast<uint32_t*>(sched), n, static_cast<uint32_t*>(t.data_ptr()), st);
+        }
         return rc ? PyLong_FromLong(rc) : THPVariable_Wrap(t);
     } catch (const std::exception& x) {
         PyErr_SetString(PyExc_RuntimeError, x.what());
