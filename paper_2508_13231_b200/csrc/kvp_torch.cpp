@@ -1,12 +1,15 @@
 // Native side of the Python binding for calls so short that Python's own work would be most of them: scoring a schedule is
 // 4 us of host time in the library, and took 25 with output tensors, stream and arguments handled in Python (2.4 us for
 // each of five torch.empty, 3.2 for the current stream). Argument handling only; the work is libkvp.so's.
+// Every function turns what torch throws into the Python exception torch itself raises for it (out of memory, no device, a
+// tensor without storage): nothing may be thrown through the interpreter, which would end the process.
 #define PY_SSIZE_T_CLEAN
 #include <Python.h>
 
 #include <ATen/core/Tensor.h>
 #include <ATen/cuda/EmptyTensor.h>
 #include <c10/cuda/CUDAStream.h>
+#include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
 
 #include "../../include/kvp.h"
@@ -80,6 +83,7 @@ bool put(PyObject* dict, PyObject* key, const at::Tensor& t)
 // eval(problem, steps, w32, schedules, want_steps, want_seconds, stream or None) -> dict of tensors, or an error code
 PyObject* eval(PyObject*, PyObject* const* args, Py_ssize_t nargs)
 {
+    HANDLE_TH_ERRORS
     if (nargs != 7) return value_error("eval takes 7 arguments");
     kvp_problem* p;
     unsigned long long S, w32;
@@ -89,39 +93,36 @@ PyObject* eval(PyObject*, PyObject* const* args, Py_ssize_t nargs)
     const bool steps = PyObject_IsTrue(args[4]), seconds = PyObject_IsTrue(args[5]);
     const c10::Device dev = THPVariable_Unpack(args[3]).device();
     if (!stream_of(args[6], dev.index(), &st)) return nullptr;
-    try {
-        at::Tensor a, b, c, d, e;
-        const int64_t rows[2] = {(int64_t)n, (int64_t)S}, one[1] = {(int64_t)n};
-        int rc;
-        {
-            Unlocked unlocked;
-            if (steps) a = make(rows, at::kLong, dev);
-            b = make(one, at::kLong, dev);
-            if (steps && seconds) c = make(rows, at::kDouble, dev);
-            if (seconds) d = make(one, at::kDouble, dev);
-            e = make(one, at::kInt, dev);
-            rc = kvp_eval(p, static_cast<uint32_t*>(sched), n, steps ? static_cast<uint64_t*>(a.data_ptr()) : nullptr,
-                          static_cast<uint64_t*>(b.data_ptr()), c.defined() ? static_cast<double*>(c.data_ptr()) : nullptr,
-                          seconds ? static_cast<double*>(d.data_ptr()) : nullptr, static_cast<int32_t*>(e.data_ptr()), st);
-        }
-        if (rc) return PyLong_FromLong(rc);
-        PyObject* out = PyDict_New();
-        if (!out || !put(out, k_step_ticks, a) || !put(out, k_total_ticks, b) || !put(out, k_step_seconds, c) ||
-            !put(out, k_total_seconds, d) || !put(out, k_bad_step, e)) {
-            Py_XDECREF(out);
-            return nullptr;
-        }
-        return out;
-    } catch (const std::exception& x) {
-        PyErr_SetString(PyExc_RuntimeError, x.what());
+    at::Tensor a, b, c, d, e;
+    const int64_t rows[2] = {(int64_t)n, (int64_t)S}, one[1] = {(int64_t)n};
+    int rc;
+    {
+        Unlocked unlocked;
+        if (steps) a = make(rows, at::kLong, dev);
+        b = make(one, at::kLong, dev);
+        if (steps && seconds) c = make(rows, at::kDouble, dev);
+        if (seconds) d = make(one, at::kDouble, dev);
+        e = make(one, at::kInt, dev);
+        rc = kvp_eval(p, static_cast<uint32_t*>(sched), n, steps ? static_cast<uint64_t*>(a.data_ptr()) : nullptr,
+                      static_cast<uint64_t*>(b.data_ptr()), c.defined() ? static_cast<double*>(c.data_ptr()) : nullptr,
+                      seconds ? static_cast<double*>(d.data_ptr()) : nullptr, static_cast<int32_t*>(e.data_ptr()), st);
+    }
+    if (rc) return PyLong_FromLong(rc);
+    PyObject* out = PyDict_New();
+    if (!out || !put(out, k_step_ticks, a) || !put(out, k_total_ticks, b) || !put(out, k_step_seconds, c) ||
+        !put(out, k_total_seconds, d) || !put(out, k_bad_step, e)) {
+        Py_XDECREF(out);
         return nullptr;
     }
+    return out;
+    END_HANDLE_TH_ERRORS
 }
 
 // eval_noalloc(problem, steps, w32, schedules, step_ticks, total_ticks, step_seconds, total_seconds, bad_step, stream or
 // None) -> error code
 PyObject* eval_noalloc(PyObject*, PyObject* const* args, Py_ssize_t nargs)
 {
+    HANDLE_TH_ERRORS
     if (nargs != 10) return value_error("eval_noalloc takes 10 arguments");
     kvp_problem* p;
     unsigned long long S, w32;
@@ -138,11 +139,13 @@ PyObject* eval_noalloc(PyObject*, PyObject* const* args, Py_ssize_t nargs)
                               static_cast<double*>(o[2]), static_cast<double*>(o[3]), static_cast<int32_t*>(o[4]), st);
     }
     return PyLong_FromLong(rc);
+    END_HANDLE_TH_ERRORS
 }
 
 // eval_counts(problem, steps, w32, schedules, stream or None) -> tensor, or an error code
 PyObject* eval_counts(PyObject*, PyObject* const* args, Py_ssize_t nargs)
 {
+    HANDLE_TH_ERRORS
     if (nargs != 5) return value_error("eval_counts takes 5 arguments");
     kvp_problem* p;
     unsigned long long S, w32;
@@ -151,24 +154,25 @@ PyObject* eval_counts(PyObject*, PyObject* const* args, Py_ssize_t nargs)
     if (!problem_of(args, &p, &S, &w32) || !batch_of(args[3], S * w32, &n) || !device_ptr(args[3], at::kInt, true, &sched)) return nullptr;
     const c10::Device dev = THPVariable_Unpack(args[3]).device();
     if (!stream_of(args[4], dev.index(), &st)) return nullptr;
-    try {
-        const int64_t shape[3] = {(int64_t)n, (int64_t)S, 4};
-        at::Tensor t;
-        int rc;
-        {
-            Unlocked unlocked;
-            t = make(shape, at::kInt, dev);
-            rc = kvp_eval_counts(p, static_cast<uint32_t*>(sched), n, static_cast<uint32_t*>(t.data_ptr()), st);
-        }
-        return rc ? PyLong_FromLong(rc) : THPVariable_Wrap(t);
-    } catch (const std::exception& x) {
-        PyErr_SetString(PyExc_RuntimeError, x.what());
-        return nullptr;
+    const int64_t shape[3] = {(int64_t)n, (int64_t)S, 4};
+    at::Tensor t;
+    int rc;
+    {
+        Unlocked unlocked;
+        t = make(shape, at::kInt, dev);
+        rc = kvp_eval_counts(p, static_cast<uint32_t*>(sched), n, static_cast<uint32_t*>(t.data_ptr()), st);
     }
+    return rc ? PyLong_FromLong(rc) : THPVariable_Wrap(t);
+    END_HANDLE_TH_ERRORS
 }
 
 // current_stream() -> the cudaStream_t of the current device's current stream
-PyObject* current_stream(PyObject*, PyObject*) { return PyLong_FromVoidPtr(c10::cuda::getCurrentCUDAStream().stream()); }
+PyObject* current_stream(PyObject*, PyObject*)
+{
+    HANDLE_TH_ERRORS
+    return PyLong_FromVoidPtr(c10::cuda::getCurrentCUDAStream().stream());
+    END_HANDLE_TH_ERRORS
+}
 
 PyMethodDef methods[] = {
     {"current_stream", current_stream, METH_NOARGS, nullptr},

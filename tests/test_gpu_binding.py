@@ -60,3 +60,23 @@ def test_other_threads_run_during_a_scoring_call(tmp_path):
     subprocess.check_call(["gcc", "-shared", "-fPIC", "-w", "-Wl,-soname,libkvp.so", str(src), "-o", str(lib)])
     out = subprocess.run([sys.executable, "-c", CALLS, str(lib), build.BINDING], capture_output=True, text=True, timeout=300, cwd=ROOT)
     assert out.returncode == 0 and out.stdout.split() == ["ok"] * 3, out.stdout + out.stderr
+
+
+def test_out_of_memory_is_torchs_exception():
+    """The outputs come from torch's allocator: when it has nothing left the call raises what torch.empty would."""
+    import torch
+
+    from paper_2508_13231_b200 import kvp
+    access = torch.randint(0, 2 ** 16, (32, 1), dtype=torch.int32, device="cuda")
+    prob = kvp.Problem(16, 8192, 32, access, 6, 8, 1, 1)
+    schedules = torch.zeros((1 << 17, 32, 1), dtype=torch.int32, device="cuda")    # 34 MB of ticks
+    torch.cuda.empty_cache()
+    torch.cuda.set_per_process_memory_fraction(1e-4)
+    try:
+        with pytest.raises(torch.OutOfMemoryError):
+            prob.eval(schedules)
+        with pytest.raises(torch.OutOfMemoryError):
+            prob.eval_counts(schedules)
+    finally:
+        torch.cuda.set_per_process_memory_fraction(1.0)
+    assert prob.eval(schedules)["total_ticks"].unique().numel() == 1
