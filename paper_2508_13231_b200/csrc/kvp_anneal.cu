@@ -38,7 +38,7 @@ struct ExchangeArgs {
 
 // Byte offsets of the parts of a chain's shared memory (see chain_layout).
 struct ChainLayout {
-    uint32_t occ, full, lead, hb, have, work;
+    uint32_t occ, full, lead, out, in, hb, have, work;
 };
 
 struct ChainParams {
@@ -606,12 +606,18 @@ int validate(const kvp_problem* p, const kvp_anneal_params* a)
 
 typedef void (*ChainKernel)(const ChainParams);
 
-ChainKernel narrow_kernel_for(bool psmem, bool asmem, uint32_t S32, bool solo)
+template <bool LIN>
+ChainKernel narrow_pick(bool psmem, bool asmem, uint32_t S32, bool solo)
 {
-    if (psmem && solo) return asmem ? narrow_chain_kernel<true, true, true, 0> : narrow_chain_kernel<true, true, false, 0>;
-    if (psmem) return asmem ? narrow_chain_kernel<false, true, true, 0> : narrow_chain_kernel<false, true, false, 0>;
-    return S32 == 2 ? narrow_chain_kernel<false, false, false, 2> : S32 == 4 ? narrow_chain_kernel<false, false, false, 4>
-                                                                             : narrow_chain_kernel<false, false, false, 0>;
+    if (psmem && solo) return asmem ? narrow_chain_kernel<true, true, true, LIN, 0> : narrow_chain_kernel<true, true, false, LIN, 0>;
+    if (psmem) return asmem ? narrow_chain_kernel<false, true, true, LIN, 0> : narrow_chain_kernel<false, true, false, LIN, 0>;
+    return S32 == 2 ? narrow_chain_kernel<false, false, false, LIN, 2> : S32 == 4 ? narrow_chain_kernel<false, false, false, LIN, 4>
+                                                                                  : narrow_chain_kernel<false, false, false, LIN, 0>;
+}
+
+ChainKernel narrow_kernel_for(bool psmem, bool asmem, bool lin, uint32_t S32, bool solo)
+{
+    return lin ? narrow_pick<true>(psmem, asmem, S32, solo) : narrow_pick<false>(psmem, asmem, S32, solo);
 }
 
 template <bool PSMEM, bool ASMEM, bool LIN, int COLV>
@@ -637,14 +643,14 @@ ChainKernel wide_kernel_for(bool psmem, bool asmem, bool grow, bool lin, uint32_
 ChainKernel kernel_of(const Ctx& c, bool psmem, bool asmem, uint32_t W)
 {
     return c.wide ? wide_kernel_for(psmem, asmem, c.grow, c.lin, c.S32, c.rows)
-                  : narrow_kernel_for(psmem, asmem, c.S32, c.solo);
+                  : narrow_kernel_for(psmem, asmem, c.lin, c.S32, c.solo);
 }
 
 int launch_chains(const Ctx& c, ChainParams& prm, uint32_t count)
 {
     {
         const bool rounds = prm.rung_hist != nullptr;
-        prm.lay = !c.wide ? narrow_layout(prm.S, prm.S32, c.psmem, c.psmem ? 0u : c.cow_slots4) : chain_layout(prm.S, prm.S32, c.grow, c.psmem, c.lin, c.psmem ? 0u : c.cow_slots4);
+        prm.lay = !c.wide ? narrow_layout(prm.S, prm.S32, c.psmem, c.lin, c.psmem ? 0u : c.cow_slots4) : chain_layout(prm.S, prm.S32, c.grow, c.psmem, c.lin, c.psmem ? 0u : c.cow_slots4);
         prm.seg_len = rounds ? prm.exch_every : prm.per_level;
         const uint32_t batch = c.wide ? 32u * c.rows : 32u;
         prm.seg_bat = (uint32_t)((prm.seg_len + batch - 1) / batch);
@@ -740,7 +746,7 @@ int prepare(kvp_problem* p, const kvp_anneal_params* a, cudaStream_t st, Ctx& c,
     c.asmem = false;
     auto fixed_bytes = [&](uint32_t warps, bool shared) {
         if (c.wide) return chain_bytes(p->S, p->S32, c.grow, shared, c.lin, shared ? 0u : c.cow_slots4, warps, c.rows);
-        return narrow_bytes(p->S, p->S32, shared, shared ? 0u : c.cow_slots4, warps);
+        return narrow_bytes(p->S, p->S32, shared, c.lin, shared ? 0u : c.cow_slots4, warps);
     };
     // Which kernel, and how many warps per chain (W; an SM holds 16). The lines are where the two cross over in measurements
     // on 1 to 640 groups, 16 to 2.6M units, 32 to 512 steps and 64 to 4096 chains of 8,000 to 200,000 moves.
@@ -775,7 +781,7 @@ int prepare(kvp_problem* p, const kvp_anneal_params* a, cudaStream_t st, Ctx& c,
         const bool ladders = c.psmem && rungs <= 16 && rungs * (fixed_bytes(1, true) + pbytes) + 16 <= budget;
         c.wide = !ladders || hooks.warps_per_chain == 3 || (hooks.warps_per_chain >= 16 && hooks.warps_per_chain < 32);
     }
-    if (!c.lin || c.grow) c.wide = true;                          // the narrow kernel does not serve these
+    if (c.grow) c.wide = true;                                    // the narrow kernel does not serve these
     if (c.wide) c.psmem = fixed_bytes(1, true) + pbytes + 16 <= budget / 2 && p->U < 65536u;
     const uint32_t forced = hooks.warps_per_chain == 3 ? 1u : hooks.warps_per_chain >= 16 ? hooks.warps_per_chain & 15u : hooks.warps_per_chain;
     const uint32_t full = 16;
@@ -994,7 +1000,7 @@ int prepare(kvp_problem* p, const kvp_anneal_params* a, cudaStream_t st, Ctx& c,
     float* const bounds = reinterpret_cast<float*>(shifts + a->levels);
     if ((rc = kvp_accept_table(c.temps.data(), a->levels, table, shifts))) return rc;
     // the lower bounds of kvp_chain.cuh are sums of at most 31 steps' changes in 32 bits
-    const uint64_t step_max = 4ull * std::max(p->K.khF, p->K.kdF) + std::max(p->K.kh, p->K.ke) + 2ull * std::max(p->K.kh, p->K.kd);
+    const uint64_t step_max = 4ull * std::max({p->K.khF, p->K.kdF, p->K.kkF}) + std::max(p->K.kh, p->K.ke) + 2ull * std::max(p->K.kh, p->K.kd);
     const bool bounded = 31 * step_max < (1ull << 30);
     for (uint32_t j = 0; j < a->levels; ++j) bounds[j] = bounded ? (float)((c.temps[j] >= 1.0 ? c.temps[j] : 1.0) * 0.69314718) : INFINITY;
     KVP_CUDA(cudaMemcpyAsync(c.table, table, table_bytes(a->levels), cudaMemcpyHostToDevice, st));

@@ -15,30 +15,35 @@
 // The kernel before evaluated its 32 proposals in full, ahead of the commits, through a work queue of (proposal, step)
 // items, one move applied per pass. Measured (B200), before and now: 256 units x 512 steps at p0 = 0.8, 1024
 // chains x 100,000 moves: 25.5 -> 13.6 ms; 16 x 32, 64 x 10,000: 0.43 -> 0.35; 16,384 x 256, 1024 x 200,000: 15.4 -> 11.5.
+// A link slower than the DRAM channels (not LIN), which for a while only the wide kernel served, without a bound: 256 x 512,
+// 1024 x 20,000 at p0 = 0.8: 8.5 -> 3.2 ms (the kernel before 4.4); 16,384 x 256, 1024 x 100,000: 12.3 -> 7.0 (7.3).
 #pragma once
 
 namespace kvp {
 
 namespace {
 
-constexpr uint32_t kPrepared4 = 4 * 32;                   // uint4 slots of a warp's prepared proposals
+// uint4 slots of a warp's prepared proposals
+__host__ __device__ constexpr uint32_t prepared4(bool lin) { return lin ? 4 * 32 : 5 * 32; }
 
-inline ChainLayout narrow_layout(uint32_t S, uint32_t S32, bool psmem, uint32_t cow4)
+inline ChainLayout narrow_layout(uint32_t S, uint32_t S32, bool psmem, bool lin, uint32_t cow4)
 {
     ChainLayout l;
-    uint32_t at = sizeof(ChainShared) + 16 * ((S + 1) / 2);       // {th, te} of every step
+    uint32_t at = sizeof(ChainShared) + 16 * (lin ? (S + 1) / 2 : S);   // {th, te}, or {th, te without migrations, in, out}
     auto take = [&](uint32_t n4) { const uint32_t p = at; at += 16 * n4; return p; };
     l.occ = take(psmem ? (S + 7) / 8 : (S + 3) / 4);
     l.full = take((S32 + 4) / 4);                         // (a bitmap is followed by a readable word)
     l.lead = take((S32 + 4) / 4);
+    l.out = take(lin ? 0u : (S32 + 4) / 4);
+    l.in = take(lin ? 0u : (S32 + 4) / 4);
     l.have = take(cow4);
     l.hb = l.work = at;
     return l;
 }
 // bytes of a chain of W warps, without a schedule in shared memory
-inline size_t narrow_bytes(uint32_t S, uint32_t S32, bool psmem, uint32_t cow4, uint32_t W)
+inline size_t narrow_bytes(uint32_t S, uint32_t S32, bool psmem, bool lin, uint32_t cow4, uint32_t W)
 {
-    return narrow_layout(S, S32, psmem, cow4).work + (size_t)W * kPrepared4 * 16;
+    return narrow_layout(S, S32, psmem, lin, cow4).work + (size_t)W * prepared4(lin) * 16;
 }
 
 // where a chain and a warp of it keep their state in shared memory
@@ -49,26 +54,68 @@ struct Narrow {
     uint32_t cb, wb;             // byte offsets: the chain's state, the warp's prepared proposals
     template <typename T> __device__ __forceinline__ T* at(uint32_t off) const { return reinterpret_cast<T*>(chain_smem + off); }
     __device__ __forceinline__ ChainShared* sc() const { return at<ChainShared>(cb); }
-    __device__ __forceinline__ int2* tt() const { return at<int2>(cb + (uint32_t)sizeof(ChainShared)); }   // [S] {th, te}
+    // [S] {th, te}, or {th, te without its migration term, units moved in, units moved out}
+    template <typename Sides> __device__ __forceinline__ Sides* sides() const { return at<Sides>(cb + (uint32_t)sizeof(ChainShared)); }
     __device__ __forceinline__ Occ* occ() const { return at<Occ>(cb + prm.lay.occ); }              // [S]
     __device__ __forceinline__ uint32_t* full() const { return at<uint32_t>(cb + prm.lay.full); }  // [S32] bit t: occ[t] == cap
     __device__ __forceinline__ uint32_t* lead() const { return at<uint32_t>(cb + prm.lay.lead); }  // [S32] bit t: te[t] >= th[t]
+    // not LIN: [S32] bit t: the link's outbound (inbound) traffic is the largest term of Eq. 4's maximum (see term_leads)
+    __device__ __forceinline__ uint32_t* out() const { return at<uint32_t>(cb + prm.lay.out); }
+    __device__ __forceinline__ uint32_t* in() const { return at<uint32_t>(cb + prm.lay.in); }
     __device__ __forceinline__ uint32_t* have() const { return at<uint32_t>(cb + prm.lay.have); }  // not PSMEM: buckets the slice holds
     // [4][32] prepared proposals: {s0 | end << 16, hit, lost, one}, {two, neg, largest accepted change, changed},
-    // {u, v, D's two words}, {D, placement after, Metropolis uniform}
+    // {u, v, D's two words}, {D, placement after, Metropolis uniform}; not LIN: one, two and neg are of the units moved in,
+    // and a fifth row has those of the units moved out
     __device__ __forceinline__ uint4* rec() const { return at<uint4>(wb); }
 };
 
-// Only for weights with kappa_d >= kappa_k (th and te are linear in hits and migrations, see kvp_chain.cuh) and fixed
-// populations; the wide kernel serves the others.
+// By how much a count rises at each step, given the up to two events that add to it after (na, nb) and before (oa, ob) a
+// move, one bit a step: one and two are the bits of the absolute value, neg its sign.
+struct Rise { uint32_t one, two, neg; };
+__device__ __forceinline__ Rise rise_of(uint32_t na, uint32_t nb, uint32_t oa, uint32_t ob)
+{
+    const uint32_t n1 = na ^ nb, n2 = na & nb, o1 = oa ^ ob, o2 = oa & ob;
+    Rise r;
+    r.two = (n2 & ~(o1 | o2)) | (o2 & ~(n1 | n2));
+    r.one = n1 ^ o1;
+    r.neg = (o2 & ~n2) | (o1 & ~(n1 | n2));
+    return r;
+}
+// its sum over the steps of a mask
+__device__ __forceinline__ int rise_over(const Rise& r, uint32_t m)
+{
+    return __popc(r.one & m) + 2 * (__popc(r.two & m) - __popc(r.one & r.neg & m)) - 4 * __popc(r.two & r.neg & m);
+}
+// its value at a step
+__device__ __forceinline__ int rise_at(uint32_t one, uint32_t two, uint32_t neg, uint32_t bit)
+{
+    const int n = (int)((one >> bit) & 1u) + 2 * (int)((two >> bit) & 1u);
+    return (neg >> bit) & 1u ? -n : n;
+}
+
+// The sides of a step by the step bitmaps: bit 0: te leads, bit 1: the link's outbound term is the largest of Eq. 4's three,
+// bit 2: the inbound one is.
+__device__ __forceinline__ uint32_t term_leads(const int4 f, const StepC c, const CostK K)
+{
+    const int e1 = (int)c.y + (int)K.kkF * f.w, e2 = (int)K.kkF * f.z, e3 = (int)c.z + (int)K.kdF * (f.z + f.w);
+    const bool out = e1 >= e2 && e1 >= e3, in = !out && e2 >= e3;
+    return (f.y + max(max(e1, e2), e3) >= f.x ? 1u : 0u) | (out ? 2u : 0u) | (in ? 4u : 0u);
+}
+
+// Only for fixed populations; the wide kernel serves the others.
 // PSMEM: schedules in shared memory; otherwise a chain's slice of global scratch is a copy-on-write overlay of the initial
 // schedule. ASMEM: the access bitmap staged there, too. SOLO: one warp per chain (W == 1).
-template <bool SOLO, bool PSMEM, bool ASMEM, int COLV>
+// LIN: kappa_d >= kappa_k, th and te are linear in hits and migrations (see kvp_chain.cuh). Otherwise te is the largest of
+// three linear terms, migrations in and out count separately, and the lower bound follows the term that leads at each step:
+// th, or Eq. 4 with the term that is the largest of its three (the new maximum is at least that one's new value).
+template <bool SOLO, bool PSMEM, bool ASMEM, bool LIN, int COLV>
 __global__ void __launch_bounds__(SOLO ? 256 : 512, 1)
 narrow_chain_kernel(const __grid_constant__ ChainParams prm)
 {
     static_assert(PSMEM ? COLV == 0 : !ASMEM && !SOLO, "vector columns only for schedules in global scratch");
     constexpr int kSide = SOLO ? 2 : 1;                           // (registers: 157; two in the other variants spill)
+    constexpr uint32_t kPrepared4 = prepared4(LIN);
+    using Sides = typename std::conditional<LIN, int2, int4>::type;
     using Occ = typename Narrow<PSMEM>::Occ;
     const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5, W = SOLO ? 1u : prm.warps;
     const uint32_t cpb = (blockDim.x >> 5) / W, cic = warp / W, sub = warp % W;   // chains per CTA; chain; warp of the chain
@@ -92,11 +139,20 @@ narrow_chain_kernel(const __grid_constant__ ChainParams prm)
             const uint32_t t = w * 32 + lane, i = min(t, S - 1);
             const uint4 n = __ldg(prm.counters0 + i);             // {hr, mi, mo, occ}
             const StepC k = __ldg(prm.stepc + i);
-            const int2 f = make_int2((int)(k.x + prm.K.kh * n.x + prm.K.khF * (n.y + n.z)),
-                                     (int)(k.w - prm.K.ke * n.x) + ext_term((int)n.y, (int)n.z, 0, k, prm.K));
-            if (t < S) { c.tt()[t] = f; c.occ()[t] = (Occ)n.w; }
-            const uint32_t F = __ballot_sync(0xFFFFFFFFu, t < S && n.w == prm.cap), T = __ballot_sync(0xFFFFFFFFu, t < S && f.y >= f.x);
+            const int4 f = make_int4((int)(k.x + prm.K.kh * n.x + prm.K.khF * (n.y + n.z)), (int)(k.w - prm.K.ke * n.x), (int)n.y, (int)n.z);
+            const int te = f.y + ext_term(f.z, f.w, 0, k, prm.K);
+            if (t < S) {
+                if constexpr (LIN) c.template sides<int2>()[t] = make_int2(f.x, te);
+                else c.template sides<int4>()[t] = f;
+                c.occ()[t] = (Occ)n.w;
+            }
+            const uint32_t F = __ballot_sync(0xFFFFFFFFu, t < S && n.w == prm.cap), T = __ballot_sync(0xFFFFFFFFu, t < S && te >= f.x);
             if (lane == 0) { c.full()[w] = F; c.lead()[w] = T; }
+            if constexpr (!LIN) {
+                const uint32_t by = term_leads(f, k, prm.K);
+                const uint32_t O = __ballot_sync(0xFFFFFFFFu, t < S && (by & 2u)), I = __ballot_sync(0xFFFFFFFFu, t < S && (by & 4u));
+                if (lane == 0) { c.out()[w] = O; c.in()[w] = I; }
+            }
         }
         if (sub == 0 && lane == 0) {
             ChainShared z = {};
@@ -141,7 +197,7 @@ narrow_chain_kernel(const __grid_constant__ ChainParams prm)
     bool unsaved = false;                                         // the best state is the current one and not saved yet
 
     uint32_t n_same = 0, n_inf = 0;                               // per lane
-    const int kh = (int)prm.K.kh, ke = (int)prm.K.ke, khF = (int)prm.K.khF, kdF = (int)prm.K.kdF;
+    const int kh = (int)prm.K.kh, ke = (int)prm.K.ke, khF = (int)prm.K.khF, kdF = (int)prm.K.kdF, kkF = (int)prm.K.kkF;
     const bool exchange = prm.rung_hist != nullptr;               // a level is a round of a replica-exchange run
     bool over = !active, silent = false;                          // this warp is done with its chain; because a wait ran out
     for (uint32_t level = 0; level < prm.seg1; ++level) {
@@ -233,14 +289,22 @@ narrow_chain_kernel(const __grid_constant__ ChainParams prm)
                     }
                     const uint32_t hit = (Au ^ Av) & D, lost = hit & (Au ^ Nu);
                     const uint32_t eun = Nu ^ (Nu << 1), euo = wu ^ (wu << 1), evn = Nv ^ (Nv << 1), evo = Wv ^ (Wv << 1);
-                    // migrations gained at a step: (eun + evn) - (euo + evo), as sign and two bits of the absolute value
-                    const uint32_t n1 = (eun ^ evn) & Sb, n2 = eun & evn & Sb, o1 = (euo ^ evo) & Sb, o2 = euo & evo & Sb;
-                    const uint32_t two = (n2 & ~(o1 | o2)) | (o2 & ~(n1 | n2)), one = n1 ^ o1;
-                    const uint32_t neg = (o2 & ~n2) | (o1 & ~(n1 | n2));
                     const int ht = __popc(hit & T) - 2 * __popc(lost & T), hs = __popc(hit) - 2 * __popc(lost) - ht;
-                    const int mt = __popc(one & T) + 2 * (__popc(two & T) - __popc(one & neg & T)) - 4 * __popc(two & neg & T);
-                    const int ms = __popc(one) + 2 * (__popc(two) - __popc(one & neg)) - 4 * __popc(two & neg) - mt;
-                    const int lb = kdF * mt - ke * ht + khF * ms + kh * hs;   // the change of the side that leads
+                    int lb = kh * hs - ke * ht;                   // the change of the side that leads
+                    Rise go, leave;                               // migrations gained at a step; not LIN: into HBM, out of it
+                    if constexpr (LIN) {
+                        go = rise_of(eun & Sb, evn & Sb, euo & Sb, evo & Sb);
+                        const int mt = rise_over(go, T), ms = rise_over(go, 0xFFFFFFFFu) - mt;
+                        lb += kdF * mt + khF * ms;
+                    } else {
+                        go = rise_of(eun & Nu & Sb, evn & Nv & Sb, euo & wu & Sb, evo & Wv & Sb);
+                        leave = rise_of(eun & ~Nu & Sb, evn & ~Nv & Sb, euo & ~wu & Sb, evo & ~Wv & Sb);
+                        const uint32_t O = window_at<0>(c.out(), wp), I = window_at<0>(c.in(), wp), C = T & ~(O | I);
+                        lb += khF * (rise_over(go, ~T) + rise_over(leave, ~T)) + kkF * (rise_over(leave, T & O) + rise_over(go, T & I)) +
+                              kdF * (rise_over(go, C) + rise_over(leave, C));
+                    }
+                    uint32_t turns = hit | go.one | go.two;
+                    if constexpr (!LIN) turns |= leave.one | leave.two;
                     __syncwarp();
                     if ((prep >> lane) & 1u) {
                         Wu = wu;
@@ -248,8 +312,9 @@ narrow_chain_kernel(const __grid_constant__ ChainParams prm)
                         bad = !swap && (~wu & D & W2) != 0u;      // a flip may not raise a full step (Eq. 5)
                         rejected = bounded && lb > dmax && (uint32_t)(lb - dmax) > bin;
                         const uint32_t d = s0 ? D : D >> 1;       // aligned to step s0 - 1 (0)
-                        c.rec()[lane] = make_uint4(s0 | (s0 + 31u - __clz(D)) << 16, hit, lost, one);
-                        c.rec()[32 + lane] = make_uint4(two, neg, (uint32_t)dmax, hit | one | two | (swap ? 1u : 0u));   // (bit 0 is no step)
+                        c.rec()[lane] = make_uint4(s0 | (s0 + 31u - __clz(D)) << 16, hit, lost, go.one);
+                        c.rec()[32 + lane] = make_uint4(go.two, go.neg, (uint32_t)dmax, turns | (swap ? 1u : 0u));   // (bit 0 is no step)
+                        if constexpr (!LIN) c.rec()[128 + lane] = make_uint4(leave.one, leave.two, leave.neg, 0u);
                         c.rec()[64 + lane] = make_uint4(u, v, d << wp.sh, wp.sh ? d >> (32u - wp.sh) : 0u);
                         c.rec()[96 + lane] = make_uint4(D, Nu, mv.w, 0u);
                     } else if ((check >> lane) & 1u) {
@@ -312,7 +377,7 @@ narrow_chain_kernel(const __grid_constant__ ChainParams prm)
 #pragma unroll 1
                 while (survivors) {
                     // up to kSide of the survivors: cost changes against the present state
-                    int2 g[kSide], f[kSide];
+                    Sides g[kSide], f[kSide];
                     uint32_t id[kSide], t[kSide], chg[kSide], steps[kSide];
                     int delta[kSide], most[kSide];
                     uint32_t rest = survivors;
@@ -324,11 +389,19 @@ narrow_chain_kernel(const __grid_constant__ ChainParams prm)
                         const uint4 a = c.rec()[k], b = c.rec()[32 + k];
                         chg[j] = b.w; steps[j] = a.x; most[j] = (int)b.z;
                         t[j] = min((a.x & 0xFFFFu) + max(lane, 1u) - 1u, S - 1u);   // lane l: window bit l, step s0 - 1 + l
-                        f[j] = c.tt()[t[j]];
-                        const int h = (a.y >> lane) & 1u, mg = (int)((a.w >> lane) & 1u) + 2 * (int)((b.x >> lane) & 1u);
-                        const int hr = (a.z >> lane) & 1u ? -h : h, mm = (b.y >> lane) & 1u ? -mg : mg;
-                        g[j] = make_int2(f[j].x + kh * hr + khF * mm, f[j].y - ke * hr + kdF * mm);
-                        delta[j] = max(g[j].x, g[j].y) - max(f[j].x, f[j].y);   // 0 where nothing changes
+                        f[j] = c.template sides<Sides>()[t[j]];
+                        const int h = (a.y >> lane) & 1u, hr = (a.z >> lane) & 1u ? -h : h, mi = rise_at(a.w, b.x, b.y, lane);
+                        if constexpr (LIN) {
+                            g[j] = make_int2(f[j].x + kh * hr + khF * mi, f[j].y - ke * hr + kdF * mi);
+                            delta[j] = max(g[j].x, g[j].y) - max(f[j].x, f[j].y);   // 0 where nothing changes
+                        } else {
+                            const uint4 o = c.rec()[128 + k];
+                            const int mo = rise_at(o.x, o.y, o.z, lane);
+                            const StepC sc = __ldg(prm.stepc + t[j]);
+                            g[j] = make_int4(f[j].x + kh * hr + khF * (mi + mo), f[j].y - ke * hr, f[j].z + mi, f[j].w + mo);
+                            delta[j] = max(g[j].x, g[j].y + ext_term(g[j].z, g[j].w, 0, sc, prm.K)) -
+                                       max(f[j].x, f[j].y + ext_term(f[j].z, f[j].w, 0, sc, prm.K));
+                        }
                     }
 #pragma unroll
                     for (int j = 0; j < kSide; ++j) delta[j] = __reduce_add_sync(0xFFFFFFFFu, delta[j]);
@@ -353,9 +426,17 @@ narrow_chain_kernel(const __grid_constant__ ChainParams prm)
                         const bool sw = chg[j] & 1u, mine = lane != 0u && (chg[j] >> lane) & 1u;
                         const uint32_t bit0 = b0 ? b0 - 1u : 0u;
                         __syncwarp();
-                        if (mine) c.tt()[t[j]] = g[j];
-                        const uint32_t lturn = __ballot_sync(0xFFFFFFFFu, mine && (g[j].y >= g[j].x) != (f[j].y >= f[j].x));
-                        uint32_t fturn = 0u;
+                        if (mine) c.template sides<Sides>()[t[j]] = g[j];
+                        uint32_t lturn, oturn = 0u, iturn = 0u, fturn = 0u;   // steps at which the bitmaps turn
+                        if constexpr (LIN) {
+                            lturn = __ballot_sync(0xFFFFFFFFu, mine && (g[j].y >= g[j].x) != (f[j].y >= f[j].x));
+                        } else {
+                            const StepC sc = __ldg(prm.stepc + t[j]);
+                            const uint32_t turn = mine ? term_leads(g[j], sc, prm.K) ^ term_leads(f[j], sc, prm.K) : 0u;
+                            lturn = __ballot_sync(0xFFFFFFFFu, turn & 1u);
+                            oturn = __ballot_sync(0xFFFFFFFFu, turn & 2u);
+                            iturn = __ballot_sync(0xFFFFFFFFu, turn & 4u);
+                        }
                         if (!sw) {                                // a flip: occupancy and the full-step bitmap
                             const uint2 e = *reinterpret_cast<const uint2*>(c.rec() + 96 + id[j]);
                             const bool in = (e.x >> lane) & 1u;
@@ -395,10 +476,12 @@ narrow_chain_kernel(const __grid_constant__ ChainParams prm)
                         a.steps = b0 | bend << 16;
                         a.units = (r.x & 0xFFFFu) | r.y << 16;
                         a.bits = a.fulls = 0xFFFFu;
-                        if (lturn | fturn) {
-                            const uint32_t sh = bit0 & 31u, x0 = lane < 2 ? lturn : fturn, x = b0 ? x0 : x0 >> 1;
+                        if (lturn | fturn | oturn | iturn) {
+                            const uint32_t sh = bit0 & 31u, x0 = lane < 2 ? lturn : lane < 4 || LIN ? fturn : lane < 6 ? oturn : iturn, x = b0 ? x0 : x0 >> 1;
                             const uint32_t part = lane & 1u ? (sh ? x >> (32u - sh) : 0u) : x << sh;
-                            if (lane < 4 && part) (lane < 2 ? c.lead() : c.full())[(bit0 >> 5) + (lane & 1u)] ^= part;
+                            if (lane < (LIN ? 4u : 8u) && part)
+                                (lane < 2 ? c.lead() : lane < 4 || LIN ? c.full() : lane < 6 ? c.out() : c.in())[(bit0 >> 5) + (lane & 1u)] ^= part;
+                            lturn |= oturn | iturn;
                             if (lturn) a.bits = (b0 + __ffs(lturn) - 2u) | (b0 + 30u - __clz(lturn)) << 16;
                             if (fturn) a.fulls = (b0 + __ffs(fturn) - 2u) | (b0 + 30u - __clz(fturn)) << 16;
                         }

@@ -1,7 +1,7 @@
 """The chain kernels' variants at the sizes where they can go wrong, against the oracle bit for bit: every number of warps
 per chain, window edges (steps around multiples of 32), vector columns (two and four words), columns longer than half a
-warp, schedules in shared and in global memory, weights for which the narrow kernel is not built, replica exchange inside
-CTAs and in launches."""
+warp, schedules in shared and in global memory, weights for which the cost is not linear in migrations, replica exchange
+inside CTAs and in launches."""
 import numpy as np
 import pytest
 
@@ -47,6 +47,35 @@ def test_weights(kvp, oracle, hooks, bw, flags):
     for warps in (2, 18):
         hooks(warps_per_chain=warps)
         _same(g, o, chains=6, moves=2000, seed=4, levels=4, p0=0.3)
+
+
+@pytest.mark.parametrize("warps", (0,) + NARROW + (18,))
+@pytest.mark.parametrize("U,S,cap", [(31, 32, 9), (40, 33, 40), (65, 64, 20), (33, 97, 10), (7000, 64, 2000), (5000, 128, 900),
+                                     (3000, 257, 700)])
+def test_link_slower_than_dram(kvp, oracle, hooks, warps, U, S, cap):
+    """Eq. 4's maximum is over three terms then, each of which leads at some steps: the link in either direction, the DRAM
+    channels. Written units on either side shift which one does."""
+    hooks(warps_per_chain=warps)
+    A = wl.random_access(U, S, 0.2, seed=U + S)
+    rng = np.random.default_rng(U)
+    hw, ew = rng.integers(0, 3, S), rng.integers(0, 4, S) * (rng.random(S) < 0.5)
+    g, o = both_problems(kvp, oracle, U, 8192, S, A, cap, (4900 * GB, 500 * GB, 700 * GB), hw=hw, ew=ew)
+    for p0 in (0.8, 1e-4):
+        _same(g, o, chains=5, moves=1500, seed=U, levels=6, p0=p0, early_stop_permille=1, early_stop_from_level=4)
+
+
+@pytest.mark.parametrize("warps", [0, 2, 3])
+@pytest.mark.parametrize("chains,rungs", [(24, 3), (40, 20)])
+def test_exchange_with_slow_link(kvp, oracle, hooks, warps, chains, rungs):
+    hooks(warps_per_chain=warps)
+    A = wl.random_access(120, 90, 0.25, seed=2)
+    g, o = both_problems(kvp, oracle, 120, 8192, 90, A, 30, (8000 * GB, 400 * GB, 900 * GB))
+    kw = dict(chains=chains, moves=701, seed=9, levels=rungs, p0=1e-2, alpha=0.7)
+    out = g.anneal_exchange(g.make_params(**kw), rungs, 100)
+    ref = o.anneal_exchange(o.make_params(**kw), rungs, 100, want_best=True)
+    assert [r.astuple() for r in out["per_chain"]] == [r.astuple() for r in ref["per_chain"]]
+    assert out["final_rung"] == ref["final_rung"].tolist()
+    assert np.array_equal(to_np(out["best_schedule"]), ref["best_schedule"])
 
 
 @pytest.mark.parametrize("warps", [0, 2, 3, 18])
