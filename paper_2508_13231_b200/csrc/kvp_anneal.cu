@@ -1000,7 +1000,7 @@ int prepare(kvp_problem* p, const kvp_anneal_params* a, cudaStream_t st, Ctx& c,
     float* const bounds = reinterpret_cast<float*>(shifts + a->levels);
     if ((rc = kvp_accept_table(c.temps.data(), a->levels, table, shifts))) return rc;
     // the lower bounds of kvp_chain.cuh are sums of at most 31 steps' changes in 32 bits
-    const uint64_t step_max = 4ull * std::max({p->K.khF, p->K.kdF, p->K.kkF}) + std::max(p->K.kh, p->K.ke) + 2ull * std::max(p->K.kh, p->K.kd);
+    const uint64_t step_max = 4ull * std::max({p->K.khF, p->K.kdF, p->K.kkF}) + std::max(p->K.kh, p->K.ke) + 2ull * std::max(p->K.kh, p->K.ke);
     const bool bounded = 31 * step_max < (1ull << 30);
     for (uint32_t j = 0; j < a->levels; ++j) bounds[j] = bounded ? (float)((c.temps[j] >= 1.0 ? c.temps[j] : 1.0) * 0.69314718) : INFINITY;
     KVP_CUDA(cudaMemcpyAsync(c.table, table, table_bytes(a->levels), cudaMemcpyHostToDevice, st));

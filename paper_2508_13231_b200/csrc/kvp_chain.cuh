@@ -93,6 +93,8 @@ inline ChainLayout chain_layout(uint32_t S, uint32_t S32, bool grow, bool psmem,
     l.occ = take(psmem ? (S + 7) / 8 : (S + 3) / 4);
     l.full = take((S32 + 3) / 4);
     l.lead = take((S32 + 3) / 4);
+    l.out = take(lin ? 0u : (S32 + 3) / 4);
+    l.in = take(lin ? 0u : (S32 + 3) / 4);
     l.hb = take(grow && !lin ? (S + 3) / 4 : 0u);
     l.have = take(cow4);
     l.work = at;                                          // what outlives a batch ends here
@@ -122,6 +124,9 @@ struct Chain {
     __device__ __forceinline__ Occ* occ() const { return at<Occ>(cb + prm.lay.occ); }              // [S]
     __device__ __forceinline__ uint32_t* full() const { return at<uint32_t>(cb + prm.lay.full); }  // [S32] bit t: occ[t] == cap
     __device__ __forceinline__ uint32_t* lead() const { return at<uint32_t>(cb + prm.lay.lead); }  // [S32] bit t: te[t] >= th[t]
+    // not LIN: [S32] bit t: the link's outbound (inbound) traffic is the largest term of Eq. 4's maximum (see term_leads)
+    __device__ __forceinline__ uint32_t* out() const { return at<uint32_t>(cb + prm.lay.out); }
+    __device__ __forceinline__ uint32_t* in() const { return at<uint32_t>(cb + prm.lay.in); }
     __device__ __forceinline__ uint32_t* hb() const { return at<uint32_t>(cb + prm.lay.hb); }      // not LIN, GROW: [S] written to HBM at birth
     __device__ __forceinline__ uint32_t* have() const { return at<uint32_t>(cb + prm.lay.have); }  // not PSMEM: buckets present in the slice
     __device__ __forceinline__ uint4* ring() const { return at<uint4>(wb); }                       // [kRing] {pk | id << 24, u, v, w}
@@ -241,6 +246,15 @@ __device__ __forceinline__ int ext_term(int mi, int mo, int hb, const StepC c, c
     const int e3 = (int)c.z - (int)K.kd * hb + (int)K.kdF * (mi + mo);
     return max(max(e1, e2), e3);
 }
+// The terms of a step by the step bitmaps, f = {th, te without its migration term, in, out}: bit 0: te leads; bit 1: the
+// link's outbound term is the largest of Eq. 4's three; bit 2: the inbound one is.
+__device__ __forceinline__ uint32_t term_leads(const int4 f, int hb, const StepC c, const CostK K)
+{
+    const int e1 = (int)c.y - (int)K.kk * hb + (int)K.kkF * f.w, e2 = (int)K.kkF * f.z;
+    const int e3 = (int)c.z - (int)K.kd * hb + (int)K.kdF * (f.z + f.w);
+    const bool out = e1 >= e2 && e1 >= e3, in = !out && e2 >= e3;
+    return (f.y + max(max(e1, e2), e3) >= f.x ? 1u : 0u) | (out ? 2u : 0u) | (in ? 4u : 0u);
+}
 
 // What a warp needs to evaluate, constant over a temperature level or longer.
 struct EvalCtx {
@@ -291,19 +305,34 @@ __device__ __forceinline__ void judge(const Chain<PSMEM, GROW, LIN, COLV, R>& c,
     const uint32_t av = window_at<COLV>(x.Acol + (size_t)(swap ? a.z : a.y) * prm.S32, wp);   // a flip reads unit u twice
     const uint32_t Av = swap ? av : 0u;
     const Effect e = effect_of<GROW, LIN>(prm.birth, S, pk, a.y, a.z, b.x, b.y, Au, Av);
-    bool keep = live;
+    const uint32_t T = window_at<0>((const uint32_t*)c.lead(), wp);          // steps where te leads
+    const int hits_t = __popc(e.won & T) - __popc(e.lost & T), hits = __popc(e.won) - __popc(e.lost);
+    int lb;
     if (LIN) {
-        const uint32_t T = window_at<0>((const uint32_t*)c.lead(), wp);      // steps where te leads
-        const int hits_t = __popc(e.won & T) - __popc(e.lost & T), hits = __popc(e.won) - __popc(e.lost);
         const int mm_t = __popc(e.eun & T) + __popc(e.evn & T) - __popc(e.euo & T) - __popc(e.evo & T);
         const int mm = __popc(e.eun) + __popc(e.evn) - __popc(e.euo) - __popc(e.evo);
-        int lb = kdF * mm_t - ke * hits_t + khF * (mm - mm_t) + kh * (hits - hits_t);
+        lb = kdF * mm_t - ke * hits_t + khF * (mm - mm_t) + kh * (hits - hits_t);
         if (GROW) {
             if (e.Bu) lb += ((e.Nu & e.Bu) != 0 ? 1 : -1) * ((T & e.Bu) != 0 ? -kd : kh);
             if (e.Bv) lb += ((e.Nv & e.Bv) != 0 ? 1 : -1) * ((T & e.Bv) != 0 ? -kd : kh);
         }
-        keep = live && (float)lb <= x.bound * (32.001f - __log2f((float)max(a.w, 1u))) + __uint_as_float((127u + x.shift) << 23);
+    } else {
+        // migrations count in the direction of the term that leads (both where th or the DRAM channels do)
+        const uint32_t O = T & window_at<0>((const uint32_t*)c.out(), wp), I = T & window_at<0>((const uint32_t*)c.in(), wp);
+        const uint32_t iu = e.eun & e.Nu, iv = e.evn & e.Nv, ju = e.euo & b.x, jv = e.evo & b.y;    // into HBM: after, before
+        const uint32_t ou = e.eun ^ iu, ov = e.evn ^ iv, pu = e.euo ^ ju, pv = e.evo ^ jv;          // out of it
+        auto in = [&](uint32_t m) { return __popc(iu & m) + __popc(iv & m) - __popc(ju & m) - __popc(jv & m); };
+        auto out = [&](uint32_t m) { return __popc(ou & m) + __popc(ov & m) - __popc(pu & m) - __popc(pv & m); };
+        const uint32_t C = T & ~(O | I);
+        const int kk = (int)prm.K.kk, kkF = (int)prm.K.kkF;
+        lb = kh * (hits - hits_t) - ke * hits_t + khF * (in(~T) + out(~T)) + kkF * (out(O) + in(I)) + kdF * (in(C) + out(C));
+        if (GROW) {
+            auto write = [&](uint32_t B) { return (T & B) == 0 ? kh : (O & B) != 0 ? -kk : (I & B) != 0 ? 0 : -kd; };
+            if (e.Bu) lb += ((e.Nu & e.Bu) != 0 ? 1 : -1) * write(e.Bu);
+            if (e.Bv) lb += ((e.Nv & e.Bv) != 0 ? 1 : -1) * write(e.Bv);
+        }
     }
+    const bool keep = live && (float)lb <= x.bound * (32.001f - __log2f((float)max(a.w, 1u))) + __uint_as_float((127u + x.shift) << 23);
     const uint32_t kb = __ballot_sync(0xFFFFFFFFu, keep);
     if (!kb) return;
     if (keep) atomicOr(c.close() + (pk >> 29), 1u << ((pk >> 24) & 31u));
@@ -461,7 +490,8 @@ __device__ __forceinline__ uint32_t apply(const Chain<PSMEM, GROW, LIN, COLV, R>
     const uint32_t j = valid ? lane : 1u, t = s0 + j - 1;
     const BitChange d = bit_change<GROW>(e, j);
     const CostK& K = prm.K;
-    bool lead = false, led = false;                               // not LIN: the bitmap is not used
+    bool lead = false, led = false;                               // LIN: te leads, led before
+    uint32_t by = 0u, was = 0u;                                   // not LIN: which terms lead, led before
     if (LIN) {
         int2 f = c.tt()[t];
         led = f.y >= f.x;
@@ -471,14 +501,19 @@ __device__ __forceinline__ uint32_t apply(const Chain<PSMEM, GROW, LIN, COLV, R>
         lead = f.y >= f.x;
     } else {
         int4 f = c.tm()[t];
+        const StepC sc = __ldg(prm.stepc + t);
+        const int hb = GROW ? (int)c.hb()[t] : 0;
         int mi, mo;
         edge_change(e, win.x, win.y, j, mi, mo);
+        was = term_leads(f, hb, sc, K);
         f.x += (int)K.kh * (d.hr + d.hb) + (int)K.khF * (mi + mo);
         f.y -= (int)K.ke * d.hr;
         f.z += mi; f.w += mo;
+        by = term_leads(f, hb + d.hb, sc, K);
+        lead = by & 1u; led = was & 1u;
         if (valid) {
             c.tm()[t] = f;
-            if (GROW) c.hb()[t] += (uint32_t)d.hb;
+            if (GROW) c.hb()[t] = (uint32_t)(hb + d.hb);
         }
     }
     uint32_t occ = c.occ()[t];
@@ -486,12 +521,17 @@ __device__ __forceinline__ uint32_t apply(const Chain<PSMEM, GROW, LIN, COLV, R>
     occ += ((e.Nu >> j) & 1u) + ((e.Nv >> j) & 1u) - ((win.x >> j) & 1u) - ((win.y >> j) & 1u);
     if (valid) c.occ()[t] = (typename Chain<PSMEM, GROW, LIN, COLV, R>::Occ)occ;
     uint32_t F = __ballot_sync(0xFFFFFFFFu, valid && occ == prm.cap), T = __ballot_sync(0xFFFFFFFFu, valid && lead);
-    const uint32_t turned = __ballot_sync(0xFFFFFFFFu, valid && (lead != led || (occ == prm.cap) != was_full));
+    uint32_t O = 0u, I = 0u;
+    if (!LIN) {
+        O = __ballot_sync(0xFFFFFFFFu, valid && (by & 2u));
+        I = __ballot_sync(0xFFFFFFFFu, valid && (by & 4u));
+    }
+    const uint32_t turned = __ballot_sync(0xFFFFFFFFu, valid && (lead != led || by != was || (occ == prm.cap) != was_full));
     c.own(u, lane);
     if (swap) c.own(v, lane);
     if (lane < 2) {
         uint32_t M = ((1u << run) - 1u) << 1, V = ((1u << nl) - 1u) << 1, NU = e.Nu, NV = e.Nv, sbit = s0 - 1;
-        if (s0 == 0) { F >>= 1; T >>= 1; V >>= 1; M >>= 1; NU >>= 1; NV >>= 1; sbit = 0; }
+        if (s0 == 0) { F >>= 1; T >>= 1; O >>= 1; I >>= 1; V >>= 1; M >>= 1; NU >>= 1; NV >>= 1; sbit = 0; }
         const uint32_t wj = (sbit >> 5) + lane, sh = sbit & 31u;
         if (wj < S32 && (lane == 0 || sh != 0)) {
             // lane 0 holds the part of the window that falls into the first word, lane 1 the spill-over
@@ -499,7 +539,11 @@ __device__ __forceinline__ uint32_t apply(const Chain<PSMEM, GROW, LIN, COLV, R>
             const uint32_t Vx = part(V), Mx = part(M);
             if (Vx) {
                 c.full()[wj] = (c.full()[wj] & ~Vx) | (part(F) & Vx);
-                if (LIN) c.lead()[wj] = (c.lead()[wj] & ~Vx) | (part(T) & Vx);
+                c.lead()[wj] = (c.lead()[wj] & ~Vx) | (part(T) & Vx);
+                if (!LIN) {
+                    c.out()[wj] = (c.out()[wj] & ~Vx) | (part(O) & Vx);
+                    c.in()[wj] = (c.in()[wj] & ~Vx) | (part(I) & Vx);
+                }
             }
             if (Mx) {
                 uint32_t* const pu = c.P() + (size_t)u * S32 + wj;
@@ -669,6 +713,11 @@ wide_chain_kernel(const __grid_constant__ ChainParams prm)
             const uint32_t F = __ballot_sync(0xFFFFFFFFu, t < S && n.w == prm.cap);
             const uint32_t T = __ballot_sync(0xFFFFFFFFu, t < S && base + ext >= th);
             if (lane == 0) { c.full()[w] = F; c.lead()[w] = T; }
+            if (!LIN) {
+                const uint32_t by = term_leads(make_int4(th, base, (int)n.y, (int)n.z), (int)hb, k, prm.K);
+                const uint32_t O = __ballot_sync(0xFFFFFFFFu, t < S && (by & 2u)), I = __ballot_sync(0xFFFFFFFFu, t < S && (by & 4u));
+                if (lane == 0) { c.out()[w] = O; c.in()[w] = I; }
+            }
         }
         if (tid == 0) {
             ChainShared z = {};

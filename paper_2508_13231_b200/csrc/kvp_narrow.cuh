@@ -93,15 +93,6 @@ __device__ __forceinline__ int rise_at(uint32_t one, uint32_t two, uint32_t neg,
     return (neg >> bit) & 1u ? -n : n;
 }
 
-// The sides of a step by the step bitmaps: bit 0: te leads, bit 1: the link's outbound term is the largest of Eq. 4's three,
-// bit 2: the inbound one is.
-__device__ __forceinline__ uint32_t term_leads(const int4 f, const StepC c, const CostK K)
-{
-    const int e1 = (int)c.y + (int)K.kkF * f.w, e2 = (int)K.kkF * f.z, e3 = (int)c.z + (int)K.kdF * (f.z + f.w);
-    const bool out = e1 >= e2 && e1 >= e3, in = !out && e2 >= e3;
-    return (f.y + max(max(e1, e2), e3) >= f.x ? 1u : 0u) | (out ? 2u : 0u) | (in ? 4u : 0u);
-}
-
 // Only for fixed populations; the wide kernel serves the others.
 // PSMEM: schedules in shared memory; otherwise a chain's slice of global scratch is a copy-on-write overlay of the initial
 // schedule. ASMEM: the access bitmap staged there, too. SOLO: one warp per chain (W == 1).
@@ -149,7 +140,7 @@ narrow_chain_kernel(const __grid_constant__ ChainParams prm)
             const uint32_t F = __ballot_sync(0xFFFFFFFFu, t < S && n.w == prm.cap), T = __ballot_sync(0xFFFFFFFFu, t < S && te >= f.x);
             if (lane == 0) { c.full()[w] = F; c.lead()[w] = T; }
             if constexpr (!LIN) {
-                const uint32_t by = term_leads(f, k, prm.K);
+                const uint32_t by = term_leads(f, 0, k, prm.K);
                 const uint32_t O = __ballot_sync(0xFFFFFFFFu, t < S && (by & 2u)), I = __ballot_sync(0xFFFFFFFFu, t < S && (by & 4u));
                 if (lane == 0) { c.out()[w] = O; c.in()[w] = I; }
             }
@@ -432,7 +423,7 @@ narrow_chain_kernel(const __grid_constant__ ChainParams prm)
                             lturn = __ballot_sync(0xFFFFFFFFu, mine && (g[j].y >= g[j].x) != (f[j].y >= f[j].x));
                         } else {
                             const StepC sc = __ldg(prm.stepc + t[j]);
-                            const uint32_t turn = mine ? term_leads(g[j], sc, prm.K) ^ term_leads(f[j], sc, prm.K) : 0u;
+                            const uint32_t turn = mine ? term_leads(g[j], 0, sc, prm.K) ^ term_leads(f[j], 0, sc, prm.K) : 0u;
                             lturn = __ballot_sync(0xFFFFFFFFu, turn & 1u);
                             oturn = __ballot_sync(0xFFFFFFFFu, turn & 2u);
                             iturn = __ballot_sync(0xFFFFFFFFu, turn & 4u);

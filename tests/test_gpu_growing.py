@@ -19,9 +19,8 @@ def kvp():
 
 @pytest.fixture(params=[3, 1, 2], ids=["wide", "narrow1", "narrow2"])
 def warps_per_chain(request, hooks):
-    """The wide chain kernel (one warp per chain, four proposals per lane; the library's choice for jobs of many
-    chains) and both forms of the narrow one (one proposal per lane; one warp per chain, or two warps that take a
-    chain's batches in turn; the choice for few chains)."""
+    """The wide chain kernel, the only one that serves growing caches: one warp per chain (3 and 1) and two warps that take a
+    chain's batches in turn (2)."""
     hooks(warps_per_chain=request.param)
     return request.param
 
@@ -217,6 +216,21 @@ def test_anneal_growing_global_state(kvp, oracle, warps_per_chain):
         out = _check_chains(g, o, g.make_params(**kw), o.make_params(**kw))
         if p0 < 0.1:                                          # the near-greedy run improves on its start: the winner
             assert out["stats"].best_move != 2 ** 64 - 1      # is a walked-back state, not the initial schedule
+
+
+@pytest.mark.parametrize("layers,heads,n,prompt,cap", [(3, 1, 45, 20, 30), (4, 4, 256, 200, 800)], ids=["shared", "global"])
+def test_anneal_growing_slow_link(kvp, oracle, warps_per_chain, layers, heads, n, prompt, cap):
+    """A link slower than the DRAM channels: three terms in Eq. 4's maximum, two of which a write to DRAM counts in."""
+    cfg, groups, U, S, birth = _shape(layers, heads, n, prompt)
+    rng = np.random.default_rng(n)
+    alive = birth[None, :] <= np.arange(S)[:, None]
+    A = wl.pack_bits(((rng.random((S, U)) < 0.2) & alive).astype(np.uint8))
+    hw, ew = (np.arange(S) % 2).astype(np.uint32), (np.arange(S) % 5).astype(np.uint32)
+    for bw in ((4900, 500, 700), (3, 1, 2)):
+        g, o = _problems(kvp, oracle, U, 512, S, A, cap, tuple(b * GB for b in bw), birth, hw=hw, ew=ew)
+        for p0 in (0.5, 1e-4):
+            kw = dict(chains=5, moves=3000, seed=8, p0=p0, levels=6)
+            _check_chains(g, o, g.make_params(**kw), o.make_params(**kw))
 
 
 def test_anneal_growing_8b_sampled_chains(kvp, oracle):
