@@ -606,18 +606,19 @@ int validate(const kvp_problem* p, const kvp_anneal_params* a)
 
 typedef void (*ChainKernel)(const ChainParams);
 
-template <bool LIN>
+template <bool GROW, bool LIN>
 ChainKernel narrow_pick(bool psmem, bool asmem, uint32_t S32, bool solo)
 {
-    if (psmem && solo) return asmem ? narrow_chain_kernel<true, true, true, LIN, 0> : narrow_chain_kernel<true, true, false, LIN, 0>;
-    if (psmem) return asmem ? narrow_chain_kernel<false, true, true, LIN, 0> : narrow_chain_kernel<false, true, false, LIN, 0>;
-    return S32 == 2 ? narrow_chain_kernel<false, false, false, LIN, 2> : S32 == 4 ? narrow_chain_kernel<false, false, false, LIN, 4>
-                                                                                  : narrow_chain_kernel<false, false, false, LIN, 0>;
+    if (psmem && solo) return asmem ? narrow_chain_kernel<true, true, true, GROW, LIN, 0> : narrow_chain_kernel<true, true, false, GROW, LIN, 0>;
+    if (psmem) return asmem ? narrow_chain_kernel<false, true, true, GROW, LIN, 0> : narrow_chain_kernel<false, true, false, GROW, LIN, 0>;
+    return S32 == 2 ? narrow_chain_kernel<false, false, false, GROW, LIN, 2> : S32 == 4 ? narrow_chain_kernel<false, false, false, GROW, LIN, 4>
+                                                                                        : narrow_chain_kernel<false, false, false, GROW, LIN, 0>;
 }
 
-ChainKernel narrow_kernel_for(bool psmem, bool asmem, bool lin, uint32_t S32, bool solo)
+ChainKernel narrow_kernel_for(bool psmem, bool asmem, bool grow, bool lin, uint32_t S32, bool solo)
 {
-    return lin ? narrow_pick<true>(psmem, asmem, S32, solo) : narrow_pick<false>(psmem, asmem, S32, solo);
+    if (grow) return lin ? narrow_pick<true, true>(psmem, asmem, S32, solo) : narrow_pick<true, false>(psmem, asmem, S32, solo);
+    return lin ? narrow_pick<false, true>(psmem, asmem, S32, solo) : narrow_pick<false, false>(psmem, asmem, S32, solo);
 }
 
 template <bool PSMEM, bool ASMEM, bool LIN, int COLV>
@@ -643,14 +644,14 @@ ChainKernel wide_kernel_for(bool psmem, bool asmem, bool grow, bool lin, uint32_
 ChainKernel kernel_of(const Ctx& c, bool psmem, bool asmem, uint32_t W)
 {
     return c.wide ? wide_kernel_for(psmem, asmem, c.grow, c.lin, c.S32, c.rows)
-                  : narrow_kernel_for(psmem, asmem, c.lin, c.S32, c.solo);
+                  : narrow_kernel_for(psmem, asmem, c.grow, c.lin, c.S32, c.solo);
 }
 
 int launch_chains(const Ctx& c, ChainParams& prm, uint32_t count)
 {
     {
         const bool rounds = prm.rung_hist != nullptr;
-        prm.lay = !c.wide ? narrow_layout(prm.S, prm.S32, c.psmem, c.lin, c.psmem ? 0u : c.cow_slots4) : chain_layout(prm.S, prm.S32, c.grow, c.psmem, c.lin, c.psmem ? 0u : c.cow_slots4);
+        prm.lay = !c.wide ? narrow_layout(prm.S, prm.S32, c.grow, c.psmem, c.lin, c.psmem ? 0u : c.cow_slots4) : chain_layout(prm.S, prm.S32, c.grow, c.psmem, c.lin, c.psmem ? 0u : c.cow_slots4);
         prm.seg_len = rounds ? prm.exch_every : prm.per_level;
         const uint32_t batch = c.wide ? 32u * c.rows : 32u;
         prm.seg_bat = (uint32_t)((prm.seg_len + batch - 1) / batch);
@@ -746,7 +747,7 @@ int prepare(kvp_problem* p, const kvp_anneal_params* a, cudaStream_t st, Ctx& c,
     c.asmem = false;
     auto fixed_bytes = [&](uint32_t warps, bool shared) {
         if (c.wide) return chain_bytes(p->S, p->S32, c.grow, shared, c.lin, shared ? 0u : c.cow_slots4, warps, c.rows);
-        return narrow_bytes(p->S, p->S32, shared, c.lin, shared ? 0u : c.cow_slots4, warps);
+        return narrow_bytes(p->S, p->S32, c.grow, shared, c.lin, shared ? 0u : c.cow_slots4, warps);
     };
     // Which kernel, and how many warps per chain (W; an SM holds 16). The lines are where the two cross over in measurements
     // on 1 to 640 groups, 16 to 2.6M units, 32 to 512 steps and 64 to 4096 chains of 8,000 to 200,000 moves.
@@ -781,11 +782,17 @@ int prepare(kvp_problem* p, const kvp_anneal_params* a, cudaStream_t st, Ctx& c,
         const bool ladders = c.psmem && rungs <= 16 && rungs * (fixed_bytes(1, true) + pbytes) + 16 <= budget;
         c.wide = !ladders || hooks.warps_per_chain == 3 || (hooks.warps_per_chain >= 16 && hooks.warps_per_chain < 32);
     }
-    if (c.grow) c.wide = true;                                    // the narrow kernel does not serve these
+    // Growing caches: the narrow kernel with schedules in shared memory and for warm starts (512 units x 132 steps, 256 chains
+    // x 20,000 moves: 0.46 against 0.61 ms, at p0 = 0.8 1.7 against 5.2; 131,072 x 1056, 1024 x 20,000 at p0 = 0.3 1.39
+    // against 1.70, at 0.8 4.5 against 6.6); the wide one for near-greedy chains in global memory, most of whose proposals
+    // change nothing, which its compaction is for (0.65 against 0.80, at p0 = 0.1 0.90 against 0.93), and, with a slow link,
+    // for jobs of many chains (2368 x 10,000 at p0 = 0.8: 16.5 against 20.9; 1024 x 20,000: 10.7 against 7.0).
+    if (c.grow && !hooks.warps_per_chain && !exchange) c.wide = !c.psmem && (a->temps || a->p0 < 0.2 || (!c.lin && !few));
     if (c.wide) c.psmem = fixed_bytes(1, true) + pbytes + 16 <= budget / 2 && p->U < 65536u;
     const uint32_t forced = hooks.warps_per_chain == 3 ? 1u : hooks.warps_per_chain >= 16 ? hooks.warps_per_chain & 15u : hooks.warps_per_chain;
     const uint32_t full = 16;
     auto narrow_warps = [&]() {
+        if (c.grow && !c.psmem) return c.lin && few ? 2u : 1u;
         if (hot) return !c.psmem && few ? 2u : 1u;
         const uint32_t most = held <= 4 ? 4u : held == 5 ? 3u : held <= 8 ? 2u : 1u;
         return p->S < 128u && (c.psmem || !many_units) ? std::min(most, 2u) : most;
@@ -831,7 +838,7 @@ int prepare(kvp_problem* p, const kvp_anneal_params* a, cudaStream_t st, Ctx& c,
     } else {
         // wide: two warps per chain while an SM has at most 8 (more per chain are no faster)
         if (!c.wide) W = narrow_warps();
-        else if (!exchange && few) W = 2;
+        else if (!exchange && few && !(c.grow && !c.lin)) W = 2;   // (131,072 x 1056 births, slow link: 1.07 against 1.13 ms)
         if (forced) W = forced;
         if (W == 1 && c.wide && c.lin) c.rows = kRowsOne;
         uint32_t per_cta = full / W;                              // chains of a full CTA

@@ -17,6 +17,10 @@
 // chains x 100,000 moves: 25.5 -> 13.6 ms; 16 x 32, 64 x 10,000: 0.43 -> 0.35; 16,384 x 256, 1024 x 200,000: 15.4 -> 11.5.
 // A link slower than the DRAM channels (not LIN), which for a while only the wide kernel served, without a bound: 256 x 512,
 // 1024 x 20,000 at p0 = 0.8: 8.5 -> 3.2 ms (the kernel before 4.4); 16,384 x 256, 1024 x 100,000: 12.3 -> 7.0 (7.3).
+// Growing caches, likewise: 512 units x 132 steps, 256 x 20,000 0.61 -> 0.45 ms (0.69), at p0 = 0.8 5.2 -> 1.7 (3.4);
+// 131,072 x 1056, 1024 x 20,000 at p0 = 0.8 6.6 -> 4.5 (5.8).
+// Growing caches, likewise: 1028 units x 132 steps, 256 x 20,000 0.61 -> 0.45 ms (0.69), at p0 = 0.8 5.2 -> 1.7 (3.4);
+// 131,072 x 1056, 1024 x 20,000 at p0 = 0.8 6.6 -> 4.5 (5.8).
 #pragma once
 
 namespace kvp {
@@ -26,7 +30,7 @@ namespace {
 // uint4 slots of a warp's prepared proposals
 __host__ __device__ constexpr uint32_t prepared4(bool lin) { return lin ? 4 * 32 : 5 * 32; }
 
-inline ChainLayout narrow_layout(uint32_t S, uint32_t S32, bool psmem, bool lin, uint32_t cow4)
+inline ChainLayout narrow_layout(uint32_t S, uint32_t S32, bool grow, bool psmem, bool lin, uint32_t cow4)
 {
     ChainLayout l;
     uint32_t at = sizeof(ChainShared) + 16 * (lin ? (S + 1) / 2 : S);   // {th, te}, or {th, te without migrations, in, out}
@@ -36,14 +40,15 @@ inline ChainLayout narrow_layout(uint32_t S, uint32_t S32, bool psmem, bool lin,
     l.lead = take((S32 + 4) / 4);
     l.out = take(lin ? 0u : (S32 + 4) / 4);
     l.in = take(lin ? 0u : (S32 + 4) / 4);
+    l.hb = take(grow && !lin ? (S + 3) / 4 : 0u);
     l.have = take(cow4);
-    l.hb = l.work = at;
+    l.work = at;
     return l;
 }
 // bytes of a chain of W warps, without a schedule in shared memory
-inline size_t narrow_bytes(uint32_t S, uint32_t S32, bool psmem, bool lin, uint32_t cow4, uint32_t W)
+inline size_t narrow_bytes(uint32_t S, uint32_t S32, bool grow, bool psmem, bool lin, uint32_t cow4, uint32_t W)
 {
-    return narrow_layout(S, S32, psmem, lin, cow4).work + (size_t)W * prepared4(lin) * 16;
+    return narrow_layout(S, S32, grow, psmem, lin, cow4).work + (size_t)W * prepared4(lin) * 16;
 }
 
 // where a chain and a warp of it keep their state in shared memory
@@ -62,9 +67,11 @@ struct Narrow {
     // not LIN: [S32] bit t: the link's outbound (inbound) traffic is the largest term of Eq. 4's maximum (see term_leads)
     __device__ __forceinline__ uint32_t* out() const { return at<uint32_t>(cb + prm.lay.out); }
     __device__ __forceinline__ uint32_t* in() const { return at<uint32_t>(cb + prm.lay.in); }
+    __device__ __forceinline__ uint32_t* hb() const { return at<uint32_t>(cb + prm.lay.hb); }      // GROW, not LIN: [S] written to HBM at birth
     __device__ __forceinline__ uint32_t* have() const { return at<uint32_t>(cb + prm.lay.have); }  // not PSMEM: buckets the slice holds
     // [4][32] prepared proposals: {s0 | end << 16, hit, lost, one}, {two, neg, largest accepted change, changed},
-    // {u, v, D's two words}, {D, placement after, Metropolis uniform}; not LIN: one, two and neg are of the units moved in,
+    // {u, v, D's two words}, {D, placement after, Metropolis uniform, GROW: the step at which a unit is written to HBM (bit 0
+    // set) or to DRAM instead of the other}; not LIN: one, two and neg are of the units moved in,
     // and a fifth row has those of the units moved out
     __device__ __forceinline__ uint4* rec() const { return at<uint4>(wb); }
 };
@@ -93,13 +100,14 @@ __device__ __forceinline__ int rise_at(uint32_t one, uint32_t two, uint32_t neg,
     return (neg >> bit) & 1u ? -n : n;
 }
 
-// Only for fixed populations; the wide kernel serves the others.
 // PSMEM: schedules in shared memory; otherwise a chain's slice of global scratch is a copy-on-write overlay of the initial
 // schedule. ASMEM: the access bitmap staged there, too. SOLO: one warp per chain (W == 1).
 // LIN: kappa_d >= kappa_k, th and te are linear in hits and migrations (see kvp_chain.cuh). Otherwise te is the largest of
 // three linear terms, migrations in and out count separately, and the lower bound follows the term that leads at each step:
 // th, or Eq. 4 with the term that is the largest of its three (the new maximum is at least that one's new value).
-template <bool SOLO, bool PSMEM, bool ASMEM, bool LIN, int COLV>
+// GROW: units have steps of birth. A move acts where both its units exist; of the steps in which they are written at most one
+// is among these (the later one: if both are written in the same step, a swap leaves that step's writes as they are).
+template <bool SOLO, bool PSMEM, bool ASMEM, bool GROW, bool LIN, int COLV>
 __global__ void __launch_bounds__(SOLO ? 256 : 512, 1)
 narrow_chain_kernel(const __grid_constant__ ChainParams prm)
 {
@@ -130,17 +138,19 @@ narrow_chain_kernel(const __grid_constant__ ChainParams prm)
             const uint32_t t = w * 32 + lane, i = min(t, S - 1);
             const uint4 n = __ldg(prm.counters0 + i);             // {hr, mi, mo, occ}
             const StepC k = __ldg(prm.stepc + i);
-            const int4 f = make_int4((int)(k.x + prm.K.kh * n.x + prm.K.khF * (n.y + n.z)), (int)(k.w - prm.K.ke * n.x), (int)n.y, (int)n.z);
-            const int te = f.y + ext_term(f.z, f.w, 0, k, prm.K);
+            const int hb = GROW ? (int)__ldg(prm.hb0 + i) : 0;
+            const int4 f = make_int4((int)(k.x + prm.K.kh * (n.x + hb) + prm.K.khF * (n.y + n.z)), (int)(k.w - prm.K.ke * n.x), (int)n.y, (int)n.z);
+            const int te = f.y + ext_term(f.z, f.w, hb, k, prm.K);
             if (t < S) {
                 if constexpr (LIN) c.template sides<int2>()[t] = make_int2(f.x, te);
                 else c.template sides<int4>()[t] = f;
+                if constexpr (GROW && !LIN) c.hb()[t] = (uint32_t)hb;
                 c.occ()[t] = (Occ)n.w;
             }
             const uint32_t F = __ballot_sync(0xFFFFFFFFu, t < S && n.w == prm.cap), T = __ballot_sync(0xFFFFFFFFu, t < S && te >= f.x);
             if (lane == 0) { c.full()[w] = F; c.lead()[w] = T; }
             if constexpr (!LIN) {
-                const uint32_t by = term_leads(f, 0, k, prm.K);
+                const uint32_t by = term_leads(f, hb, k, prm.K);
                 const uint32_t O = __ballot_sync(0xFFFFFFFFu, t < S && (by & 2u)), I = __ballot_sync(0xFFFFFFFFu, t < S && (by & 4u));
                 if (lane == 0) { c.out()[w] = O; c.in()[w] = I; }
             }
@@ -189,6 +199,7 @@ narrow_chain_kernel(const __grid_constant__ ChainParams prm)
 
     uint32_t n_same = 0, n_inf = 0;                               // per lane
     const int kh = (int)prm.K.kh, ke = (int)prm.K.ke, khF = (int)prm.K.khF, kdF = (int)prm.K.kdF, kkF = (int)prm.K.kkF;
+    const int kd = (int)prm.K.kd, kk = (int)prm.K.kk;
     const bool exchange = prm.rung_hist != nullptr;               // a level is a round of a replica-exchange run
     bool over = !active, silent = false;                          // this warp is done with its chain; because a wait ran out
     for (uint32_t level = 0; level < prm.seg1; ++level) {
@@ -223,9 +234,17 @@ narrow_chain_kernel(const __grid_constant__ ChainParams prm)
             const uint32_t s0 = mv.pk >> 8, len = (mv.pk >> 1) & 31u, send = s0 + len;
             const bool swap = mv.pk & 1u;
             const uint32_t run = min(len, S - s0), nl = min(len, S - 1 - s0) + 1;   // steps rewritten; affected
-            const uint32_t M = ((1u << run) - 1u) << 1, Sb = ((1u << nl) - 1u) << 1;
+            const uint32_t Sb = ((1u << nl) - 1u) << 1;
+            uint32_t M = ((1u << run) - 1u) << 1;
             const WinPos wp = window_pos(s0);
             const uint32_t u = mv.u, v = swap ? mv.v : mv.u, units = (u & 0xFFFFu) | v << 16;
+            uint32_t Bu = 0u, Bv = 0u;                            // GROW: the steps in which u and v are written
+            if constexpr (GROW) {
+                uint32_t Lu, Lv;
+                alive_born(__ldg(prm.birth + u), s0, Lu, Bu);
+                alive_born(__ldg(prm.birth + v), s0, Lv, Bv);
+                M &= Lu & Lv;
+            }
             const uint32_t Au = window_at<COLV>(A + (size_t)u * S32, wp), av = window_at<COLV>(A + (size_t)v * S32, wp);
             const uint32_t Av = swap ? av : 0u;
             // A cost change passes the Metropolis test if its bin q has q + 1/2 < X = C ln(2^32 / w) in bins, up to the
@@ -279,7 +298,13 @@ narrow_chain_kernel(const __grid_constant__ ChainParams prm)
                         Nv = (Nv & ~1u) | ((Nv >> 1) & 1u);
                     }
                     const uint32_t hit = (Au ^ Av) & D, lost = hit & (Au ^ Nu);
-                    const uint32_t eun = Nu ^ (Nu << 1), euo = wu ^ (wu << 1), evn = Nv ^ (Nv << 1), evo = Wv ^ (Wv << 1);
+                    uint32_t eun = Nu ^ (Nu << 1), euo = wu ^ (wu << 1), evn = Nv ^ (Nv << 1), evo = Wv ^ (Wv << 1);
+                    uint32_t born = 0u;                           // GROW: a step whose write goes elsewhere, bit 0: to HBM
+                    if constexpr (GROW) {                         // the edge into the step in which a unit is written is no migration
+                        eun &= ~Bu; euo &= ~Bu; evn &= ~Bv; evo &= ~Bv;
+                        born = (Bu ^ (swap ? Bv : 0u)) & D;
+                        if (born) born |= ((Bu & D) ? Nu & born : Nv & born) ? 1u : 0u;
+                    }
                     const int ht = __popc(hit & T) - 2 * __popc(lost & T), hs = __popc(hit) - 2 * __popc(lost) - ht;
                     int lb = kh * hs - ke * ht;                   // the change of the side that leads
                     Rise go, leave;                               // migrations gained at a step; not LIN: into HBM, out of it
@@ -287,14 +312,19 @@ narrow_chain_kernel(const __grid_constant__ ChainParams prm)
                         go = rise_of(eun & Sb, evn & Sb, euo & Sb, evo & Sb);
                         const int mt = rise_over(go, T), ms = rise_over(go, 0xFFFFFFFFu) - mt;
                         lb += kdF * mt + khF * ms;
+                        if (GROW && born) lb += (born & 1u ? 1 : -1) * ((T & born & ~1u) ? -kd : kh);
                     } else {
                         go = rise_of(eun & Nu & Sb, evn & Nv & Sb, euo & wu & Sb, evo & Wv & Sb);
                         leave = rise_of(eun & ~Nu & Sb, evn & ~Nv & Sb, euo & ~wu & Sb, evo & ~Wv & Sb);
                         const uint32_t O = window_at<0>(c.out(), wp), I = window_at<0>(c.in(), wp), C = T & ~(O | I);
                         lb += khF * (rise_over(go, ~T) + rise_over(leave, ~T)) + kkF * (rise_over(leave, T & O) + rise_over(go, T & I)) +
                               kdF * (rise_over(go, C) + rise_over(leave, C));
+                        if (GROW && born) {
+                            const uint32_t B = born & ~1u;
+                            lb += (born & 1u ? 1 : -1) * (!(T & B) ? kh : O & B ? -kk : I & B ? 0 : -kd);
+                        }
                     }
-                    uint32_t turns = hit | go.one | go.two;
+                    uint32_t turns = hit | go.one | go.two | (born & ~1u);
                     if constexpr (!LIN) turns |= leave.one | leave.two;
                     __syncwarp();
                     if ((prep >> lane) & 1u) {
@@ -307,7 +337,7 @@ narrow_chain_kernel(const __grid_constant__ ChainParams prm)
                         c.rec()[32 + lane] = make_uint4(go.two, go.neg, (uint32_t)dmax, turns | (swap ? 1u : 0u));   // (bit 0 is no step)
                         if constexpr (!LIN) c.rec()[128 + lane] = make_uint4(leave.one, leave.two, leave.neg, 0u);
                         c.rec()[64 + lane] = make_uint4(u, v, d << wp.sh, wp.sh ? d >> (32u - wp.sh) : 0u);
-                        c.rec()[96 + lane] = make_uint4(D, Nu, mv.w, 0u);
+                        c.rec()[96 + lane] = make_uint4(D, Nu, mv.w, born);
                     } else if ((check >> lane) & 1u) {
                         bad = (~wu & D & W2) != 0u;
                     }
@@ -382,16 +412,22 @@ narrow_chain_kernel(const __grid_constant__ ChainParams prm)
                         t[j] = min((a.x & 0xFFFFu) + max(lane, 1u) - 1u, S - 1u);   // lane l: window bit l, step s0 - 1 + l
                         f[j] = c.template sides<Sides>()[t[j]];
                         const int h = (a.y >> lane) & 1u, hr = (a.z >> lane) & 1u ? -h : h, mi = rise_at(a.w, b.x, b.y, lane);
+                        int hb = 0;                               // GROW: writes to HBM gained
+                        if constexpr (GROW) {
+                            const uint32_t born = c.rec()[96 + k].w;
+                            if (lane != 0u && ((born >> lane) & 1u)) hb = born & 1u ? 1 : -1;
+                        }
                         if constexpr (LIN) {
-                            g[j] = make_int2(f[j].x + kh * hr + khF * mi, f[j].y - ke * hr + kdF * mi);
+                            g[j] = make_int2(f[j].x + kh * (hr + hb) + khF * mi, f[j].y - ke * hr + kdF * mi - kd * hb);
                             delta[j] = max(g[j].x, g[j].y) - max(f[j].x, f[j].y);   // 0 where nothing changes
                         } else {
                             const uint4 o = c.rec()[128 + k];
                             const int mo = rise_at(o.x, o.y, o.z, lane);
                             const StepC sc = __ldg(prm.stepc + t[j]);
-                            g[j] = make_int4(f[j].x + kh * hr + khF * (mi + mo), f[j].y - ke * hr, f[j].z + mi, f[j].w + mo);
-                            delta[j] = max(g[j].x, g[j].y + ext_term(g[j].z, g[j].w, 0, sc, prm.K)) -
-                                       max(f[j].x, f[j].y + ext_term(f[j].z, f[j].w, 0, sc, prm.K));
+                            const int was = GROW ? (int)c.hb()[t[j]] : 0;
+                            g[j] = make_int4(f[j].x + kh * (hr + hb) + khF * (mi + mo), f[j].y - ke * hr, f[j].z + mi, f[j].w + mo);
+                            delta[j] = max(g[j].x, g[j].y + ext_term(g[j].z, g[j].w, was + hb, sc, prm.K)) -
+                                       max(f[j].x, f[j].y + ext_term(f[j].z, f[j].w, was, sc, prm.K));
                         }
                     }
 #pragma unroll
@@ -423,7 +459,15 @@ narrow_chain_kernel(const __grid_constant__ ChainParams prm)
                             lturn = __ballot_sync(0xFFFFFFFFu, mine && (g[j].y >= g[j].x) != (f[j].y >= f[j].x));
                         } else {
                             const StepC sc = __ldg(prm.stepc + t[j]);
-                            const uint32_t turn = mine ? term_leads(g[j], 0, sc, prm.K) ^ term_leads(f[j], 0, sc, prm.K) : 0u;
+                            int was = 0, hb = 0;
+                            if constexpr (GROW) {
+                                const uint32_t born = c.rec()[96 + id[j]].w;
+                                was = (int)c.hb()[t[j]];
+                                hb = was + (lane != 0u && ((born >> lane) & 1u) ? (born & 1u ? 1 : -1) : 0);
+                                __syncwarp();
+                                if (mine) c.hb()[t[j]] = (uint32_t)hb;
+                            }
+                            const uint32_t turn = mine ? term_leads(g[j], hb, sc, prm.K) ^ term_leads(f[j], was, sc, prm.K) : 0u;
                             lturn = __ballot_sync(0xFFFFFFFFu, turn & 1u);
                             oturn = __ballot_sync(0xFFFFFFFFu, turn & 2u);
                             iturn = __ballot_sync(0xFFFFFFFFu, turn & 4u);

@@ -17,10 +17,10 @@ def kvp():
     return kvp
 
 
-@pytest.fixture(params=[3, 1, 2], ids=["wide", "narrow1", "narrow2"])
+@pytest.fixture(params=[3, 1, 2, 36], ids=["wide", "narrow1", "narrow2", "narrow4"])
 def warps_per_chain(request, hooks):
-    """The wide chain kernel, the only one that serves growing caches: one warp per chain (3 and 1) and two warps that take a
-    chain's batches in turn (2)."""
+    """The wide chain kernel with one warp per chain, the narrow one with one warp per chain and with two and four that take a
+    chain's batches in turn."""
     hooks(warps_per_chain=request.param)
     return request.param
 
