@@ -737,7 +737,6 @@ int prepare(kvp_problem* p, const kvp_anneal_params* a, cudaStream_t st, Ctx& c,
     const bool exchange = rungs != 0;
     const uint32_t chains_per_sm = (a->chains + sms - 1) / sms;
     const size_t pbytes = (size_t)p->U * p->S32 * 4;
-    const bool hot = !a->temps && a->p0 >= 0.5;
     c.lin = p->K.kd >= p->K.kk;
     c.ladder_ctas = c.solo = false;
     c.rows = kRowsMany;
@@ -749,31 +748,35 @@ int prepare(kvp_problem* p, const kvp_anneal_params* a, cudaStream_t st, Ctx& c,
         if (c.wide) return chain_bytes(p->S, p->S32, c.grow, shared, c.lin, shared ? 0u : c.cow_slots4, warps, c.rows);
         return narrow_bytes(p->S, p->S32, c.grow, shared, c.lin, shared ? 0u : c.cow_slots4, warps);
     };
-    // Which kernel, and how many warps per chain (W; an SM holds 16). The lines are where the two cross over in measurements
-    // on 1 to 640 groups, 16 to 2.6M units, 32 to 512 steps and 64 to 4096 chains of 8,000 to 200,000 moves.
-    //  - Hot starts (C_0 from p0 >= 0.5: a fifth of the proposals change the schedule): the narrow kernel. Schedules in
-    //    shared memory: one warp, 13.5 ms on 256 units x 512 steps, 1024 chains x 100,000 moves (two: 22, hand-overs are
-    //    too many; wide kernel: 32). In global memory two warps while an SM has at most 8 chains (equal or 5% better).
-    //  - Otherwise, at most 8 chains per SM: the narrow kernel with as many warps as fit, four at most, two at most on
-    //    short horizons, where moves meet more often (16,384 units x 256 steps, 1024 chains x 200,000 moves: 11.5 against
-    //    14.3 ms; 65,536 x 128, 64 chains x 20,000: 0.48 with four warps, 0.76 with two). But where a batch has few
-    //    proposals to judge, that is with many units, the wide kernel's compaction pays off as soon as an SM has more than
-    //    5 chains (262,144 x 64, 1036 chains x 50,000: 1.33 against 1.77 ms).
-    //  - More chains per SM: the wide kernel with one warp per chain; but the narrow one on schedules in global memory of
-    //    few units, whose chains apply many moves (16,384 x 256, 1480 chains x 20,000: 2.2 against 3.7 ms), and on short
-    //    horizons in shared memory (64 x 64: 0.89 against 1.04 ms; 64 x 512: 0.82 against 0.77).
-    // What counts as chains of an SM is how many it holds at a time, when their schedules take its shared memory.
+    // Which kernel, and how many warps per chain (W; an SM holds 16). Measured on problems of 64 to 524,288 units x 32 to 512
+    // steps, 5 to 20% of the units read per step, 10 to 35% in HBM, even and Zipf importance, 64 to 2368 chains of 10,000 to
+    // 15,000 moves, p0 = 1e-6, 0.03 and 0.3; in brackets what the other choice takes, as geometric mean over such jobs.
+    //  - What decides is how many proposals change the schedule. Many do at a warm start, and at any where the HBM side of Eq. 2
+    //    is the larger one in the static placement (busy): such a schedule gets better by moving units out of HBM, and 2 to 14%
+    //    of a near-greedy chain's first 20,000 proposals change it, elsewhere 0.02 to 1%. Quiet chains with few units in HBM
+    //    (up to a quarter) have few proposals to judge, which the wide kernel's compaction is for.
+    //  - Schedules in shared memory: quiet near-greedy chains, more than 8 per SM: the wide kernel (narrow: 1.10). Everything else
+    //    the narrow one (wide: 1.18 to 2.35; but 0.92 to 0.94 on quiet near-greedy chains up to 8 per SM), from p0 = 0.02 on with
+    //    one warp per chain (two: 1.09 at 0.03, 1.32 at 0.3), below with as many as fit, four at most, two at most on horizons
+    //    below 128 steps, where moves meet more often.
+    //  - In global memory: quiet near-greedy chains, more than 5 per SM: the wide kernel with two warps per chain (narrow: 1.07),
+    //    from 9 per SM on with one (narrow: 1.38). Everything else the narrow one (wide: 2.1 to 2.2 on busy chains, 1.03 to 1.46
+    //    at warm starts), with four warps per chain up to 4 per SM, two up to 8 and one beyond, and two at most on busy chains
+    //    (four: 1.77).
+    // What counts as chains of an SM (held) is how many it holds at a time when their state takes its shared memory, the waves
+    // of the job taken equally large. A ladder given as temperatures is taken for a near-greedy one: what share of the
+    // proposals it accepts is not known (256 x 512, 1024 chains x 100,000 moves with the ladder of p0 = 0.8: 23.3 instead of
+    // 13.6 ms).
     // kvp_set_test_hooks can force the choice (warps_per_chain 1, 2 or 32 + w: narrow; 3 or 16 + w: wide).
-    const bool many_units = p->U >= 32768u;
+    const double p0 = a->temps ? 0.0 : a->p0;
+    const bool busy = (double)p->kh * (double)p->static_hits >= 0.9 * (double)p->ke * (double)(p->total_accessed - p->static_hits);
     c.wide = false;                                               // (for the bytes of a chain)
     c.psmem = fixed_bytes(1, true) + pbytes + 16 <= budget / 2 && p->U < 65536u;
-    uint32_t held = chains_per_sm;
-    if (c.psmem) {
-        const uint32_t fit = (uint32_t)((budget - 16) / (fixed_bytes(1, true) + pbytes));
-        if (held > fit) held = fit > 8 && fit < 12 ? 8u : fit;    // eight with two warps each do more than eleven with one
-    }
-    const bool few = held <= 8;
-    if (!hot) c.wide = c.psmem ? !few && p->S >= 256u : many_units && held > 5;
+    const uint32_t fit = (uint32_t)((budget - 16) / (c.psmem ? fixed_bytes(1, true) + pbytes : fixed_bytes(1, false) + kCowBitsMin / 8));
+    const uint32_t at_a_time = std::min(std::max(fit, 1u), 16u);
+    const uint32_t turns = (chains_per_sm + at_a_time - 1) / at_a_time;
+    const uint32_t held = turns > 1 ? (chains_per_sm + turns - 1) / turns : chains_per_sm;
+    if (!busy && p0 < 0.02 && p->cap <= p->U / 4) c.wide = held > (c.psmem ? 8u : 5u);
     if (hooks.warps_per_chain) c.wide = hooks.warps_per_chain == 3 || (hooks.warps_per_chain >= 16 && hooks.warps_per_chain < 32);
     if (exchange) {
         // Whole ladders in a CTA: every round waits for the hottest rungs, which apply the most moves, and one warp per chain
@@ -787,19 +790,19 @@ int prepare(kvp_problem* p, const kvp_anneal_params* a, cudaStream_t st, Ctx& c,
     // against 1.70, at 0.8 4.5 against 6.6); the wide one for near-greedy chains in global memory, most of whose proposals
     // change nothing, which its compaction is for (0.65 against 0.80, at p0 = 0.1 0.90 against 0.93), and, with a slow link,
     // for jobs of many chains (2368 x 10,000 at p0 = 0.8: 16.5 against 20.9; 1024 x 20,000: 10.7 against 7.0).
-    if (c.grow && !hooks.warps_per_chain && !exchange) c.wide = !c.psmem && (a->temps || a->p0 < 0.2 || (!c.lin && !few));
+    if (c.grow && !hooks.warps_per_chain && !exchange) c.wide = !c.psmem && (p0 < 0.2 || (!c.lin && chains_per_sm > 8));
     if (c.wide) c.psmem = fixed_bytes(1, true) + pbytes + 16 <= budget / 2 && p->U < 65536u;
     const uint32_t forced = hooks.warps_per_chain == 3 ? 1u : hooks.warps_per_chain >= 16 ? hooks.warps_per_chain & 15u : hooks.warps_per_chain;
     const uint32_t full = 16;
     auto narrow_warps = [&]() {
-        if (c.grow && !c.psmem) return c.lin && few ? 2u : 1u;
-        if (hot) return !c.psmem && few ? 2u : 1u;
+        if (c.psmem && (p0 >= 0.02 || (!c.lin && held > 4))) return 1u;
         const uint32_t most = held <= 4 ? 4u : held == 5 ? 3u : held <= 8 ? 2u : 1u;
-        return p->S < 128u && (c.psmem || !many_units) ? std::min(most, 2u) : most;
+        if (c.grow && !c.psmem) return c.lin ? std::min(most, 2u) : 1u;
+        return (c.psmem ? p->S < 128u : busy || p0 >= 0.5) ? std::min(most, 2u) : most;
     };
     uint32_t W = 1;
     if (c.psmem) {
-        uint32_t want = chains_per_sm < 1 ? 1 : chains_per_sm;
+        uint32_t want = held;
         if (exchange) want = (want + rungs - 1) / rungs * rungs;  // whole ladders
         // bytes with the access bitmap staged; columns are followed by readable bytes
         auto with_a = [&](uint32_t chains, uint32_t warps) {
@@ -838,7 +841,7 @@ int prepare(kvp_problem* p, const kvp_anneal_params* a, cudaStream_t st, Ctx& c,
     } else {
         // wide: two warps per chain while an SM has at most 8 (more per chain are no faster)
         if (!c.wide) W = narrow_warps();
-        else if (!exchange && few && !(c.grow && !c.lin)) W = 2;   // (131,072 x 1056 births, slow link: 1.07 against 1.13 ms)
+        else if (!exchange && chains_per_sm <= 8 && !(c.grow && !c.lin)) W = 2;   // (131,072 x 1056 births, slow link: 1.07 against 1.13 ms)
         if (forced) W = forced;
         if (W == 1 && c.wide && c.lin) c.rows = kRowsOne;
         uint32_t per_cta = full / W;                              // chains of a full CTA

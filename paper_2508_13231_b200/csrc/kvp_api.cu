@@ -130,7 +130,8 @@ static int create_impl(kvp_problem* p, const uint32_t* access, const uint32_t* h
     auto take = [&](size_t bytes) { size_t o = off; off += (bytes + 255) & ~(size_t)255; return o; };
     const size_t oA = take(nw * 4), oAcol = take((size_t)p->U * p->S32 * 4);
     const size_t osc = take((size_t)p->S * sizeof(StepC)), orf = take((size_t)p->W32 * 4);
-    const size_t oa = take((size_t)p->S * 4), ouc = take((size_t)p->U * 4), ofr = take(static_freq_words(p) * 4);
+    const size_t hits_at = ((size_t)p->S * 4 + 7) & ~(size_t)7;   // behind |A[s]|: the accesses of the static row
+    const size_t oa = take(hits_at + 8), ouc = take((size_t)p->U * 4), ofr = take(static_freq_words(p) * 4);
     const size_t owr = take(hw || ew ? (size_t)p->S * 8 : 0);
     KVP_CUDA(cudaMallocAsync(&p->d_block, off, st));
     char* base = static_cast<char*>(p->d_block);
@@ -145,12 +146,13 @@ static int create_impl(kvp_problem* p, const uint32_t* access, const uint32_t* h
     }
     if ((rc = launch_open(p, access, st))) return rc;
     if ((rc = launch_stepc(p->d_stepc, writes, p->d_a, p->S, p->K, st))) return rc;
-    if ((rc = launch_static_freq_row(p, (uint32_t*)(base + ofr), p->d_row_freq, st))) return rc;
-    std::vector<uint32_t> a(p->S);
-    KVP_CUDA(cudaMemcpyAsync(a.data(), p->d_a, (size_t)p->S * 4, cudaMemcpyDeviceToHost, st));
+    if ((rc = launch_static_freq_row(p, (uint32_t*)(base + ofr), p->d_row_freq, (unsigned long long*)(base + oa + hits_at), st))) return rc;
+    std::vector<uint32_t> a(hits_at / 4 + 2);
+    KVP_CUDA(cudaMemcpyAsync(a.data(), p->d_a, hits_at + 8, cudaMemcpyDeviceToHost, st));
     KVP_CUDA(cudaStreamSynchronize(st));                 // the host vectors go out of scope
     p->total_accessed = 0;
     for (uint32_t s = 0; s < p->S; ++s) p->total_accessed += a[s];
+    memcpy(&p->static_hits, a.data() + hits_at / 4, 8);
     return KVP_OK;
 }
 

@@ -123,6 +123,7 @@ struct kvp_problem {
     uint32_t* d_ucnt;    // [U]        accesses per unit over all steps
     uint32_t* d_row_freq;// [W32]      STATIC_FREQ row
     uint64_t total_accessed;
+    uint64_t static_hits;      // of them, those that the STATIC_FREQ row serves (units there from the start)
     // growing cache (kvp_set_births); all null for a fixed population
     uint32_t* d_birth;   // [U]        step at which a unit is written, 0 = there from the start
     uint32_t* dL;        // [S][W32]   bit u of row s set iff unit u exists at step s
@@ -171,7 +172,7 @@ int launch_clean_copy(const uint32_t* in, uint32_t* out, uint32_t S, uint32_t W3
 int launch_open(const kvp_problem* p, const uint32_t* access, cudaStream_t st);
 int launch_stepc(StepC* stepc, const uint32_t* writes, const uint32_t* a, uint32_t S, const CostK& K, cudaStream_t st);
 size_t static_freq_words(const kvp_problem* p);
-int launch_static_freq_row(const kvp_problem* p, uint32_t* scratch, uint32_t* row, cudaStream_t st);
+int launch_static_freq_row(const kvp_problem* p, uint32_t* scratch, uint32_t* row, unsigned long long* hits, cudaStream_t st);
 int launch_static_first_row(const kvp_problem* p, uint32_t* row, cudaStream_t st);
 int launch_broadcast_row(const uint32_t* row, uint32_t S, uint32_t W32, uint32_t* sched, cudaStream_t st);
 int launch_initial_schedule(const kvp_problem* p, const uint32_t* row, uint32_t* sched, uint32_t* Pcol, cudaStream_t st);

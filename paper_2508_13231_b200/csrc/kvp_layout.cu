@@ -146,11 +146,11 @@ __global__ void stepc_kernel(StepC* __restrict__ stepc, const uint32_t* __restri
 //
 // First, a histogram of the counts (bins 0..S). Few bins and millions of units: every CTA counts its units in shared
 // memory (when the bins fit) and adds only its non-empty bins to the global histogram. The last CTA then finds the
-// threshold: sel = {threshold count, number of ties to take}.
+// threshold: sel = {threshold count, number of ties to take}, and with it the row's accesses over all steps (hits).
 constexpr uint32_t kHistBins = 8192;
 __global__ void __launch_bounds__(1024)
 static_threshold_kernel(const uint32_t* __restrict__ ucnt, uint32_t U, uint32_t S, uint32_t cap, uint32_t* __restrict__ hist,
-                        uint32_t* __restrict__ sel, uint32_t* __restrict__ ticket)
+                        uint32_t* __restrict__ sel, uint32_t* __restrict__ ticket, unsigned long long* __restrict__ hits)
 {
     __shared__ uint32_t local[kHistBins];
     __shared__ uint32_t s_thr, s_take, s_found, s_last;
@@ -179,6 +179,7 @@ static_threshold_kernel(const uint32_t* __restrict__ ucnt, uint32_t U, uint32_t 
     // counts run 0..S; descend, 1024 counts at a time (thread i looks at count top - i), until the capacity is reached
     if (cap != 0) {
         uint32_t above = 0;                               // units with a count above this chunk
+        unsigned long long got = 0;                       // accesses of the units this thread's counts contribute
         for (int64_t top = S; top >= 0; top -= 1024) {
             const int64_t c = top - (int64_t)threadIdx.x;
             const uint32_t h = c >= 0 ? __ldcg(hist + c) : 0u;
@@ -198,12 +199,16 @@ static_threshold_kernel(const uint32_t* __restrict__ ucnt, uint32_t U, uint32_t 
             }
             incl += before + above;
             const uint32_t excl = incl - h;
+            if (c > 0 && excl < cap) got += (unsigned long long)c * (min(incl, cap) - excl);
             if (c >= 0 && excl < cap && incl >= cap) { s_thr = (uint32_t)c; s_take = cap - excl; s_found = 1; }   // one thread at most
             __syncthreads();
             if (s_found) break;
             above += total;
             __syncthreads();
         }
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) got += __shfl_xor_sync(0xFFFFFFFFu, got, off);
+        if (lane == 0 && got) atomicAdd(hits, got);
     }
     if (threadIdx.x == 0) { sel[0] = s_thr; sel[1] = s_take; }
 }
@@ -427,8 +432,8 @@ size_t static_freq_words(const kvp_problem* p)
 }
 
 // scratch: static_freq_words, of which the first S + 2 are zero: the histogram (S + 1 bins), the ticket of the first kernel,
-// the selection (2 words) and the tie counts of the chunks
-int launch_static_freq_row(const kvp_problem* p, uint32_t* scratch, uint32_t* row, cudaStream_t st)
+// the selection (2 words) and the tie counts of the chunks. hits (zero before): the accesses of the row's units over all steps
+int launch_static_freq_row(const kvp_problem* p, uint32_t* scratch, uint32_t* row, unsigned long long* hits, cudaStream_t st)
 {
     uint32_t* hist = scratch;
     uint32_t* sel = hist + ((p->S + 2 + 3) & ~3u);
@@ -436,7 +441,7 @@ int launch_static_freq_row(const kvp_problem* p, uint32_t* scratch, uint32_t* ro
     const uint32_t span = static_span(p), chunks = (p->W32 * 32 + 32 * span - 1) / (32 * span);
     uint32_t hgrid = (p->U + 8191) / 8192;
     if (hgrid > 148) hgrid = 148;
-    static_threshold_kernel<<<hgrid, 1024, 0, st>>>(p->d_ucnt, p->U, p->S, p->cap, hist, sel, hist + p->S + 1);
+    static_threshold_kernel<<<hgrid, 1024, 0, st>>>(p->d_ucnt, p->U, p->S, p->cap, hist, sel, hist + p->S + 1, hits);
     KVP_CUDA(cudaGetLastError());
     static_ties_kernel<<<chunks, 1024, 0, st>>>(p->d_ucnt, sel, p->U, span, ties);
     KVP_CUDA(cudaGetLastError());

@@ -93,6 +93,31 @@ def test_exchange_rounds(kvp, oracle, hooks, warps, chains, rungs):
     assert np.array_equal(to_np(out["best_schedule"]), ref["best_schedule"])
 
 
+@pytest.mark.parametrize("busy", [False, True])
+@pytest.mark.parametrize("p0,init", [(1e-6, 1), (1e-6, 0), (0.3, 1)])
+def test_choice_in_global_memory(kvp, oracle, busy, p0, init):
+    """The library's own choice between the kernels: by the start temperature and by which side of Eq. 2 is the larger one in
+    the most-accessed placement, whatever placement the chains start from. Both give the oracle's chains."""
+    U, S, cap = 16384, 64, 1600
+    A = wl.random_access(U, S, 0.05, seed=4)
+    if busy:
+        rng = np.random.default_rng(3)
+        hot = rng.permutation(U) < 1700                       # the same tenth of the units at every step, most of it in HBM
+        A = wl.pack_bits(np.broadcast_to(hot, (S, U)) & (rng.random((S, U)) < 0.95))
+    g, o = both_problems(kvp, oracle, U, 8192, S, A, cap, (8000 * GB, 900 * GB, 900 * GB))
+    ratio = g.weights["kh"] / g.weights["ke"]
+    counts = g.eval_counts(g.chain_state(g.make_params(1, 1, temps=[1.0], levels=1), 0, 0)[0])[0].cpu().numpy().astype(np.int64)
+    hits, reads = counts[:, 0].sum(), wl.unpack_bits(A, U).sum(dtype=np.int64)
+    assert (hits * ratio >= 0.9 * (reads - hits)) == busy
+    kw = dict(chains=1184, moves=400, seed=2, levels=4, p0=p0, init_mode=init)
+    out = g.anneal(g.make_params(**kw), want_per_chain=True)
+    assert out["stats"].wide_kernel == (0 if busy or p0 > 0.1 else 1)
+    op = o.make_params(**kw)
+    for c in (0, 591, 1183):
+        want, _, _ = o.anneal_chains(op, c, 1)
+        assert out["per_chain"][c].astuple() == want[0].astuple(), c
+
+
 @pytest.mark.parametrize("scale", [1, 2 ** 10, 2 ** 20])
 def test_accept_table_rows(kvp, oracle, scale):
     """Rows built as geometric sequences against exp() for every entry, at temperatures around powers of two."""
