@@ -803,7 +803,9 @@ int prepare(kvp_problem* p, const kvp_anneal_params* a, cudaStream_t st, Ctx& c,
     uint32_t W = 1;
     if (c.psmem) {
         uint32_t want = held;
-        if (exchange) want = (want + rungs - 1) / rungs * rungs;  // whole ladders
+        // whole ladders, where a CTA can hold one (256 x 512, 92 ladders of 11, which it cannot: 93 CTAs of 11 chains would
+        // leave a third of the SMs idle)
+        if (exchange && rungs <= full && rungs * (fixed_bytes(1, true) + pbytes) + 16 <= budget) want = (want + rungs - 1) / rungs * rungs;
         // bytes with the access bitmap staged; columns are followed by readable bytes
         auto with_a = [&](uint32_t chains, uint32_t warps) {
             const size_t a_off = ((size_t)chains * (pbytes / 4) + 3) & ~(size_t)3, c_off = (a_off + pbytes / 4 + 3) & ~(size_t)3;
@@ -811,8 +813,10 @@ int prepare(kvp_problem* p, const kvp_anneal_params* a, cudaStream_t st, Ctx& c,
         };
         if (c.wide) {
             // two warps per chain, four where an SM has three chains or fewer (256 units x 512 steps, 50,000 moves, 148 and
-            // 740 chains: one warp 1.62 and 1.79 ms, two 1.12 and 1.34, four 1.05 and 2.40)
+            // 740 chains: one warp 1.62 and 1.79 ms, two 1.12 and 1.34, four 1.05 and 2.40); half of that for replica exchange,
+            // whose hot rungs apply many moves (20 rungs, 200 and 1020 chains x 50,000: one 5.01 and 5.54, two 4.73 and 5.65)
             W = chains_per_sm <= 3 ? 4 : 2;
+            if (exchange) W /= 2;
             while (W > 1 && (want * W > full || with_a(want, W) > budget)) W /= 2;
         } else {
             W = exchange ? 1u : narrow_warps();
