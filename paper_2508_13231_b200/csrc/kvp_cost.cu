@@ -1,7 +1,7 @@
 // Cost kernels: per-step cardinalities of a schedule (popc over mask AND placement words) and Eq. 1-5.
 //
-// Three forms. Small schedules, where launches and latency are all there is: score_kernel, one CTA per schedule, groups of
-// lanes own whole rows, everything in one launch. Large ones, HBM-bound: count_wide_kernel, in which a warp owns 64
+// Four forms. Small schedules, where launches and latency are all there is: score_kernel, one CTA per schedule, groups of
+// lanes own whole rows, everything in one launch; score_long_kernel, the same where they have many steps. Large ones, HBM-bound: count_wide_kernel, in which a warp owns 64
 // consecutive 16-byte vectors of every row of a step chunk, carries P[s-1] in registers (every word of A and P is read once)
 // and adds its per-step counts to global counters; the last CTA of a schedule, or a second launch, turns them into ticks.
 // Large batches: count_staged_kernel, the same with rows fetched ahead into shared memory.
@@ -454,14 +454,107 @@ score_kernel(const uint32_t* __restrict__ A, const uint32_t* __restrict__ Ps, ui
     if (out.stepc) score_total(out, i, sum);
 }
 
+// The same for schedules of many steps whose rows take 8 lanes or more (and a vector per lane at most). There the lanes that
+// hold a row's counts, one in LPR, are too few to score it: the counts go to shared memory, kChunk rows at a time, and every
+// thread scores a row. (400 schedules of 2048 units x 2048 steps: 165 -> 89 us, 1024 of 416 x 512: 56 -> 38, 6 of 416 x 2048:
+// 35 -> 19; with rows that follow one another in a group, P[s-1] in registers, 155, and 19: too many streams at a time.)
+constexpr uint32_t kChunk = 1024;
+template <int VEC, bool GROW>
+__global__ void __launch_bounds__(1024)
+score_long_kernel(const uint32_t* __restrict__ A, const uint32_t* __restrict__ Ps, uint32_t S, uint32_t W32, uint32_t WV, uint32_t LPR,
+                  uint32_t pad_mask, const uint32_t* __restrict__ L, uint32_t* __restrict__ counts, uint32_t* __restrict__ hbc, const ScoreOut out)
+{
+    __shared__ uint4 s_counts[kChunk];
+    __shared__ uint32_t s_hb[GROW ? kChunk : 1];
+    const uint32_t groups = blockDim.x / LPR, g = threadIdx.x / LPR, l = threadIdx.x % LPR, i = blockIdx.x;
+    const uint32_t* __restrict__ P = Ps + (size_t)i * S * W32;
+    const bool mine = l < WV;
+    const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
+    auto count = [](uint4 v) {
+        if (VEC == 1) return (uint32_t)__popc(v.x);
+        uint32_t twos, ones;
+        csa(twos, ones, v.x, v.y, v.z);
+        return (uint32_t)(__popc(ones) + 2 * __popc(twos) + __popc(v.w));
+    };
+    auto row = [&](const uint32_t* m, uint32_t s) { return mine ? load_vec<VEC>(m, W32, s, l) : zero; };
+    ScoreSum sum;
+    for (uint32_t c0 = 0; c0 < S; c0 += kChunk) {
+        const uint32_t rows = min(kChunk, S - c0);
+#pragma unroll 4
+        for (uint32_t r0 = 0; r0 < rows; r0 += groups) {          // (all lanes of a warp go through the sums)
+            const uint32_t r = r0 + g, s = min(c0 + r, S - 1), sp = s ? s - 1 : 0;   // rows beyond the chunk: counted and dropped
+            const uint4 a = row(A, s);
+            uint4 p = mask_last<VEC>(row(P, s), l, WV, pad_mask), q = mask_last<VEC>(row(P, sp), l, WV, pad_mask);
+            uint32_t hb = 0;
+            if (GROW) {
+                const uint4 lq = row(L, sp);
+                p = and4(p, row(L, s));
+                q = and4(q, lq);
+                hb = count(andn4(p, lq));                         // written in HBM, not migrated in
+            }
+            uint32_t x = count(and4(a, p)) | (count(andn4(p, q)) - hb) << 16, y = count(andn4(q, p)) | count(p) << 16;   // at most 4096 each
+            for (uint32_t off = LPR / 2; off > 0; off >>= 1) {
+                x += __shfl_xor_sync(0xFFFFFFFFu, x, off);
+                y += __shfl_xor_sync(0xFFFFFFFFu, y, off);
+                if (GROW) hb += __shfl_xor_sync(0xFFFFFFFFu, hb, off);
+            }
+            if (l == 0 && r < rows) {
+                s_counts[r] = make_uint4(x & 0xFFFFu, x >> 16, y & 0xFFFFu, y >> 16);
+                if (GROW) s_hb[r] = hb;
+            }
+        }
+        __syncthreads();
+        for (uint32_t r = threadIdx.x; r < rows; r += blockDim.x) {
+            const uint4 c = s_counts[r];
+            const uint32_t hb = GROW ? s_hb[r] : 0u;
+            if (counts) reinterpret_cast<uint4*>(counts)[(size_t)i * S + c0 + r] = c;
+            if (GROW && hbc) hbc[(size_t)i * S + c0 + r] = hb;
+            if (out.stepc) score_step<GROW>(out, i, S, c0 + r, c, hb, sum);
+        }
+        __syncthreads();
+    }
+    if (out.stepc) score_total(out, i, sum);
+}
+
 }  // namespace
 
-// A schedule is small when one CTA is done with it before a grid of CTAs would have started: up to 512 KB (of one SM's some
-// 200 GB/s, beside a second and a third launch). Many of them with long rows go to the streaming kernel, which reads P once.
+// lanes of a row in score_kernel
+static uint32_t lanes_per_row(uint32_t WV)
+{
+    uint32_t n = 1;
+    while (n < 32 && n < WV) n *= 2;
+    return n;
+}
+
+// threads of score_kernel and score_long_kernel: one CTA per SM or fewer: as many rows side by side as there are; many CTAs:
+// smaller ones. lots: which of the two.
+static uint32_t score_threads(const kvp_problem* p, uint32_t n, uint32_t WV, uint32_t LPR, bool* lots)
+{
+    const uint64_t lanes = (uint64_t)p->S * LPR;
+    uint32_t T = (uint32_t)std::min<uint64_t>(n <= 148 ? 1024 : 256, (lanes + 31) / 32 * 32);
+    *lots = LPR >= 8 && WV <= LPR && lanes >= 8ull * T;
+    if (*lots && n > 148 && n <= 4 * 148) T = 512;
+    return T;
+}
+
+// Schedules are small when a CTA for each is done with them before the streaming kernel would be. Both estimates in us, from 721
+// batches of 1 to 1024 schedules of 32 to 2048 steps x 1 to 2048 words (the choice takes 1.2 times the better kernel's time at
+// most, but for two of them; 6 x 6816 units x 512 steps: one CTA each 43.3, streaming 9.9; 148 x 8192 x 128: 12.8, 40.2):
+//  - one CTA each: the launch, then by rounds of its threads, longer when the SMs hold more than 1024 threads; at most 2 TB/s;
+//  - streaming: the launch and the clearing of the counters, then by steps of a schedule: rows narrower than a CTA's tile (2048
+//    words in vectors, 512 in single words) cost as much as a tile.
+// Beyond 512 KB a schedule whose rows take a CTA's lanes several times round is no work for one SM (64 x 16,384 x 2048: 239, 173).
 static bool is_small(const kvp_problem* p, uint32_t n)
 {
-    const size_t bytes = (size_t)p->S * p->W32 * 4;
-    return (bytes <= (512u << 10) && (p->W32 <= 64 || n * bytes <= ((size_t)16 << 20))) || (p->W32 <= 64 && n >= 148);
+    const bool vec4 = p->W32 % 4 == 0;
+    const uint32_t WV = vec4 ? p->W32 / 4 : p->W32, LPR = lanes_per_row(WV), per_sm = (n + 147) / 148;
+    bool lots;
+    const uint32_t T = score_threads(p, n, WV, LPR, &lots);
+    const double steps = (double)n * p->S, rounds = (double)(((uint64_t)p->S * LPR + T - 1) / T), more = (WV + LPR - 1) / LPR - 1;
+    const double round = lots ? (vec4 ? 0.7 : 0.53) : vec4 ? 1.1 + 0.5 * more : 0.95 + 0.25 * more;
+    const double one = 4.0 + std::max(rounds * round * std::max(1.0, per_sm * T / 1024.0), steps * p->W32 * 2e-6);
+    const double streaming = 9.5 + steps * (vec4 ? std::max(1.3e-3, 1.4e-6 * p->W32) : 0.47e-3 * ((p->W32 + 511) / 512));
+    return one <= streaming && (more == 0 || (size_t)p->S * p->W32 * 4 <= (512u << 10));
 }
 
 size_t score_scratch_bytes(const kvp_problem* p, uint32_t n)
@@ -471,20 +564,19 @@ size_t score_scratch_bytes(const kvp_problem* p, uint32_t n)
 
 // counts [n][S][4] = {hr, mi, mo, occ}, or null if score_scratch_bytes(p, n) is 0; hbc [n][S] for a problem with births,
 // likewise; tickets [n] behind counts and hbc, or null. out.stepc null: only the counts are wanted.
-static int launch_score_impl(const kvp_problem* p, const uint32_t* schedules, uint32_t n, uint32_t* counts, uint32_t* hbc,
+static int launch_score_impl(const kvp_problem* p, const uint32_t* schedules, uint32_t n, bool small, uint32_t* counts, uint32_t* hbc,
                              uint32_t* tickets, const ScoreOut& out, cudaStream_t st, uint32_t* launches)
 {
     const bool grow = p->dL != nullptr;
     const bool vec4 = (p->W32 % 4 == 0) && ((reinterpret_cast<uintptr_t>(schedules) & 15) == 0);
     const uint32_t WV = vec4 ? p->W32 / 4 : p->W32;
     if (launches) *launches += 1;
-    if (is_small(p, n)) {
-        uint32_t LPR = 1;
-        while (LPR < 32 && LPR < WV) LPR *= 2;
-        // one CTA per SM or fewer: as many rows side by side as there are; many CTAs: smaller ones
-        uint32_t T = (uint32_t)std::min<uint64_t>(n <= 148 ? 1024 : 256, ((uint64_t)p->S * LPR + 31) / 32 * 32);
+    if (small) {
+        const uint32_t LPR = lanes_per_row(WV);
+        bool lots;
+        const uint32_t T = score_threads(p, n, WV, LPR, &lots);
 #define KVP_SCORE(VEC, GROW) \
-        score_kernel<VEC, GROW><<<n, T, 0, st>>>(p->dA, schedules, p->S, p->W32, WV, LPR, p->pad_mask, p->dL, counts, hbc, out)
+        (lots ? score_long_kernel<VEC, GROW> : score_kernel<VEC, GROW>)<<<n, T, 0, st>>>(p->dA, schedules, p->S, p->W32, WV, LPR, p->pad_mask, p->dL, counts, hbc, out)
         if (grow) { if (vec4) KVP_SCORE(4, true); else KVP_SCORE(1, true); }
         else { if (vec4) KVP_SCORE(4, false); else KVP_SCORE(1, false); }
 #undef KVP_SCORE
@@ -556,9 +648,10 @@ int launch_score(const kvp_problem* p, const uint32_t* schedules, uint32_t n, vo
     uint32_t* counts = static_cast<uint32_t*>(scratch);
     uint32_t* hbc = counts && p->dL ? counts + (size_t)n * p->S * 4 : nullptr;
     uint32_t* tickets = counts ? counts + (size_t)n * p->S * (p->dL ? 5 : 4) : nullptr;
-    if (is_small(p, n)) { counts = counts_out; hbc = hbc_out; }
-    int rc = launch_score_impl(p, schedules, n, counts, hbc, tickets, o, st, launches);
-    if (rc || is_small(p, n)) return rc;
+    const bool small = is_small(p, n);
+    if (small) { counts = counts_out; hbc = hbc_out; }
+    int rc = launch_score_impl(p, schedules, n, small, counts, hbc, tickets, o, st, launches);
+    if (rc || small) return rc;
     if (counts_out && counts_out != counts) KVP_CUDA(cudaMemcpyAsync(counts_out, counts, (size_t)n * p->S * 16, cudaMemcpyDeviceToDevice, st));
     if (hbc_out && hbc && hbc_out != hbc) KVP_CUDA(cudaMemcpyAsync(hbc_out, hbc, (size_t)n * p->S * 4, cudaMemcpyDeviceToDevice, st));
     return KVP_OK;
@@ -568,7 +661,7 @@ int launch_counts(const kvp_problem* p, const uint32_t* schedules, uint32_t n, u
 {
     ScoreOut none;
     memset(&none, 0, sizeof none);
-    return launch_score_impl(p, schedules, n, counts, nullptr, nullptr, none, st, nullptr);
+    return launch_score_impl(p, schedules, n, is_small(p, n), counts, nullptr, nullptr, none, st, nullptr);
 }
 
 }  // namespace kvp

@@ -119,6 +119,23 @@ def test_eval_growing(kvp, oracle, layers, heads, n, prompt):
         g.close()
 
 
+@pytest.mark.parametrize("layers,heads,n,prompt", [(17, 1, 40, 0), (32, 1, 40, 8)], ids=["single words", "vectors"])
+def test_eval_growing_batch_of_many_steps(kvp, oracle, layers, heads, n, prompt):
+    """A CTA per schedule, its counts scored by other threads than those that counted."""
+    cfg, groups, U, S, birth = _shape(layers, heads, n, prompt)
+    rng = np.random.default_rng(S)
+    alive = birth[None, :] <= np.arange(S)[:, None]
+    A = wl.pack_bits(((rng.random((S, U)) < 0.2) & alive).astype(np.uint8))
+    g, o = _problems(kvp, oracle, U, 512, S, A, U // 3, (4900 * GB, 900 * GB, 500 * GB), birth)
+    scheds = rng.integers(0, 2 ** 32, (40, S, A.shape[1]), dtype=np.uint64).astype(np.uint32)
+    scheds &= rng.integers(0, 2 ** 32, scheds.shape, dtype=np.uint64).astype(np.uint32)     # a quarter of the bits
+    out = g.eval(to_dev(scheds))
+    for i in (0, 19, 39):
+        ref = o.eval(scheds[i])
+        assert np.array_equal(u64(out["step_ticks"])[i], ref["step_ticks"])
+        assert int(u64(out["total_ticks"])[i]) == ref["total_ticks"] and int(out["bad_step"][i]) == ref["bad_step"]
+
+
 def test_eval_growing_8b(kvp, oracle):
     g, o, cfg, A, birth = _named(kvp, oracle, "growing_8b")
     groups, U, S = wl.growing_shape(cfg)
