@@ -18,6 +18,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <new>
 #include <type_traits>
 #include <vector>
 
@@ -1043,7 +1044,7 @@ using namespace kvp;
 
 extern "C" int kvp_anneal(kvp_problem* p, const kvp_anneal_params* a, uint32_t* best_schedule, uint64_t* best_ticks,
                           double* best_seconds, kvp_anneal_stats* stats, void* stream)
-{
+try {
     Ctx c;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     int rc = validate(p, a);
@@ -1169,11 +1170,13 @@ extern "C" int kvp_anneal(kvp_problem* p, const kvp_anneal_params* a, uint32_t* 
         stats->work_again = work[0]; stats->work_listed = work[1]; stats->work_items = work[2];
     }
     return ok ? KVP_OK : KVP_ERR_INTERNAL;
+} catch (const std::bad_alloc&) {
+    return KVP_ERR_NOMEM;
 }
 
 extern "C" int kvp_anneal_chain_state(kvp_problem* p, const kvp_anneal_params* a, uint32_t chain, uint64_t upto_moves,
                                       uint32_t* schedule, kvp_chain_result* result, void* stream)
-{
+try {
     if (!schedule) return KVP_ERR_ARG;
     Ctx c;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
@@ -1193,6 +1196,8 @@ extern "C" int kvp_anneal_chain_state(kvp_problem* p, const kvp_anneal_params* a
     KVP_CUDA(cudaMemcpyAsync(&gave_up, c.prm.err, 4, cudaMemcpyDeviceToHost, st));
     KVP_CUDA(cudaStreamSynchronize(st));
     return gave_up ? KVP_ERR_TIMEOUT : KVP_OK;
+} catch (const std::bad_alloc&) {
+    return KVP_ERR_NOMEM;
 }
 
 extern "C" void kvp_set_test_hooks(const kvp_test_hooks* hooks)
@@ -1217,7 +1222,7 @@ extern "C" int kvp_exchange_temps(const double* temps, uint32_t rungs, double* p
 extern "C" int kvp_anneal_exchange(kvp_problem* p, const kvp_anneal_params* a, const kvp_exchange_params* xp,
                                    uint32_t* best_schedule, uint64_t* best_ticks, double* best_seconds,
                                    kvp_anneal_stats* stats, uint32_t* final_rung, uint32_t* n_exchanged, void* stream)
-{
+try {
     Ctx c;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     int rc = validate(p, a);
@@ -1377,4 +1382,6 @@ extern "C" int kvp_anneal_exchange(kvp_problem* p, const kvp_anneal_params* a, c
         stats->exchange_rounds = rounds; stats->exchanges_tried = xcounts[0]; stats->exchanges_accepted = xcounts[1];
     }
     return ok ? KVP_OK : KVP_ERR_INTERNAL;
+} catch (const std::bad_alloc&) {
+    return KVP_ERR_NOMEM;
 }

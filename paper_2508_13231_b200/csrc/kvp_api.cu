@@ -4,6 +4,7 @@
 #include <stdlib.h>
 #include <string.h>
 
+#include <new>
 #include <vector>
 
 #include "kvp_common.cuh"
@@ -107,7 +108,7 @@ extern "C" void kvp_destroy(kvp_problem* p)
 }
 
 static int create_impl(kvp_problem* p, const uint32_t* access, const uint32_t* hw, const uint32_t* ew, cudaStream_t st)
-{
+try {
     const size_t nw = (size_t)p->S * p->W32;
     // Everything the cost function adds up must stay below 2^31 so that the annealer can work in 32-bit arithmetic.
     uint64_t wmax = 0;
@@ -154,6 +155,8 @@ static int create_impl(kvp_problem* p, const uint32_t* access, const uint32_t* h
     for (uint32_t s = 0; s < p->S; ++s) p->total_accessed += a[s];
     memcpy(&p->static_hits, a.data() + hits_at / 4, 8);
     return KVP_OK;
+} catch (const std::bad_alloc&) {
+    return KVP_ERR_NOMEM;
 }
 
 extern "C" int kvp_create(kvp_problem** out, uint32_t units, uint64_t bytes_per_unit, uint32_t steps,
@@ -191,7 +194,7 @@ extern "C" int kvp_create(kvp_problem** out, uint32_t units, uint64_t bytes_per_
 }
 
 extern "C" int kvp_set_births(kvp_problem* p, const uint32_t* birth, void* stream)
-{
+try {
     if (!p || !birth || p->dL) return KVP_ERR_ARG;
     KVP_CUDA(cudaSetDevice(p->device));
     cudaStream_t st = static_cast<cudaStream_t>(stream);
@@ -200,13 +203,13 @@ extern "C" int kvp_set_births(kvp_problem* p, const uint32_t* birth, void* strea
     size_t off = 0;
     auto take = [&](size_t bytes) { size_t o = off; off += (bytes + 255) & ~(size_t)255; return o; };
     const size_t ob = take((size_t)p->U * 4), oL = take(nw * 4), onb = take((size_t)p->S * 4 + 4);
+    std::vector<uint32_t> nb((size_t)p->S + 1);
     void* block = nullptr;
     KVP_CUDA(cudaMallocAsync(&block, off, st));
     char* base = static_cast<char*>(block);
     uint32_t* d_birth = (uint32_t*)(base + ob);
     uint32_t* dL = (uint32_t*)(base + oL);
     uint32_t* d_nb = (uint32_t*)(base + onb);            // [S] births per step, then the check flags
-    std::vector<uint32_t> nb((size_t)p->S + 1);
     int rc = KVP_OK;
     auto fail = [&](int code) { cudaFreeAsync(block, st); return code; };
     if (cudaMemcpyAsync(d_birth, birth, (size_t)p->U * 4, cudaMemcpyDeviceToDevice, st) != cudaSuccess ||
@@ -228,6 +231,8 @@ extern "C" int kvp_set_births(kvp_problem* p, const uint32_t* birth, void* strea
     if ((rc = launch_stepc_births(p->d_stepc, d_nb, p->S, p->K.kk, p->K.kd, st))) return fail(rc);
     p->d_grow_block = block; p->d_birth = d_birth; p->dL = dL;
     return KVP_OK;
+} catch (const std::bad_alloc&) {
+    return KVP_ERR_NOMEM;
 }
 
 extern "C" int kvp_get_info(const kvp_problem* p, kvp_info* info)

@@ -16,6 +16,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <new>
 #include <vector>
 
 #include "kvp_common.cuh"
@@ -663,7 +664,7 @@ extern "C" int kvp_wr_grid(kvp_problem* p, uint32_t init_mode, uint32_t w_max, u
 
 extern "C" int kvp_wr_anneal(const uint64_t* table, uint32_t w_max, uint32_t n_ratio, const kvp_wr_params* wp,
                              kvp_wr_result* results, kvp_wr_result* best, void* stream)
-{
+try {
     if (!table || !wp || w_max < 1 || n_ratio < 2) return KVP_ERR_ARG;
     if (!wp->chains || !wp->levels || wp->levels > 4096 || !wp->iters || wp->reserved) return KVP_ERR_ARG;
     if (wp->w0 < 1 || wp->w0 > w_max || wp->r0 >= n_ratio) return KVP_ERR_ARG;
@@ -699,6 +700,7 @@ extern "C" int kvp_wr_anneal(const uint64_t* table, uint32_t w_max, uint32_t n_r
     std::vector<uint32_t> acc((size_t)wp->levels * KVP_TABLE_Q), shifts(wp->levels);
     int rc = kvp_accept_table(temps.data(), wp->levels, acc.data(), shifts.data());
     if (rc) return rc;
+    std::vector<kvp_wr_result> host(wp->chains);
     char* dev = nullptr;
     const size_t acc_bytes = acc.size() * 4, sh_bytes = (shifts.size() * 4 + 255) & ~(size_t)255;
     const size_t res_bytes = (size_t)wp->chains * sizeof(kvp_wr_result);
@@ -721,7 +723,6 @@ extern "C" int kvp_wr_anneal(const uint64_t* table, uint32_t w_max, uint32_t n_r
     if (row_bytes + tab_bytes <= 48 * 1024) wr_anneal_kernel<true><<<wp->chains, 32, row_bytes + tab_bytes, st>>>(k, d_res);
     else wr_anneal_kernel<false><<<wp->chains, 32, row_bytes, st>>>(k, d_res);
     cudaError_t le = cudaGetLastError();
-    std::vector<kvp_wr_result> host(wp->chains);
     if (le == cudaSuccess) le = cudaMemcpyAsync(host.data(), d_res, res_bytes, cudaMemcpyDeviceToHost, st);
     cudaFreeAsync(dev, st);
     KVP_CUDA(le);
@@ -733,4 +734,6 @@ extern "C" int kvp_wr_anneal(const uint64_t* table, uint32_t w_max, uint32_t n_r
             if (host[c].best_ticks < best->best_ticks) *best = host[c];
     }
     return KVP_OK;
+} catch (const std::bad_alloc&) {
+    return KVP_ERR_NOMEM;
 }

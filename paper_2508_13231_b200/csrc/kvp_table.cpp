@@ -4,6 +4,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <new>
 #include <thread>
 #include <vector>
 
@@ -79,7 +80,7 @@ void accept_rows(const double* temps, const uint32_t* shifts, const uint32_t* ro
 }  // namespace
 
 extern "C" int kvp_accept_table(const double* temps, uint32_t levels, uint32_t* table, uint32_t* shifts)
-{
+try {
     if (!temps || !table || !shifts || !levels) return KVP_ERR_ARG;
     // A level whose (clamped) temperature equals that of the level before it has the same row: a ladder that has
     // cooled below one tick repeats its last row, often for a third of its levels. Only the others are computed.
@@ -118,4 +119,6 @@ extern "C" int kvp_accept_table(const double* temps, uint32_t levels, uint32_t* 
         memcpy(table + (size_t)j * KVP_TABLE_Q, table + (size_t)(j - 1) * KVP_TABLE_Q, KVP_TABLE_Q * sizeof(uint32_t));
     }
     return KVP_OK;
+} catch (const std::bad_alloc&) {
+    return KVP_ERR_NOMEM;
 }

@@ -75,3 +75,23 @@ def test_no_gpu_means_error_not_fallback(lib):
     rc = lib.kvp_create(ctypes.byref(h), 16, ctypes.c_uint64(8192), 4, dummy.ctypes.data_as(ctypes.c_void_p), 4,
                         ctypes.byref(ms), None, None, None)
     assert rc in (-4, -5)      # KVP_ERR_CUDA: no device, and no CPU path to fall back to
+
+
+NO_ROOM = r"""
+import ctypes, resource, sys
+lib = ctypes.CDLL(sys.argv[1])
+temps, table, shifts = (ctypes.c_double * 4)(1, 1, 1, 1), (ctypes.c_uint32 * 4096)(), (ctypes.c_uint32 * 4)()
+used = [int(l.split()[1]) * 1024 for l in open("/proc/self/status") if l.startswith("VmSize")][0]
+resource.setrlimit(resource.RLIMIT_AS, (used + (1 << 28), resource.RLIM_INFINITY))
+print(lib.kvp_accept_table(temps, ctypes.c_uint32(1 << 30), table, shifts), lib.kvp_accept_table(temps, 4, table, shifts))
+"""
+
+
+def test_no_host_memory_is_an_error_code(lib):
+    """A failed host allocation inside the library comes back as KVP_ERR_NOMEM; nothing is thrown through the C interface."""
+    import subprocess
+    import sys
+
+    from paper_2508_13231_b200 import build
+    r = subprocess.run([sys.executable, "-c", NO_ROOM, build.LIB], capture_output=True, text=True, timeout=120)
+    assert r.returncode == 0 and r.stdout.split() == ["-5", "0"], r.stdout + r.stderr
