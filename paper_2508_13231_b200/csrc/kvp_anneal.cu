@@ -558,6 +558,12 @@ struct Ctx {
     char* host;              // host side of the copies: 256 bytes for `small`, then the tables
     size_t host_bytes;
     std::vector<char> host_own;
+    // The next call of this thread uses the same block: no way out of a call may leave a copy from or to it in flight.
+    struct InFlight {
+        cudaStream_t st = nullptr;
+        bool any = false;
+        ~InFlight() { if (any) cudaStreamSynchronize(st); }
+    } copies;
     uint64_t* host_small() const { return reinterpret_cast<uint64_t*>(host); }
     uint32_t* table; uint32_t* shifts;
     kvp_chain_result* results;
@@ -685,8 +691,9 @@ int run_chains(Ctx& c, uint32_t first, uint32_t count, uint32_t result_base, kvp
 size_t table_bytes(uint32_t levels) { return (size_t)levels * (KVP_TABLE_Q + 2) * 4; }
 
 // Host side of a call's copies: page-locked, so that a copy neither waits for a staging copy nor holds the host up (the
-// tables of 64 levels, 262 KB in three pageable copies: 40 us of a call of 540). Every call ends with a synchronisation,
-// so one block per thread is enough; it is kept up to 1 MB and freed with the thread. Larger calls use ordinary memory.
+// tables of 64 levels, 262 KB in three pageable copies: 40 us of a call of 540). Every call ends with a synchronisation, one
+// that fails half-way too (Ctx::copies), so one block per thread is enough; it is kept up to 1 MB and freed with the thread.
+// Larger calls use ordinary memory.
 struct Staging {
     char* p = nullptr;
     size_t bytes = 0;
@@ -996,6 +1003,8 @@ int prepare(kvp_problem* p, const kvp_anneal_params* a, cudaStream_t st, Ctx& c,
         ++c.launches;
     }
     uint64_t* const host_small = c.host_small();
+    c.copies.st = st;
+    c.copies.any = true;
     KVP_CUDA(cudaMemcpyAsync(host_small, c.small, 64, cudaMemcpyDeviceToHost, st));
     KVP_CUDA(cudaStreamSynchronize(st));
     if ((int32_t)(host_small[2] & 0xFFFFFFFFu) >= 0) return KVP_ERR_CAPACITY;   // Eq. 5 on the initial schedule
@@ -1146,6 +1155,7 @@ try {
                                  cudaMemcpyDeviceToHost, st));
     KVP_CUDA(cudaEventRecord(ev[3], st));
     KVP_CUDA(cudaStreamSynchronize(st));
+    c.copies.any = false;
     memcpy(&red, host_small + 8, sizeof red);
     if (red.pad) return KVP_ERR_TIMEOUT;
     red.best_chain += a->first_chain;                      // the reduction works on call-local indices
@@ -1195,6 +1205,7 @@ try {
     uint32_t gave_up = 0;
     KVP_CUDA(cudaMemcpyAsync(&gave_up, c.prm.err, 4, cudaMemcpyDeviceToHost, st));
     KVP_CUDA(cudaStreamSynchronize(st));
+    c.copies.any = false;
     return gave_up ? KVP_ERR_TIMEOUT : KVP_OK;
 } catch (const std::bad_alloc&) {
     return KVP_ERR_NOMEM;
@@ -1356,6 +1367,7 @@ try {
     if (n_exchanged) KVP_CUDA(cudaMemcpyAsync(n_exchanged, nex, (size_t)chains * 4, cudaMemcpyDeviceToHost, st));
     KVP_CUDA(cudaEventRecord(ev[3], st));
     KVP_CUDA(cudaStreamSynchronize(st));
+    c.copies.any = false;
     if (final_rung)
         for (uint32_t i = 0; i < chains; ++i) final_rung[i] = last_row[i];
     memcpy(&red, host_small + 8, sizeof red);

@@ -126,3 +126,20 @@ def test_exchange_argument_errors(kvp, oracle):
         with pytest.raises(kvp.KvpError) as e:
             g.anneal_exchange(g.make_params(**kw), rungs, every)
         assert e.value.code == kvp.ERR_ARG
+
+
+def test_failed_call_leaves_nothing_in_flight(kvp, oracle):
+    """A call that fails after its device work has begun (the ladder turns out to rise) has waited for its copies, and the same
+    thread's next call, on another stream, is exact."""
+    A = wl.random_access(64, 20, 0.3, seed=1)
+    g, o = both_problems(kvp, oracle, 64, 8192, 20, A, 16, (8000 * GB, 900 * GB, 900 * GB))
+    first, second = torch.cuda.Stream(), torch.cuda.Stream()
+    rising = [100.0] * 119 + [200.0]
+    kw = dict(chains=6, moves=500, seed=3, levels=100, p0=0.3)
+    ref = o.anneal(o.make_params(**kw))
+    for _ in range(10):
+        with pytest.raises(kvp.KvpError):
+            g.anneal_exchange(g.make_params(chains=120, moves=10, levels=120, temps=rising), 120, 5, stream=first)
+        assert first.query()
+        out = g.anneal(g.make_params(**kw), want_per_chain=True, stream=second)
+        assert [r.astuple() for r in out["per_chain"]] == [r.astuple() for r in ref["per_chain"]]
