@@ -68,23 +68,22 @@ struct ChainParams {
     uint32_t early_permille, early_from;
     PhiloxKeys keys;             // round keys of the seed
     uint64_t per_level, upto, init_ticks;
-    uint32_t* cow_out;           // wide kernel, schedules in global scratch: [slots][cow_slots4 * 4] which buckets of
+    uint32_t* cow_out;           // schedules in global scratch: [slots][cow_slots4 * 4] which buckets of
                                  // units a slot's slice holds when its chain ends (the rest is the initial schedule)
     uint32_t cow_shift;          // a bucket is 2^cow_shift consecutive units
     unsigned long long* work;    // wide kernel: [3] sums over the chains of {n_again, n_listed, n_items}
-    // Replica exchange (wide kernel): the call runs rounds round0 .. round1-1; in round t chain c proposes moves
+    // Replica exchange: the call runs rounds round0 .. round1-1; in round t chain c proposes moves
     // t * exch_every .. (t + 1) * exch_every - 1 (up to `upto`) with the table row of the rung it holds,
     // rung_hist[t * hist_stride + (c - hist_base)].
     uint8_t* rung_hist;          // null: the ordinary cooling schedule by temperature levels
     uint64_t exch_every;
     uint32_t round0, round1, hist_stride, hist_base;
-    uint4* state;                // if set: [chains][state4] the chain's persistent shared-memory state (and its
+    uint4* state;                // wide kernel, if set: [chains][state4] the chain's persistent shared-memory state (and its
                                  // schedule, when that lives in shared memory), indexed like rung_hist
     uint32_t state4;             // uint4 slots per chain in `state`
     uint32_t resume;             // 1: start from `state` instead of the initial schedule
-    uint32_t cow_slots4;         // schedules in global scratch: uint4 slots of a chain's bucket bitmap; 0 (narrow kernel
-                                 // only): plain slices, each a whole copy of the initial schedule
-    // wide kernel: segments seg0 .. seg1 - 1 of seg_len moves (the last one takes what is left up to `upto`), each of
+    uint32_t cow_slots4;         // schedules in global scratch: uint4 slots of a chain's bucket bitmap
+    // segments seg0 .. seg1 - 1 of seg_len moves (the last one takes what is left up to `upto`), each of
     // seg_bat batches: the temperature levels of the cooling schedule, or rounds of a replica-exchange run
     uint32_t seg0, seg1, seg_bat;
     uint64_t seg_len;
@@ -98,11 +97,10 @@ struct ChainParams {
 };
 
 // A proposal as its lane keeps it in registers: the Philox words and, after evaluation, the verdict.
-// The placement windows live in shared memory (ChainView::win), 8 words per proposal:
-//   {Wu, Wv, Nu, Nv} = placement of units u, v before (W) and after (N) the move, {Au, Av} = access bits,
-//   then s0. Window convention: bit k belongs to step s0 - 1 + k, so bit 0 is the step before the run (for
-//   s0 == 0 it repeats step 0, because P[-1] := P[0]), bits 1..run are the run, and the affected steps
-//   s0..last are bits 1..nl <= 31. Run lengths stop at 30 so that every vector fits one 32-bit register.
+// Windows of it: Wu, Wv, Nu, Nv = placement of units u, v before (W) and after (N) the move, Au, Av = access bits. Bit k
+// belongs to step s0 - 1 + k, so bit 0 is the step before the run (for s0 == 0 it repeats step 0, because P[-1] := P[0]),
+// bits 1..run are the run, and the affected steps s0..last are bits 1..nl <= 31. Run lengths stop at 30 so that every
+// window fits one 32-bit register.
 struct LaneMove {
     uint32_t pk, u, v, w;        // packed (swap | len << 1 | s0 << 8), units, Metropolis uniform
     int delta;
@@ -405,26 +403,18 @@ undo_kernel(const ChainParams prm, uint32_t slot)
     // the schedule itself is copied out by gather_slice_kernel, on the whole GPU
 }
 
-// The schedule a slice of global scratch stands for, copied to dst: a plain slice (have == null) word for word; a
-// copy-on-write slice bucket by bucket, from the slice where it holds the bucket and from the initial schedule
-// elsewhere. A warp per bucket (per 1024 words of a plain slice).
+// The schedule a copy-on-write slice of global scratch stands for, copied to dst bucket by bucket, from the slice where it
+// holds the bucket and from the initial schedule elsewhere. A warp per bucket.
 __global__ void __launch_bounds__(256)
 gather_slice_kernel(uint32_t* __restrict__ dst, const uint32_t* __restrict__ mine, const uint32_t* __restrict__ p0,
                     const uint32_t* __restrict__ have, uint32_t shift, uint32_t U, uint32_t S32)
 {
     const uint32_t lane = threadIdx.x & 31, warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const uint32_t nwarps = (gridDim.x * blockDim.x) >> 5;
-    if (have) {
-        const uint32_t nb = (U + (1u << shift) - 1u) >> shift;
-        for (uint32_t b = warp; b < nb; b += nwarps) {
-            const size_t lo = (size_t)(b << shift) * S32, hi = (size_t)min(U, (b + 1u) << shift) * S32;
-            const uint32_t* src = (have[b >> 5] >> (b & 31u)) & 1u ? mine : p0;
-            for (size_t i = lo + lane; i < hi; i += 32) dst[i] = src[i];
-        }
-    } else {
-        const size_t n = (size_t)U * S32;
-        for (size_t lo = (size_t)warp * 1024; lo < n; lo += (size_t)nwarps * 1024)
-            for (size_t i = lo + lane; i < min(n, lo + 1024); i += 32) dst[i] = mine[i];
+    const uint32_t nwarps = (gridDim.x * blockDim.x) >> 5, nb = (U + (1u << shift) - 1u) >> shift;
+    for (uint32_t b = warp; b < nb; b += nwarps) {
+        const size_t lo = (size_t)(b << shift) * S32, hi = (size_t)min(U, (b + 1u) << shift) * S32;
+        const uint32_t* src = (have[b >> 5] >> (b & 31u)) & 1u ? mine : p0;
+        for (size_t i = lo + lane; i < hi; i += 32) dst[i] = src[i];
     }
 }
 
@@ -577,7 +567,7 @@ struct Ctx {
     uint64_t* undo_log;      // undo logs (global variant), or null
     uint32_t* undo_len;
     uint32_t undo_cap;
-    uint32_t* cow_out;       // wide kernel, global variant: bucket bitmaps of the slices, or null
+    uint32_t* cow_out;       // global variant: bucket bitmaps of the slices, or null
     uint32_t cow_shift;
     uint32_t cow_slots4;     // uint4 slots of a chain's bucket bitmap
     bool psmem;
@@ -648,7 +638,7 @@ ChainKernel wide_kernel_for(bool psmem, bool asmem, bool grow, bool lin, uint32_
     return lin ? wide_pick<true, false, true, 0>(grow, rows) : wide_pick<true, false, false, 0>(grow, rows);
 }
 
-ChainKernel kernel_of(const Ctx& c, bool psmem, bool asmem, uint32_t W)
+ChainKernel kernel_of(const Ctx& c, bool psmem, bool asmem)
 {
     return c.wide ? wide_kernel_for(psmem, asmem, c.grow, c.lin, c.S32, c.rows)
                   : narrow_kernel_for(psmem, asmem, c.grow, c.lin, c.S32, c.solo);
@@ -669,7 +659,7 @@ int launch_chains(const Ctx& c, ChainParams& prm, uint32_t count)
     }
     const uint32_t grid = (count + c.wpb - 1) / c.wpb;
     const size_t smem = (size_t)c.wpb * c.smem_per_warp + c.smem_shared;
-    kernel_of(c, c.psmem, c.asmem, c.wpc)<<<grid, c.wpb * c.wpc * 32, smem, c.st>>>(prm);
+    kernel_of(c, c.psmem, c.asmem)<<<grid, c.wpb * c.wpc * 32, smem, c.st>>>(prm);
     KVP_CUDA(cudaGetLastError());
     return KVP_OK;
 }
@@ -849,7 +839,7 @@ int prepare(kvp_problem* p, const kvp_anneal_params* a, cudaStream_t st, Ctx& c,
         if (c.asmem) {
             c.smem_shared = with_a(c.wpb, W) - (size_t)c.wpb * c.smem_per_warp;
         }
-        KVP_CUDA(cudaFuncSetAttribute(kernel_of(c, true, c.asmem, W), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)budget));
+        KVP_CUDA(cudaFuncSetAttribute(kernel_of(c, true, c.asmem), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)budget));
     } else {
         // wide: two warps per chain while an SM has at most 8 (more per chain are no faster)
         if (!c.wide) W = narrow_warps();
@@ -877,9 +867,9 @@ int prepare(kvp_problem* p, const kvp_anneal_params* a, cudaStream_t st, Ctx& c,
         c.wpc = W;
         uint32_t wcap = (uint32_t)(budget / c.smem_per_warp);     // chains per CTA at most
         if (wcap > full / W) wcap = full / W;
-        KVP_CUDA(cudaFuncSetAttribute(kernel_of(c, false, false, W), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)budget));
+        KVP_CUDA(cudaFuncSetAttribute(kernel_of(c, false, false), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)budget));
         int ctas = 0;
-        KVP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ctas, kernel_of(c, false, false, W), (int)(wcap * W * 32),
+        KVP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ctas, kernel_of(c, false, false), (int)(wcap * W * 32),
                                                                wcap * c.smem_per_warp));
         if (ctas < 1) return KVP_ERR_RANGE;
         uint32_t per_sm = (uint32_t)ctas * wcap;                   // resident chains per SM, at most 32 warps
@@ -933,8 +923,7 @@ int prepare(kvp_problem* p, const kvp_anneal_params* a, cudaStream_t st, Ctx& c,
     c.undo_cap = c.psmem ? 0u : 4096u;
     const size_t o_ulog = take((size_t)c.resident * c.undo_cap * 8), o_ulen = take(c.psmem ? 0 : (size_t)c.resident * 4);
     // Which buckets of its slice a chain has taken over, for the walk back of the winner.
-    const bool cow = !c.psmem && c.cow_slots4 != 0;
-    const size_t o_cow = take(cow ? (size_t)c.resident * c.cow_slots4 * 16 : 0);
+    const size_t o_cow = take(c.psmem ? 0 : (size_t)c.resident * c.cow_slots4 * 16);
     rc = ensure_chain_ws(p, off, st);
     if (rc) return rc;
     char* base = static_cast<char*>(p->d_chain_ws);
@@ -946,7 +935,7 @@ int prepare(kvp_problem* p, const kvp_anneal_params* a, cudaStream_t st, Ctx& c,
     c.hb0 = c.grow ? c.counts0 + (size_t)p->S * 4 : nullptr;
     c.full0 = (uint32_t*)(base + o_full); c.snap = snapshots ? (uint32_t*)(base + o_snap) : nullptr;
     c.undo_log = c.psmem ? nullptr : (uint64_t*)(base + o_ulog); c.undo_len = c.psmem ? nullptr : (uint32_t*)(base + o_ulen);
-    c.cow_out = cow ? (uint32_t*)(base + o_cow) : nullptr;
+    c.cow_out = c.psmem ? nullptr : (uint32_t*)(base + o_cow);
 
     // initial schedule in both layouts
     KVP_CUDA(cudaMemsetAsync(c.small, 0, 256, st));
@@ -1106,7 +1095,7 @@ try {
                     else undo_kernel<false><<<1, 32, 0, st>>>(prm, wslot);
                     KVP_CUDA(cudaGetLastError());
                     gather_slice_kernel<<<148 * 4, 256, 0, st>>>(c.dumpcol, c.slots + (size_t)wslot * p->U * p->S32, c.Pcol0,
-                                                                 c.cow_out ? c.cow_out + (size_t)wslot * (c.cow_slots4 * 4) : nullptr,
+                                                                 c.cow_out + (size_t)wslot * (c.cow_slots4 * 4),
                                                                  c.cow_shift, p->U, p->S32);
                     KVP_CUDA(cudaGetLastError());
                     c.launches += 2;

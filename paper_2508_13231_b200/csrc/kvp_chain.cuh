@@ -64,7 +64,6 @@ struct ChainShared {
     uint32_t rung, n_exchanged;  // replica exchange
     Applied applog[kLog];
 };
-constexpr uint32_t kShared4 = sizeof(ChainShared) / 16;
 static_assert(sizeof(ChainShared) % 16 == 0, "uint4 slots");
 
 // Work area of a warp: a ring of listed proposals with their placement windows, the accepted ones that change the schedule
