@@ -477,7 +477,8 @@ typedef struct {
                                    accepted moves instead of 6                                                    */
     uint32_t resident;          /* n: at most n chains whose schedules live in global memory run at a time, so
                                    that a small job comes in several waves                                       */
-    uint32_t overlay;           /* without effect: schedules in global memory are always copy-on-write slices     */
+    uint32_t overlay;           /* 2: the copy-on-write slices of schedules in global memory come in buckets of 8
+                                   units at least, as those of large problems do                                 */
 } kvp_test_hooks;
 void kvp_set_test_hooks(const kvp_test_hooks* hooks);
 

@@ -78,7 +78,7 @@ struct ChainParams {
     uint8_t* rung_hist;          // null: the ordinary cooling schedule by temperature levels
     uint64_t exch_every;
     uint32_t round0, round1, hist_stride, hist_base;
-    uint4* state;                // wide kernel, if set: [chains][state4] the chain's persistent shared-memory state (and its
+    uint4* state;                // if set: [chains][state4] the chain's persistent shared-memory state (and its
                                  // schedule, when that lives in shared memory), indexed like rung_hist
     uint32_t state4;             // uint4 slots per chain in `state`
     uint32_t resume;             // 1: start from `state` instead of the initial schedule
@@ -87,6 +87,7 @@ struct ChainParams {
     // seg_bat batches: the temperature levels of the cooling schedule, or rounds of a replica-exchange run
     uint32_t seg0, seg1, seg_bat;
     uint64_t seg_len;
+    uint64_t move0;              // narrow kernel: it counts segments from 0, this is the first one's first move
     ChainLayout lay;
     uint32_t warps;              // warps per chain
     uint32_t carry;              // room for accepted proposals: kAccepted (less in tests)
@@ -659,7 +660,13 @@ int launch_chains(const Ctx& c, ChainParams& prm, uint32_t count)
     }
     const uint32_t grid = (count + c.wpb - 1) / c.wpb;
     const size_t smem = (size_t)c.wpb * c.smem_per_warp + c.smem_shared;
-    kernel_of(c, c.psmem, c.asmem)<<<grid, c.wpb * c.wpc * 32, smem, c.st>>>(prm);
+    ChainParams k = prm;
+    if (!c.wide) {
+        k.move0 = k.seg0 * k.seg_len;
+        k.seg1 -= k.seg0;
+        if (k.rung_hist) k.rung_hist += (size_t)k.seg0 * k.hist_stride;
+    }
+    kernel_of(c, c.psmem, c.asmem)<<<grid, c.wpb * c.wpc * 32, smem, c.st>>>(k);
     KVP_CUDA(cudaGetLastError());
     return KVP_OK;
 }
@@ -776,13 +783,11 @@ int prepare(kvp_problem* p, const kvp_anneal_params* a, cudaStream_t st, Ctx& c,
     const uint32_t held = turns > 1 ? (chains_per_sm + turns - 1) / turns : chains_per_sm;
     if (!busy && p0 < 0.02 && p->cap <= p->U / 4) c.wide = held > (c.psmem ? 8u : 5u);
     if (hooks.warps_per_chain) c.wide = hooks.warps_per_chain == 3 || (hooks.warps_per_chain >= 16 && hooks.warps_per_chain < 32);
-    if (exchange) {
-        // Whole ladders in a CTA: every round waits for the hottest rungs, which apply the most moves, and one warp per chain
-        // is fastest there (128 ladders of 8 on 256 units x 512 steps, 100,000 moves: 4.5 ms, two warps 5.1, wide kernel 7.5;
-        // 7 of 4 on 46 x 61, 38,619 moves: 3.5, 5.4, 11.2).
-        const bool ladders = c.psmem && rungs <= 16 && rungs * (fixed_bytes(1, true) + pbytes) + 16 <= budget;
-        c.wide = !ladders || hooks.warps_per_chain == 3 || (hooks.warps_per_chain >= 16 && hooks.warps_per_chain < 32);
-    }
+    // Replica exchange: every round waits for the hottest rungs, which apply the most moves: the narrow kernel, with one warp per
+    // chain where schedules live in shared memory. Whole ladders in a CTA (128 of 8 on 256 units x 512 steps, 100,000 moves: 4.5
+    // ms, two warps 5.1, wide kernel 7.5; 7 of 4 on 46 x 61, 38,619 moves: 3.5, 5.4, 11.2), or rounds of launches (51 of 20,
+    // 50,000 moves: 3.4 ms, wide kernel 5.5; with a slow link 5.2 and 9.8; 128 of 8 on 16,384 x 256, 20,000 moves: 3.8 and 8.0).
+    if (exchange && !hooks.warps_per_chain) c.wide = false;
     // Growing caches: the narrow kernel with schedules in shared memory and for warm starts (512 units x 132 steps, 256 chains
     // x 20,000 moves: 0.46 against 0.61 ms, at p0 = 0.8 1.7 against 5.2; 131,072 x 1056, 1024 x 20,000 at p0 = 0.3 1.39
     // against 1.70, at 0.8 4.5 against 6.6); the wide one for near-greedy chains in global memory, most of whose proposals
@@ -811,10 +816,8 @@ int prepare(kvp_problem* p, const kvp_anneal_params* a, cudaStream_t st, Ctx& c,
         };
         if (c.wide) {
             // two warps per chain, four where an SM has three chains or fewer (256 units x 512 steps, 50,000 moves, 148 and
-            // 740 chains: one warp 1.62 and 1.79 ms, two 1.12 and 1.34, four 1.05 and 2.40); half of that for replica exchange,
-            // whose hot rungs apply many moves (20 rungs, 200 and 1020 chains x 50,000: one 5.01 and 5.54, two 4.73 and 5.65)
+            // 740 chains: one warp 1.62 and 1.79 ms, two 1.12 and 1.34, four 1.05 and 2.40)
             W = chains_per_sm <= 3 ? 4 : 2;
-            if (exchange) W /= 2;
             while (W > 1 && (want * W > full || with_a(want, W) > budget)) W /= 2;
         } else {
             W = exchange ? 1u : narrow_warps();
@@ -859,6 +862,7 @@ int prepare(kvp_problem* p, const kvp_anneal_params* a, cudaStream_t st, Ctx& c,
             if (bits < kCowBitsMin) bits = kCowBitsMin;
             if (bits > kCowBitsMax) bits = kCowBitsMax;
             while (((uint64_t)p->U + (1ull << c.cow_shift) - 1) >> c.cow_shift > bits) ++c.cow_shift;
+            if (hooks.overlay == 2 && c.cow_shift < 3) c.cow_shift = 3;   // test hook
             const uint64_t buckets = ((uint64_t)p->U + (1ull << c.cow_shift) - 1) >> c.cow_shift;
             c.cow_slots4 = (uint32_t)((buckets + 127) / 128);
         }
@@ -1256,7 +1260,8 @@ try {
     if ((rc = kvp_accept_table(pair_temps.data(), pairs, xtable, xshifts))) return rc;
 
     // workspace of the run: rung history, holders, exchange counts, thresholds, the chains' saved states
-    const uint32_t persist4 = chain_layout(p->S, p->S32, c.grow, c.psmem, c.lin, c.psmem ? 0u : c.cow_slots4).work / 16;
+    const uint32_t cow4 = c.psmem ? 0u : c.cow_slots4;
+    const uint32_t persist4 = (c.wide ? chain_layout(p->S, p->S32, c.grow, c.psmem, c.lin, cow4) : narrow_layout(p->S, p->S32, c.grow, c.psmem, c.lin, cow4)).work / 16;
     const size_t pwords = (size_t)p->U * p->S32;
     const uint32_t state4 = persist4 + (c.psmem ? (uint32_t)((pwords + 3) / 4) : 0u);
     size_t off = 0;

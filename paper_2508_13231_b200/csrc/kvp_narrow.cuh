@@ -133,7 +133,15 @@ narrow_chain_kernel(const __grid_constant__ ChainParams prm)
         copy_words(a_s, prm.Acol, pwords, threadIdx.x, blockDim.x);
         A = a_s;
     }
-    if (active) {
+    // rounds of launches: what the chain left behind in the round before (see ChainParams::state)
+    const bool resumed = prm.resume != 0u;
+    if (active && resumed) {
+        if (sub == 0) {
+            const uint32_t* const saved = reinterpret_cast<const uint32_t*>(prm.state + (size_t)(chain - prm.hist_base) * prm.state4);
+            copy_words_cold(c.template at<uint32_t>(cb), saved, prm.lay.work / 4, lane);
+            if (PSMEM) copy_words_cold(P, saved + prm.lay.work / 4, pwords, lane);
+        }
+    } else if (active) {
         for (uint32_t w = sub; w < S32; w += W) {                 // 32 steps at a time, for the two bitmaps
             const uint32_t t = w * 32 + lane, i = min(t, S - 1);
             const uint4 n = __ldg(prm.counters0 + i);             // {hr, mi, mo, occ}
@@ -196,6 +204,11 @@ narrow_chain_kernel(const __grid_constant__ ChainParams prm)
     // The chain's scalars: SOLO in registers, otherwise in `sc`.
     uint64_t cur = prm.init_ticks, best = cur, best_move = ~0ull, hash = 0, n_chg = 0;
     bool unsaved = false;                                         // the best state is the current one and not saved yet
+    if (SOLO && resumed) {
+        const ChainShared* const was = c.sc();
+        cur = was->cur; best = was->best; best_move = was->best_move; hash = was->hash; n_chg = was->n_chg;
+        unsaved = was->snap_dirty != 0u;
+    }
 
     uint32_t n_same = 0, n_inf = 0;                               // per lane
     const int kh = (int)prm.K.kh, ke = (int)prm.K.ke, khF = (int)prm.K.khF, kdF = (int)prm.K.kdF, kkF = (int)prm.K.kkF;
@@ -204,7 +217,7 @@ narrow_chain_kernel(const __grid_constant__ ChainParams prm)
     bool over = !active, silent = false;                          // this warp is done with its chain; because a wait ran out
     for (uint32_t level = 0; level < prm.seg1; ++level) {
         if (over && !fused) break;
-        const uint64_t lvl_start = level * prm.seg_len, lvl_len = min(level + 1 == prm.seg1 ? ~(uint64_t)0 : prm.seg_len, prm.upto - lvl_start);
+        const uint64_t lvl_start = prm.move0 + level * prm.seg_len, lvl_len = min(level + 1 == prm.seg1 ? ~(uint64_t)0 : prm.seg_len, prm.upto - lvl_start);
         const uint32_t nbat = (uint32_t)((lvl_len + 31) / 32), last_nb = (uint32_t)(lvl_len - (uint64_t)(nbat - 1) * 32);
         const uint32_t base = level * prm.seg_bat;                // index of the level's first batch (mod 2^32)
         // row of the acceptance table
@@ -580,10 +593,17 @@ narrow_chain_kernel(const __grid_constant__ ChainParams prm)
     if (lane == 0) {
         kvp_chain_result res;
         res.best_ticks = c.sc()->best; res.best_move = c.sc()->best_move; res.final_ticks = c.sc()->cur;
-        res.moves_done = c.sc()->m_end ? c.sc()->m_end : min(prm.upto, exchange ? prm.seg1 * prm.seg_len : ~(uint64_t)0);
+        res.moves_done = c.sc()->m_end ? c.sc()->m_end : min(prm.upto, exchange ? prm.move0 + prm.seg1 * prm.seg_len : ~(uint64_t)0);
         res.n_accepted = c.sc()->n_same + c.sc()->n_chg; res.n_changed = c.sc()->n_chg; res.n_infeasible = c.sc()->n_inf; res.traj_hash = c.sc()->hash;
         prm.results[chain - prm.result_base] = res;
         if (prm.n_exchanged) prm.n_exchanged[chain - prm.hist_base] = c.sc()->n_exchanged;
+        c.sc()->turn = 0u; c.sc()->napplied = 0u; c.sc()->left = 0u;   // the hand-over of a chain taken up again starts anew
+    }
+    __syncwarp();
+    if (prm.state) {                                              // the next round goes on from here
+        uint32_t* const saved = reinterpret_cast<uint32_t*>(prm.state + (size_t)(chain - prm.hist_base) * prm.state4);
+        copy_words_cold(saved, c.template at<uint32_t>(cb), prm.lay.work / 4, lane);
+        if (PSMEM) copy_words_cold(saved + prm.lay.work / 4, P, pwords, lane);
     }
     if (prm.snap && c.sc()->snap_dirty) copy_words_cold(prm.snap + (size_t)slot * pwords, P, pwords, lane);
     if (prm.undo_log && lane == 0) prm.undo_len[slot] = c.sc()->ulen;

@@ -255,13 +255,13 @@ def test_global_state_winner_paths(kvp, oracle, warps_per_chain):
         assert np.array_equal(to_np(out["best_schedule"]), bst[0]) and out["best_ticks"] == ref[0].best_ticks
 
 
-@pytest.mark.parametrize("overlay", [1, 2], ids=["overlay", "plain"])
+@pytest.mark.parametrize("overlay", [1, 2], ids=["columns", "buckets"])
 def test_later_waves_start_afresh(kvp, oracle, hooks, warps_per_chain, overlay):
     """More chains than are resident at once: a chain of a later wave takes over a slice of global scratch that holds
-    the final state of an earlier chain. With copy-on-write slices it starts from an empty overlay of the initial
-    schedule, with plain slices from a fresh copy (the narrow kernel has both forms, test hook; the wide kernel always
-    the first). Chains of every wave against the oracle, after a warm start with few rewritten units and after a hot
-    one that rewrites most of them."""
+    the final state of an earlier chain, and starts from an empty overlay of the initial schedule. Slices in buckets of one
+    unit, which the narrow kernel takes over and rewrites in one go, and of eight (test hook), which are copied first. Chains
+    of every wave against the oracle, after a warm start with few rewritten units and after a hot one that rewrites most of
+    them."""
     hooks(overlay=overlay)
     g, o, cfg, A = named_problem(kvp, oracle, "layer_8b")
     for kw, hot in ((dict(chains=5000, moves=2000, seed=7, p0=0.3, levels=4), False),
@@ -280,12 +280,12 @@ def test_later_waves_start_afresh(kvp, oracle, hooks, warps_per_chain, overlay):
         assert np.array_equal(to_np(out["best_schedule"]), bst[0]) and out["best_ticks"] == ref[0].best_ticks
 
 
-@pytest.mark.parametrize("overlay", [1, 2], ids=["overlay", "plain"])
+@pytest.mark.parametrize("overlay", [1, 2], ids=["columns", "buckets"])
 @pytest.mark.parametrize("resident", [1, 3, 4])
 def test_small_job_in_several_waves(kvp, oracle, hooks, resident, warps_per_chain, overlay):
     """Schedules in global memory, at most `resident` chains at a time (test hook): every chain but the first ones
-    starts in a slice that an earlier chain left behind, as a copy-on-write overlay of the initial schedule or as a
-    plain copy of it (test hook; the narrow kernel has both forms). All chains, the bound and the winner's schedule
+    starts in a slice that an earlier chain left behind, as an empty overlay of the initial schedule in buckets of one unit
+    or of eight (test hook). All chains, the bound and the winner's schedule
     (walked back in its slice) against the oracle, at a hot and a cold start, with the stop rule, and with a winner
     that an early wave produced."""
     hooks(resident=resident, overlay=overlay)
@@ -330,11 +330,11 @@ def test_two_warp_chains_repeat_exactly(kvp, oracle, hooks, name, p0):
         assert torch.equal(out["best_schedule"], ref["best_schedule"])
 
 
-@pytest.mark.parametrize("split", [0, 20, 64])
+@pytest.mark.parametrize("split", [0, 2, 5])
 def test_work_queue_in_two_halves(kvp, oracle, hooks, split, warps_per_chain):
-    """Chains in shared memory with the access bitmap staged beside them keep half a work queue and work a batch
-    with more items than it holds off in two halves. Ordinary inputs never fill it, so the hook lowers the limit:
-    dense accesses, a churning initial schedule and a hot start give batches of a few hundred items."""
+    """The wide kernel keeps the accepted proposals of a batch in a list of six and stops to commit when it is full. Near-greedy
+    chains seldom fill it; dense accesses, a churning initial schedule and a hot start do, and the hook lowers the limit to one
+    and three."""
     hooks(split_queue=split)
     U, S, cap = 64, 200, 32
     A = wl.random_access(U, S, 0.5, seed=9)

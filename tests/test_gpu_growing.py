@@ -250,6 +250,25 @@ def test_anneal_growing_slow_link(kvp, oracle, warps_per_chain, layers, heads, n
             _check_chains(g, o, g.make_params(**kw), o.make_params(**kw))
 
 
+@pytest.mark.parametrize("layers,heads,n,prompt,cap", [(3, 1, 45, 20, 30), (4, 4, 256, 200, 800)], ids=["shared", "global"])
+@pytest.mark.parametrize("chains,rungs", [(12, 3), (40, 20)])
+@pytest.mark.parametrize("link", [900, 300])
+def test_exchange_growing(kvp, oracle, hooks, layers, heads, n, prompt, cap, chains, rungs, link):
+    cfg, groups, U, S, birth = _shape(layers, heads, n, prompt)
+    rng = np.random.default_rng(n)
+    alive = birth[None, :] <= np.arange(S)[:, None]
+    A = wl.pack_bits(((rng.random((S, U)) < 0.2) & alive).astype(np.uint8))
+    g, o = _problems(kvp, oracle, U, 512, S, A, cap, (4900 * GB, link * GB, 500 * GB), birth)
+    kw = dict(chains=chains, moves=700, seed=9, levels=rungs, p0=1e-2, alpha=0.7)
+    ref = o.anneal_exchange(o.make_params(**kw), rungs, 100, want_best=True)
+    for warps in (0, 3):
+        hooks(warps_per_chain=warps)
+        out = g.anneal_exchange(g.make_params(**kw), rungs, 100)
+        assert [r.astuple() for r in out["per_chain"]] == [r.astuple() for r in ref["per_chain"]]
+        assert out["final_rung"] == ref["final_rung"].tolist() and out["n_exchanged"] == ref["n_exchanged"].tolist()
+        assert np.array_equal(to_np(out["best_schedule"]), ref["best_schedule"])
+
+
 def test_anneal_growing_8b_sampled_chains(kvp, oracle):
     g, o, cfg, A, birth = _named(kvp, oracle, "growing_8b")
     kw = dict(chains=16, moves=20000, seed=0, p0=cfg["p0"])
