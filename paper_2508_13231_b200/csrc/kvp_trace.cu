@@ -78,11 +78,14 @@ __device__ __forceinline__ void select_reset(SelectSmem& sm)
 // What bounds it: instructions per key, then the latency of the barriers. So keys that cannot be picked are dropped first.
 // Every warp looks at the largest key of each lane and finds, by six ballots, a value that `want` = ceil(k / warps) of them
 // reach; the smallest such value over the warps is reached by at least k keys of the step, so the k-th largest is not
-// below it. (Where that would take more than 24 of the 32 lanes, `want` is 0 and the bound is the smallest key.) Keys from
+// below it. (Where that would take more than 24 of the 32 lanes, `want` is 0 and the bound is the smallest key; so it is with
+// fewer than eight keys per thread, where the search costs more than it saves: 411 groups of 268 units 171 against 161 us.) Keys from
 // the bound up, about 9% of them at k = 5%, are counted per digit of (key - bound) in a shared-memory histogram, one
 // warp walks it from the top until the counts reach what is needed, and the keys of the bin found there, a few, are
 // ranked against each other. A bin with many keys (ties) takes more histogram passes, eight bits each.
 // 640 groups of 4096 units x 64 steps, 205 picked: 323 us with every key in the histogram and eight keys per thread, 240 now.
+// Groups that do not begin at a word set their bits by two atomics per 32 units (123 groups of 2326 units x 106 steps, the whole
+// call: 166 us, 273 when they took the way of the ties, 186 with an atomic per bit).
 // FULL: the CTA's UPT * T slots are exactly the n units, so no slot needs a bounds test.
 template <int UPT, bool FULL = false>
 __device__ __forceinline__ void select_step(const int32_t (&key)[UPT], const TraceK& k, uint32_t want, uint32_t topk, uint32_t gbase,
@@ -95,7 +98,7 @@ __device__ __forceinline__ void select_step(const int32_t (&key)[UPT], const Tra
         for (int j = 1; j < UPT; ++j) mine = max(mine, key[j]);
         const int32_t mx = __reduce_max_sync(0xFFFFFFFFu, mine);
         int32_t bound;
-        if (UPT >= 4 && want) {
+        if (UPT >= 8 && want) {
             const int32_t mn = __reduce_min_sync(0xFFFFFFFFu, mine);
             const uint32_t d = (uint32_t)mine - (uint32_t)mn;
             const int shift = max(26 - __clz((uint32_t)mx - (uint32_t)mn), 0);
@@ -198,7 +201,7 @@ __device__ __forceinline__ void select_step(const int32_t (&key)[UPT], const Tra
     const uint32_t take = need;                              // ties to admit, lowest unit index first
     const bool rank_ties = equal != take;                    // and when all keys from the bound up are equal
     uint32_t* row = k.out + (size_t)t * k.W32;
-    if (!rank_ties && k.aligned) {                           // the usual case, kept apart so that its loop stays small
+    if (!rank_ties) {                                        // the usual case, kept apart so that its loop stays small
         uint32_t word = 0;                                   // lane j keeps and stores round j's word
 #pragma unroll
         for (int j = 0; j < UPT; ++j) {
@@ -206,7 +209,16 @@ __device__ __forceinline__ void select_step(const int32_t (&key)[UPT], const Tra
             if (lane == (uint32_t)j) word = bits;
         }
         const uint32_t i = lane * T + (tid & ~31u);
-        if (lane < UPT && (FULL || i < k.n)) row[(gbase + i) >> 5] = word;
+        if (lane < UPT && (FULL || i < k.n)) {
+            uint32_t* const to = row + ((gbase + i) >> 5);
+            const uint32_t sh = (gbase + i) & 31u;
+            if (k.aligned) {
+                *to = word;
+            } else {                                         // its bits in two words of the row, which groups share
+                if (word << sh) atomicOr(to, word << sh);
+                if (sh && word >> (32u - sh)) atomicOr(to + 1, word >> (32u - sh));
+            }
+        }
         return;
     }
     if (tid == 0) sm.run = 0;
@@ -287,7 +299,7 @@ trace_kernel(const TraceK k)
             born[j] = i < k.n ? __ldg(k.birth + gbase + i) : 0u;
         }
     }
-    const uint32_t want = UPT >= 4 ? select_want(k.topk, T) : 0u;
+    const uint32_t want = UPT >= 8 ? select_want(k.topk, T) : 0u;
     for (uint32_t tok = 0, t = layer; t < k.steps; ++tok, t += k.layers) {
         select_reset(sm);
         int32_t key[UPT];
