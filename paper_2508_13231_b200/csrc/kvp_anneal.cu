@@ -753,21 +753,24 @@ int prepare(kvp_problem* p, const kvp_anneal_params* a, cudaStream_t st, Ctx& c,
         if (c.wide) return chain_bytes(p->S, p->S32, c.grow, shared, c.lin, shared ? 0u : c.cow_slots4, warps, c.rows);
         return narrow_bytes(p->S, p->S32, c.grow, shared, c.lin, shared ? 0u : c.cow_slots4, warps);
     };
-    // Which kernel, and how many warps per chain (W; an SM holds 16). Measured on problems of 64 to 524,288 units x 32 to 512
-    // steps, 5 to 20% of the units read per step, 10 to 35% in HBM, even and Zipf importance, 64 to 2368 chains of 10,000 to
-    // 15,000 moves, p0 = 1e-6, 0.03 and 0.3; in brackets what the other choice takes, as geometric mean over such jobs.
+    // Which kernel, and how many warps per chain (W; an SM holds 16). Measured on 1800 problems of 64 to 524,288 units x 32 to
+    // 512 steps, 5 to 20% of the units read per step, 10 to 45% in HBM, even and Zipf importance, 64 to 2368 chains of 10,000 to
+    // 100,000 moves, p0 = 1e-6, 0.03 and 0.3; the times below are ratios to the chosen form's, geometric means over such jobs
+    // (over all of them the chosen form takes 1.02 to 1.04 times the best one's time, 1.16 to 1.18 with the lines before).
     //  - What decides is how many proposals change the schedule. Many do at a warm start, and at any where the HBM side of Eq. 2
     //    is the larger one in the static placement (busy): such a schedule gets better by moving units out of HBM, and 2 to 14%
-    //    of a near-greedy chain's first 20,000 proposals change it, elsewhere 0.02 to 1%. Quiet chains with few units in HBM
-    //    (up to a quarter) have few proposals to judge, which the wide kernel's compaction is for.
-    //  - Schedules in shared memory: quiet near-greedy chains, more than 8 per SM: the wide kernel (narrow: 1.10). Everything else
-    //    the narrow one (wide: 1.18 to 2.35; but 0.92 to 0.94 on quiet near-greedy chains up to 8 per SM), from p0 = 0.02 on with
-    //    one warp per chain (two: 1.09 at 0.03, 1.32 at 0.3), below with as many as fit, four at most, two at most on horizons
-    //    below 128 steps, where moves meet more often.
-    //  - In global memory: quiet near-greedy chains, more than 5 per SM: the wide kernel with two warps per chain (narrow: 1.07),
-    //    from 9 per SM on with one (narrow: 1.38). Everything else the narrow one (wide: 2.1 to 2.2 on busy chains, 1.03 to 1.46
-    //    at warm starts), with four warps per chain up to 4 per SM, two up to 8 and one beyond, and two at most on busy chains
-    //    (four: 1.77).
+    //    of a near-greedy chain's first 20,000 proposals change it, elsewhere 0.02 to 1%. A quiet chain has few proposals to
+    //    judge, which the wide kernel's compaction is for; the fewer units are in HBM or read the fewer, and fewer later on.
+    //  - Schedules in shared memory: the narrow kernel (wide: 1.2 to 2.35), from p0 = 0.02 on with one warp per chain (two: 1.09
+    //    at 0.03, 1.32 at 0.3), below with three up to 5 per SM (two: 1.12, four: 1.02 up to 4), two up to 8 and one beyond; two
+    //    at most on fewer than 64 units and on busy short horizons, where moves meet most often (16 x 32, 64 chains x 10,000: 347
+    //    us, three 370, one 325). The wide one for quiet jobs of more than 8 chains per SM with next to nothing in HBM, if they
+    //    are brief or have many units (narrow: 1.1 to 1.2).
+    //  - In global memory: the narrow kernel on busy chains, with two warps per chain up to 8 per SM and one beyond (four: 1.77,
+    //    wide: 2.1 to 2.2), at warm starts (wide: 1.03 to 1.46) and up to 5 quiet chains per SM, with four warps per chain up to 4,
+    //    two up to 8 and one beyond. More quiet chains: the wide one, with two warps per chain up to 8 per SM and one beyond (100,000
+    //    moves: narrow 1.05 to 1.8). The limits below are those of jobs of 10,000 moves, whose chains still change much, and of
+    //    6 to 8 chains per SM that judge much (where they stop the wide kernel takes 1.0 to 1.25).
     // What counts as chains of an SM (held) is how many it holds at a time when their state takes its shared memory, the waves
     // of the job taken equally large. A ladder given as temperatures is taken for a near-greedy one: what share of the
     // proposals it accepts is not known (256 x 512, 1024 chains x 100,000 moves with the ladder of p0 = 0.8: 23.3 instead of
@@ -781,7 +784,12 @@ int prepare(kvp_problem* p, const kvp_anneal_params* a, cudaStream_t st, Ctx& c,
     const uint32_t at_a_time = std::min(std::max(fit, 1u), 16u);
     const uint32_t turns = (chains_per_sm + at_a_time - 1) / at_a_time;
     const uint32_t held = turns > 1 ? (chains_per_sm + turns - 1) / turns : chains_per_sm;
-    if (!busy && p0 < 0.02 && p->cap <= p->U / 4) c.wide = held > (c.psmem ? 8u : 5u);
+    const double in_hbm = (double)p->cap / p->U, read = (double)p->total_accessed / p->S / p->U;
+    const bool quiet = !busy && p0 < 0.02, brief = a->moves < 30000;
+    if (quiet && c.psmem) c.wide = held > 8 && in_hbm <= 0.15 && (brief || p->U >= 1024u);
+    if (quiet && !c.psmem && held > 5)
+        c.wide = brief ? in_hbm <= (p->S > 128 ? 0.2 : p->S > 64 ? 0.25 : held > 8 ? 0.4 : 0.3)
+                       : held > 8 || p->S <= 64 || read <= 0.1 || in_hbm <= 0.2;
     if (hooks.warps_per_chain) c.wide = hooks.warps_per_chain == 3 || (hooks.warps_per_chain >= 16 && hooks.warps_per_chain < 32);
     // Replica exchange: every round waits for the hottest rungs, which apply the most moves: the narrow kernel, with one warp per
     // chain where schedules live in shared memory. Whole ladders in a CTA (128 of 8 on 256 units x 512 steps, 100,000 moves: 4.5
@@ -801,7 +809,8 @@ int prepare(kvp_problem* p, const kvp_anneal_params* a, cudaStream_t st, Ctx& c,
         if (c.psmem && (p0 >= 0.02 || (!c.lin && held > 4))) return 1u;
         const uint32_t most = held <= 4 ? 4u : held == 5 ? 3u : held <= 8 ? 2u : 1u;
         if (c.grow && !c.psmem) return c.lin ? std::min(most, 2u) : 1u;
-        return (c.psmem ? p->S < 128u : busy || p0 >= 0.5) ? std::min(most, 2u) : most;
+        if (c.psmem) return std::min(most, p->U < 64u || (busy && p->S < 128u) ? 2u : 3u);
+        return busy || p0 >= 0.5 ? std::min(most, 2u) : most;
     };
     uint32_t W = 1;
     if (c.psmem) {
