@@ -304,7 +304,7 @@ def cost_kernel_record(steps, warmup):
     alg_bytes = (n + 1) * S * W32 * 4
     peak, src = _hbm_peak()
     achieved = alg_bytes / (ms * 1e-3) / 1e9
-    return {"kernel": "count_wide_kernel + score_counts_kernel (kvp_eval)", "metric": "schedules_scored_per_sec",
+    return {"kernel": "count_staged_kernel + score_counts_kernel (kvp_eval)", "metric": "schedules_scored_per_sec",
             "value": n / (ms * 1e-3), "unit": "schedules/s", "ms_per_call": ms, "steps": steps,
             "config": {"workload": name, "batch": n, "words_per_row": W32, "rows": S, "l2": FLUSH_NOTE},
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
@@ -521,8 +521,8 @@ class PathBench:
         out = prob.anneal(prm, want_per_chain=want_per_chain)
         if dist is not None:          # the cross-rank part of the reduction: MIN over one (ticks, chain) pair per rank
             out["global_best"] = self.sharding.combine_best(dist, out["best_ticks"], out["stats"].best_chain, device="cuda")
-        # kernels: 2 trace (scores, select) + 6 create (clean, popcount, transpose, unit counts, histogram,
-        #          static row) + 2 eval (count, finish) + those kvp_anneal reports
+        # kernels: 2 trace (scores, select) + 5 create (copy with transpose and counts, step constants, the three of the static
+        #          row) + 1 eval (counts and totals of two schedules) + those kvp_anneal reports
         self.launches = 2 + 5 + 1 + out["stats"].kernel_launches
         prob.close()
         return out

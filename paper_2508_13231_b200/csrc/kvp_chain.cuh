@@ -4,7 +4,8 @@
 // step the two sides of Eq. 2, th (Eq. 3) and te (Eq. 4), the occupancy, one bit "HBM is full" and one bit "te >= th".
 // When a DRAM channel is no faster than the link (kappa_d >= kappa_k, LIN) the third term of Eq. 4's maximum is always
 // the largest, so th and te are linear in the number of hits and of migrations of a step, and the pair is all a
-// proposal's cost needs; otherwise (not LIN) the migrations in both directions are kept beside it.
+// proposal's cost needs; otherwise (not LIN) the migrations in both directions are kept beside it, and two more step bitmaps
+// that say which of the three terms is the largest (the bound of step 3 then takes that term's change where te leads).
 //
 // A warp takes a batch of 32 * R consecutive moves:
 //   1. draw: a Philox block per proposal.
@@ -23,11 +24,11 @@
 // Several warps may serve one chain: they take its batches in turn and evaluate ahead of each other's commits (see
 // ChainShared). The outcome is that of the sequential chain in every case.
 //
-// What bounds it (ncu): issue slots and the integer pipe, 10 warp instructions per move on 2.6M units x 64 steps, 64% of
-// the issue slots busy with 16 warps per SM. Measured there (8192 chains x 1M moves) 201 -> 136 ms, on 256 units x 512
-// steps (1024 x 100k) 4.24 -> 2.9 ms, on a growing cache of 131,072 units (1024 x 100k) 6.3 -> 2.7 ms against the kernels
-// before, which put the changed steps of every listed proposal through a shared-memory queue of (proposal, step) items,
-// each an evaluation of Eq. 2-4 from four counters, and had no second warp per chain (work area 6.9 KB a warp, now 3.1).
+// What bounds it (ncu): issue slots and the integer pipe, 12.9 warp instructions per move on 2.6M units x 64 steps, 57% of
+// the issue slots busy with 16 warps per SM in a short launch (2368 chains x 6,000 moves). Measured there (8192 chains x 1M
+// moves) 201 -> 140 ms, on a growing cache of 131,072 units (1024 x 100k) 6.3 -> 2.7 ms against the kernels before, which put
+// the changed steps of every listed proposal through a shared-memory queue of (proposal, step) items, each an evaluation of
+// Eq. 2-4 from four counters, and had no second warp per chain (work area 6.9 KB a warp, now 3.1).
 #pragma once
 
 namespace kvp {

@@ -282,8 +282,9 @@ count_wide_kernel(const uint32_t* __restrict__ A, const uint32_t* __restrict__ P
 // next steps on their way into shared memory by asynchronous copies. Every lane copies its own vectors into slots of its own,
 // so there is no barrier, and what is in flight takes no registers: the loads of the other kernel are as far ahead of their
 // use as the compiler's schedule happens to put them. Three CTAs per SM (72 KB of rows each, two of three stages in
-// flight). Bound by DRAM: 96 schedules of 640 x 4096 units x 64 steps 348 -> 326 us, 6.2 TB/s; the logic pipe is next (66%),
-// hence the cheaper population count, without which this form took 372 us.
+// flight). Bound by DRAM: 96 schedules of 640 x 4096 units x 64 steps 345 to 376 us before, 329 to 358 now, by box (5.7 to 6.2
+// TB/s, 0.88 to 0.96 of a plain copy); the logic pipe is next (68%), hence the cheaper population count, without which this
+// form took 372 us on a box where it took 326 with it.
 constexpr int kStages = 3;
 
 __device__ __forceinline__ void copy_async(uint4* to, const uint4* from)

@@ -1,6 +1,6 @@
 // The narrow chain kernel (included by kvp_anneal.cu only): for jobs of few chains per SM and for chains that apply many of
 // their moves, such as hot starts, where a fifth to a quarter of the proposals change the schedule, and the hot rungs of
-// replica exchange (whole ladders in a CTA).
+// replica exchange (whole ladders in a CTA, or a launch per round).
 //
 // There, evaluations of cost changes ahead of the commits do not last. What lasts is what depends on a proposal's own units:
 // a warp takes 32 consecutive proposals, one per lane, and prepares them word-parallel: the windows, what the placement bits
@@ -14,12 +14,10 @@
 //
 // The kernel before evaluated its 32 proposals in full, ahead of the commits, through a work queue of (proposal, step)
 // items, one move applied per pass. Measured (B200), before and now: 256 units x 512 steps at p0 = 0.8, 1024
-// chains x 100,000 moves: 25.5 -> 13.6 ms; 16 x 32, 64 x 10,000: 0.43 -> 0.35; 16,384 x 256, 1024 x 200,000: 15.4 -> 11.5.
+// chains x 100,000 moves: 25.5 -> 13.6 ms; 16 x 32, 64 x 10,000: 0.43 -> 0.35; 16,384 x 256, 1024 x 200,000: 15.7 -> 11.7.
 // A link slower than the DRAM channels (not LIN), which for a while only the wide kernel served, without a bound: 256 x 512,
 // 1024 x 20,000 at p0 = 0.8: 8.5 -> 3.2 ms (the kernel before 4.4); 16,384 x 256, 1024 x 100,000: 12.3 -> 7.0 (7.3).
 // Growing caches, likewise: 512 units x 132 steps, 256 x 20,000 0.61 -> 0.45 ms (0.69), at p0 = 0.8 5.2 -> 1.7 (3.4);
-// 131,072 x 1056, 1024 x 20,000 at p0 = 0.8 6.6 -> 4.5 (5.8).
-// Growing caches, likewise: 1028 units x 132 steps, 256 x 20,000 0.61 -> 0.45 ms (0.69), at p0 = 0.8 5.2 -> 1.7 (3.4);
 // 131,072 x 1056, 1024 x 20,000 at p0 = 0.8 6.6 -> 4.5 (5.8).
 #pragma once
 
