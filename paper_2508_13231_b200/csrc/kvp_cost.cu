@@ -458,7 +458,8 @@ score_kernel(const uint32_t* __restrict__ A, const uint32_t* __restrict__ Ps, ui
 // The same for schedules of many steps whose rows take 8 lanes or more (and a vector per lane at most). There the lanes that
 // hold a row's counts, one in LPR, are too few to score it: the counts go to shared memory, kChunk rows at a time, and every
 // thread scores a row. (400 schedules of 2048 units x 2048 steps: 165 -> 89 us, 1024 of 416 x 512: 56 -> 38, 6 of 416 x 2048:
-// 35 -> 19; with rows that follow one another in a group, P[s-1] in registers, 155, and 19: too many streams at a time.)
+// 35 -> 21; with rows that follow one another in a group, P[s-1] in registers, 155, 38 and 21: too many streams at a time. It
+// waits for its loads first; issue slots 65% busy.)
 constexpr uint32_t kChunk = 1024;
 template <int VEC, bool GROW>
 __global__ void __launch_bounds__(1024)
