@@ -143,3 +143,16 @@ def test_failed_call_leaves_nothing_in_flight(kvp, oracle):
         assert first.query()
         out = g.anneal(g.make_params(**kw), want_per_chain=True, stream=second)
         assert [r.astuple() for r in out["per_chain"]] == [r.astuple() for r in ref["per_chain"]]
+
+
+def test_exchange_of_as_many_chains_as_fit(kvp, oracle):
+    """4200 steps: four chains of one warp fill an SM's shared memory, with four warps each only three would fit; a job of nearly
+    four per SM is served all the same."""
+    U, S = 220, 4200
+    A = wl.random_access(U, S, 0.05, seed=3)
+    g, o = both_problems(kvp, oracle, U, 8192, S, A, 20, (8000 * GB, 900 * GB, 900 * GB))
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    kw = dict(moves=40, seed=9, levels=4, temps=[900.0, 300.0, 100.0, 30.0])
+    out = g.anneal_exchange(g.make_params(chains=4 * sms - 4, **kw), 4, 10)
+    ref = o.anneal_exchange(o.make_params(chains=8, **kw), 4, 10)
+    assert [r.astuple() for r in out["per_chain"][:8]] == [r.astuple() for r in ref["per_chain"]]
