@@ -856,6 +856,7 @@ int prepare(kvp_problem* p, const kvp_anneal_params* a, cudaStream_t st, Ctx& c,
         // wide: two warps per chain while an SM has at most 8 (more per chain are no faster)
         if (!c.wide) W = narrow_warps();
         else if (!exchange && chains_per_sm <= 8 && !(c.grow && !c.lin)) W = 2;   // (131,072 x 1056 births, slow link: 1.07 against 1.13 ms)
+        while (W > 1 && fixed_bytes(W, false) + kCowBitsMin / 8 > budget) --W;   // very long horizons
         // replica exchange keeps every chain resident: no more warps than leave room for all of them
         while (exchange && W > 1 && std::min<size_t>(full / W, budget / (fixed_bytes(W, false) + kCowBitsMin / 8)) * sms < a->chains) --W;
         if (forced) W = forced;

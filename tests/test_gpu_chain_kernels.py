@@ -93,6 +93,19 @@ def test_exchange_rounds(kvp, oracle, hooks, warps, chains, rungs):
     assert np.array_equal(to_np(out["best_schedule"]), ref["best_schedule"])
 
 
+@pytest.mark.parametrize("chains", [3, 1184])
+def test_horizon_that_fills_shared_memory(kvp, oracle, chains):
+    """18,600 steps: the state of one chain takes all of an SM's shared memory with one warp and does not fit with four."""
+    U, S = 40, 18600
+    A = wl.random_access(U, S, 0.1, seed=3)
+    g, o = both_problems(kvp, oracle, U, 8192, S, A, 8, (8000 * GB, 900 * GB, 900 * GB))
+    kw = dict(chains=chains, moves=60, seed=9, levels=2, p0=1e-4)
+    out = g.anneal(g.make_params(**kw), want_per_chain=True)
+    for c in (0, 1, chains - 1):
+        want, _, _ = o.anneal_chains(o.make_params(**kw), c, 1)
+        assert out["per_chain"][c].astuple() == want[0].astuple()
+
+
 @pytest.mark.parametrize("busy", [False, True])
 @pytest.mark.parametrize("p0,init", [(1e-6, 1), (1e-6, 0), (0.3, 1)])
 def test_choice_in_global_memory(kvp, oracle, busy, p0, init):
