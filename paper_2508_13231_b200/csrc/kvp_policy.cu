@@ -1,17 +1,18 @@
 // Policy kernels: the look-ahead placement policy of Section III-B (window W, migration ratio R) for many (W, R) pairs
 // at once, the comparison strategies of Section IV-A, and the paper's own annealer that walks the (W, R) grid.
 //
-// A policy is sequential in the steps, so what counts is the latency of one step. A warp (up to 4096 units; several
-// warps of one CTA above that) holds the whole population in registers, 32 units to a word: the resident bitmap H and
-// the units' keys (accesses in the window, reads of the page, time of last use) as bit planes, plane b holding bit b of
-// every unit's key. Then
+// A policy is sequential in the steps, so what counts is the latency of one step. The warps of a CTA hold the whole
+// population in registers, 32 units to a word: the resident bitmap H and the units' keys (accesses in the window, reads of
+// the page, time of last use) as bit planes, plane b holding bit b of every unit's key. Then
 //   - a window slides by a bit-sliced add of the entering and the leaving access row,
-//   - the k-th largest (smallest) key of a set is found from the top plane down, one popc count of the set per plane and
-//     one warp reduction, which also leaves the set of units beyond the threshold and the set of ties at it,
+//   - the k-th largest (smallest) key of a set is the one of the step before or close to it: the sets above and at it come
+//     from a bit-sliced comparison, their sizes from one reduction; else it is found from the top plane down, a count of
+//     the set per plane,
 //   - ties go by unit index: a prefix sum over the lanes, then the lowest bits of one word.
 // Measured on 4096 units x 512 steps (B200): a CTA of 1024 threads with a frequency byte and a shared-memory histogram
 // update per unit and one thread walking the histograms took 9.5 us per step (4.9 ms for one pair, 24.4 ms for the
-// 64 x 11 grid, which is 4.8 CTAs per SM); this form is bound by the latency of its ~20 dependent reductions per step.
+// 64 x 11 grid); a warp with ~20 dependent reductions per step 1.5 us (0.76 and 1.14 ms); this form 0.67 us (0.34 and
+// 0.81), some 300 instructions a warp and step of which a lone warp issues one in four cycles.
 #include <math.h>
 #include <string.h>
 
@@ -32,40 +33,60 @@ constexpr int kFreqPlanes = 7;                           // frequencies are at m
 constexpr int kStampPlanes = 15;                         // times of last use are below 32768
 constexpr uint32_t kPolicyMaxWarps = 8;                  // x 32 lanes x 4 words x 32 units = kPolicyMaxUnits
 
-// Sums over the CTA of a packed pair of 16-bit counts (two sets of units are disjoint and hold at most 32768 units
-// together, so neither field overflows). One warp: a reduction; several: one barrier, the partial sums double-buffered.
+// Sums over the CTA of packed pairs of 16-bit counts (two sets of units are disjoint and hold at most 32768 units
+// together, so neither field overflows). One warp: reductions; several: one barrier, the partial sums double-buffered.
 template <bool MULTI>
 struct CtaSum {
-    uint32_t* buf;                                       // MULTI: [2][kPolicyMaxWarps] shared
+    uint4* buf;                                          // MULTI: [2][kPolicyMaxWarps] shared, zero at first
     uint32_t flip;
+    // Three sums at once, so that what a step wants to know costs one round trip. What does not depend on them goes between
+    // begin and end: it is worked on while the sums are on their way.
+    __device__ __forceinline__ void begin(uint32_t& x, uint32_t& y, uint32_t& z)
+    {
+        x = __reduce_add_sync(0xFFFFFFFFu, x);
+        y = __reduce_add_sync(0xFFFFFFFFu, y);
+        z = __reduce_add_sync(0xFFFFFFFFu, z);
+    }
+    // by, bz: of y and z, what the warps before this one counted
+    __device__ __forceinline__ void end(uint32_t& x, uint32_t& y, uint32_t& z, uint32_t& by, uint32_t& bz)
+    {
+        by = bz = 0u;
+        if (!MULTI) return;
+        const uint32_t warp = threadIdx.x >> 5;
+        uint4* const b = buf + (flip ^= kPolicyMaxWarps);
+        if ((threadIdx.x & 31) == 0) b[warp] = make_uint4(x, y, z, 0u);
+        __syncthreads();
+        x = y = z = 0u;
+#pragma unroll
+        for (uint32_t h = 0; h < kPolicyMaxWarps; h += 4) {   // the slots of absent warps stay 0
+            if (h * 32 >= blockDim.x) break;
+#pragma unroll
+            for (uint32_t w = h; w < h + 4; ++w) {
+                const uint4 v = b[w];
+                if (w == warp) { by = y; bz = z; }
+                x += v.x; y += v.y; z += v.z;
+            }
+        }
+    }
+    __device__ __forceinline__ void end(uint32_t& x, uint32_t& y, uint32_t& z)
+    {
+        uint32_t by, bz;
+        end(x, y, z, by, bz);
+    }
     __device__ __forceinline__ uint32_t operator()(uint32_t v)
     {
-        v = __reduce_add_sync(0xFFFFFFFFu, v);
-        if (!MULTI) return v;
-        uint32_t* b = buf + (flip ^= kPolicyMaxWarps);
-        if ((threadIdx.x & 31) == 0) b[threadIdx.x >> 5] = v;
-        __syncthreads();
-        const uint4 x = *reinterpret_cast<const uint4*>(b), y = *reinterpret_cast<const uint4*>(b + 4);
-        return x.x + x.y + x.z + x.w + y.x + y.y + y.z + y.w;   // the slots of absent warps stay 0
+        uint32_t y = 0u, z = 0u;
+        begin(v, y, z);
+        end(v, y, z);
+        return v;
     }
-    // sum over the threads before this one (threads own ascending unit indices)
-    __device__ __forceinline__ uint32_t before(uint32_t v)
+    // the same and what the warps before this one counted
+    __device__ __forceinline__ uint32_t operator()(uint32_t v, uint32_t& before)
     {
-        const uint32_t lane = threadIdx.x & 31;
-        uint32_t incl = v;
-#pragma unroll
-        for (int off = 1; off < 32; off <<= 1) {
-            const uint32_t o = __shfl_up_sync(0xFFFFFFFFu, incl, off);
-            if (lane >= (uint32_t)off) incl += o;
-        }
-        uint32_t base = 0;
-        if (MULTI) {
-            uint32_t* b = buf + (flip ^= kPolicyMaxWarps);
-            if (lane == 31) b[threadIdx.x >> 5] = incl;
-            __syncthreads();
-            for (uint32_t w = 0; w < (threadIdx.x >> 5); ++w) base += b[w];
-        }
-        return base + incl - v;
+        uint32_t x = 0u, z = 0u, bz;
+        begin(x, v, z);
+        end(x, v, z, before, bz);
+        return v;
     }
 };
 
@@ -78,27 +99,35 @@ __device__ __forceinline__ uint32_t popcn(const uint32_t (&m)[WPL])
     return c;
 }
 
-// the r lowest set bits of w (0 < r < popc(w))
-__device__ __forceinline__ uint32_t lowest_bits(uint32_t w, uint32_t r)
-{
-    uint32_t pos = 0;                                    // the largest cut with at most r bits below it
-#pragma unroll
-    for (uint32_t step = 16; step > 0; step >>= 1)
-        if (__popc(w & ((1u << (pos + step)) - 1u)) <= r) pos += step;
-    return w & ((1u << pos) - 1u);
-}
-
-// Leaves in m its first `take` bits in unit order, given how many bits of the set lie in the threads before this one.
+// Leaves in m, a set of units, its first `take` units in unit order; `before` of them are in the warps before this one.
 template <int WPL>
-__device__ __forceinline__ void first_bits(uint32_t (&m)[WPL], uint32_t before, uint32_t take)
+__device__ __forceinline__ void first_units(uint32_t (&m)[WPL], uint32_t take, uint32_t before)
 {
-    int r = (int)take - (int)before;
+    const uint32_t lane = threadIdx.x & 31, mine = popcn(m);
+    uint32_t upto = mine;                                // threads own ascending unit indices
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+        const uint32_t o = __shfl_up_sync(0xFFFFFFFFu, upto, off);
+        if (lane >= (uint32_t)off) upto += o;
+    }
+    int r = (int)(take - before - (upto - mine));
+    uint32_t part = 0, left = 0;                         // the word that is cut, in one lane at most: what stays of it
+    int at = -1;
 #pragma unroll
     for (int j = 0; j < WPL; ++j) {
         const int c = __popc(m[j]);
-        if (r <= 0) m[j] = 0u;
-        else if (r < c) m[j] = lowest_bits(m[j], (uint32_t)r);
+        if (r > 0 && r < c) { part = m[j]; left = (uint32_t)r; at = j; }
+        if (r < c) m[j] = 0u;
         r -= c;
+    }
+    const uint32_t who = __ballot_sync(0xFFFFFFFFu, at >= 0);
+    if (who) {                                           // warp-uniform; its bits are looked at by a lane each
+        const int src = __ffs(who) - 1;
+        const uint32_t w = __shfl_sync(0xFFFFFFFFu, part, src), n = __shfl_sync(0xFFFFFFFFu, left, src);
+        const uint32_t stay = __ballot_sync(0xFFFFFFFFu, ((w >> lane) & 1u) && (uint32_t)__popc(w & ((1u << lane) - 1u)) < n);
+#pragma unroll
+        for (int j = 0; j < WPL; ++j)
+            if (j == at) m[j] = stay;
     }
 }
 
@@ -140,74 +169,205 @@ __device__ __forceinline__ void slide(uint32_t (&plane)[NP][WPL], int np, const 
     }
 }
 
-// One step of the look-ahead rule: at most `want` of the candidates move in, the best first; they take the free
-// capacity, then the next ones replace residents of lower key, lowest first. H is updated; I units came in, `swaps` of
-// them for a resident. kb = want less the free capacity bounds the swaps from one side, the keys from the other: m swaps
-// are possible iff some threshold t has insf + m candidates with key >= t and m residents with key < t, so their number
-// is the maximum over t of min(C(t) - insf, R(t)), C falling and R rising in t, reached where the two cross.
-//   quota: the want-th best candidate and the kb-th lowest resident, both descents side by side; right when the first
-//          key is above the second.
-//   cross: the crossing, one descent over both sets; right when it gives at most kb swaps, and then its threshold cuts
-//          both sets: candidates above it and residents below it move, of those at it as many as are still to move.
-// Either is one count per plane. `limited` remembers which was right at the step before and goes first.
-template <int WPL, int NP, bool MULTI>
-__device__ __forceinline__ void exchange_units(const uint32_t (&plane)[NP][WPL], int np, const uint32_t (&cand)[WPL],
-                                               uint32_t want, uint32_t free_slots, uint32_t (&H)[WPL],
-                                               CtaSum<MULTI>& sum, bool& limited, uint32_t& I, uint32_t& swaps)
+// the units whose key is above k, and those whose key is k
+template <int WPL, int NP>
+__device__ __forceinline__ void split_keys(const uint32_t (&plane)[NP][WPL], uint32_t k, uint32_t (&gt)[WPL], uint32_t (&eq)[WPL])
 {
-    const uint32_t insf = min(want, free_slots), kb = want - insf;
-    uint32_t mc[WPL], mr[WPL], in[WPL], out[WPL], needC, needR;   // ties at the thresholds, units beyond them
-    for (bool quota = limited || kb == 0;; quota = !quota) {      // two passes at most
 #pragma unroll
-        for (int j = 0; j < WPL; ++j) { mc[j] = cand[j]; mr[j] = H[j]; in[j] = 0u; out[j] = 0u; }
-        uint32_t above = 0, below = 0, keyC = 0, keyR = 0;
-        needC = want; needR = kb;
+    for (int j = 0; j < WPL; ++j) { gt[j] = 0u; eq[j] = 0xFFFFFFFFu; }
 #pragma unroll
-        for (int b = NP - 1; b >= 0; --b) {
-            if (b >= np) continue;
-            uint32_t c = 0;
+    for (int b = NP - 1; b >= 0; --b) {
+        const uint32_t kb = (uint32_t)((int)(k << (31 - b)) >> 31);
 #pragma unroll
-            for (int j = 0; j < WPL; ++j) c += (__popc(mc[j] & plane[b][j]) << 16) + __popc(mr[j] & ~plane[b][j]);
-            c = sum(c);
-            const uint32_t cc = c >> 16, cr = c & 0xFFFFu;
-            uint32_t tc, tr;                              // all ones: go on among the set bits (C), among the clear ones (R)
-            if (quota) {
-                tc = needC <= cc ? 0xFFFFFFFFu : 0u;
-                tr = needR <= cr ? 0xFFFFFFFFu : 0u;
-                needC -= cc & ~tc; needR -= cr & ~tr;
-                keyC |= tc & (1u << b); keyR |= ~tr & (1u << b);
-            } else {
-                tc = above + cc >= insf + below + cr ? 0xFFFFFFFFu : 0u;
-                tr = ~tc;
-                above += cc & ~tc; below += cr & tc;
-            }
-#pragma unroll
-            for (int j = 0; j < WPL; ++j) {
-                const uint32_t p = plane[b][j];
-                in[j] |= mc[j] & p & ~tc;
-                mc[j] &= ~(p ^ tc);
-                out[j] |= mr[j] & ~p & ~tr;
-                mr[j] &= p ^ tr;
-            }
-        }
-        if (quota) {
-            swaps = kb;
-            if (kb == 0 || keyC > keyR) break;
-            limited = false;
-        } else {
-            swaps = max(below, above > insf ? above - insf : 0u);
-            needC = insf + swaps - above; needR = swaps - below;
-            if (swaps <= kb) break;
-            limited = true;
+        for (int j = 0; j < WPL; ++j) {
+            gt[j] |= eq[j] & plane[b][j] & ~kb;
+            eq[j] &= ~(plane[b][j] ^ kb);
         }
     }
-    I = insf + swaps;
-    if (!I) return;
-    const uint32_t bf = sum.before((popcn(mc) << 16) + popcn(mr));
-    first_bits(mc, bf >> 16, needC);
-    first_bits(mr, bf & 0xFFFFu, needR);
+}
+
+// The look-ahead rule: of the nC candidates (units outside HBM with a key above 0) at most want = nC * permille / 1000 move
+// in, the best first; they take the free capacity, then the next ones replace residents of lower key, lowest first.
+// kb = want less the free capacity bounds the swaps from one side, the keys from the other: m swaps are possible iff some
+// threshold t has insf + m candidates with key >= t and m residents with key < t, so their number is the maximum over t of
+// min(C(t) - insf, R(t)), C falling and R rising in t, reached where the two cross.
+//   quota: the want-th best candidate and the kb-th lowest resident; right when the first key is above the second.
+//   cross: the crossing, the largest t with C(t) >= insf + R(t); right when it gives at most kb swaps, and then its
+//          threshold cuts both sets: candidates above it and residents below it move, of those at it as many as are still
+//          to move.
+// The thresholds of a sliding window seldom move from step to step, so those of the step before are tried first: one
+// reduction of the counts above and at them shows whether they hold, and which way to go where they do not. What the
+// comparison needs of the keys alone (Keyed) is worked out a step ahead, while the reduction is under way. Where the
+// thresholds do not hold, they are moved a few times, then found from the top plane down, a count per plane.
+// Measured on 4096 units x 512 steps, the descent in every step against this: one policy 760 -> 342 us, the 64 x 11 grid
+// 1143 -> 811; page granularity 463 -> 275. The thresholds hold in 19 of 20 steps at windows of 16 and 32, in 9 of 10 at 64.
+struct Cut {
+    uint32_t c, r;                                       // thresholds: of the candidates, of the residents (cross: the same)
+    bool quota;
+};
+
+template <int WPL>
+struct Keyed {                                           // units with a key above 0; candidates: above, at; residents: below, level
+    uint32_t any[WPL], above[WPL], at[WPL], below[WPL], level[WPL];
+};
+
+template <int WPL, int NP>
+__device__ __forceinline__ void compare_keys(const uint32_t (&plane)[NP][WPL], const Cut& cut, Keyed<WPL>& k)
+{
 #pragma unroll
-    for (int j = 0; j < WPL; ++j) H[j] = (H[j] & ~(out[j] | mr[j])) | in[j] | mc[j];
+    for (int j = 0; j < WPL; ++j) {
+        k.any[j] = plane[0][j];
+#pragma unroll
+        for (int b = 1; b < NP; ++b) k.any[j] |= plane[b][j];
+    }
+    split_keys(plane, cut.c, k.above, k.at);
+    if (cut.r == cut.c) {                                // CTA-uniform
+#pragma unroll
+        for (int j = 0; j < WPL; ++j) { k.below[j] = ~(k.above[j] | k.at[j]); k.level[j] = k.at[j]; }
+    } else {
+        split_keys(plane, cut.r, k.below, k.level);
+#pragma unroll
+        for (int j = 0; j < WPL; ++j) k.below[j] = ~(k.below[j] | k.level[j]);
+    }
+}
+
+// What a step comes to: the counts, and how many of the ties at the thresholds move.
+struct Exchange {
+    uint32_t want, insf, kb, swaps, needC, needR;
+    bool found, splitC, splitR;                          // the thresholds hold; some of the ties move and some do not
+};
+// Judges the thresholds by the counts (CTA-uniform) and moves them where they do not hold. False: give up moving.
+__device__ __forceinline__ bool judge_cut(Cut& cut, uint32_t top, uint32_t above, uint32_t at, uint32_t below, uint32_t level, Exchange& e)
+{
+    if (cut.quota) {
+        const int dc = above >= e.want ? 1 : above + at < e.want ? -1 : 0;
+        const int dr = !e.kb ? 0 : below >= e.kb ? -1 : below + level < e.kb ? 1 : 0;
+        e.swaps = e.kb;
+        e.needC = e.want - above; e.needR = e.kb ? e.kb - below : 0u;
+        e.found = !dc && !dr && (!e.kb || cut.c > cut.r);
+        if (!e.found) {
+            if (!dc && !dr) { cut.quota = false; cut.c = cut.r; }
+            cut.c += dc; cut.r += dr;
+        }
+    } else {
+        const int d = above + at < e.insf + below ? -1 : above >= e.insf + below + level ? 1 : 0;
+        e.swaps = max(below, above > e.insf ? above - e.insf : 0u);
+        e.needC = e.insf + e.swaps - above; e.needR = e.swaps - below;
+        e.found = !d && e.swaps <= e.kb;
+        if (!d && !e.found) cut.quota = true;
+        cut.c = cut.r = cut.c + d;
+    }
+    e.splitC = e.needC != 0u && e.needC != at;
+    e.splitR = e.needR != 0u && e.needR != level;
+    return cut.c <= top && cut.r <= top;                 // (beyond: fewer residents than places, or none)
+}
+
+// One step: H is updated, I units came in, `swaps` of them for a resident. k: of this step's keys, for `cut`; ahead():
+// works on the next step meanwhile, and again if the thresholds moved; back(): takes the planes back to this step. hits: a count of the caller's, summed.
+template <int WPL, int NP, bool MULTI, typename Ahead, typename Back>
+__device__ __forceinline__ void exchange_units(uint32_t (&plane)[NP][WPL], int np, const Keyed<WPL>& k, uint32_t permille,
+                                               uint32_t free_slots, uint32_t (&H)[WPL], CtaSum<MULTI>& sum, Cut& cut,
+                                               uint32_t& I, uint32_t& swaps, uint32_t& hits, Ahead ahead, Back back)
+{
+    const uint32_t top = (1u << np) - 1u;
+    uint32_t mc[WPL], mr[WPL], in[WPL], out[WPL];        // ties at the thresholds, units beyond them
+    uint32_t nc = 0, c, r;
+#pragma unroll
+    for (int j = 0; j < WPL; ++j) {
+        in[j] = k.above[j] & ~H[j]; mc[j] = k.at[j] & k.any[j] & ~H[j];
+        out[j] = k.below[j] & H[j]; mr[j] = k.level[j] & H[j];
+        nc += __popc(k.any[j] & ~H[j]);
+    }
+    nc = nc << 16 | hits;
+    c = popcn(in) << 16 | popcn(mc); r = popcn(out) << 16 | popcn(mr);
+    uint32_t bc, br;                                      // of the ties, those of the warps before this one
+    sum.begin(nc, c, r);
+    ahead();
+    sum.end(nc, c, r, bc, br);
+    hits = nc & 0xFFFFu;
+    Exchange e;
+    e.want = (nc >> 16) * permille / 1000u;
+    I = swaps = 0;
+    if (!e.want) return;
+    e.insf = min(e.want, free_slots); e.kb = e.want - e.insf;
+    const Cut was = cut;
+    if (!e.kb) cut.quota = true;                          // nobody has to leave
+    bool go = judge_cut(cut, top, c >> 16, c & 0xFFFFu, r >> 16, r & 0xFFFFu, e);
+    if (!e.found) {                                       // CTA-uniform
+        back();
+        uint32_t cand[WPL];
+#pragma unroll
+        for (int j = 0; j < WPL; ++j) cand[j] = k.any[j] & ~H[j];
+#pragma unroll 1
+        for (int t = 0; t < 2 && go && !e.found; ++t) {
+            Keyed<WPL> n;
+            compare_keys(plane, cut, n);
+#pragma unroll
+            for (int j = 0; j < WPL; ++j) { in[j] = cand[j] & n.above[j]; mc[j] = cand[j] & n.at[j]; out[j] = H[j] & n.below[j]; mr[j] = H[j] & n.level[j]; }
+            c = popcn(in) << 16 | popcn(mc); r = popcn(out) << 16 | popcn(mr);
+            uint32_t none = 0;
+            sum.begin(none, c, r);
+            sum.end(none, c, r, bc, br);
+            go = judge_cut(cut, top, c >> 16, c & 0xFFFFu, r >> 16, r & 0xFFFFu, e);
+        }
+        for (bool quota = cut.quota || e.kb == 0; !e.found; quota = !quota) {   // two passes at most
+#pragma unroll
+            for (int j = 0; j < WPL; ++j) { mc[j] = cand[j]; mr[j] = H[j]; in[j] = 0u; out[j] = 0u; }
+            uint32_t above = 0, below = 0;
+            cut.quota = quota; cut.c = cut.r = 0;
+            e.needC = e.want; e.needR = e.kb;
+#pragma unroll
+            for (int b = NP - 1; b >= 0; --b) {
+                if (b >= np) continue;
+                uint32_t n = 0;
+#pragma unroll
+                for (int j = 0; j < WPL; ++j) n += (__popc(mc[j] & plane[b][j]) << 16) + __popc(mr[j] & ~plane[b][j]);
+                n = sum(n);
+                const uint32_t cc = n >> 16, cr = n & 0xFFFFu;
+                uint32_t tc, tr;                          // all ones: go on among the set bits (C), among the clear ones (R)
+                if (quota) {
+                    tc = e.needC <= cc ? 0xFFFFFFFFu : 0u;
+                    tr = e.needR <= cr ? 0xFFFFFFFFu : 0u;
+                    e.needC -= cc & ~tc; e.needR -= cr & ~tr;
+                } else {
+                    tc = above + cc >= e.insf + below + cr ? 0xFFFFFFFFu : 0u;
+                    tr = ~tc;
+                    above += cc & ~tc; below += cr & tc;
+                }
+                cut.c |= tc & (1u << b); cut.r |= ~tr & (1u << b);   // (cross: the same)
+#pragma unroll
+                for (int j = 0; j < WPL; ++j) {
+                    const uint32_t p = plane[b][j];
+                    in[j] |= mc[j] & p & ~tc;
+                    mc[j] &= ~(p ^ tc);
+                    out[j] |= mr[j] & ~p & ~tr;
+                    mr[j] &= p ^ tr;
+                }
+            }
+            sum((popcn(mc) << 16) + popcn(mr), bc);
+            br = bc; bc >>= 16;
+            e.splitC = e.splitR = true;
+            if (quota) {
+                e.swaps = e.kb;
+                e.found = e.kb == 0 || cut.c > cut.r;
+            } else {
+                e.swaps = max(below, above > e.insf ? above - e.insf : 0u);
+                e.needC = e.insf + e.swaps - above; e.needR = e.swaps - below;
+                e.found = e.swaps <= e.kb;
+            }
+        }
+    }
+    if (cut.c != was.c || cut.r != was.r) ahead();
+    swaps = e.swaps;
+    I = e.insf + swaps;
+    if (!I) return;
+    if (e.splitC) first_units(mc, e.needC, bc & 0xFFFFu);  // CTA-uniform
+    if (e.splitR) first_units(mr, e.needR, br & 0xFFFFu);
+#pragma unroll
+    for (int j = 0; j < WPL; ++j) {
+        const uint32_t gone = e.kb ? out[j] | (e.needR ? mr[j] : 0u) : 0u;
+        H[j] = (H[j] & ~gone) | in[j] | (e.needC ? mc[j] : 0u);
+    }
 }
 
 // the static placement of this thread's words: the row, or the first `cap` of `entities` where there is none
@@ -238,9 +398,9 @@ lookahead_kernel(const uint32_t* __restrict__ A, const uint32_t* __restrict__ ro
                  uint32_t n_ratio, const __grid_constant__ PolicyPairs pairs, uint32_t* __restrict__ out,
                  const StepC* __restrict__ stepc, CostK K, uint64_t* __restrict__ totals)
 {
-    __shared__ __align__(16) uint32_t s_part[2 * kPolicyMaxWarps];
+    __shared__ uint4 s_part[2 * kPolicyMaxWarps];
     if (MULTI) {
-        if (threadIdx.x < 2 * kPolicyMaxWarps) s_part[threadIdx.x] = 0u;
+        if (threadIdx.x < 2 * kPolicyMaxWarps) s_part[threadIdx.x] = make_uint4(0u, 0u, 0u, 0u);
         __syncthreads();
     }
     CtaSum<MULTI> sum{s_part, 0u};
@@ -264,45 +424,43 @@ lookahead_kernel(const uint32_t* __restrict__ A, const uint32_t* __restrict__ ro
             load_row(A + (size_t)t * W32, W32, w0, a);
             slide(plane, np, a, none);
         }
-    bool limited = permille < 1000;
+    Cut cut = {1u, 1u, permille < 1000};
     uint64_t total = 0;
     uint32_t mi = 0, mo = 0, hits = 0;                   // of the step before (its hits are reduced with the next step's count)
-    uint32_t enter[WPL], leave[WPL] = {}, now[WPL];      // rows s + W - 1, s - 1 and s
+    uint32_t enter[WPL], now[WPL];                       // rows s + W and s
+    Keyed<WPL> k;
     load_row(A + (size_t)min(W - 1, S - 1) * W32, W <= S ? W32 : 0u, w0, enter);
+    if (permille) slide(plane, np, enter, none);
+    compare_keys(plane, cut, k);
+    load_row(A + (size_t)min(W, S - 1) * W32, W < S ? W32 : 0u, w0, enter);
     load_row(A, W32, w0, now);
     for (uint32_t s = 0; s < S; ++s) {
         // the rows of the next step are on their way while this one is worked on
-        uint32_t enter2[WPL], now2[WPL];
-        load_row(A + (size_t)min(s + W, S - 1) * W32, s + W < S ? W32 : 0u, w0, enter2);
+        uint32_t enter2[WPL], now2[WPL], I = 0, swaps = 0;
+        load_row(A + (size_t)min(s + 1 + W, S - 1) * W32, s + 1 + W < S ? W32 : 0u, w0, enter2);
         load_row(A + (size_t)min(s + 1, S - 1) * W32, W32, w0, now2);
-        uint32_t cand[WPL], I = 0, swaps = 0;
         if (permille) {
-            slide(plane, np, enter, leave);
-#pragma unroll
-            for (int j = 0; j < WPL; ++j) {
-                uint32_t any = plane[0][j];
-#pragma unroll
-                for (int b = 1; b < kFreqPlanes; ++b) any |= plane[b][j];
-                cand[j] = any & ~H[j];
-            }
+            const Keyed<WPL> of_now = k;
+            bool moved = false;                          // the planes are the next step's
+            exchange_units(plane, np, of_now, permille, cap - nR, H, sum, cut, I, swaps, hits,
+                           [&] {
+                               if (!moved) slide(plane, np, enter, now);
+                               moved = true;
+                               compare_keys(plane, cut, k);
+                           },
+                           [&] { slide(plane, np, now, enter); moved = false; });
+            if (!moved) { slide(plane, np, enter, now); compare_keys(plane, cut, k); }
         } else {
-#pragma unroll
-            for (int j = 0; j < WPL; ++j) cand[j] = 0u;
+            hits = sum(hits);
         }
-        const uint32_t both = sum((popcn(cand) << 16) + hits);
-        const uint32_t nC = both >> 16;
-        if (totals && s) total += step_cost(both & 0xFFFFu, mi, mo, __ldg(stepc + s - 1), K);
-        const uint32_t want = nC * permille / 1000u;
-        if (want) {
-            exchange_units(plane, np, cand, want, cap - nR, H, sum, limited, I, swaps);
-            nR += I - swaps;
-        }
+        if (totals && s) total += step_cost(hits, mi, mo, __ldg(stepc + s - 1), K);
+        nR += I - swaps;
         mi = s ? I : 0u; mo = s ? swaps : 0u;            // the migrations of step 0 are free
         hits = 0;
 #pragma unroll
         for (int j = 0; j < WPL; ++j) {
             hits += __popc(now[j] & H[j]);
-            leave[j] = now[j]; now[j] = now2[j]; enter[j] = enter2[j];
+            now[j] = now2[j]; enter[j] = enter2[j];
         }
         if (mine) store_row(mine + (size_t)s * W32, W32, w0, H);
     }
@@ -339,37 +497,39 @@ template <int WPL, bool MULTI>
 __global__ void __launch_bounds__(MULTI ? 32 * kPolicyMaxWarps : 32)
 page_kernel(const uint32_t* __restrict__ planes, int np, uint32_t S, uint32_t EW32, uint32_t cap, uint32_t* __restrict__ pages)
 {
-    __shared__ __align__(16) uint32_t s_part[2 * kPolicyMaxWarps];
+    __shared__ uint4 s_part[2 * kPolicyMaxWarps];
     if (MULTI) {
-        if (threadIdx.x < 2 * kPolicyMaxWarps) s_part[threadIdx.x] = 0u;
+        if (threadIdx.x < 2 * kPolicyMaxWarps) s_part[threadIdx.x] = make_uint4(0u, 0u, 0u, 0u);
         __syncthreads();
     }
     CtaSum<MULTI> sum{s_part, 0u};
     const uint32_t w0 = threadIdx.x * WPL;
-    uint32_t H[WPL], plane[kPagePlanes][WPL], next[kPagePlanes][WPL];
+    uint32_t H[WPL], plane[kPagePlanes][WPL], next[kPagePlanes][WPL], after[kPagePlanes][WPL];   // of this step, the next, the one after
     initial_row<WPL>(nullptr, EW32, w0, cap, H);
     uint32_t nR = sum(popcn(H));
     auto fetch = [&](uint32_t s) {
 #pragma unroll
-        for (int b = 0; b < kPagePlanes; ++b) load_row(planes + ((size_t)s * np + min(b, np - 1)) * EW32, b < np ? EW32 : 0u, w0, next[b]);
+        for (int b = 0; b < kPagePlanes; ++b) load_row(planes + ((size_t)s * np + min(b, np - 1)) * EW32, b < np ? EW32 : 0u, w0, after[b]);
     };
     fetch(0);
-    bool limited = false;
+#pragma unroll
+    for (int b = 0; b < kPagePlanes; ++b)
+#pragma unroll
+        for (int j = 0; j < WPL; ++j) next[b][j] = after[b][j];
+    fetch(min(1u, S - 1));
+    Cut cut = {1u, 1u, false};
+    Keyed<WPL> k;
+    compare_keys(next, cut, k);
     for (uint32_t s = 0; s < S; ++s) {
-        uint32_t cand[WPL], I = 0, swaps = 0;
+        const Keyed<WPL> mine = k;
+        uint32_t I, swaps, none = 0;
 #pragma unroll
-        for (int j = 0; j < WPL; ++j) {
-            uint32_t any = 0;
+        for (int b = 0; b < kPagePlanes; ++b)
 #pragma unroll
-            for (int b = 0; b < kPagePlanes; ++b) { plane[b][j] = next[b][j]; any |= next[b][j]; }
-            cand[j] = any & ~H[j];
-        }
-        fetch(min(s + 1, S - 1));
-        const uint32_t nC = sum(popcn(cand));
-        if (nC) {
-            exchange_units(plane, np, cand, nC, cap - nR, H, sum, limited, I, swaps);
-            nR += I - swaps;
-        }
+            for (int j = 0; j < WPL; ++j) { plane[b][j] = next[b][j]; next[b][j] = after[b][j]; }
+        fetch(min(s + 2, S - 1));
+        exchange_units(plane, np, mine, 1000u, cap - nR, H, sum, cut, I, swaps, none, [&] { compare_keys(next, cut, k); }, [] {});
+        nR += I - swaps;
         store_row(pages + (size_t)s * EW32, EW32, w0, H);
     }
 }
@@ -401,9 +561,9 @@ __global__ void __launch_bounds__(MULTI ? 32 * kPolicyMaxWarps : 32)
 reactive_kernel(const uint32_t* __restrict__ A, const uint32_t* __restrict__ row0, uint32_t S, uint32_t W32, uint32_t cap,
                 uint32_t* __restrict__ out)
 {
-    __shared__ __align__(16) uint32_t s_part[2 * kPolicyMaxWarps];
+    __shared__ uint4 s_part[2 * kPolicyMaxWarps];
     if (MULTI) {
-        if (threadIdx.x < 2 * kPolicyMaxWarps) s_part[threadIdx.x] = 0u;
+        if (threadIdx.x < 2 * kPolicyMaxWarps) s_part[threadIdx.x] = make_uint4(0u, 0u, 0u, 0u);
         __syncthreads();
     }
     CtaSum<MULTI> sum{s_part, 0u};
@@ -425,11 +585,13 @@ reactive_kernel(const uint32_t* __restrict__ A, const uint32_t* __restrict__ row
         load_row(A + (size_t)(s + 1) * W32, W32, w0, a2);
 #pragma unroll
         for (int j = 0; j < WPL; ++j) { miss[j] = a[j] & ~H[j]; oldest[j] &= ~a[j]; }
-        const uint32_t both = sum((popcn(miss) << 16) + popcn(oldest));
+        uint32_t ahead;                                  // of the two, what the warps before this one have
+        const uint32_t both = sum((popcn(miss) << 16) + popcn(oldest), ahead);
         const uint32_t nM = both >> 16;
         uint32_t n_old = both & 0xFFFFu;
         const uint32_t promoted = min(nM, cap), free_slots = cap - nR;
-        if (promoted < nM) first_bits(miss, sum.before(popcn(miss)), promoted);   // CTA-uniform
+        if (promoted < nM) first_units(miss, promoted, ahead >> 16);   // CTA-uniform
+        ahead &= 0xFFFFu;
 #pragma unroll
         for (int b = 0; b < kStampPlanes; ++b) {
             if (b >= np) continue;
@@ -455,14 +617,14 @@ reactive_kernel(const uint32_t* __restrict__ A, const uint32_t* __restrict__ row
                     if (b < np) other |= plane[b][j] ^ ((tau >> b) & 1u ? 0xFFFFFFFFu : 0u);
                 oldest[j] = H[j] & ~other;
             }
-            n_old = sum(popcn(oldest));
+            n_old = sum(popcn(oldest), ahead);
             if (tau > s + 1) break;                      // never reached: the keys of the residents end at s + 1
         }
         if (evict) {                                     // CTA-uniform
             uint32_t gone[WPL];
 #pragma unroll
             for (int j = 0; j < WPL; ++j) gone[j] = oldest[j];
-            first_bits(gone, sum.before(popcn(gone)), evict);
+            if (evict < n_old) first_units(gone, evict, ahead);   // CTA-uniform
 #pragma unroll
             for (int j = 0; j < WPL; ++j) { H[j] &= ~gone[j]; oldest[j] &= ~gone[j]; }
         }
@@ -485,9 +647,11 @@ struct WRK {
 
 // The paper's annealer over (W, R): one warp per chain, the objective is a table lookup. The lanes hold the chain's next
 // 32 proposals and test all of them against the present point; the first one that is accepted is taken, and the lanes
-// after it test again from there. A walk of n iterations so costs n / 32 draws plus one short round per accepted move (a
-// few tests in flight at once, 0.1 us) instead of n times the latency of a draw and two lookups (0.25 us).
-// TSMEM: the table is staged in shared memory. The level's acceptance row always is.
+// after it test again from there. What bounds a walk is the latency of a round, one per accepted move, so all that does not
+// depend on the point is worked out when the proposals are drawn: the largest change each lets pass (a search in the level's
+// row of thresholds, which fall). A round is then one lookup, a compare, a vote and the shuffles that tell the new point: 64
+// walks of 2000 iterations over a 64 x 11 grid 312 -> 193 us (before, each round looked a threshold up behind the cost).
+// TSMEM: the table is staged in shared memory. The level's acceptance row always is; the next one is on its way meanwhile.
 template <bool TSMEM>
 __global__ void __launch_bounds__(32)
 wr_anneal_kernel(const WRK k, kvp_wr_result* __restrict__ results)
@@ -499,23 +663,32 @@ wr_anneal_kernel(const WRK k, kvp_wr_result* __restrict__ results)
     if (TSMEM)
         for (uint32_t i = lane; i < k.w_max * k.n_ratio; i += 32) tab_s[i] = __ldg(k.table + i);
     const uint64_t* const tab = TSMEM ? tab_s : k.table;
+    constexpr uint32_t kRow4 = KVP_TABLE_Q / 128;        // uint4 of a row in each lane
+    const uint4* const rows = reinterpret_cast<const uint4*>(k.acc) + lane;
+    uint4 row[kRow4];
+#pragma unroll
+    for (uint32_t q = 0; q < kRow4; ++q) row[q] = __ldg(rows + q * 32);
+    uint32_t shift = __ldg(k.shifts);
     __syncwarp();
-    uint32_t w = k.w0, r = k.r0;
-    uint64_t cur = tab[(size_t)(w - 1) * k.n_ratio + r];
+    int w = (int)k.w0 - 1, r = (int)k.r0;                // the point, from 0
+    const int w_max = (int)k.w_max, n_ratio = (int)k.n_ratio;
+    uint64_t cur = tab[(size_t)w * n_ratio + r];
     kvp_wr_result res;
-    res.best_ticks = cur; res.best_w = w; res.best_r = r; res.n_accepted = 0;
-    uint64_t bab = cur, i = 0;
+    res.best_ticks = cur; res.best_w = k.w0; res.best_r = k.r0; res.n_accepted = 0;
+    uint64_t bab = res.best_ticks, i = 0;
     for (uint32_t level = 0; level < k.levels && i < k.iters; ++level) {
         if (level) {
             if (k.early_permille && (bab - res.best_ticks) * 1000ull < bab * (uint64_t)k.early_permille) break;
             bab = res.best_ticks;
         }
         __syncwarp();
-        const uint4* src = reinterpret_cast<const uint4*>(k.acc + (size_t)level * KVP_TABLE_Q);
 #pragma unroll
-        for (uint32_t q = 0; q < KVP_TABLE_Q / 128; ++q) reinterpret_cast<uint4*>(acc)[q * 32 + lane] = __ldg(src + q * 32 + lane);
+        for (uint32_t q = 0; q < kRow4; ++q) reinterpret_cast<uint4*>(acc)[q * 32 + lane] = row[q];
         __syncwarp();
-        const uint32_t shift = __ldg(k.shifts + level);
+        const uint32_t bin = shift, next = min(level + 1, k.levels - 1);
+#pragma unroll
+        for (uint32_t q = 0; q < kRow4; ++q) row[q] = __ldg(rows + (size_t)next * (KVP_TABLE_Q / 4) + q * 32);
+        shift = __ldg(k.shifts + next);
         const uint64_t end = level + 1 < k.levels ? min(i + k.per_level, k.iters) : k.iters;
         for (; i < end; i += 32) {
             const uint64_t it = i + lane;
@@ -524,28 +697,33 @@ wr_anneal_kernel(const WRK k, kvp_wr_result* __restrict__ results)
             const uint32_t sel = x[0] & 255u, d = (x[0] >> 8) & 3u;
             const int dw = sel < 102u || sel >= 204u ? (int)d - (d < 2u ? 2 : 1) : 0;   // window, diagonal: {-2, -1, 1, 2}
             const int dr = sel < 102u ? 0 : ((x[0] >> 10) & 1u) ? 1 : -1;               // ratio, diagonal
+            // Metropolis: a change passes if it is 0 or less, or if its bin is among the first `bins`, whose thresholds are
+            // above the proposal's uniform
+            uint32_t bins = 0;
+#pragma unroll
+            for (uint32_t step = KVP_TABLE_Q / 2; step > 0; step >>= 1)
+                if (x[3] < acc[bins + step - 1]) bins += step;
+            if (x[3] < acc[bins]) ++bins;                // (at most KVP_TABLE_Q - 1 before)
+            const uint64_t pass = (uint64_t)bins << bin;
             uint32_t open = end - i >= 32 ? 0xFFFFFFFFu : (1u << (uint32_t)(end - i)) - 1u;
             for (;;) {
-                const int nw = (int)w + dw, nr = (int)r + dr;
-                const bool on = nw >= 1 && nw <= (int)k.w_max && nr >= 0 && nr < (int)k.n_ratio;   // off the grid: discarded
-                const uint64_t cand = tab[on ? (size_t)(nw - 1) * k.n_ratio + nr : 0];
-                const uint64_t q = cand <= cur ? 0 : (cand - cur) >> shift;
-                const uint32_t thr = acc[min(q, (uint64_t)KVP_TABLE_Q - 1)];
-                const bool accept = on && (cand <= cur || (q < KVP_TABLE_Q && x[3] < thr));        // Metropolis
-                const uint32_t yes = __ballot_sync(0xFFFFFFFFu, accept) & open;
+                const int nw = w + dw, nr = r + dr;
+                const bool on = (uint32_t)nw < (uint32_t)w_max && (uint32_t)nr < (uint32_t)n_ratio;   // off the grid: discarded
+                const uint64_t cand = tab[on ? (size_t)nw * n_ratio + nr : 0];
+                const uint32_t yes = __ballot_sync(0xFFFFFFFFu, on && (cand <= cur || cand - cur < pass)) & open;
                 if (!yes) break;
                 const int j = __ffs(yes) - 1;
-                w = __shfl_sync(0xFFFFFFFFu, (uint32_t)nw, j);
-                r = __shfl_sync(0xFFFFFFFFu, (uint32_t)nr, j);
+                w = __shfl_sync(0xFFFFFFFFu, nw, j);
+                r = __shfl_sync(0xFFFFFFFFu, nr, j);
                 cur = __shfl_sync(0xFFFFFFFFu, cand, j);
                 ++res.n_accepted;
-                if (cur < res.best_ticks) { res.best_ticks = cur; res.best_w = w; res.best_r = r; }
+                if (cur < res.best_ticks) { res.best_ticks = cur; res.best_w = (uint32_t)w + 1u; res.best_r = (uint32_t)r; }
                 open &= 0xFFFFFFFEu << j;                // the proposals after the accepted one
             }
         }
         i = end;
     }
-    res.iters_done = i; res.final_ticks = cur; res.final_w = w; res.final_r = r;
+    res.iters_done = i; res.final_ticks = cur; res.final_w = (uint32_t)w + 1u; res.final_r = (uint32_t)r;
     if (lane == 0) results[c] = res;
 }
 
@@ -554,15 +732,17 @@ wr_anneal_kernel(const WRK k, kvp_wr_result* __restrict__ results)
 }  // namespace kvp
 
 using namespace kvp;
-
-// Words per thread and threads of a policy CTA: one warp holds up to 128 words (4096 units); more warps above that.
+// Words per thread and threads of a policy CTA. A word to a thread up to 8 warps (8192 units), four above that: what a step
+// costs is a warp's instructions, most of them per word. Against a single warp of two or four words to a thread up to 4096
+// units and two warps of four up to 8192, on 4096 units x 512 steps: reactive 397 -> 299 us, one policy 530 -> 342, the 704 of
+// a grid 955 -> 811 (two warps of two words 791, but on 2470 units x 192 steps 752 against 691 us a search); 6693 x 166: a
+// whole search 760 -> 650 us.
 #define KVP_POLICY(kernel, words, grid, ...)                                                                    \
     do {                                                                                                        \
-        const uint32_t words_ = (words);                                                                        \
-        if (words_ <= 32) kernel<1, false><<<grid, 32, 0, st>>>(__VA_ARGS__);                                   \
-        else if (words_ <= 64) kernel<2, false><<<grid, 32, 0, st>>>(__VA_ARGS__);                              \
-        else if (words_ <= 128) kernel<4, false><<<grid, 32, 0, st>>>(__VA_ARGS__);                             \
-        else kernel<4, true><<<grid, (words_ + 127) / 128 * 32, 0, st>>>(__VA_ARGS__);                          \
+        const uint32_t words_ = (words), grid_ = (grid);                                                        \
+        if (words_ <= 32) kernel<1, false><<<grid_, 32, 0, st>>>(__VA_ARGS__);                                  \
+        else if (words_ <= 32 * kPolicyMaxWarps) kernel<1, true><<<grid_, (words_ + 31) / 32 * 32, 0, st>>>(__VA_ARGS__); \
+        else kernel<4, true><<<grid_, (words_ + 127) / 128 * 32, 0, st>>>(__VA_ARGS__);                         \
         KVP_CUDA(cudaGetLastError());                                                                           \
     } while (0)
 

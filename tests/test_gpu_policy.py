@@ -103,3 +103,34 @@ def test_named_policies(kvp, oracle):
     g, o, cfg, A = named_problem(kvp, oracle, "layer_8b")
     assert np.array_equal(to_np(g.policy_reactive()), oracle.policy_reactive(o))
     assert np.array_equal(to_np(g.policy_page(16)), oracle.policy_page(o, 16))
+
+
+@pytest.mark.parametrize("U", [1024, 1056, 4096, 8192, 8224])
+def test_keys_that_jump(kvp, oracle, U):
+    """Steps that read next to nothing or nearly everything, so that the thresholds of the step before do not hold; the last
+    population of one warp, of words of one to a thread and the first of several words, and the one before each."""
+    S = 40
+    rng = np.random.default_rng(U)
+    rate = rng.choice([0.0, 0.01, 0.3, 0.9], size=S)
+    bits = rng.random((S, U)) < rate[:, None] * rng.choice([0.3, 1.0], size=U)
+    A = np.packbits(bits, axis=1, bitorder="little").view(np.uint32)
+    for cap in (0, U // 50, U // 3, U):
+        g, o = both_problems(kvp, oracle, U, 8192, S, A, cap, (8000 * GB, 900 * GB, 900 * GB))
+        pairs = [(1, 1000), (2, 40), (3, 999), (8, 500), (40, 70), (64, 1000)]
+        got = to_np(g.policy_lookahead([w for w, _ in pairs], [r for _, r in pairs]))
+        for i, (w, r) in enumerate(pairs):
+            assert np.array_equal(got[i], oracle.policy_lookahead(o, w, r)), (cap, w, r)
+        assert np.array_equal(to_np(g.policy_reactive()), oracle.policy_reactive(o)), cap
+        for page in (2, 32):
+            assert np.array_equal(to_np(g.policy_page(page)), oracle.policy_page(o, page)), (cap, page)
+        assert np.array_equal(u64(g.wr_grid(5, 4)), oracle.wr_grid(o, 5, 4)), cap
+
+
+@pytest.mark.parametrize("w_max,n_ratio,top", [(64, 101, 10 ** 6), (5, 2, 3), (20, 11, 2 ** 42), (7, 7, 1)])
+def test_walk_on_any_table(kvp, oracle, w_max, n_ratio, top):
+    """Tables beyond shared memory, of equal costs, of costs far apart and of large ones (their differences decide)."""
+    T = np.random.default_rng(w_max).integers(0, top, size=(w_max, n_ratio), dtype=np.uint64) + np.uint64(2 ** 63 if top == 3 else 5)
+    dev = torch.from_numpy(T.view(np.int64)).cuda()
+    for kw in (dict(chains=9, iters=3001, seed=3, levels=8), dict(chains=2, iters=40, seed=4, levels=64, p0=0.01, alpha=0.5)):
+        res, best = kvp.wr_anneal(dev, kvp.wr_params(**kw))
+        assert [r.astuple() for r in res] == [r.astuple() for r in oracle.wr_anneal(T, oracle.wr_params(**kw))]
