@@ -70,17 +70,24 @@ static_assert(sizeof(ChainShared) % 16 == 0, "uint4 slots");
 // Work area of a warp: a ring of listed proposals with their placement windows, the accepted ones that change the schedule
 // in move order, by proposal of the batch what spoiled needs and (when it is evaluated again) what became of it, and the
 // list of those to evaluate again. A batch with more accepted ones than fit goes on where they end once these are applied.
-// Rows of 32 proposals a warp works on side by side: with schedules in global memory two, so that their loads overlap
-// (144 against 168 ms on the largest configuration, four: 148); with births, whose loads come first, one (2.7 against 4.6
-// ms); in shared memory one, for there the instruction cache counts (four rows: 2000 instructions in a batch's path, and
-// a warp waited for the next one a quarter of the time).
+// Rows of 32 proposals a warp works on side by side: with schedules in global memory and columns of two words two, so that
+// their loads overlap (144 against 168 ms on the largest configuration, four: 148); in shared memory one, for there the
+// instruction cache counts (four rows: 2000 instructions in a batch's path, and a warp waited for the next one a quarter of
+// the time); with births, whose loads come first, one (2.7 against 4.6 ms).
+// Columns of other lengths, whose loads take longer, are loaded a row ahead (load_ahead): while a row is listed and judged the
+// next one's columns are on their way. 32,768 units x 256 steps, 2368 chains x 50,000: 3.17 -> 2.31 ms (two rows ahead: 2.62);
+// 131,072 x 100, 1500 x 50,000: 1.87 -> 1.80; 65,536 x 128, 2368 x 50,000: 2.63 -> 2.54. Not where a column is two words: its
+// loads stay in flight for less than the longer path costs (131,072 x 64, 2368 x 20,000: 0.75 -> 0.79 ms).
 constexpr uint32_t kAccepted = 6;
-__host__ __device__ constexpr int rows_at_a_time(bool psmem, bool grow) { return psmem || grow ? 1 : 2; }
-__host__ __device__ constexpr uint32_t ring_size(bool psmem, bool grow) { return rows_at_a_time(psmem, grow) > 1 ? 128u : 64u; }
-__host__ __device__ constexpr uint32_t work4(bool psmem, bool grow, int rows)   // uint4 slots of it
+__host__ __device__ constexpr bool load_ahead(bool psmem, bool grow, int colv) { return !psmem && !grow && colv != 2; }
+__host__ __device__ constexpr int rows_at_a_time(bool psmem, bool grow, int colv) { return !psmem && !grow && colv == 2 ? 2 : 1; }
+__host__ __device__ constexpr uint32_t ring_size(bool psmem, bool grow, int colv) { return rows_at_a_time(psmem, grow, colv) > 1 ? 128u : 64u; }
+__host__ __device__ constexpr uint32_t work4(bool psmem, bool grow, int colv, int rows)   // uint4 slots of it
 {
-    return ring_size(psmem, grow) * 3 / 2 + 2 * kAccepted + 2 * (uint32_t)rows * 8 + 2 * (uint32_t)rows * 2 + 2;
+    return ring_size(psmem, grow, colv) * 3 / 2 + 2 * kAccepted + 2 * (uint32_t)rows * 8 + 2 * (uint32_t)rows * 2 + 2;
 }
+// words of a column that come with one vector load (see window_at), else 0
+__host__ __device__ constexpr int column_vector(bool psmem, bool lin, uint32_t S32) { return !psmem && lin && (S32 == 2 || S32 == 4) ? (int)S32 : 0; }
 constexpr uint32_t kSame = 1u, kInf = 2u;                 // proposal states: changes nothing (accepted); infeasible
 
 // Byte offsets of the parts of a chain's shared memory. They are kernel parameters, so that a chain's state costs its
@@ -103,7 +110,7 @@ inline ChainLayout chain_layout(uint32_t S, uint32_t S32, bool grow, bool psmem,
 // bytes of a chain of W warps, without a schedule in shared memory
 inline size_t chain_bytes(uint32_t S, uint32_t S32, bool grow, bool psmem, bool lin, uint32_t cow4, uint32_t W, int rows)
 {
-    return chain_layout(S, S32, grow, psmem, lin, cow4).work + (size_t)W * work4(psmem, grow, rows) * 16;
+    return chain_layout(S, S32, grow, psmem, lin, cow4).work + (size_t)W * work4(psmem, grow, column_vector(psmem, lin, S32), rows) * 16;
 }
 
 extern __shared__ char chain_smem[];
@@ -111,7 +118,7 @@ extern __shared__ char chain_smem[];
 template <bool PSMEM, bool GROW, bool LIN, int COLV, int R>
 struct Chain {
     using Occ = typename std::conditional<PSMEM, uint16_t, uint32_t>::type;   // PSMEM: fewer than 2^16 units
-    static constexpr uint32_t kRing = ring_size(PSMEM, GROW), kBatch = 32 * R;
+    static constexpr uint32_t kRing = ring_size(PSMEM, GROW, COLV), kBatch = 32 * R;
     const ChainParams& prm;
     uint32_t cb, wb, pb;         // byte offsets in shared memory: the chain's state, the warp's work area, PSMEM: the schedule
     uint32_t* slice;             // not PSMEM: the chain's slice of global scratch
@@ -154,7 +161,6 @@ struct Chain {
     // Before unit u is rewritten: its bucket is copied into the slice if it is not there yet (all lanes, u uniform).
     __device__ __forceinline__ void own(uint32_t u, uint32_t lane) const
     {
-        if (PSMEM) return;
         const uint32_t b = u >> prm.cow_shift, S32 = prm.S32;
         if ((have()[b >> 5] >> (b & 31u)) & 1u) return;
         const size_t lo = (size_t)(b << prm.cow_shift) * S32, hi = (size_t)min(prm.U, (b + 1u) << prm.cow_shift) * S32;
@@ -163,6 +169,18 @@ struct Chain {
         __syncwarp();
         if (lane == 0) have()[b >> 5] |= 1u << (b & 31u);
         __syncwarp();
+    }
+    // Before units u and v (u again for a flip) are rewritten. Growing caches change few units: one after the other, in less
+    // code (3.17 against 3.28 ms on 131,072 units x 1056 steps, 1024 chains x 100,000).
+    __device__ __forceinline__ void own(uint32_t u, uint32_t v, uint32_t lane) const
+    {
+        if (PSMEM) return;
+        if (GROW) {
+            own(u, lane);
+            if (v != u) own(v, lane);
+        } else {
+            own_buckets(slice, prm.Pcol0, have(), prm.cow_shift, prm.U, prm.S32, u, v, lane);
+        }
     }
 };
 
@@ -387,6 +405,32 @@ __device__ __forceinline__ void judge(const Chain<PSMEM, GROW, LIN, COLV, R>& c,
     __syncwarp();
 }
 
+// the words of a column that a window is cut from (see window_at)
+template <int COLV>
+struct Words { using type = uint2; };
+template <>
+struct Words<4> { using type = uint4; };
+template <int COLV, typename Ptr>
+__device__ __forceinline__ typename Words<COLV>::type words_at(Ptr col, const WinPos p)
+{
+    typename Words<COLV>::type x;
+    if constexpr (COLV == 0) { x.x = col[p.w]; x.y = col[p.w + 1]; }
+    else x = *reinterpret_cast<const typename Words<COLV>::type*>(col);
+    return x;
+}
+template <int COLV>
+__device__ __forceinline__ uint32_t cut(const typename Words<COLV>::type q, const WinPos p)
+{
+    uint32_t lo, hi;
+    if constexpr (COLV == 0) { lo = q.x; hi = q.y; }
+    else if constexpr (COLV == 2) { lo = p.w ? q.y : q.x; hi = q.y; }
+    else {
+        lo = p.w == 0 ? q.x : p.w == 1 ? q.y : p.w == 2 ? q.z : q.w;
+        hi = p.w == 0 ? q.y : p.w == 1 ? q.z : q.w;
+    }
+    return p.first ? ((lo << 1) | (lo & 1u)) : __funnelshift_r(lo, hi, p.sh);
+}
+
 // Evaluation of `count` proposals of the batch that starts at move m, against the current state: all of them from the
 // first on (fresh), or those listed in c.again(). Draws them, settles what the placement bits settle (into the row masks
 // same and inf of a fresh batch, into c.state() otherwise) and judges the rest. The accepted ones that change the schedule
@@ -398,36 +442,65 @@ __device__ __forceinline__ uint32_t evaluate(const Chain<PSMEM, GROW, LIN, COLV,
 {
     const ChainParams& prm = c.prm;
     const uint32_t S = prm.S;
-    constexpr int UNR = rows_at_a_time(PSMEM, GROW);
+    constexpr int UNR = rows_at_a_time(PSMEM, GROW, COLV);
+    constexpr bool kAhead = load_ahead(PSMEM, GROW, COLV);
     uint32_t head = 0, listed = 0, late = kNone;
     kept = 0;
+    auto id_of = [&](uint32_t i) { return fresh ? i : (uint32_t)c.again()[i < count ? i : 0u]; };
+    auto draw = [&](uint32_t id, uint32_t& pk, uint32_t& u, uint32_t& v, uint32_t& w) {
+        uint32_t r[4];
+        const uint64_t mine = m + id;
+        philox4x32_10((uint32_t)mine, (uint32_t)(mine >> 32), chain, TAG_MOVE, prm.keys, r);
+        LaneMove mv;
+        decode_move(r, prm.p_swap_256, prm.len_choices, S, prm.U, mv);
+        pk = mv.pk; u = mv.u; v = mv.v; w = mv.w;
+    };
+    // kAhead: the row drawn last, its columns under way while the row before it is listed and judged
+    uint32_t npk, nu, nv, nw;
+    typename Words<COLV>::type qu, qv;
+    auto fetch = [&](uint32_t q) {
+        draw(id_of(q + lane), npk, nu, nv, nw);
+        const WinPos wp = window_pos(npk >> 8);
+        qu = words_at<COLV>(c.col(nu), wp);
+        if (npk & 1u) qv = words_at<COLV>(c.col(nv), wp);
+    };
+    if constexpr (kAhead) fetch(0);
 #pragma unroll 1
     for (uint32_t q = 0; q < count; q += 32 * UNR) {
         uint32_t id[UNR], pk[UNR], u[UNR], v[UNR], w[UNR], Wu[UNR], W2[UNR], live[UNR];
-#pragma unroll
-        for (int j = 0; j < UNR; ++j) {
-            const uint32_t i = q + 32u * j + lane;
-            id[j] = fresh ? i : c.again()[i < count ? i : 0u];
-            uint32_t r[4];
-            const uint64_t mine = m + id[j];
-            philox4x32_10((uint32_t)mine, (uint32_t)(mine >> 32), chain, TAG_MOVE, prm.keys, r);
-            LaneMove mv;
-            decode_move(r, prm.p_swap_256, prm.len_choices, S, prm.U, mv);
-            pk[j] = mv.pk; u[j] = mv.u; v[j] = mv.v; w[j] = mv.w;
-        }
-#pragma unroll
-        for (int j = 0; j < UNR; ++j) {
-            const WinPos wp = window_pos(pk[j] >> 8);
-            const bool swap = pk[j] & 1u;
-            Wu[j] = window_at<COLV>(c.col(u[j]), wp);
+        if constexpr (kAhead) {
+            static_assert(UNR == 1, "one row at a time");
+            id[0] = id_of(q + lane); pk[0] = npk; u[0] = nu; v[0] = nv; w[0] = nw; live[0] = 0xFFFFFFFFu;
+            const WinPos wp = window_pos(npk >> 8);
             // the second window: the other unit's placement for a swap, the full-step bitmap for a flip
-            W2[j] = window_at<COLV>(swap ? c.col(v[j]) : (const uint32_t*)c.full(), wp);
-            live[j] = 0xFFFFFFFFu;
-            if (GROW) {
-                uint32_t La, Lb, Bu, Bv;
-                alive_born(__ldg(prm.birth + u[j]), pk[j] >> 8, La, Bu);
-                alive_born(__ldg(prm.birth + (swap ? v[j] : u[j])), pk[j] >> 8, Lb, Bv);
-                live[j] = La & Lb;
+            Wu[0] = cut<COLV>(qu, wp);
+            W2[0] = npk & 1u ? cut<COLV>(qv, wp) : window_at<0>((const uint32_t*)c.full(), wp);
+            if (q + 32 < count) fetch(q + 32);
+        } else {
+#pragma unroll
+            for (int j = 0; j < UNR; ++j) {
+                const uint32_t i = q + 32u * j + lane;
+                id[j] = fresh ? i : c.again()[i < count ? i : 0u];
+                uint32_t r[4];
+                const uint64_t mine = m + id[j];
+                philox4x32_10((uint32_t)mine, (uint32_t)(mine >> 32), chain, TAG_MOVE, prm.keys, r);
+                LaneMove mv;
+                decode_move(r, prm.p_swap_256, prm.len_choices, S, prm.U, mv);
+                pk[j] = mv.pk; u[j] = mv.u; v[j] = mv.v; w[j] = mv.w;
+            }
+#pragma unroll
+            for (int j = 0; j < UNR; ++j) {
+                const WinPos wp = window_pos(pk[j] >> 8);
+                const bool swap = pk[j] & 1u;
+                Wu[j] = window_at<COLV>(c.col(u[j]), wp);
+                W2[j] = window_at<COLV>(swap ? c.col(v[j]) : (const uint32_t*)c.full(), wp);
+                live[j] = 0xFFFFFFFFu;
+                if (GROW) {
+                    uint32_t La, Lb, Bu, Bv;
+                    alive_born(__ldg(prm.birth + u[j]), pk[j] >> 8, La, Bu);
+                    alive_born(__ldg(prm.birth + (swap ? v[j] : u[j])), pk[j] >> 8, Lb, Bv);
+                    live[j] = La & Lb;
+                }
             }
         }
         if (lane == 0) x.n_listed -= listed;                      // (what was left over is counted again below)
@@ -527,11 +600,10 @@ __device__ __forceinline__ uint32_t apply(const Chain<PSMEM, GROW, LIN, COLV, R>
         I = __ballot_sync(0xFFFFFFFFu, valid && (by & 4u));
     }
     const uint32_t turned = __ballot_sync(0xFFFFFFFFu, valid && (lead != led || by != was || (occ == prm.cap) != was_full));
-    c.own(u, lane);
-    if (swap) c.own(v, lane);
+    c.own(u, swap ? v : u, lane);
     if (lane < 2) {
-        uint32_t M = ((1u << run) - 1u) << 1, V = ((1u << nl) - 1u) << 1, NU = e.Nu, NV = e.Nv, sbit = s0 - 1;
-        if (s0 == 0) { F >>= 1; T >>= 1; O >>= 1; I >>= 1; V >>= 1; M >>= 1; NU >>= 1; NV >>= 1; sbit = 0; }
+        uint32_t M = ((1u << run) - 1u) << 1, V = ((1u << nl) - 1u) << 1, NU = e.Nu, NV = e.Nv, D = win.x ^ NU, sbit = s0 - 1;
+        if (s0 == 0) { F >>= 1; T >>= 1; O >>= 1; I >>= 1; V >>= 1; M >>= 1; NU >>= 1; NV >>= 1; D >>= 1; sbit = 0; }
         const uint32_t wj = (sbit >> 5) + lane, sh = sbit & 31u;
         if (wj < S32 && (lane == 0 || sh != 0)) {
             // lane 0 holds the part of the window that falls into the first word, lane 1 the spill-over
@@ -545,12 +617,15 @@ __device__ __forceinline__ uint32_t apply(const Chain<PSMEM, GROW, LIN, COLV, R>
                     c.in()[wj] = (c.in()[wj] & ~Vx) | (part(I) & Vx);
                 }
             }
-            if (Mx) {
+            if (Mx) {                                             // (many moves in global memory: atomics, which are not waited for)
                 uint32_t* const pu = c.P() + (size_t)u * S32 + wj;
-                *pu = (*pu & ~Mx) | (part(NU) & Mx);
-                if (swap) {
-                    uint32_t* const pv = c.P() + (size_t)v * S32 + wj;
-                    *pv = (*pv & ~Mx) | (part(NV) & Mx);
+                uint32_t* const pv = c.P() + (size_t)v * S32 + wj;
+                if (PSMEM || GROW) {
+                    *pu = (*pu & ~Mx) | (part(NU) & Mx);
+                    if (swap) *pv = (*pv & ~Mx) | (part(NV) & Mx);
+                } else if (const uint32_t x = part(D) & Mx) {     // a swap toggles the same bits of both
+                    atomicXor(pu, x);
+                    if (swap) atomicXor(pv, x);
                 }
             }
         }
@@ -681,8 +756,8 @@ wide_chain_kernel(const __grid_constant__ ChainParams prm)
     const uint32_t S = prm.S, S32 = prm.S32, U = prm.U;
     const size_t pwords = (size_t)U * S32;
     const uint32_t cow_words = PSMEM ? 0u : prm.cow_slots4 * 4;
-    const uint32_t stride = prm.lay.work + W * work4(PSMEM, GROW, R) * 16;       // bytes of a chain
-    Chain<PSMEM, GROW, LIN, COLV, R> c{prm, cic * stride, cic * stride + prm.lay.work + sub * work4(PSMEM, GROW, R) * 16,
+    const uint32_t stride = prm.lay.work + W * work4(PSMEM, GROW, COLV, R) * 16;       // bytes of a chain
+    Chain<PSMEM, GROW, LIN, COLV, R> c{prm, cic * stride, cic * stride + prm.lay.work + sub * work4(PSMEM, GROW, COLV, R) * 16,
                                        cpb * stride + cic * U * S32 * 4, PSMEM ? nullptr : prm.ws + (size_t)slot * pwords};
     ChainShared* const sc = c.sc();
     EvalCtx x;

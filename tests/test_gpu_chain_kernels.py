@@ -39,6 +39,18 @@ def test_shapes(kvp, oracle, hooks, warps, U, S, cap):
         _same(g, o, chains=5, moves=1500, seed=U, levels=6, p0=p0, early_stop_permille=1, early_stop_from_level=4)
 
 
+@pytest.mark.parametrize("warps", (3, 18))
+@pytest.mark.parametrize("U,S", [(7000, 64), (7001, 63), (5003, 97), (3001, 129), (3003, 257)])
+def test_buckets_of_eight_columns(kvp, oracle, hooks, warps, U, S):
+    """Buckets of a slice taken over as vectors (7000 x 2 words, 5003 x 4) and word by word (slices or buckets that do not begin
+    at a vector), the last one shorter than the others; columns of 2, 4, 5 and 9 words, loaded a row ahead from 4 on."""
+    hooks(warps_per_chain=warps, overlay=2)
+    A = wl.random_access(U, S, 0.2, seed=U + S)
+    g, o = both_problems(kvp, oracle, U, 8192, S, A, U // 3, (8000 * GB, 900 * GB, 900 * GB))
+    for p0 in (0.8, 1e-4):
+        _same(g, o, chains=5, moves=1500, seed=U, levels=6, p0=p0)
+
+
 @pytest.mark.parametrize("bw,flags", [((4900, 500, 900), 3), ((4900, 500, 900), 1), ((3, 1, 1), 0)])
 def test_weights(kvp, oracle, hooks, bw, flags):
     """A link slower than the DRAM channels (the cost is not linear in migrations), migrations free on a side or both."""
