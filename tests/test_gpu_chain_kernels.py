@@ -143,6 +143,21 @@ def test_choice_in_global_memory(kvp, oracle, busy, p0, init):
         assert out["per_chain"][c].astuple() == want[0].astuple(), c
 
 
+@pytest.mark.parametrize("U,S,cap,chains", [(63, 63, 20, 200), (64, 63, 20, 200), (63, 64, 20, 200),    # one warp, two, two
+                                            (90, 70, 12, 889), (90, 70, 12, 888), (90, 70, 80, 1184)])
+def test_choice_of_warps_in_shared_memory(kvp, oracle, U, S, cap, chains):
+    """Both sides of the lines below which a near-greedy chain has one warp: units and steps, chains per SM, the share of the
+    reads that the static placement serves (a little above cap / U here)."""
+    A = wl.random_access(U, S, 0.2, seed=U + S)
+    g, o = both_problems(kvp, oracle, U, 8192, S, A, cap, (8000 * GB, 900 * GB, 900 * GB))
+    kw = dict(chains=chains, moves=1200, seed=3, levels=4, p0=1e-6)
+    out = g.anneal(g.make_params(**kw), want_per_chain=True)
+    op = o.make_params(**kw)
+    for c in (0, 1, chains // 2, chains - 1):
+        want, _, _ = o.anneal_chains(op, c, 1)
+        assert out["per_chain"][c].astuple() == want[0].astuple(), c
+
+
 @pytest.mark.parametrize("scale", [1, 2 ** 10, 2 ** 20])
 def test_accept_table_rows(kvp, oracle, scale):
     """Rows built as geometric sequences against exp() for every entry, at temperatures around powers of two."""
