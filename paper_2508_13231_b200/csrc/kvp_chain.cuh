@@ -26,7 +26,7 @@
 //
 // What bounds it (ncu): issue slots and the integer pipe, 12.9 warp instructions per move on 2.6M units x 64 steps, 57% of
 // the issue slots busy with 16 warps per SM in a short launch (2368 chains x 6,000 moves). Measured there (8192 chains x 1M
-// moves) 201 -> 140 ms, on a growing cache of 131,072 units (1024 x 100k) 6.3 -> 2.7 ms against the kernels before, which put
+// moves) 201 -> 133 ms, on a growing cache of 131,072 units (1024 x 100k) 6.3 -> 2.7 ms against the kernels before, which put
 // the changed steps of every listed proposal through a shared-memory queue of (proposal, step) items, each an evaluation of
 // Eq. 2-4 from four counters, and had no second warp per chain (work area 6.9 KB a warp, now 3.1).
 #pragma once
@@ -75,9 +75,11 @@ static_assert(sizeof(ChainShared) % 16 == 0, "uint4 slots");
 // instruction cache counts (four rows: 2000 instructions in a batch's path, and a warp waited for the next one a quarter of
 // the time); with births, whose loads come first, one (2.7 against 4.6 ms).
 // Columns of other lengths, whose loads take longer, are loaded a row ahead (load_ahead): while a row is listed and judged the
-// next one's columns are on their way. 32,768 units x 256 steps, 2368 chains x 50,000: 3.17 -> 2.31 ms (two rows ahead: 2.62);
-// 131,072 x 100, 1500 x 50,000: 1.87 -> 1.80; 65,536 x 128, 2368 x 50,000: 2.63 -> 2.54. Not where a column is two words: its
-// loads stay in flight for less than the longer path costs (131,072 x 64, 2368 x 20,000: 0.75 -> 0.79 ms).
+// next one's columns are on their way. 32,768 units x 256 steps, 2368 chains x 50,000: 3.17 -> 2.27 ms (two rows ahead: 2.62);
+// 131,072 x 100, 1500 x 50,000: 1.87 -> 1.73; 65,536 x 128, 2368 x 50,000: 2.63 -> 2.49. Not where a column is two words, whose
+// loads stay in flight for less than a single row at a time costs (131,072 x 64, 2368 x 20,000: 0.74 -> 0.82 ms; the largest
+// configuration 132 -> 138), nor with births (131,072 x 1056: 2.71 -> 2.76). The second load takes its address from a select: with a
+// branch around it, since a flip has no second column, the three first lines took 2.30, 1.81 and 2.55 ms.
 constexpr uint32_t kAccepted = 6;
 __host__ __device__ constexpr bool load_ahead(bool psmem, bool grow, int colv) { return !psmem && !grow && colv != 2; }
 __host__ __device__ constexpr int rows_at_a_time(bool psmem, bool grow, int colv) { return !psmem && !grow && colv == 2 ? 2 : 1; }
@@ -140,9 +142,9 @@ struct Chain {
     __device__ __forceinline__ uint2* ring_win() const { return at<uint2>(wb + 16 * kRing); }      // [kRing] {Wu, Wv}
     // [kAccepted][2] {pk | id << 24, u, v, cost change}, {Wu, Wv, Au, Av}
     __device__ __forceinline__ uint4* acc() const { return at<uint4>(wb + 24 * kRing); }
-    __device__ __forceinline__ uint32_t* range() const { return at<uint32_t>(wb + 24 * kRing + 32 * kAccepted); }   // [kBatch] s0 | (s0 + len) << 16
-    __device__ __forceinline__ uint32_t* units() const { return range() + kBatch; }                // [kBatch] low halves of u | v << 16 (u twice for a flip)
-    __device__ __forceinline__ uint32_t* close() const { return units() + kBatch; }                // [R] bit: this proposal's steps were looked at one by one
+    // [kBatch] {s0 | (s0 + len) << 16, low halves of u | v << 16 (u twice for a flip)}
+    __device__ __forceinline__ uint2* reach() const { return at<uint2>(wb + 24 * kRing + 32 * kAccepted); }
+    __device__ __forceinline__ uint32_t* close() const { return at<uint32_t>(wb + 24 * kRing + 32 * kAccepted + 8 * kBatch); }   // [R] bit: this proposal's steps were looked at one by one
     // [kBatch] of proposals evaluated again: kSame, kInf or 0
     __device__ __forceinline__ uint8_t* state() const { return at<uint8_t>(wb + 24 * kRing + 32 * kAccepted + 8 * kBatch + 32); }
     __device__ __forceinline__ uint8_t* again() const { return state() + kBatch; }                 // [kBatch] ids to evaluate again, ascending
@@ -462,7 +464,8 @@ __device__ __forceinline__ uint32_t evaluate(const Chain<PSMEM, GROW, LIN, COLV,
         draw(id_of(q + lane), npk, nu, nv, nw);
         const WinPos wp = window_pos(npk >> 8);
         qu = words_at<COLV>(c.col(nu), wp);
-        if (npk & 1u) qv = words_at<COLV>(c.col(nv), wp);
+        // the second window: the other unit's placement for a swap, the full-step bitmap for a flip (one address, no branch)
+        qv = words_at<COLV>(npk & 1u ? c.col(nv) : (const uint32_t*)c.full(), wp);
     };
     if constexpr (kAhead) fetch(0);
 #pragma unroll 1
@@ -472,9 +475,8 @@ __device__ __forceinline__ uint32_t evaluate(const Chain<PSMEM, GROW, LIN, COLV,
             static_assert(UNR == 1, "one row at a time");
             id[0] = id_of(q + lane); pk[0] = npk; u[0] = nu; v[0] = nv; w[0] = nw; live[0] = 0xFFFFFFFFu;
             const WinPos wp = window_pos(npk >> 8);
-            // the second window: the other unit's placement for a swap, the full-step bitmap for a flip
             Wu[0] = cut<COLV>(qu, wp);
-            W2[0] = npk & 1u ? cut<COLV>(qv, wp) : window_at<0>((const uint32_t*)c.full(), wp);
+            W2[0] = cut<COLV>(qv, wp);
             if (q + 32 < count) fetch(q + 32);
         } else {
 #pragma unroll
@@ -516,8 +518,7 @@ __device__ __forceinline__ uint32_t evaluate(const Chain<PSMEM, GROW, LIN, COLV,
             const bool bad = !swap && (~Wu[j] & D & W2[j]) != 0;  // a flip may not raise a full step (Eq. 5)
             const bool more = named && !none && !bad;
             if (named) {
-                c.range()[id[j]] = s0 | (s0 + len) << 16;
-                c.units()[id[j]] = (u[j] & 0xFFFFu) | (swap ? v[j] : u[j]) << 16;
+                c.reach()[id[j]] = make_uint2(s0 | (s0 + len) << 16, (u[j] & 0xFFFFu) | (swap ? v[j] : u[j]) << 16);
                 if (fresh) {                                      // row (q >> 5) + j of this lane
                     const uint32_t bit = 1u << ((q >> 5) + j);
                     if (none) same |= bit;
@@ -655,7 +656,8 @@ __device__ __forceinline__ uint32_t spoiled(const Chain<PSMEM, GROW, LIN, COLV, 
     uint32_t rows = 0;
 #pragma unroll
     for (int h = 0; h < R; ++h) {
-        const uint32_t r = c.range()[h * 32 + lane], w = c.units()[h * 32 + lane], lo = w & 0xFFFFu, hi = w >> 16;
+        const uint2 x = c.reach()[h * 32 + lane];
+        const uint32_t r = x.x, lo = x.y & 0xFFFFu, hi = x.y >> 16;
         const bool meets = (r & 0xFFFFu) <= endb + 1u && s0b <= (r >> 16);
         const bool shares = lo == bu || lo == bv || hi == bu || hi == bv;
         const bool turned = first <= (r >> 16) && (r & 0xFFFFu) <= last && !((same >> h) & 1u);
