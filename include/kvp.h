@@ -245,7 +245,11 @@ typedef struct {
     uint32_t chain_launches;    /* launches of the chain kernel (waves of resident chains)         */
     uint32_t resident_chains;   /* chains per wave                                                 */
     uint32_t wide_kernel;       /* 1: the wide chain kernel ran (many chains), 0: the narrow one   */
-    uint32_t reserved;
+    /* The form the chain kernel ran in: */
+    uint8_t  warps_per_chain;
+    uint8_t  shared_schedules;  /* 1: the chains' schedules in shared memory, 0: as overlays in global memory */
+    uint8_t  bucket_log2;       /* of an overlay: a bucket is 2^bucket_log2 units                  */
+    uint8_t  columns_ahead;     /* wide kernel, global memory: 1: placement columns loaded a row ahead */
     /* What the evaluations of the wide kernel amounted to, summed over the chains (0 for the narrow kernel): */
     uint64_t work_again;        /* proposals evaluated a second time after a move was applied in their batch   */
     uint64_t work_listed;       /* evaluations that needed more than the placement bits (a cost evaluation)    */

@@ -687,6 +687,15 @@ ChainKernel kernel_of(const Ctx& c, bool psmem, bool asmem)
                   : narrow_kernel_for(psmem, asmem, c.grow, c.lin, c.S32, c.solo);
 }
 
+void report_form(const Ctx& c, kvp_anneal_stats* stats)
+{
+    stats->wide_kernel = c.wide ? 1u : 0u;
+    stats->warps_per_chain = (uint8_t)c.wpc;
+    stats->shared_schedules = c.psmem ? 1u : 0u;
+    stats->bucket_log2 = (uint8_t)(c.psmem ? 0u : c.cow_shift);
+    stats->columns_ahead = c.wide && load_ahead(c.psmem, c.grow, column_vector(c.psmem, c.lin, c.S32)) ? 1u : 0u;
+}
+
 int launch_chains(const Ctx& c, ChainParams& prm, uint32_t count)
 {
     {
@@ -1226,7 +1235,7 @@ try {
         cudaEventElapsedTime(&stats->ms_finish, ev[2], ev[3]);
         stats->kernel_launches = c.launches;
         stats->chain_launches = waves; stats->resident_chains = c.resident;
-        stats->wide_kernel = c.wide ? 1u : 0u;
+        report_form(c, stats);
         stats->work_again = work[0]; stats->work_listed = work[1]; stats->work_items = work[2];
     }
     return ok ? KVP_OK : KVP_ERR_INTERNAL;
@@ -1440,7 +1449,8 @@ try {
         cudaEventElapsedTime(&stats->ms_chains, ev[1], ev[2]);
         cudaEventElapsedTime(&stats->ms_finish, ev[2], ev[3]);
         stats->kernel_launches = c.launches;
-        stats->chain_launches = rounds; stats->resident_chains = chains; stats->wide_kernel = c.wide ? 1u : 0u;
+        stats->chain_launches = rounds; stats->resident_chains = chains;
+        report_form(c, stats);
         stats->work_again = work[0]; stats->work_listed = work[1]; stats->work_items = work[2];
         stats->exchange_rounds = rounds; stats->exchanges_tried = xcounts[0]; stats->exchanges_accepted = xcounts[1];
     }

@@ -75,7 +75,8 @@ class AnnealStats(C.Structure):
         ("winner_hits", C.c_uint64), ("winner_accessed", C.c_uint64),
         ("ms_init", C.c_float), ("ms_chains", C.c_float), ("ms_finish", C.c_float), ("kernel_launches", C.c_uint32),
         ("per_chain", C.POINTER(ChainResult)), ("chain_launches", C.c_uint32), ("resident_chains", C.c_uint32),
-        ("wide_kernel", C.c_uint32), ("reserved", C.c_uint32),
+        ("wide_kernel", C.c_uint32), ("warps_per_chain", C.c_uint8), ("shared_schedules", C.c_uint8), ("bucket_log2", C.c_uint8),
+        ("columns_ahead", C.c_uint8),
         ("work_again", C.c_uint64), ("work_listed", C.c_uint64), ("work_items", C.c_uint64),
         ("exchanges_tried", C.c_uint64), ("exchanges_accepted", C.c_uint64), ("exchange_rounds", C.c_uint32),
         ("reserved2", C.c_uint32),

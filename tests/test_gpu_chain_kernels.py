@@ -4,6 +4,7 @@ warp, schedules in shared and in global memory, weights for which the cost is no
 inside CTAs and in launches."""
 import numpy as np
 import pytest
+import torch
 
 from paper_2508_13231_b200 import workloads as wl
 from gpu_util import both_problems, to_np
@@ -19,36 +20,51 @@ def kvp():
     return kvp
 
 
+def _warps(hook):
+    """Warps per chain that a value of the hook stands for."""
+    return 1 if hook == 3 else hook & 15 if hook >= 16 else hook
+
+
 def _same(g, o, **kw):
     out = g.anneal(g.make_params(**kw), want_per_chain=True)
     ref = o.anneal(o.make_params(**kw))
     assert [r.astuple() for r in out["per_chain"]] == [r.astuple() for r in ref["per_chain"]]
     assert np.array_equal(to_np(out["best_schedule"]), ref["best_schedule"])
+    return out["stats"]
+
+
+SHARED = [(2, 2, 1), (31, 32, 9), (40, 31, 0), (40, 33, 40), (65, 64, 20), (33, 97, 10), (7000, 64, 2000), (5000, 128, 900),
+          (3000, 257, 700), (300, 2050, 90)]
+# above what two chains of an SM can hold in shared memory: columns of 1, 2, 3, 4, 5, 9 and 65 words
+GLOBAL = [(30011, 32, 9000), (15004, 64, 4000), (10001, 90, 900), (8003, 128, 1500), (6001, 129, 2000), (3601, 257, 700), (500, 2050, 90)]
 
 
 @pytest.mark.parametrize("warps", NARROW + WIDE)
-@pytest.mark.parametrize("U,S,cap", [
-    (2, 2, 1), (31, 32, 9), (40, 31, 0), (40, 33, 40), (65, 64, 20), (33, 97, 10),   # schedules in shared memory
-    (7000, 64, 2000), (5000, 128, 900), (3000, 257, 700), (300, 2050, 90),           # in global memory: 2, 4, 9, 65 words
-])
+@pytest.mark.parametrize("U,S,cap", SHARED + GLOBAL)
 def test_shapes(kvp, oracle, hooks, warps, U, S, cap):
     hooks(warps_per_chain=warps)
     A = wl.random_access(U, S, 0.2, seed=U + S)
     g, o = both_problems(kvp, oracle, U, 8192, S, A, cap, (4900 * GB, 900 * GB, 500 * GB))
     for p0 in (0.8, 1e-4):
-        _same(g, o, chains=5, moves=1500, seed=U, levels=6, p0=p0, early_stop_permille=1, early_stop_from_level=4)
+        st = _same(g, o, chains=5, moves=1500, seed=U, levels=6, p0=p0, early_stop_permille=1, early_stop_from_level=4)
+        assert (st.wide_kernel, st.warps_per_chain) == (warps in WIDE, _warps(warps))
+        assert st.shared_schedules == ((U, S, cap) in SHARED) and st.bucket_log2 == 0
 
 
+@pytest.mark.parametrize("link", [900, 500])
 @pytest.mark.parametrize("warps", (3, 18))
-@pytest.mark.parametrize("U,S", [(7000, 64), (7001, 63), (5003, 97), (3001, 129), (3003, 257)])
-def test_buckets_of_eight_columns(kvp, oracle, hooks, warps, U, S):
-    """Buckets of a slice taken over as vectors (7000 x 2 words, 5003 x 4) and word by word (slices or buckets that do not begin
-    at a vector), the last one shorter than the others; columns of 2, 4, 5 and 9 words, loaded a row ahead from 4 on."""
+@pytest.mark.parametrize("U,S", [(30011, 32), (30004, 30), (15004, 64), (15001, 63), (10001, 90), (10004, 90), (7503, 97), (6001, 129),
+                                 (3301, 257)])
+def test_buckets_of_eight_columns(kvp, oracle, hooks, warps, U, S, link):
+    """Buckets of a slice in global memory taken over as vectors (30004, 15004, 10004 and 7503 units) and word by word (slices
+    that do not begin at a vector), the last one shorter than the others; columns of 1, 2, 3, 4, 5 and 9 words; one and two
+    warps per chain; a link faster and slower than the DRAM channels."""
     hooks(warps_per_chain=warps, overlay=2)
     A = wl.random_access(U, S, 0.2, seed=U + S)
-    g, o = both_problems(kvp, oracle, U, 8192, S, A, U // 3, (8000 * GB, 900 * GB, 900 * GB))
+    g, o = both_problems(kvp, oracle, U, 8192, S, A, U // 3, (8000 * GB, link * GB, 900 * GB))
     for p0 in (0.8, 1e-4):
-        _same(g, o, chains=5, moves=1500, seed=U, levels=6, p0=p0)
+        st = _same(g, o, chains=5, moves=1500, seed=U, levels=6, p0=p0)
+        assert (st.wide_kernel, st.warps_per_chain, st.shared_schedules, st.bucket_log2) == (1, _warps(warps), 0, 3) and U % 8
 
 
 @pytest.mark.parametrize("bw,flags", [((4900, 500, 900), 3), ((4900, 500, 900), 1), ((3, 1, 1), 0)])
@@ -63,7 +79,7 @@ def test_weights(kvp, oracle, hooks, bw, flags):
 
 @pytest.mark.parametrize("warps", (0,) + NARROW + (18,))
 @pytest.mark.parametrize("U,S,cap", [(31, 32, 9), (40, 33, 40), (65, 64, 20), (33, 97, 10), (7000, 64, 2000), (5000, 128, 900),
-                                     (3000, 257, 700)])
+                                     (3000, 257, 700), (15004, 64, 4000), (8003, 128, 1500), (3601, 257, 700)])
 def test_link_slower_than_dram(kvp, oracle, hooks, warps, U, S, cap):
     """Eq. 4's maximum is over three terms then, each of which leads at some steps: the link in either direction, the DRAM
     channels. Written units on either side shift which one does."""
@@ -73,7 +89,8 @@ def test_link_slower_than_dram(kvp, oracle, hooks, warps, U, S, cap):
     hw, ew = rng.integers(0, 3, S), rng.integers(0, 4, S) * (rng.random(S) < 0.5)
     g, o = both_problems(kvp, oracle, U, 8192, S, A, cap, (4900 * GB, 500 * GB, 700 * GB), hw=hw, ew=ew)
     for p0 in (0.8, 1e-4):
-        _same(g, o, chains=5, moves=1500, seed=U, levels=6, p0=p0, early_stop_permille=1, early_stop_from_level=4)
+        st = _same(g, o, chains=5, moves=1500, seed=U, levels=6, p0=p0, early_stop_permille=1, early_stop_from_level=4)
+        assert st.shared_schedules == (U * ((S + 31) // 32) < 25000)      # words of a schedule
 
 
 @pytest.mark.parametrize("warps", [0, 2, 3])
@@ -143,15 +160,20 @@ def test_choice_in_global_memory(kvp, oracle, busy, p0, init):
         assert out["per_chain"][c].astuple() == want[0].astuple(), c
 
 
-@pytest.mark.parametrize("U,S,cap,chains", [(63, 63, 20, 200), (64, 63, 20, 200), (63, 64, 20, 200),    # one warp, two, two
-                                            (90, 70, 12, 889), (90, 70, 12, 888), (90, 70, 80, 1184)])
-def test_choice_of_warps_in_shared_memory(kvp, oracle, U, S, cap, chains):
+@pytest.mark.parametrize("U,S,cap,chains,warps", [
+    (63, 63, 20, 200, 1), (64, 63, 20, 200, 3), (63, 64, 20, 200, 2),          # units and steps
+    (90, 70, 12, 889, 1), (90, 70, 12, 888, 2),                                # chains per SM: 7 and 6
+    (90, 70, 80, 1184, 2)])                                                    # a placement that serves more than half of the reads
+def test_choice_of_warps_in_shared_memory(kvp, oracle, U, S, cap, chains, warps):
     """Both sides of the lines below which a near-greedy chain has one warp: units and steps, chains per SM, the share of the
     reads that the static placement serves (a little above cap / U here)."""
+    if torch.cuda.get_device_properties(0).multi_processor_count != 148:
+        warps = None                                                           # (the chains per SM are others)
     A = wl.random_access(U, S, 0.2, seed=U + S)
     g, o = both_problems(kvp, oracle, U, 8192, S, A, cap, (8000 * GB, 900 * GB, 900 * GB))
     kw = dict(chains=chains, moves=1200, seed=3, levels=4, p0=1e-6)
     out = g.anneal(g.make_params(**kw), want_per_chain=True)
+    assert not out["stats"].wide_kernel and out["stats"].shared_schedules and warps in (None, out["stats"].warps_per_chain)
     op = o.make_params(**kw)
     for c in (0, 1, chains // 2, chains - 1):
         want, _, _ = o.anneal_chains(op, c, 1)

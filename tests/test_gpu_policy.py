@@ -126,6 +126,23 @@ def test_keys_that_jump(kvp, oracle, U):
         assert np.array_equal(u64(g.wr_grid(5, 4)), oracle.wr_grid(o, 5, 4)), cap
 
 
+@pytest.mark.parametrize("U", [20001, 32768])
+def test_largest_populations(kvp, oracle, U):
+    """Five and eight warps of four words to a thread, a row that is no whole number of threads' words; steps that read every
+    unit, so that counts reach the top of their fields."""
+    S = 7
+    rng = np.random.default_rng(U)
+    A = wl.pack_bits(rng.random((S, U)) < np.array([1.0, 0.3, 0.0, 1.0, 0.9, 0.02, 1.0])[:, None])
+    for cap in (0, U // 3, U):
+        g, o = both_problems(kvp, oracle, U, 8192, S, A, cap, (8000 * GB, 900 * GB, 900 * GB))
+        pairs = [(1, 1000), (2, 500), (9, 1000)]
+        got = to_np(g.policy_lookahead([w for w, _ in pairs], [r for _, r in pairs]))
+        for i, (w, r) in enumerate(pairs):
+            assert np.array_equal(got[i], oracle.policy_lookahead(o, w, r)), (cap, w, r)
+        assert np.array_equal(to_np(g.policy_reactive()), oracle.policy_reactive(o)), cap
+        assert np.array_equal(u64(g.wr_grid(4, 3)), oracle.wr_grid(o, 4, 3)), cap
+
+
 @pytest.mark.parametrize("w_max,n_ratio,top", [(64, 101, 10 ** 6), (5, 2, 3), (20, 11, 2 ** 42), (7, 7, 1)])
 def test_walk_on_any_table(kvp, oracle, w_max, n_ratio, top):
     """Tables beyond shared memory, of equal costs, of costs far apart and of large ones (their differences decide)."""
