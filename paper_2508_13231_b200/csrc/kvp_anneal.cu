@@ -625,6 +625,7 @@ struct Ctx {
     bool solo;               // narrow kernel, schedules in shared memory: the variant for one warp per chain
     bool ladder_ctas;        // replica exchange: every CTA holds whole ladders (one launch)
     int rows;                // wide kernel: rows of 32 proposals in a batch
+    bool ahead;              // wide kernel: placement columns loaded a row ahead
     bool lin;                // kappa_d >= kappa_k: see kvp_chain.cuh
     float* bounds;           // [levels]
     std::vector<double> temps;
@@ -662,28 +663,31 @@ ChainKernel narrow_kernel_for(bool psmem, bool asmem, bool grow, bool lin, uint3
 }
 
 template <bool PSMEM, bool ASMEM, bool LIN, int COLV>
-ChainKernel wide_pick(bool grow, int rows)
+ChainKernel wide_pick(bool grow, int rows, bool ahead)
 {
-    if (!PSMEM && LIN && rows == kRowsOne)
-        return grow ? wide_chain_kernel<PSMEM, true, ASMEM, LIN, COLV, !PSMEM && LIN ? kRowsOne : kRowsMany>
-                    : wide_chain_kernel<PSMEM, false, ASMEM, LIN, COLV, !PSMEM && LIN ? kRowsOne : kRowsMany>;
-    return grow ? wide_chain_kernel<PSMEM, true, ASMEM, LIN, COLV, kRowsMany> : wide_chain_kernel<PSMEM, false, ASMEM, LIN, COLV, kRowsMany>;
+    constexpr int kOne = !PSMEM && LIN ? kRowsOne : kRowsMany;
+    constexpr bool kAhead = !PSMEM && COLV != 2, kTwo = COLV != 4;     // the forms without births (see load_ahead)
+    const bool one = rows == kRowsOne;
+    if (grow) return one ? wide_chain_kernel<PSMEM, true, ASMEM, LIN, COLV, kOne, false> : wide_chain_kernel<PSMEM, true, ASMEM, LIN, COLV, kRowsMany, false>;
+    if (ahead || !kTwo)
+        return one ? wide_chain_kernel<PSMEM, false, ASMEM, LIN, COLV, kOne, kAhead> : wide_chain_kernel<PSMEM, false, ASMEM, LIN, COLV, kRowsMany, kAhead>;
+    return one ? wide_chain_kernel<PSMEM, false, ASMEM, LIN, COLV, kOne, !kTwo> : wide_chain_kernel<PSMEM, false, ASMEM, LIN, COLV, kRowsMany, !kTwo>;
 }
 
-ChainKernel wide_kernel_for(bool psmem, bool asmem, bool grow, bool lin, uint32_t S32, int rows)
+ChainKernel wide_kernel_for(bool psmem, bool asmem, bool grow, bool lin, uint32_t S32, int rows, bool ahead)
 {
     if (!psmem) {
-        if (lin && S32 == 2) return wide_pick<false, false, true, 2>(grow, rows);
-        if (lin && S32 == 4) return wide_pick<false, false, true, 4>(grow, rows);
-        return lin ? wide_pick<false, false, true, 0>(grow, rows) : wide_pick<false, false, false, 0>(grow, rows);
+        if (lin && S32 == 2) return wide_pick<false, false, true, 2>(grow, rows, ahead);
+        if (lin && S32 == 4) return wide_pick<false, false, true, 4>(grow, rows, ahead);
+        return lin ? wide_pick<false, false, true, 0>(grow, rows, ahead) : wide_pick<false, false, false, 0>(grow, rows, ahead);
     }
-    if (asmem && lin) return wide_pick<true, true, true, 0>(grow, rows);
-    return lin ? wide_pick<true, false, true, 0>(grow, rows) : wide_pick<true, false, false, 0>(grow, rows);
+    if (asmem && lin) return wide_pick<true, true, true, 0>(grow, rows, ahead);
+    return lin ? wide_pick<true, false, true, 0>(grow, rows, ahead) : wide_pick<true, false, false, 0>(grow, rows, ahead);
 }
 
 ChainKernel kernel_of(const Ctx& c, bool psmem, bool asmem)
 {
-    return c.wide ? wide_kernel_for(psmem, asmem, c.grow, c.lin, c.S32, c.rows)
+    return c.wide ? wide_kernel_for(psmem, asmem, c.grow, c.lin, c.S32, c.rows, c.ahead)
                   : narrow_kernel_for(psmem, asmem, c.grow, c.lin, c.S32, c.solo);
 }
 
@@ -693,7 +697,7 @@ void report_form(const Ctx& c, kvp_anneal_stats* stats)
     stats->warps_per_chain = (uint8_t)c.wpc;
     stats->shared_schedules = c.psmem ? 1u : 0u;
     stats->bucket_log2 = (uint8_t)(c.psmem ? 0u : c.cow_shift);
-    stats->columns_ahead = c.wide && load_ahead(c.psmem, c.grow, column_vector(c.psmem, c.lin, c.S32)) ? 1u : 0u;
+    stats->columns_ahead = c.ahead ? 1u : 0u;
 }
 
 int launch_chains(const Ctx& c, ChainParams& prm, uint32_t count)
@@ -796,12 +800,13 @@ int prepare(kvp_problem* p, const kvp_anneal_params* a, cudaStream_t st, Ctx& c,
     c.lin = p->K.kd >= p->K.kk;
     c.ladder_ctas = c.solo = false;
     c.rows = kRowsMany;
+    c.ahead = false;
     c.cow_slots4 = 0;
     c.cow_shift = 0;
     c.smem_shared = 0;
     c.asmem = false;
     auto fixed_bytes = [&](uint32_t warps, bool shared) {
-        if (c.wide) return chain_bytes(p->S, p->S32, c.grow, shared, c.lin, shared ? 0u : c.cow_slots4, warps, c.rows);
+        if (c.wide) return chain_bytes(p->S, p->S32, c.grow, shared, c.lin, shared ? 0u : c.cow_slots4, warps, c.rows, c.ahead);
         return narrow_bytes(p->S, p->S32, c.grow, shared, c.lin, shared ? 0u : c.cow_slots4, warps);
     };
     // Which kernel, and how many warps per chain (W; an SM holds 16). Measured on 1800 problems of 64 to 524,288 units x 32 to
@@ -910,19 +915,24 @@ int prepare(kvp_problem* p, const kvp_anneal_params* a, cudaStream_t st, Ctx& c,
         // wide: two warps per chain while an SM has at most 8 (more per chain are no faster)
         if (!c.wide) W = narrow_warps();
         else if (!exchange && chains_per_sm <= 8 && !(c.grow && !c.lin)) W = 2;   // (131,072 x 1056 births, slow link: 1.07 against 1.13 ms)
+        const bool may_load_ahead = c.wide && load_ahead(c.grow, c.lin, p->S32);
+        c.ahead = may_load_ahead;                                 // (the smaller work area)
         while (W > 1 && fixed_bytes(W, false) + kCowBitsMin / 8 > budget) --W;   // very long horizons
         // replica exchange keeps every chain resident: no more warps than leave room for all of them
         while (exchange && W > 1 && std::min<size_t>(full / W, budget / (fixed_bytes(W, false) + kCowBitsMin / 8)) * sms < a->chains) --W;
         if (forced) W = forced;
         if (W == 1 && c.wide && c.lin) c.rows = kRowsOne;
-        uint32_t per_cta = full / W;                              // chains of a full CTA
-        if (chains_per_sm < per_cta) per_cta = chains_per_sm ? chains_per_sm : 1u;
-        {
+        // Shares the shared memory out and returns how many chains a CTA can hold (0: not one).
+        auto share_out = [&](bool ahead) {
+            c.ahead = ahead;
+            c.cow_shift = c.cow_slots4 = 0;
+            uint32_t per_cta = full / W;                          // chains of a full CTA
+            if (chains_per_sm < per_cta) per_cta = chains_per_sm ? chains_per_sm : 1u;
             // The bucket bitmap takes what a full CTA of chains leaves of the shared memory: the smaller the buckets, the
             // fewer reads of a long chain go to its private slice.
             const size_t bare = fixed_bytes(W, false);
             if (budget / bare < per_cta) per_cta = (uint32_t)(budget / bare);
-            if (per_cta < 1) return KVP_ERR_RANGE;
+            if (per_cta < 1) return 0u;
             const size_t share = budget / per_cta;
             size_t bits = share > bare ? (share - bare) / 16 * 128 : 0;
             if (bits < kCowBitsMin) bits = kCowBitsMin;
@@ -931,12 +941,28 @@ int prepare(kvp_problem* p, const kvp_anneal_params* a, cudaStream_t st, Ctx& c,
             if (hooks.overlay == 2 && c.cow_shift < 3) c.cow_shift = 3;   // test hook
             const uint64_t buckets = ((uint64_t)p->U + (1ull << c.cow_shift) - 1) >> c.cow_shift;
             c.cow_slots4 = (uint32_t)((buckets + 127) / 128);
+            c.smem_per_warp = fixed_bytes(W, false);
+            return (uint32_t)std::min<size_t>(budget / c.smem_per_warp, full / W);
+        };
+        // Wide kernel: two rows of proposals at a time, or one whose columns were loaded a row ahead (see rows_at_a_time). The
+        // first is the faster one by itself (350 jobs: 1.02 to 1.04 in the mean of 16,000 to 50,000 moves, 0.98 to 1.11), but for
+        // columns of four words (0.88 to 0.99) and where the last row of a level stands alone in it (0.93 to 0.97 with three
+        // rows a level, 0.97 with five in batches of eight, 1.00 in batches of four). The second has the smaller work area: it is
+        // taken where a CTA of the first needs more than 196 KB, which leaves 28 KB of an SM's L1 instead of 60 (2368 chains: 1.07 to
+        // 1.6 times faster), or more waves (1.27 to 1.7).
+        const uint64_t level_rows = (a->moves / a->levels + 31) / 32;
+        const bool odd_rows = (level_rows & 1u) && level_rows < (uint64_t)c.rows;
+        uint32_t wcap = share_out(may_load_ahead && (exchange || (c.lin && p->S32 == 4) || odd_rows));   // chains per CTA at most
+        if (may_load_ahead && !c.ahead) {
+            auto waves_of = [&](uint32_t held) { return (a->chains + held * sms - 1) / (held * sms); };
+            const uint32_t waves = wcap ? waves_of(wcap) : 0u;
+            const uint32_t in_cta = waves ? ((a->chains + waves - 1) / waves + sms - 1) / sms : 0u;
+            const bool crowded = !waves || std::min(in_cta, wcap) * c.smem_per_warp + 1024 > ((size_t)196 << 10);
+            if (crowded || waves > 1) wcap = share_out(true);
+            if (!crowded && waves > 1 && waves_of(wcap) == waves) wcap = share_out(false);
         }
-        c.smem_per_warp = fixed_bytes(W, false);
-        if (c.smem_per_warp > budget) return KVP_ERR_RANGE;
+        if (wcap < 1) return KVP_ERR_RANGE;
         c.wpc = W;
-        uint32_t wcap = (uint32_t)(budget / c.smem_per_warp);     // chains per CTA at most
-        if (wcap > full / W) wcap = full / W;
         KVP_CUDA(cudaFuncSetAttribute(kernel_of(c, false, false), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)budget));
         int ctas = 0;
         KVP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ctas, kernel_of(c, false, false), (int)(wcap * W * 32),

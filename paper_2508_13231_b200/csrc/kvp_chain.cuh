@@ -70,26 +70,24 @@ static_assert(sizeof(ChainShared) % 16 == 0, "uint4 slots");
 // Work area of a warp: a ring of listed proposals with their placement windows, the accepted ones that change the schedule
 // in move order, by proposal of the batch what spoiled needs and (when it is evaluated again) what became of it, and the
 // list of those to evaluate again. A batch with more accepted ones than fit goes on where they end once these are applied.
-// Rows of 32 proposals a warp works on side by side: with schedules in global memory and columns of two words two, so that
-// their loads overlap (144 against 168 ms on the largest configuration, four: 148); in shared memory one, for there the
-// instruction cache counts (four rows: 2000 instructions in a batch's path, and a warp waited for the next one a quarter of
-// the time); with births, whose loads come first, one (2.7 against 4.6 ms).
-// Columns of other lengths, whose loads take longer, are loaded a row ahead (load_ahead): while a row is listed and judged the
-// next one's columns are on their way. 32,768 units x 256 steps, 2368 chains x 50,000: 3.17 -> 2.27 ms (two rows ahead: 2.62);
-// 131,072 x 100, 1500 x 50,000: 1.87 -> 1.73; 65,536 x 128, 2368 x 50,000: 2.63 -> 2.49. Not where a column is two words, whose
-// loads stay in flight for less than a single row at a time costs (131,072 x 64, 2368 x 20,000: 0.74 -> 0.82 ms; the largest
-// configuration 132 -> 138), nor with births (131,072 x 1056: 2.71 -> 2.76). The second load takes its address from a select: with a
-// branch around it, since a flip has no second column, the three first lines took 2.30, 1.81 and 2.55 ms.
+// Rows of 32 proposals a warp works on side by side: with schedules in global memory two, so that their loads overlap (144
+// against 168 ms on the largest configuration, four: 148); in shared memory one, for there the instruction cache counts (four
+// rows: 2000 instructions in a batch's path, and a warp waited for the next one a quarter of the time); with births, whose loads
+// come first, one (2.7 against 4.6 ms).
+// Or, in global memory, one row whose columns were loaded while the row before it was listed and judged (AHEAD), which takes half
+// the ring: the choice, and what either measured, is where the shared memory is shared out. Never for columns that are one
+// vector of two words, whose loads stay in flight for less than a single row at a time costs (131,072 units x 64 steps, 2368 chains
+// x 20,000: 0.74 -> 0.82 ms; the largest configuration 132 -> 138), nor with births (131,072 x 1056: 2.71 -> 2.76); always for
+// vectors of four. The second load takes its address from a select: with a branch around it, since a flip has no second column,
+// 32,768 x 256, 2368 x 50,000 took 2.30 ms instead of 2.27.
 constexpr uint32_t kAccepted = 6;
-__host__ __device__ constexpr bool load_ahead(bool psmem, bool grow, int colv) { return !psmem && !grow && colv != 2; }
-__host__ __device__ constexpr int rows_at_a_time(bool psmem, bool grow, int colv) { return !psmem && !grow && colv == 2 ? 2 : 1; }
-__host__ __device__ constexpr uint32_t ring_size(bool psmem, bool grow, int colv) { return rows_at_a_time(psmem, grow, colv) > 1 ? 128u : 64u; }
-__host__ __device__ constexpr uint32_t work4(bool psmem, bool grow, int colv, int rows)   // uint4 slots of it
+constexpr bool load_ahead(bool grow, bool lin, uint32_t S32) { return !grow && !(lin && S32 == 2); }   // whether it may be
+__host__ __device__ constexpr int rows_at_a_time(bool psmem, bool grow, bool ahead) { return psmem || grow || ahead ? 1 : 2; }
+__host__ __device__ constexpr uint32_t ring_size(bool psmem, bool grow, bool ahead) { return rows_at_a_time(psmem, grow, ahead) > 1 ? 128u : 64u; }
+__host__ __device__ constexpr uint32_t work4(bool psmem, bool grow, bool ahead, int rows)   // uint4 slots of it
 {
-    return ring_size(psmem, grow, colv) * 3 / 2 + 2 * kAccepted + 2 * (uint32_t)rows * 8 + 2 * (uint32_t)rows * 2 + 2;
+    return ring_size(psmem, grow, ahead) * 3 / 2 + 2 * kAccepted + 2 * (uint32_t)rows * 8 + 2 * (uint32_t)rows * 2 + 2;
 }
-// words of a column that come with one vector load (see window_at), else 0
-__host__ __device__ constexpr int column_vector(bool psmem, bool lin, uint32_t S32) { return !psmem && lin && (S32 == 2 || S32 == 4) ? (int)S32 : 0; }
 constexpr uint32_t kSame = 1u, kInf = 2u;                 // proposal states: changes nothing (accepted); infeasible
 
 // Byte offsets of the parts of a chain's shared memory. They are kernel parameters, so that a chain's state costs its
@@ -110,17 +108,17 @@ inline ChainLayout chain_layout(uint32_t S, uint32_t S32, bool grow, bool psmem,
     return l;
 }
 // bytes of a chain of W warps, without a schedule in shared memory
-inline size_t chain_bytes(uint32_t S, uint32_t S32, bool grow, bool psmem, bool lin, uint32_t cow4, uint32_t W, int rows)
+inline size_t chain_bytes(uint32_t S, uint32_t S32, bool grow, bool psmem, bool lin, uint32_t cow4, uint32_t W, int rows, bool ahead)
 {
-    return chain_layout(S, S32, grow, psmem, lin, cow4).work + (size_t)W * work4(psmem, grow, column_vector(psmem, lin, S32), rows) * 16;
+    return chain_layout(S, S32, grow, psmem, lin, cow4).work + (size_t)W * work4(psmem, grow, ahead, rows) * 16;
 }
 
 extern __shared__ char chain_smem[];
 
-template <bool PSMEM, bool GROW, bool LIN, int COLV, int R>
+template <bool PSMEM, bool GROW, bool LIN, int COLV, int R, bool AHEAD>
 struct Chain {
     using Occ = typename std::conditional<PSMEM, uint16_t, uint32_t>::type;   // PSMEM: fewer than 2^16 units
-    static constexpr uint32_t kRing = ring_size(PSMEM, GROW, COLV), kBatch = 32 * R;
+    static constexpr uint32_t kRing = ring_size(PSMEM, GROW, AHEAD), kBatch = 32 * R;
     const ChainParams& prm;
     uint32_t cb, wb, pb;         // byte offsets in shared memory: the chain's state, the warp's work area, PSMEM: the schedule
     uint32_t* slice;             // not PSMEM: the chain's slice of global scratch
@@ -285,8 +283,8 @@ struct EvalCtx {
 };
 
 // Cost change of the step at window bit k, step t.
-template <bool PSMEM, bool GROW, bool LIN, int COLV, int R>
-__device__ __forceinline__ int step_change(const Chain<PSMEM, GROW, LIN, COLV, R>& c, const Effect& e, uint32_t Wu, uint32_t Wv, uint32_t k,
+template <bool PSMEM, bool GROW, bool LIN, int COLV, int R, bool AHEAD>
+__device__ __forceinline__ int step_change(const Chain<PSMEM, GROW, LIN, COLV, R, AHEAD>& c, const Effect& e, uint32_t Wu, uint32_t Wv, uint32_t k,
                                            uint32_t t)
 {
     const ChainParams& prm = c.prm;
@@ -307,8 +305,8 @@ __device__ __forceinline__ int step_change(const Chain<PSMEM, GROW, LIN, COLV, R
 
 // Steps 3 and 4 for up to 32 listed proposals, from ring position `head` on, one per lane. The accepted ones go to
 // c.acc() from `kept` on; where there is no room for all of them, `late` becomes the id of the first that found none.
-template <bool PSMEM, bool GROW, bool LIN, int COLV, int R>
-__device__ __forceinline__ void judge(const Chain<PSMEM, GROW, LIN, COLV, R>& c, EvalCtx& x, uint32_t head, uint32_t count, uint32_t lane,
+template <bool PSMEM, bool GROW, bool LIN, int COLV, int R, bool AHEAD>
+__device__ __forceinline__ void judge(const Chain<PSMEM, GROW, LIN, COLV, R, AHEAD>& c, EvalCtx& x, uint32_t head, uint32_t count, uint32_t lane,
                                       uint32_t& kept, uint32_t& late)
 {
     const ChainParams& prm = c.prm;
@@ -438,14 +436,13 @@ __device__ __forceinline__ uint32_t cut(const typename Words<COLV>::type q, cons
 // same and inf of a fresh batch, into c.state() otherwise) and judges the rest. The accepted ones that change the schedule
 // are left in c.acc() in move order (`kept` of them). Returns the id from which on nothing was evaluated (kNone:
 // everything was). One copy of this code for every use keeps the path through a batch short.
-template <bool PSMEM, bool GROW, bool LIN, int COLV, int R>
-__device__ __forceinline__ uint32_t evaluate(const Chain<PSMEM, GROW, LIN, COLV, R>& c, EvalCtx& x, uint64_t m, uint32_t chain, bool fresh,
+template <bool PSMEM, bool GROW, bool LIN, int COLV, int R, bool AHEAD>
+__device__ __forceinline__ uint32_t evaluate(const Chain<PSMEM, GROW, LIN, COLV, R, AHEAD>& c, EvalCtx& x, uint64_t m, uint32_t chain, bool fresh,
                                              uint32_t count, uint32_t lane, uint32_t& kept, uint32_t& same, uint32_t& inf)
 {
     const ChainParams& prm = c.prm;
     const uint32_t S = prm.S;
-    constexpr int UNR = rows_at_a_time(PSMEM, GROW, COLV);
-    constexpr bool kAhead = load_ahead(PSMEM, GROW, COLV);
+    constexpr int UNR = rows_at_a_time(PSMEM, GROW, AHEAD);
     uint32_t head = 0, listed = 0, late = kNone;
     kept = 0;
     auto id_of = [&](uint32_t i) { return fresh ? i : (uint32_t)c.again()[i < count ? i : 0u]; };
@@ -457,7 +454,7 @@ __device__ __forceinline__ uint32_t evaluate(const Chain<PSMEM, GROW, LIN, COLV,
         decode_move(r, prm.p_swap_256, prm.len_choices, S, prm.U, mv);
         pk = mv.pk; u = mv.u; v = mv.v; w = mv.w;
     };
-    // kAhead: the row drawn last, its columns under way while the row before it is listed and judged
+    // AHEAD: the row drawn last, its columns under way while the row before it is listed and judged
     uint32_t npk, nu, nv, nw;
     typename Words<COLV>::type qu, qv;
     auto fetch = [&](uint32_t q) {
@@ -467,11 +464,11 @@ __device__ __forceinline__ uint32_t evaluate(const Chain<PSMEM, GROW, LIN, COLV,
         // the second window: the other unit's placement for a swap, the full-step bitmap for a flip (one address, no branch)
         qv = words_at<COLV>(npk & 1u ? c.col(nv) : (const uint32_t*)c.full(), wp);
     };
-    if constexpr (kAhead) fetch(0);
+    if constexpr (AHEAD) fetch(0);
 #pragma unroll 1
     for (uint32_t q = 0; q < count; q += 32 * UNR) {
         uint32_t id[UNR], pk[UNR], u[UNR], v[UNR], w[UNR], Wu[UNR], W2[UNR], live[UNR];
-        if constexpr (kAhead) {
+        if constexpr (AHEAD) {
             static_assert(UNR == 1, "one row at a time");
             id[0] = id_of(q + lane); pk[0] = npk; u[0] = nu; v[0] = nv; w[0] = nw; live[0] = 0xFFFFFFFFu;
             const WinPos wp = window_pos(npk >> 8);
@@ -552,8 +549,8 @@ __device__ __forceinline__ uint32_t evaluate(const Chain<PSMEM, GROW, LIN, COLV,
 
 // Apply an accepted proposal: all lanes take part, lane j updates the step of window bit j, lanes 0 and 1 rewrite the
 // words of the schedule and of the two step bitmaps. Returns the steps at which these turned (Applied::bits).
-template <bool PSMEM, bool GROW, bool LIN, int COLV, int R>
-__device__ __forceinline__ uint32_t apply(const Chain<PSMEM, GROW, LIN, COLV, R>& c, uint32_t lane, const uint4 a, const uint4 win)
+template <bool PSMEM, bool GROW, bool LIN, int COLV, int R, bool AHEAD>
+__device__ __forceinline__ uint32_t apply(const Chain<PSMEM, GROW, LIN, COLV, R, AHEAD>& c, uint32_t lane, const uint4 a, const uint4 win)
 {
     const ChainParams& prm = c.prm;
     const uint32_t pk = a.x, u = a.y, v = a.z, s0 = (pk >> 8) & 0x7FFFu, S = prm.S, S32 = prm.S32;
@@ -593,7 +590,7 @@ __device__ __forceinline__ uint32_t apply(const Chain<PSMEM, GROW, LIN, COLV, R>
     uint32_t occ = c.occ()[t];
     const bool was_full = occ == prm.cap;
     occ += ((e.Nu >> j) & 1u) + ((e.Nv >> j) & 1u) - ((win.x >> j) & 1u) - ((win.y >> j) & 1u);
-    if (valid) c.occ()[t] = (typename Chain<PSMEM, GROW, LIN, COLV, R>::Occ)occ;
+    if (valid) c.occ()[t] = (typename Chain<PSMEM, GROW, LIN, COLV, R, AHEAD>::Occ)occ;
     uint32_t F = __ballot_sync(0xFFFFFFFFu, valid && occ == prm.cap), T = __ballot_sync(0xFFFFFFFFu, valid && lead);
     uint32_t O = 0u, I = 0u;
     if (!LIN) {
@@ -648,8 +645,8 @@ __device__ __forceinline__ uint32_t first_of(uint32_t rows, uint32_t lane)
 // This lane's proposals whose evaluation an applied move spoils. The move rewrote steps s0 .. s0 + len, a proposal reads
 // steps s0 - 1 .. s0 + len. Where the two meet, what a proposal came to depends on its units' placement, on the two step
 // bitmaps and, if its steps were looked at one by one, on their th and te; on the bitmaps not if it changes nothing.
-template <bool PSMEM, bool GROW, bool LIN, int COLV, int R>
-__device__ __forceinline__ uint32_t spoiled(const Chain<PSMEM, GROW, LIN, COLV, R>& c, const Applied g, uint32_t same, uint32_t lane)
+template <bool PSMEM, bool GROW, bool LIN, int COLV, int R, bool AHEAD>
+__device__ __forceinline__ uint32_t spoiled(const Chain<PSMEM, GROW, LIN, COLV, R, AHEAD>& c, const Applied g, uint32_t same, uint32_t lane)
 {
     const uint32_t s0b = g.steps & 0xFFFFu, endb = g.steps >> 16, first = g.bits & 0xFFFFu, last = g.bits >> 16;
     const uint32_t bu = g.units & 0xFFFFu, bv = g.units >> 16;
@@ -744,7 +741,7 @@ __device__ __forceinline__ void record(const ChainParams& prm, ChainShared* sc, 
 // ASMEM (only with PSMEM): the access bitmap, which every chain of the CTA reads, is staged in shared memory.
 // COLV (only without PSMEM): 2 or 4 when every column has exactly that many words, else 0 (see window_at).
 // A CTA has blockDim / 32 / W chains of W warps each (W = prm.warps, a power of two).
-template <bool PSMEM, bool GROW, bool ASMEM, bool LIN, int COLV, int R>
+template <bool PSMEM, bool GROW, bool ASMEM, bool LIN, int COLV, int R, bool AHEAD>
 __global__ void __launch_bounds__(512, 1)
 wide_chain_kernel(const __grid_constant__ ChainParams prm)
 {
@@ -758,8 +755,8 @@ wide_chain_kernel(const __grid_constant__ ChainParams prm)
     const uint32_t S = prm.S, S32 = prm.S32, U = prm.U;
     const size_t pwords = (size_t)U * S32;
     const uint32_t cow_words = PSMEM ? 0u : prm.cow_slots4 * 4;
-    const uint32_t stride = prm.lay.work + W * work4(PSMEM, GROW, COLV, R) * 16;       // bytes of a chain
-    Chain<PSMEM, GROW, LIN, COLV, R> c{prm, cic * stride, cic * stride + prm.lay.work + sub * work4(PSMEM, GROW, COLV, R) * 16,
+    const uint32_t stride = prm.lay.work + W * work4(PSMEM, GROW, AHEAD, R) * 16;       // bytes of a chain
+    Chain<PSMEM, GROW, LIN, COLV, R, AHEAD> c{prm, cic * stride, cic * stride + prm.lay.work + sub * work4(PSMEM, GROW, AHEAD, R) * 16,
                                        cpb * stride + cic * U * S32 * 4, PSMEM ? nullptr : prm.ws + (size_t)slot * pwords};
     ChainShared* const sc = c.sc();
     EvalCtx x;
@@ -785,7 +782,7 @@ wide_chain_kernel(const __grid_constant__ ChainParams prm)
                 if (LIN) c.tt()[t] = make_int2(th, base + ext);
                 else c.tm()[t] = make_int4(th, base, (int)n.y, (int)n.z);
                 if (GROW && !LIN) c.hb()[t] = hb;
-                c.occ()[t] = (typename Chain<PSMEM, GROW, LIN, COLV, R>::Occ)n.w;
+                c.occ()[t] = (typename Chain<PSMEM, GROW, LIN, COLV, R, AHEAD>::Occ)n.w;
             }
             const uint32_t F = __ballot_sync(0xFFFFFFFFu, t < S && n.w == prm.cap);
             const uint32_t T = __ballot_sync(0xFFFFFFFFu, t < S && base + ext >= th);

@@ -180,6 +180,47 @@ def test_choice_of_warps_in_shared_memory(kvp, oracle, U, S, cap, chains, warps)
         assert out["per_chain"][c].astuple() == want[0].astuple(), c
 
 
+@pytest.mark.parametrize("U,S,link,warps,chains,moves,ahead", [
+    (10001, 90, 900, 3, 5, 640, 1), (10001, 90, 900, 3, 5, 512, 0), (10001, 90, 900, 3, 5, 1152, 0),       # rows of a level: 5, 4, 9
+    (10001, 90, 900, 18, 5, 384, 1), (10001, 90, 900, 18, 5, 640, 0), (10001, 90, 500, 3, 5, 384, 1), (10001, 90, 500, 3, 5, 640, 0),
+    (30011, 32, 900, 3, 5, 40000, 0), (15004, 64, 500, 18, 5, 512, 0),
+    (8003, 128, 900, 3, 5, 40000, 1), (8003, 128, 900, 18, 5, 512, 1), (8003, 128, 500, 18, 5, 512, 0),    # vectors of four words
+    (15004, 64, 900, 3, 5, 384, 0), (15004, 64, 900, 18, 5, 384, 0),                                       # of two
+    (20000, 1400, 900, 18, 1184, 256, 1), (20000, 1400, 900, 18, 740, 256, 0),                             # over and under 196 KB
+    (4096, 512, 500, 3, 2368, 256, 1), (65536, 512, 500, 3, 2368, 256, 0)])                                # one wave for two, two for two
+def test_choice_of_columns_ahead(kvp, oracle, hooks, U, S, link, warps, chains, moves, ahead):
+    """Both sides of the lines between two rows of proposals at a time and one whose columns were loaded a row ahead."""
+    hooks(warps_per_chain=warps)
+    A = wl.random_access(U, S, 0.1, seed=U + S)
+    g, o = both_problems(kvp, oracle, U, 8192, S, A, U // 6, (8000 * GB, link * GB, 900 * GB))
+    kw = dict(chains=chains, moves=moves, seed=3, levels=4, p0=1e-3)
+    out = g.anneal(g.make_params(**kw), want_per_chain=True)
+    st = out["stats"]
+    assert (st.wide_kernel, st.warps_per_chain, st.shared_schedules) == (1, _warps(warps), 0)
+    if chains < 148 or torch.cuda.get_device_properties(0).multi_processor_count == 148:
+        assert st.columns_ahead == ahead
+    op = o.make_params(**kw)
+    for c in sorted({0, 1, chains // 2, chains - 1}):
+        want, _, _ = o.anneal_chains(op, c, 1)
+        assert out["per_chain"][c].astuple() == want[0].astuple(), c
+
+
+@pytest.mark.parametrize("link", [900, 500])
+@pytest.mark.parametrize("warps", [3, 18])
+def test_exchange_with_columns_ahead(kvp, oracle, hooks, warps, link):
+    """Replica exchange in global memory on the wide kernel, which loads columns ahead whatever the job."""
+    hooks(warps_per_chain=warps)
+    U, S = 10001, 90
+    A = wl.random_access(U, S, 0.2, seed=2)
+    g, o = both_problems(kvp, oracle, U, 8192, S, A, 1000, (8000 * GB, link * GB, 900 * GB))
+    kw = dict(chains=20, moves=701, seed=9, levels=5, p0=0.5, alpha=0.7)
+    out = g.anneal_exchange(g.make_params(**kw), 5, 100)
+    ref = o.anneal_exchange(o.make_params(**kw), 5, 100, want_best=True)
+    assert (out["stats"].columns_ahead, out["stats"].warps_per_chain) == (1, _warps(warps))
+    assert [r.astuple() for r in out["per_chain"]] == [r.astuple() for r in ref["per_chain"]]
+    assert np.array_equal(to_np(out["best_schedule"]), ref["best_schedule"])
+
+
 @pytest.mark.parametrize("scale", [1, 2 ** 10, 2 ** 20])
 def test_accept_table_rows(kvp, oracle, scale):
     """Rows built as geometric sequences against exp() for every entry, at temperatures around powers of two."""
