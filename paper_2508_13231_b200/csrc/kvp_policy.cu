@@ -392,8 +392,10 @@ struct PolicyPairs {
     uint16_t window[kPairsPerLaunch], permille[kPairsPerLaunch];
 };
 
-template <int WPL, bool MULTI>
-__global__ void __launch_bounds__(MULTI ? 32 * kPolicyMaxWarps : 32)
+// DENSE: with four words to a thread, 128 registers, so that an SM holds 16 warps and not the 12 of the 139 it would take. What is
+// spilled costs 3 to 6% of a step.
+template <int WPL, bool MULTI, bool DENSE = false>
+__global__ void __launch_bounds__(MULTI ? 32 * kPolicyMaxWarps : 32, DENSE ? 2 : 0)
 lookahead_kernel(const uint32_t* __restrict__ A, const uint32_t* __restrict__ row0, uint32_t S, uint32_t W32, uint32_t cap,
                  uint32_t n_ratio, const __grid_constant__ PolicyPairs pairs, uint32_t* __restrict__ out,
                  const StepC* __restrict__ stepc, CostK K, uint64_t* __restrict__ totals)
@@ -746,6 +748,34 @@ using namespace kvp;
         KVP_CUDA(cudaGetLastError());                                                                           \
     } while (0)
 
+namespace {
+
+// The look-ahead policies of `grid` CTAs (see lookahead_kernel). Above 8192 units the dense form where it takes fewer waves: the
+// 704 of a 64 x 11 grid on 32,768 units x 256 steps 2.26 -> 1.73 ms, the 352 of 32 x 11 1.33 -> 1.11; the other one elsewhere (88 of
+// 8 x 11: 0.65 against 0.67).
+template <typename... Args>
+int launch_lookahead(uint32_t words, uint32_t grid, cudaStream_t st, const Args&... args)
+{
+    if (words > 32 * kPolicyMaxWarps) {
+        const uint32_t threads = (words + 127) / 128 * 32;
+        int dev = 0, sms = 0, ctas = 0, dense = 0;
+        KVP_CUDA(cudaGetDevice(&dev));
+        KVP_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+        KVP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ctas, lookahead_kernel<4, true>, threads, 0));
+        KVP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&dense, lookahead_kernel<4, true, true>, threads, 0));
+        auto waves = [&](int held) { return held > 0 ? (grid - 1) / (uint32_t)(held * sms) : 0xFFFFFFFFu; };
+        if (waves(dense) < waves(ctas)) {
+            lookahead_kernel<4, true, true><<<grid, threads, 0, st>>>(args...);
+            KVP_CUDA(cudaGetLastError());
+            return KVP_OK;
+        }
+    }
+    KVP_POLICY(lookahead_kernel, words, grid, args...);
+    return KVP_OK;
+}
+
+}  // namespace
+
 extern "C" int kvp_policy_reactive(kvp_problem* p, uint32_t init_mode, uint32_t* schedule, void* stream)
 {
     if (!p || !schedule || init_mode > KVP_INIT_STATIC_FREQ || p->dL) return KVP_ERR_ARG;   // fixed populations only
@@ -800,11 +830,11 @@ extern "C" int kvp_policy_lookahead(kvp_problem* p, uint32_t init_mode, const ui
     PolicyPairs pairs;
     uint32_t used = 0;
     auto flush = [&]() -> int {
-        if (used)
-            KVP_POLICY(lookahead_kernel, p->W32, used, p->dA, row, p->S, p->W32, p->cap, 0u, pairs, schedules, p->d_stepc, p->K,
-                       (uint64_t*)nullptr);
+        const uint32_t n_pairs = used;
         used = 0;
-        return KVP_OK;
+        return n_pairs ? launch_lookahead(p->W32, n_pairs, st, p->dA, row, p->S, p->W32, p->cap, 0u, pairs, schedules, p->d_stepc, p->K,
+                                          (uint64_t*)nullptr)
+                       : KVP_OK;
     };
     int rc;
     for (uint32_t i = 0; i < n; ++i) {
@@ -836,10 +866,9 @@ extern "C" int kvp_wr_grid(kvp_problem* p, uint32_t init_mode, uint32_t w_max, u
     p->last_stream = st;
     // every grid point is simulated and scored by one CTA; no schedule is written
     const PolicyPairs none = {};
-    KVP_POLICY(lookahead_kernel, p->W32, w_max * n_ratio, p->dA,
-               init_mode == KVP_INIT_STATIC_FREQ ? p->d_row_freq : (const uint32_t*)nullptr, p->S, p->W32, p->cap, n_ratio, none,
-               (uint32_t*)nullptr, p->d_stepc, p->K, table);
-    return KVP_OK;
+    return launch_lookahead(p->W32, w_max * n_ratio, st, p->dA,
+                            init_mode == KVP_INIT_STATIC_FREQ ? p->d_row_freq : (const uint32_t*)nullptr, p->S, p->W32, p->cap, n_ratio,
+                            none, (uint32_t*)nullptr, p->d_stepc, p->K, table);
 }
 
 extern "C" int kvp_wr_anneal(const uint64_t* table, uint32_t w_max, uint32_t n_ratio, const kvp_wr_params* wp,

@@ -141,6 +141,8 @@ def test_largest_populations(kvp, oracle, U):
             assert np.array_equal(got[i], oracle.policy_lookahead(o, w, r)), (cap, w, r)
         assert np.array_equal(to_np(g.policy_reactive()), oracle.policy_reactive(o)), cap
         assert np.array_equal(u64(g.wr_grid(4, 3)), oracle.wr_grid(o, 4, 3)), cap
+        if cap == U // 3:                                # more CTAs than fit at a time: the dense form
+            assert np.array_equal(u64(g.wr_grid(31, 11)), oracle.wr_grid(o, 31, 11))
 
 
 @pytest.mark.parametrize("w_max,n_ratio,top", [(64, 101, 10 ** 6), (5, 2, 3), (20, 11, 2 ** 42), (7, 7, 1)])
