@@ -750,22 +750,29 @@ using namespace kvp;
 
 namespace {
 
-// The look-ahead policies of `grid` CTAs (see lookahead_kernel). Above 8192 units the dense form where it takes fewer waves: the
-// 704 of a 64 x 11 grid on 32,768 units x 256 steps 2.26 -> 1.73 ms, the 352 of 32 x 11 1.33 -> 1.11; the other one elsewhere (88 of
-// 8 x 11: 0.65 against 0.67).
+// The look-ahead policies of `grid` CTAs (see lookahead_kernel), in the form that is the faster one for few CTAs (KVP_POLICY) but
+// where another takes fewer waves of them.
+//  - Up to 8192 units, six to eight warps of a word: two warps of four words, of which an SM holds six CTAs and not three or
+//    four. 8192 units x 200 steps, 64 x 11: 631 -> 508 us (two warps in every case, before: 605); 45 x 11 512 -> 429. With five
+//    warps of a word it takes longer (5000 x 166, 55 x 11: 338 -> 394).
+//  - Above, the dense form of four words: 64 x 11 on 32,768 x 256 2.26 -> 1.73 ms, 32 x 11 1.33 -> 1.11; otherwise the other one
+//    (8 x 11: 0.65 against 0.67).
 template <typename... Args>
 int launch_lookahead(uint32_t words, uint32_t grid, cudaStream_t st, const Args&... args)
 {
-    if (words > 32 * kPolicyMaxWarps) {
-        const uint32_t threads = (words + 127) / 128 * 32;
-        int dev = 0, sms = 0, ctas = 0, dense = 0;
+    if (words > 160 && grid > 1) {
+        const bool one = words <= 32 * kPolicyMaxWarps;
+        const uint32_t t4 = (words + 127) / 128 * 32;
+        const auto usual = one ? &lookahead_kernel<1, true> : &lookahead_kernel<4, true>;
+        const auto other = one ? &lookahead_kernel<4, true> : &lookahead_kernel<4, true, true>;
+        int dev = 0, sms = 0, n_usual = 0, n_other = 0;
         KVP_CUDA(cudaGetDevice(&dev));
         KVP_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-        KVP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ctas, lookahead_kernel<4, true>, threads, 0));
-        KVP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&dense, lookahead_kernel<4, true, true>, threads, 0));
+        KVP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n_usual, usual, one ? (words + 31) / 32 * 32 : t4, 0));
+        KVP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n_other, other, t4, 0));
         auto waves = [&](int held) { return held > 0 ? (grid - 1) / (uint32_t)(held * sms) : 0xFFFFFFFFu; };
-        if (waves(dense) < waves(ctas)) {
-            lookahead_kernel<4, true, true><<<grid, threads, 0, st>>>(args...);
+        if (waves(n_other) < waves(n_usual)) {
+            other<<<grid, t4, 0, st>>>(args...);
             KVP_CUDA(cudaGetLastError());
             return KVP_OK;
         }
