@@ -151,24 +151,32 @@ __device__ __forceinline__ WinPos window_pos(uint32_t s0)
 // scattered loads. (Every column then starts on an 8- or 16-byte boundary; the arrays themselves are 16-byte
 // aligned.) COLV = 0: columns of any length, the two words they need. The choice is made at compile time: a test of
 // S32 around every load breaks up the straight-line block in which all loads of a batch are issued, and was 1.5x slower.
+template <int COLV>
+struct Words { using type = uint2; };
+template <>
+struct Words<4> { using type = uint4; };
 template <int COLV, typename Ptr>
-__device__ __forceinline__ uint32_t window_at(Ptr col, const WinPos p)
+__device__ __forceinline__ typename Words<COLV>::type words_at(Ptr col, const WinPos p)
+{
+    typename Words<COLV>::type x;
+    if constexpr (COLV == 0) { x.x = col[p.w]; x.y = col[p.w + 1]; }
+    else x = *reinterpret_cast<const typename Words<COLV>::type*>(col);
+    return x;
+}
+template <int COLV>
+__device__ __forceinline__ uint32_t cut(const typename Words<COLV>::type q, const WinPos p)
 {
     uint32_t lo, hi;
-    if (COLV == 2) {
-        const uint2 q = *reinterpret_cast<const uint2*>(col);
-        lo = p.w ? q.y : q.x;
-        hi = q.y;
-    } else if (COLV == 4) {
-        const uint4 q = *reinterpret_cast<const uint4*>(col);
+    if constexpr (COLV == 0) { lo = q.x; hi = q.y; }
+    else if constexpr (COLV == 2) { lo = p.w ? q.y : q.x; hi = q.y; }
+    else {
         lo = p.w == 0 ? q.x : p.w == 1 ? q.y : p.w == 2 ? q.z : q.w;
         hi = p.w == 0 ? q.y : p.w == 1 ? q.z : q.w;
-    } else {
-        lo = col[p.w];
-        hi = col[p.w + 1];
     }
     return p.first ? ((lo << 1) | (lo & 1u)) : __funnelshift_r(lo, hi, p.sh);
 }
+template <int COLV, typename Ptr>
+__device__ __forceinline__ uint32_t window_at(Ptr col, const WinPos p) { return cut<COLV>(words_at<COLV>(col, p), p); }
 
 // born: window bit of the step in which u (low byte) and v (next byte) are written, 0 = not among bits 1..31
 struct Windows { uint32_t Wu, Wv, Nu, Nv, Au, Av, s0, born; };

@@ -405,32 +405,6 @@ __device__ __forceinline__ void judge(const Chain<PSMEM, GROW, LIN, COLV, R, AHE
     __syncwarp();
 }
 
-// the words of a column that a window is cut from (see window_at)
-template <int COLV>
-struct Words { using type = uint2; };
-template <>
-struct Words<4> { using type = uint4; };
-template <int COLV, typename Ptr>
-__device__ __forceinline__ typename Words<COLV>::type words_at(Ptr col, const WinPos p)
-{
-    typename Words<COLV>::type x;
-    if constexpr (COLV == 0) { x.x = col[p.w]; x.y = col[p.w + 1]; }
-    else x = *reinterpret_cast<const typename Words<COLV>::type*>(col);
-    return x;
-}
-template <int COLV>
-__device__ __forceinline__ uint32_t cut(const typename Words<COLV>::type q, const WinPos p)
-{
-    uint32_t lo, hi;
-    if constexpr (COLV == 0) { lo = q.x; hi = q.y; }
-    else if constexpr (COLV == 2) { lo = p.w ? q.y : q.x; hi = q.y; }
-    else {
-        lo = p.w == 0 ? q.x : p.w == 1 ? q.y : p.w == 2 ? q.z : q.w;
-        hi = p.w == 0 ? q.y : p.w == 1 ? q.z : q.w;
-    }
-    return p.first ? ((lo << 1) | (lo & 1u)) : __funnelshift_r(lo, hi, p.sh);
-}
-
 // Evaluation of `count` proposals of the batch that starts at move m, against the current state: all of them from the
 // first on (fresh), or those listed in c.again(). Draws them, settles what the placement bits settle (into the row masks
 // same and inf of a fresh batch, into c.state() otherwise) and judges the rest. The accepted ones that change the schedule
@@ -478,14 +452,8 @@ __device__ __forceinline__ uint32_t evaluate(const Chain<PSMEM, GROW, LIN, COLV,
         } else {
 #pragma unroll
             for (int j = 0; j < UNR; ++j) {
-                const uint32_t i = q + 32u * j + lane;
-                id[j] = fresh ? i : c.again()[i < count ? i : 0u];
-                uint32_t r[4];
-                const uint64_t mine = m + id[j];
-                philox4x32_10((uint32_t)mine, (uint32_t)(mine >> 32), chain, TAG_MOVE, prm.keys, r);
-                LaneMove mv;
-                decode_move(r, prm.p_swap_256, prm.len_choices, S, prm.U, mv);
-                pk[j] = mv.pk; u[j] = mv.u; v[j] = mv.v; w[j] = mv.w;
+                id[j] = id_of(q + 32u * j + lane);
+                draw(id[j], pk[j], u[j], v[j], w[j]);
             }
 #pragma unroll
             for (int j = 0; j < UNR; ++j) {
