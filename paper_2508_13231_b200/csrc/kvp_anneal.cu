@@ -828,9 +828,9 @@ int prepare(kvp_problem* p, const kvp_anneal_params* a, cudaStream_t st, Ctx& c,
     //  - Schedules in shared memory: the narrow kernel (wide: 1.2 to 2.35), from p0 = 0.02 on with one warp per chain (two: 1.09
     //    at 0.03, 1.32 at 0.3), below with three up to 5 per SM (two: 1.12, four: 1.02 up to 4), two up to 8 and one beyond; two
     //    at most on fewer than 64 units and on busy short horizons, where moves meet most often. One on fewer than 64 units and
-    //    steps (two: 1.01 at 1 or 2 chains per SM, 1.05 to 1.10 beyond; 16 x 32, 64 chains x 10,000: 365 us, two 380, three 400),
-    //    and for 7 and 8 chains per SM where the static placement serves less than half of the reads (two: 1.06 over 66 such
-    //    jobs, 0.95 to 1.18; 0.99 where it serves more, over 99). The wide one for quiet jobs of more than 8 chains per SM with next to nothing in HBM, if they
+    //    steps (two: 1.07 in the mean of 16 jobs, 0.97 to 1.22; 16 x 32, 64 chains x 10,000: 330 to 365 us by box, there 365 against two
+    //    380, three 400), and for 7 and 8 chains per SM where the static placement serves less than half of the reads (two: 1.06
+    //    over 66 such jobs, 0.95 to 1.18, on 24 others 1.10, 1.06 to 1.21; 0.99 where it serves more, over 99). The wide one for quiet jobs of more than 8 chains per SM with next to nothing in HBM, if they
     //    are brief or have many units (narrow: 1.1 to 1.2).
     //  - In global memory: the narrow kernel on busy chains, with two warps per chain up to 8 per SM and one beyond (four: 1.77,
     //    wide: 2.1 to 2.2), at warm starts (wide: 1.03 to 1.46) and up to 5 quiet chains per SM, with four warps per chain up to 4,

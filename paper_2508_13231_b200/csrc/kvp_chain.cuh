@@ -24,9 +24,9 @@
 // Several warps may serve one chain: they take its batches in turn and evaluate ahead of each other's commits (see
 // ChainShared). The outcome is that of the sequential chain in every case.
 //
-// What bounds it (ncu): issue slots and the integer pipe, 12.9 warp instructions per move on 2.6M units x 64 steps, 57% of
-// the issue slots busy with 16 warps per SM in a short launch (2368 chains x 6,000 moves). Measured there (8192 chains x 1M
-// moves) 201 -> 133 ms, on a growing cache of 131,072 units (1024 x 100k) 6.3 -> 2.7 ms against the kernels before, which put
+// What bounds it (ncu): issue slots and the integer pipe, 13.0 warp instructions per move, 59% of the issue slots busy with 16
+// warps per SM in a short launch (65,536 units x 64 steps, 2368 chains x 6,000 moves). Measured on 2.6M units x 64 steps, 8192
+// chains x 1M moves: 201 -> 133 ms, on a growing cache of 131,072 units (1024 x 100k) 6.3 -> 2.7 ms against the kernels before, which put
 // the changed steps of every listed proposal through a shared-memory queue of (proposal, step) items, each an evaluation of
 // Eq. 2-4 from four counters, and had no second warp per chain (work area 6.9 KB a warp, now 3.1).
 #pragma once
@@ -171,7 +171,7 @@ struct Chain {
         __syncwarp();
     }
     // Before units u and v (u again for a flip) are rewritten. Growing caches change few units: one after the other, in less
-    // code (3.17 against 3.28 ms on 131,072 units x 1056 steps, 1024 chains x 100,000).
+    // code (131,072 units x 1056 steps, 1024 chains x 100,000, whole call with trace and construction: 3.17 against 3.28 ms).
     __device__ __forceinline__ void own(uint32_t u, uint32_t v, uint32_t lane) const
     {
         if (PSMEM) return;

@@ -14,7 +14,7 @@
 //
 // The kernel before evaluated its 32 proposals in full, ahead of the commits, through a work queue of (proposal, step)
 // items, one move applied per pass. Measured (B200), before and now: 256 units x 512 steps at p0 = 0.8, 1024
-// chains x 100,000 moves: 25.5 -> 13.6 ms; 16 x 32, 64 x 10,000: 0.43 -> 0.33; 16,384 x 256, 1024 x 200,000: 15.7 -> 10.8.
+// chains x 100,000 moves: 25.5 -> 13.6 ms; 16 x 32, 64 x 10,000: 0.43 -> 0.33 to 0.37 by box; 16,384 x 256, 1024 x 200,000: 15.7 -> 10.8.
 // A link slower than the DRAM channels (not LIN), which for a while only the wide kernel served, without a bound: 256 x 512,
 // 1024 x 20,000 at p0 = 0.8: 8.5 -> 3.2 ms (the kernel before 4.4); 16,384 x 256, 1024 x 100,000: 12.3 -> 7.0 (7.3).
 // Growing caches, likewise: 512 units x 132 steps, 256 x 20,000 0.61 -> 0.45 ms (0.69), at p0 = 0.8 5.2 -> 1.7 (3.4);
